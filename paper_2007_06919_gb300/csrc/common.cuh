@@ -11,6 +11,17 @@ enum : uint32_t {
   kStatusDeviceCheck = 5,
 };
 
+// ---------------------------------------------------------------- division by an invariant
+
+// n / d for 0 <= n < 2^31 and 1 <= d < 2^31 with m = div_magic(d): with m = (2^64 - 1 - r) / d,
+// 0 <= r < d, floor((n + 1) m / 2^64) is floor((n + 1) / d - e), 0 < e = (n + 1)(1 + r) / (d 2^64)
+// < 1 / d, and that is floor(n / d). A few multiply-adds, where a division by a kernel argument
+// takes a reciprocal and its corrections.
+inline uint64_t div_magic(int64_t d) { return d > 0 ? ~0ull / (uint64_t)d : 0ull; }
+#ifdef __CUDACC__
+__device__ __forceinline__ int fast_div(int n, uint64_t m) { return (int)__umul64hi((uint64_t)(uint32_t)n + 1u, m); }
+#endif
+
 // ---------------------------------------------------------------- integer epilogue
 
 __device__ __forceinline__ int64_t sat32(int64_t v) {

@@ -18,16 +18,16 @@
 // bytes of each row, so its zero border lies where a byte image's does in the same workspace.
 //
 // Per CTA (one per SM, persistent over tiles of 128 output pixels x BN channels):
-//   warps 0..E-1  epilogue (E = 4 or 8): tcgen05.ld of the accumulator, integer epilogue,
-//              bit-pack, store (warp w reads TMEM lanes 32*(w%4)..; with 8 warps each takes
-//              every other 32-column group)
+//   warps 0..E-1  epilogue (E = 16, or 8 beside activation producers): tcgen05.ld of the
+//              accumulator, integer epilogue, bit-pack, store (warp w reads TMEM lanes
+//              32*(w%4)..; the E / 4 warps of a lane quarter split the columns)
 //   warp  E    TMEM allocation + one thread issuing tcgen05.mma (kind::f8f6f4, M=128)
-//   warp  E+1  one thread loading prepared weights with TMA (cp.async.bulk.tensor, SW128)
-//   warps E+2..E+5 activation producers: im2col gather of packed k-bit codes with cp.async
+//   warp  E+1.. one thread each loading operands with TMA (cp.async.bulk.tensor, SW128)
+//   then 4 warps of activation producers (in-kernel variant): im2col gather of packed k-bit codes
 //              (zero-fill = the padding code 0), unpack to E4M3 bytes, store into the
 //              128B-swizzled K-major operand layout, signal an mbarrier
 // Stages of 128 K-bytes (one 128B swizzle atom) circulate between producers and the MMA
-// thread; two TMEM accumulators let the epilogue of tile i overlap the MMAs of tile i+1.
+// thread; two or four TMEM accumulators let the epilogue of tile i overlap the next MMAs.
 // Every wait is bounded: on expiry the CTA latches kStatusTimeout and unwinds.
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -42,40 +42,25 @@
 namespace aqd {
 namespace tc {
 
-// A tile is kSub M=128 sub-tiles (each one MMA per k-step) sharing every weight stage.
-// The MMA rate is full only for N = 256 (measured: two N=128 MMAs sharing B reach ~72%,
-// one N=128 MMA ~31%), so tiles are 128 x 256 (kSub = 1) for 256-channel layers.
-#ifndef AQD_SUBTILES
-#define AQD_SUBTILES 1
-#endif
-constexpr int kSub = AQD_SUBTILES;
-constexpr int BM = 128 * kSub;     // output pixels per tile
-constexpr int kSubA = 128 * 128;   // bytes of one sub-tile's A operand per stage
-constexpr int kStageA = kSub * kSubA; // bytes of A per stage
+constexpr int BM = 128;            // output pixels per tile and CTA
+constexpr int kStageA = BM * 128;  // bytes of A per stage (128-byte K chunks)
 constexpr int BK = 128;            // K bytes per stage
-#ifndef AQD_EPI_WARPS
-#define AQD_EPI_WARPS 8
-#endif
-constexpr int kEpiWarps = AQD_EPI_WARPS;  // 4 or 8
-static_assert(kEpiWarps == 4 || kEpiWarps == 8, "epilogue warps: 4 or 8");
-constexpr int kEpiThreads = kEpiWarps * 32;
-#ifndef AQD_TMA_WARPS
-#define AQD_TMA_WARPS 1
-#endif
-constexpr int kTmaWarps = AQD_TMA_WARPS;  // weight-loading warps, alternating K chunks
-constexpr int kWarpMma = kEpiWarps;
-constexpr int kWarpTma = kEpiWarps + 1;
-constexpr int kWarpProd0 = kEpiWarps + 1 + kTmaWarps;
-constexpr int kProdWarps = 4 * kSub;  // one thread per tile row
-constexpr int kThreads = (kWarpProd0 + kProdWarps) * 32;
+// Epilogue warps. The epilogue is a chain of dependent integer instructions per output, and a
+// scheduler that holds two such warps issued in a third of its cycles; with four it covers the
+// latencies. The in-kernel-unpack variant keeps 8: its producer warps need the registers.
+__host__ __device__ constexpr int epi_warps(bool flat) { return flat ? 16 : 8; }
+constexpr int kProdWarps = 4;  // one thread per tile row
 // The expanded-activation ("flat") variant has no producer warps: TMA loads both operands,
 // two boxes per K chunk. One issuing thread sustains about one box per ~700 cycles
 // (measured), so that variant spreads the chunks over kTmaWarpsFlat threads.
 constexpr int kTmaWarpsFlat = 3;
-__host__ __device__ constexpr int tma_warps(bool flat) { return flat ? kTmaWarpsFlat : kTmaWarps; }
-__host__ __device__ constexpr int threads_for(bool flat) { return flat ? (kWarpTma + kTmaWarpsFlat) * 32 : kThreads; }
+__host__ __device__ constexpr int tma_warps(bool flat) { return flat ? kTmaWarpsFlat : 1; }
+__host__ __device__ constexpr int threads_for(bool flat) {
+  return (epi_warps(flat) + 1 + tma_warps(flat) + (flat ? 0 : kProdWarps)) * 32;
+}
+constexpr int kMaxBufs = 4;    // TMEM accumulators
 constexpr int kMaxStages = 16;
-constexpr int kStageRow = 36;  // words per row of an int32 staging block (16-byte aligned, conflict-free)
+constexpr int kStageRow = 20;  // words per row of an int32 staging block: 16 and a pad (conflict-free)
 constexpr int kQTab = 256;  // K-chunk table entries (larger K falls back to division)
 
 // One layer of a launch: its per-channel tables, the packed output of each job and the
@@ -107,6 +92,11 @@ struct Params {
   const int8_t* skip_d;
   int32_t upsample, scale_main, has_skip;
   int32_t bn, stages, tmem_cols;
+  int32_t nbuf_log2;   // log2 of the TMEM accumulators (2, or 4 where four fit)
+  // The epilogue warps of a lane quarter split a tile's 32-column groups epi_groups ways; where a
+  // tile has fewer groups than there are warps, epi_sets sets of warps take tiles in turn.
+  int32_t epi_groups, epi_sets;
+  uint64_t div_layer, div_nt;  // fast_div of layer_tiles and n_tiles
   int32_t acc_small;  // |acc| < 2^22 guaranteed by K * max|x| * max|w|
   int32_t cin_chunks; // cin / 128 (flat path)
   int32_t dp_tiles;   // tiles [0, dp_tiles) are bn wide; later ones are the two bn/2 halves
@@ -136,7 +126,7 @@ struct Params {
   uint32_t dep_target;
 };
 
-static_assert(kSubA == kMmaM * BK, "one sub-tile is one M=128 MMA operand");
+static_assert(BM == kMmaM, "a CTA's tile rows are one M=128 MMA operand");
 
 // ---------------------------------------------------------------- tile bookkeeping
 
@@ -155,7 +145,7 @@ struct FlatTile {
 };
 __device__ __forceinline__ FlatTile flat_tile(const ConvJobDev& jb, int mt, int rows = 128) {
   FlatTile f;
-  f.img = mt / jb.tpi;
+  f.img = fast_div(mt, jb.div_img);
   f.v0 = (mt - f.img * jb.tpi) * rows;
   return f;
 }
@@ -165,7 +155,7 @@ __device__ __forceinline__ FlatTile flat_tile(const ConvJobDev& jb, int mt, int 
 template <int kTileRows>
 __device__ __forceinline__ bool wait_dep_tiles(const Params& p, int l, int j, int mt, volatile int* abort_flag) {
   const ConvJobDev& jb = p.jobs[j];
-  const int img = mt / jb.tpi, m_in = mt - img * jb.tpi;
+  const int img = fast_div(mt, jb.div_img), m_in = mt - img * jb.tpi;
   const int K = 1 + jb.wp / kTileRows;
   const int lo = m_in - K < 0 ? 0 : m_in - K;
   const int hi = m_in + K > jb.tpi - 1 ? jb.tpi - 1 : m_in + K;
@@ -178,7 +168,7 @@ __device__ __forceinline__ bool wait_dep_tiles(const Params& p, int l, int j, in
 // Global tile t -> (job, M tile, channel range). Tiles past dp_tiles split the remaining
 // full tiles into two halves of N, so the last, partial wave covers more SMs.
 __device__ __forceinline__ TileInfo tile_info(const Params& p, int t) {
-  const int layer = p.nlayers > 1 ? t / p.layer_tiles : 0;
+  const int layer = p.nlayers > 1 ? fast_div(t, p.div_layer) : 0;
   t -= layer * p.layer_tiles;
   int half = -1;
   if (t >= p.dp_tiles) {
@@ -193,7 +183,7 @@ __device__ __forceinline__ TileInfo tile_info(const Params& p, int t) {
   TileInfo ti;
   ti.layer = layer;
   ti.job = j;
-  ti.mt = local / p.n_tiles;
+  ti.mt = fast_div(local, p.div_nt);
   const int nt = local - ti.mt * p.n_tiles;
   ti.bn = half < 0 ? p.bn : p.bn / 2;
   ti.brow = nt * p.bn + (half > 0 ? p.bn / 2 : 0);
@@ -204,235 +194,191 @@ __device__ __forceinline__ TileInfo tile_info(const Params& p, int t) {
   return ti;
 }
 
-// ---------------------------------------------------------------- epilogue, general case
+// ---------------------------------------------------------------- epilogue
 
-// The skip values of one row's 32-channel group (Eq. 7's second operand), loaded and
-// unpacked per skip width into registers: every index is static, nothing goes through
-// local memory. Channels past cout read 0.
-__device__ __forceinline__ void load_skip_group(const Params& p, const uint8_t* srow, int ch0, int ncols,
-                                                int32_t (&sk)[32]) {
-#pragma unroll
-  for (int i = 0; i < 32; ++i) sk[i] = 0;
-  {
-    const int sb = p.skip_bits;
-    // a whole group of 32 channels in rows whose size is a multiple of 16 bytes: 16-byte loads
-    // (the tensor base is 16-byte aligned); otherwise element by element
-    const bool whole = ncols == 32 && ch0 + 32 <= p.cout && (p.skip_row_bytes & 15) == 0;
-    if (sb == 32 && whole) {
-      const int4* s4 = reinterpret_cast<const int4*>(reinterpret_cast<const int32_t*>(srow) + ch0);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int4 v = __ldg(s4 + q);
-        sk[4 * q] = v.x; sk[4 * q + 1] = v.y; sk[4 * q + 2] = v.z; sk[4 * q + 3] = v.w;
-      }
-    } else if (sb == 32) {
-      const int32_t* s32 = reinterpret_cast<const int32_t*>(srow) + ch0;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) sk[i] = (i < ncols && ch0 + i < p.cout) ? __ldg(s32 + i) : 0;
-    } else if (sb == 8 && whole) {
-      const uint4* s16 = reinterpret_cast<const uint4*>(srow + ch0);
-      const uint4 a = __ldg(s16), b = __ldg(s16 + 1);
-      const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-#pragma unroll
-      for (int i = 0; i < 32; ++i) sk[i] = (int32_t)((w[i / 4] >> (8 * (i % 4))) & 0xFFu);
-    } else if (sb == 8) {
-      const uint8_t* s8 = srow + ch0;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) sk[i] = (i < ncols && ch0 + i < p.cout) ? (int32_t)__ldg(s8 + i) : 0;
-    } else {
-      // 2/3/4-bit codes: one whole packed group (the layout needs cout % 32 == 0)
-      const uint32_t* g32 = reinterpret_cast<const uint32_t*>(srow + (ch0 >> 5) * group_bytes(sb));
-      uint32_t g[4] = {0u, 0u, 0u, 0u};
-      if (sb == 4) {  // 16-byte groups at 16-byte offsets
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(g32));
-        g[0] = v.x; g[1] = v.y; g[2] = v.z; g[3] = v.w;
-      } else if (sb == 2) {
-        const uint2 v = __ldg(reinterpret_cast<const uint2*>(g32));
-        g[0] = v.x; g[1] = v.y;
-      } else {
-        g[0] = __ldg(g32); g[1] = __ldg(g32 + 1); g[2] = __ldg(g32 + 2);
-      }
-      uint32_t b[8];
-      if (sb == 2) unpack_group_bytes<2>(g, b);
-      else if (sb == 3) unpack_group_bytes<3>(g, b);
-      else unpack_group_bytes<4>(g, b);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) sk[i] = (int32_t)((b[i / 4] >> (8 * (i % 4))) & 0xFFu);
-    }
-  }
-}
-
-// Eq. 6 -> Eq. 7 -> Eq. 2 in int64 for 32 accumulators of one row (any shift, any skip),
-// element by element as the definition states it; the common cases take 32-bit forms.
-// (sc: the FP32 accumulator holds the integer sum / sc: 2^18 on the E4M3 pipe, 4 on the FP4 one)
-template <bool kSkip, bool kIntAcc = false>
-__device__ __forceinline__ void general_group(const Params& p, const uint32_t* v, const EpiChan* ep,
-                                              const uint8_t* srow, int ch0, int ncols, float sc, int32_t (&out)[32]) {
-  int32_t sk[32];
-  if (kSkip) load_skip_group(p, srow, ch0, ncols, sk);
-  else {
-#pragma unroll
-    for (int i = 0; i < 32; ++i) sk[i] = 0;
-  }
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    // v: FP32 accumulators of exact integers x 2^-18, or (kIntAcc) int32 sums already
-    const int64_t acc = kIntAcc ? (int64_t)(int32_t)v[i]
-                                : (int64_t)__float2int_rn(__uint_as_float(v[i]) * sc);
-    const EpiChan ec = ep[i];
-    out[i] = kSkip ? epilogue<true>(acc, sk[i], ec, p.scale_main, p.out_bits)
-                        : epilogue<false>(acc, 0, ec, p.scale_main, p.out_bits);
-  }
-}
-
-// In the 32-bit forms below, Eq. 2's clip to [0, qmax] is __vimin_s32_relu(x, qmax) =
-// max(min(x, qmax), 0), one min.relu instruction instead of a min and a max.
-
-// Skip epilogue in 32-bit arithmetic (Eq. 6, Eq. 7 with the skip rescaled, Eq. 2) when, for
-// every column of the tile, R = 31 + shift >= 33, |bias| <= 2^30 and d >= 8, and the skip
-// holds k-bit codes (s <= 255): then rhu(s * c, d) = (s * c + 2^(d-1)) >> d fits in int32,
-// acc + bias cannot overflow (|acc| < 2^24), and one saturating add gives sat32 of the
-// exact sum; the requant is the same 32-bit form as fast_requant_group.
-// (y may be sk itself: element i is read before it is written)
-__device__ __forceinline__ void fast_skip_group(const uint32_t* v, const EpiChan* ep, const int32_t (&sk)[32],
-                                                int qmax, float sc, int32_t (&y)[32]) {
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const EpiChan c = ep[i];
-    const int32_t acc = __float2int_rn(__uint_as_float(v[i]) * sc);  // exact integer
-    const int64_t sc = (int64_t)sk[i] * (int64_t)c.c;
-    const int32_t st = (int32_t)((sc + (1LL << (c.d - 1))) >> c.d);
-    const int32_t u = add_sat(acc + c.bias, st);
-    const int r = c.r;
-    y[i] = __vimin_s32_relu((__mulhi(u, c.m0) + (1 << (r - 33))) >> (r - 32), qmax);
-  }
-}
-
-// Skip epilogue for an int32 skip (a downsample branch in accumulator units), default
-// direction, when every column has R >= 33, |bias| <= 2^30 and d >= 1: Eq. 7's rescaled skip
-// rhu(s * c, d) is one 64-bit product, add and shift (|s * c| < 2^62); acc + bias fits in
-// int32 (|acc| < 2^24); the sum is saturated to int32 as in Eq. 7's int64 form, and the requant
-// is the 32-bit form of fast_requant_group.
-__device__ __forceinline__ void fast_skip32_group(const uint32_t* v, const EpiChan* ep, const int32_t (&sk)[32],
-                                                  int qmax, float sc, int32_t (&y)[32]) {
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const EpiChan c = ep[i];
-    const int32_t acc = __float2int_rn(__uint_as_float(v[i]) * sc);  // exact integer
-    const int64_t st = ((int64_t)sk[i] * (int64_t)c.c + (1LL << (c.d - 1))) >> c.d;
-    int64_t t = (int64_t)(acc + c.bias) + st;
-    t = t > 2147483647LL ? 2147483647LL : (t < -2147483648LL ? -2147483648LL : t);
-    const int32_t u = (int32_t)t;
-    const int r = c.r;
-    y[i] = __vimin_s32_relu((__mulhi(u, c.m0) + (1 << (r - 33))) >> (r - 32), qmax);
-  }
-}
+// Per-column constants of a tile's level and channel range, in shared memory: the int64 form's
+// (EpiChan), the 32-bit requant's {bias - kMagicBits, M0, 2^(R-33), R-32} and the 32-bit skip
+// rescale's {c, rounding term, shift, 0}.
+struct EpiTab {
+  uint8_t* base;
+  static constexpr size_t kBytes = 256 * (sizeof(EpiChan) + 2 * sizeof(int4));
+  __device__ __forceinline__ EpiChan* gen() const { return reinterpret_cast<EpiChan*>(base); }
+  __device__ __forceinline__ int4* fast() const { return reinterpret_cast<int4*>(base + 256 * sizeof(EpiChan)); }
+  __device__ __forceinline__ int4* skip() const { return fast() + 256; }
+};
+// What the tables of the current tile allow
+enum : int {
+  kFlagReq = 1,   // every R >= 33 and |bias| <= 2^30: the 32-bit requant
+  kFlagBias = 2,  // |bias| <= 2^30
+  kFlagSkip = 4   // the 32-bit skip rescale (skip_const below), with kFlagReq
+};
 
 // 1.5 * 2^23: adding it to an integer-valued float |x| < 2^22 puts x in the low mantissa bits
 constexpr float kMagic = 12582912.0f;
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// Fast requant of 32 accumulators of one row into one packed group (no skip, R >= 33,
-// any bias): u = sat32(acc + bias), y = clamp((mulhi(u, M0) + 2^(R-33)) >> (R-32), 0, 2^k-1).
-template <int kOut>
-__device__ __forceinline__ void fast_requant_group(const uint32_t* v, const EpiChan* ep, int g0, int qmax, float sc,
-                                                   uint32_t gw[8]) {
-#pragma unroll
-  for (int w = 0; w < 8; ++w) gw[w] = 0u;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const EpiChan c = ep[g0 + i];
-    const int32_t acc = __float2int_rn(__uint_as_float(v[i]) * sc);  // exact integer
-    const int32_t u = add_sat(acc, c.bias);
-    const int r = c.r;
-    const uint32_t y = (uint32_t)__vimin_s32_relu((__mulhi(u, c.m0) + (1 << (r - 33))) >> (r - 32), qmax);
-    if constexpr (kOut == 3) {
-      gw[i / 16] |= (y & 3u) << (8 * (i % 4) + 2 * ((i % 16) / 4));
-      gw[2] |= (y >> 2) << (8 * (i % 4) + i / 4);
-    } else {
-      constexpr int q = 32 / kOut;
-      gw[i / q] |= y << (8 * (i % 4) + kOut * ((i % q) / 4));
-    }
-  }
+// The 32-bit requant (every R = 31 + shift >= 33): rhu(u M0, R) = (mulhi(u, M0) + 2^(R-33)) >>
+// (R-32), as the low product word cannot carry into the rounded result; the clip of Eq. 2 is
+// one min.relu (max(min(x, qmax), 0)).
+__device__ __forceinline__ uint32_t requant32(int32_t u, const int4& f, int qmax) {
+  return (uint32_t)__vimin_s32_relu((__mulhi(u, f.y) + f.z) >> f.w, qmax);
 }
 
-// Fastest requant (no skip, R >= 33, |acc| < 2^22, |bias| <= 2^30) of 32 accumulators of one
-// row, straight into 8 byte-words (word j holds channels 4j..4j+3, one code per byte: the
-// layout of the chained byte image, and one step from every packed layout). One FMA turns
-// the accumulator float acc / sc into the int32 acc + 0x4B400000; c.x holds
-// bias - 0x4B400000, so one add gives acc + bias exactly (no int32 overflow under the stated
-// bounds); c.y, c.z, c.w are M0, 2^(R-33) and R-32.
-__device__ __forceinline__ void magic_requant_bytes(const uint32_t* v, const int4* f, int qmax, float sc,
-                                                    uint32_t (&bw)[8]) {
-#pragma unroll
-  for (int j = 0; j < 8; ++j) bw[j] = 0u;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) {
-    const int4 c = f[i];
-    const int32_t u = __float_as_int(__fmaf_rn(__uint_as_float(v[i]), sc, kMagic)) + c.x;
-    const uint32_t y = (uint32_t)__vimin_s32_relu((__mulhi(u, c.y) + c.z) >> c.w, qmax);
-    bw[i / 4] += y << (8 * (i % 4));  // codes < 256: the add is an or
-  }
+// Eq. 7's rescaled skip rhu(s c, d) in 32-bit arithmetic: with s pre-scaled by 2^k so that
+// |s 2^k| < 2^31, rhu(s c, d) = (mulhi(s 2^k, c) + 2^(d+k-33)) >> (d+k-32) for d + k >= 33 (the
+// same identity as the requant's). k = 24 for 2- to 4-bit codes (the code in the top byte of a
+// word: one byte permute), 23 for 8-bit codes, 3 for int32 skips below 2^28 in magnitude
+// (checked per value). A d so large that |s c| < 2^(d-1) for every s gives 0. The sum acc + bias
+// + rescaled skip then stays within int32 (|bias| <= 2^30, |acc| < 2^24, the skip term below
+// 2^29), so Eq. 7 needs no saturation.
+__device__ __forceinline__ int skip_prescale(int skip_bits) { return skip_bits == 32 ? 3 : (skip_bits == 8 ? 23 : 24); }
+__device__ __forceinline__ bool skip_const(int skip_bits, int32_t c, int d, int4& o) {
+  const int r = d + skip_prescale(skip_bits);
+  if (r < 33) return false;
+  // |s c| < 2^(bits + 31) for codes (bits <= 8), 2^59 for int32 skips below 2^28
+  if (d > (skip_bits == 32 ? 59 : skip_bits + 31)) o = make_int4(0, 0, 1, 0);
+  else o = make_int4(c, 1 << (r - 33), r - 32, 0);
+  return true;
 }
-// Byte-words of codes < 2^kBits -> the packed group (the layout of common.cuh: word w of the
-// 2/4/8-bit layout holds its channels 4k..4k+3 in bit field k of every byte; the 3-bit layout
-// is two 2-bit words of the low bits and one word of bit 2, channel i at bit 8 (i%4) + i/4).
-template <int kBits>
-__device__ __forceinline__ void pack_bytewords(const uint32_t (&bw)[8], uint32_t (&gw)[8]) {
-  if constexpr (kBits == 8) {
-#pragma unroll
-    for (int j = 0; j < 8; ++j) gw[j] = bw[j];
-  } else if constexpr (kBits == 4) {
-#pragma unroll
-    for (int w = 0; w < 4; ++w) gw[w] = bw[2 * w] | (bw[2 * w + 1] << 4);
-  } else if constexpr (kBits == 2) {
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      gw[w] = bw[4 * w] | (bw[4 * w + 1] << 2) | (bw[4 * w + 2] << 4) | (bw[4 * w + 3] << 6);
+__device__ __forceinline__ int32_t skip32(int32_t s_scaled, const int4& e) {
+  return (__mulhi(s_scaled, e.x) + e.y) >> e.z;
+}
+
+// 16 codes < 2^bits as byte-words (word j: channels 4j..4j+3, one per byte) -> their place in the
+// packed row (the layout of common.cuh: word w of the 2/4/8-bit layout holds its channels 4k..4k+3
+// in bit field k of every byte; a 3-bit group of 32 channels is two 2-bit words of the low bits
+// and one word of bit 2, channel i at bit 8 (i%4) + i/4). ch: the first channel, a multiple of
+// 16; top: bit 2 of the group's first half (3-bit codes), kept for the second.
+__device__ __forceinline__ void store_codes16(uint8_t* yrow, int ch, const uint32_t (&bw)[4], int bits, uint32_t& top) {
+  if (bits == 4) {
+    *reinterpret_cast<uint2*>(yrow + (ch >> 1)) = make_uint2(bw[0] | (bw[1] << 4), bw[2] | (bw[3] << 4));
+  } else if (bits == 2) {
+    *reinterpret_cast<uint32_t*>(yrow + (ch >> 2)) = bw[0] | (bw[1] << 2) | (bw[2] << 4) | (bw[3] << 6);
+  } else if (bits == 8) {
+    *reinterpret_cast<uint4*>(yrow + ch) = make_uint4(bw[0], bw[1], bw[2], bw[3]);
   } else {
-#pragma unroll
-    for (int w = 0; w < 2; ++w)
-      gw[w] = (bw[4 * w] & 0x03030303u) | ((bw[4 * w + 1] & 0x03030303u) << 2) |
-              ((bw[4 * w + 2] & 0x03030303u) << 4) | ((bw[4 * w + 3] & 0x03030303u) << 6);
+    const int half = (ch >> 4) & 1;
+    uint32_t* g = reinterpret_cast<uint32_t*>(yrow + (ch >> 5) * 12);
+    g[half] = (bw[0] & 0x03030303u) | ((bw[1] & 0x03030303u) << 2) | ((bw[2] & 0x03030303u) << 4) |
+              ((bw[3] & 0x03030303u) << 6);
     uint32_t h = 0u;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) h |= ((bw[j] >> 2) & 0x01010101u) << j;
-    gw[2] = h;
+    for (int j = 0; j < 4; ++j) h |= ((bw[j] >> 2) & 0x01010101u) << j;
+    if (half) g[2] = top | (h << 4);
+    else top = h;
   }
 }
-// Chained output: the 32 codes of one packed group (byte-words bw: channels 4j..4j+3 in word
-// j) at their place in the zero-padded image that the next stride-1 conv (padding out_pad)
-// reads: one byte per code, or, when that conv runs on the FP4 pipe (nib), two codes per byte
-// (channel 2k in the low nibble of byte k) in the first half of the same row.
-__device__ __forceinline__ void chain_store_bw(const Params& p, uint8_t* ws_out, int nib, const ConvJobDev& jb,
-                                               int img, int oh, int ow, int ch0, const uint32_t (&bw)[8]) {
-  const int row = jb.orow_off + (img * jb.ohp + oh + p.out_pad) * jb.owp + ow + p.out_pad;
+// Chained output: the 16 codes at their place in the row of the zero-padded image that the next
+// stride-1 conv reads: one byte per code, or, when that conv runs on the FP4 pipe (nib), two
+// codes per byte (channel 2k in the low nibble of byte k) in the first half of the row.
+__device__ __forceinline__ void store_image16(uint8_t* irow, int ch, const uint32_t (&bw)[4], int nib) {
   if (nib) {
-    uint32_t o[4];
+    // bytes 0 and 2 of t hold the nibble pairs (c0, c1) and (c2, c3) of a byte-word
+    uint32_t t[4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      // bytes 0 and 2 of t hold the nibble pairs (c0, c1) and (c2, c3) of a byte-word
-      const uint32_t t0 = bw[2 * m] | (bw[2 * m] >> 4), t1 = bw[2 * m + 1] | (bw[2 * m + 1] >> 4);
-      o[m] = __byte_perm(t0, t1, 0x6420);
-    }
-    *reinterpret_cast<uint4*>(ws_out + (size_t)row * p.cout + (ch0 >> 1)) = make_uint4(o[0], o[1], o[2], o[3]);
+    for (int j = 0; j < 4; ++j) t[j] = bw[j] | (bw[j] >> 4);
+    *reinterpret_cast<uint2*>(irow + (ch >> 1)) =
+        make_uint2(__byte_perm(t[0], t[1], 0x6420), __byte_perm(t[2], t[3], 0x6420));
   } else {
-    uint4* dst = reinterpret_cast<uint4*>(ws_out + (size_t)row * p.cout + ch0);
-    dst[0] = make_uint4(bw[0], bw[1], bw[2], bw[3]);
-    dst[1] = make_uint4(bw[4], bw[5], bw[6], bw[7]);
+    *reinterpret_cast<uint4*>(irow + ch) = make_uint4(bw[0], bw[1], bw[2], bw[3]);
   }
 }
 
-// The same from a packed group gw of out_bits codes.
-__device__ __forceinline__ void chain_store(const Params& p, uint8_t* ws_out, int nib, const ConvJobDev& jb, int img,
-                                            int oh, int ow, int ch0, const uint32_t gw[8], int out_bits) {
-  uint32_t o[8];
-  switch (out_bits) {
-    case 2: unpack_group_bytes<2>(gw, o); break;
-    case 3: unpack_group_bytes<3>(gw, o); break;
-    default: unpack_group_bytes<4>(gw, o); break;
+// The packed words of 16 skip codes of one row (2- to 4-bit codes: the layout needs cout % 32 ==
+// 0, so they all exist) from channel ch on, and their byte-words.
+__device__ __forceinline__ uint2 load_skip_words(const uint8_t* srow, int ch, int sb, bool ok) {
+  uint2 g = make_uint2(0u, 0u);
+  if (!ok) return g;
+  if (sb == 4) {
+    g = __ldg(reinterpret_cast<const uint2*>(srow + (ch >> 1)));
+  } else if (sb == 2) {
+    g.x = __ldg(reinterpret_cast<const uint32_t*>(srow + (ch >> 2)));
+  } else {
+    const uint32_t* g3 = reinterpret_cast<const uint32_t*>(srow + (ch >> 5) * 12);
+    g = make_uint2(__ldg(g3 + ((ch >> 4) & 1)), __ldg(g3 + 2) >> ((ch >> 2) & 4));
   }
-  chain_store_bw(p, ws_out, nib, jb, img, oh, ow, ch0, o);
+  return g;
+}
+__device__ __forceinline__ void skip_bytewords(const uint2& g, int sb, uint32_t (&b)[4]) {
+  if (sb == 4) {
+    b[0] = g.x & 0x0F0F0F0Fu; b[1] = (g.x >> 4) & 0x0F0F0F0Fu;
+    b[2] = g.y & 0x0F0F0F0Fu; b[3] = (g.y >> 4) & 0x0F0F0F0Fu;
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      b[j] = (g.x >> (2 * j)) & 0x03030303u;
+      if (sb == 3) b[j] |= ((g.y >> j) & 0x01010101u) << 2;
+    }
+  }
+}
+
+// 16 columns of one row in the general form.
+struct GenCols {
+  uint32_t taddr;       // TMEM address of the first column
+  uint32_t taddr_hi;    // split weights: of the w_hi accumulator
+  const EpiChan* ep;    // the columns' constants
+  const uint8_t* srow;  // the skip's row (kSkip)
+  uint8_t* yrow;        // the output's row
+  int ch0, nc, flags;   // first channel, channels that exist
+  bool row_ok;
+};
+
+// Eq. 6 -> Eq. 7 -> Eq. 2 as the definition states them, element by element in int64 (any shift,
+// any skip direction and width, any row size), with the 32-bit requant where the tables allow it
+// and there is no skip (accumulators too large for the common form). Returns the codes as
+// byte-words; int32 outputs and 8-bit rows of no whole groups are stored here. Not inlined: its
+// registers and code stay out of the common forms.
+template <bool kSkip, bool kSplit>
+__device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, float sc) {
+  uint32_t v[16];
+  tmem_ld16(u.taddr, v);
+  tmem_wait_ld();
+  reg_fence16(v);
+  int32_t acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = __float2int_rn(__uint_as_float(v[i]) * sc);
+  if constexpr (kSplit) {
+    tmem_ld16(u.taddr_hi, v);
+    tmem_wait_ld();
+    reg_fence16(v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
+  }
+  if (!u.row_ok) return make_uint4(0u, 0u, 0u, 0u);
+  if (!kSkip && (u.flags & kFlagReq) && p.out_bits != 32) {
+    const int qmax = (1 << p.out_bits) - 1;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const EpiChan c = u.ep[i];
+      acc[i] = i < u.nc ? __vimin_s32_relu((__mulhi(add_sat(acc[i], c.bias), c.m0) + (1 << (c.r - 33))) >> (c.r - 32), qmax) : 0;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      if (i < u.nc) {
+        const int32_t s = kSkip ? read_code(u.srow, u.ch0 + i, p.skip_bits, false) : 0;
+        acc[i] = epilogue<kSkip>(acc[i], s, u.ep[i], p.scale_main, p.out_bits);
+      } else {
+        acc[i] = 0;
+      }
+    }
+  }
+  if (p.out_bits == 32) {
+    int32_t* yr = reinterpret_cast<int32_t*>(u.yrow) + u.ch0;
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < u.nc) yr[i] = acc[i];
+  } else if (p.out_bits == 8 && (p.cout & 31) != 0) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < u.nc) u.yrow[u.ch0 + i] = (uint8_t)acc[i];
+  }
+  uint32_t bw[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    bw[j] = (uint32_t)acc[4 * j] | ((uint32_t)acc[4 * j + 1] << 8) | ((uint32_t)acc[4 * j + 2] << 16) |
+            ((uint32_t)acc[4 * j + 3] << 24);
+  return make_uint4(bw[0], bw[1], bw[2], bw[3]);
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -508,9 +454,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   static_assert(!kFp4 || (kFlat && kBK == BK && !kSplit), "the FP4 pipe reads nibble images in 128-byte chunks");
   // the FP32 accumulator holds the integer sum / kAccSc
   constexpr float kAccSc = kFp4 ? 4.0f : 262144.0f;
-  // bytes of one stage's A operand: kSub sub-tiles of 128 rows x kBK bytes
-  constexpr int kStA = kSub * 128 * kBK;
+  constexpr int kStA = BM * kBK;  // bytes of one stage's A operand
   constexpr int kTma = tma_warps(kFlat);
+  constexpr int kEpiWarps = epi_warps(kFlat);
+  constexpr int kEpiThreads = kEpiWarps * 32;
+  constexpr int kWarpMma = kEpiWarps, kWarpTma = kEpiWarps + 1, kWarpProd0 = kWarpTma + kTma;
   // CTA pair: this CTA's rank; the even CTA issues the MMAs; a tile has 256 rows
   const uint32_t rank = kPair ? cluster_ctarank() : 0u;
   const bool leader = rank == 0;
@@ -522,16 +470,17 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   const uint32_t sbase = smem_u32(smem);
   const uint32_t s_a = sbase;
   const uint32_t s_b = sbase + p.off_b;
-  EpiChan* epi = reinterpret_cast<EpiChan*>(smem + p.off_epi);
+  const EpiTab epi{smem + p.off_epi};
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
-  // barrier slots: full[0..S), empty[0..S), tfull[2], tempty[2], final
+  // barrier slots: full[0..S), empty[0..S), tfull[nbuf], tempty[nbuf], final (kMaxBufs each)
   const int S = p.stages;
   const uint32_t b_full = smem_u32(bars);
   const uint32_t b_empty = b_full + 8 * S;
   const uint32_t b_tfull = b_empty + 8 * S;
-  const uint32_t b_tempty = b_tfull + 16;
-  const uint32_t b_final = b_tempty + 16;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 5);
+  const uint32_t b_tempty = b_tfull + 8 * kMaxBufs;
+  const uint32_t b_final = b_tempty + 8 * kMaxBufs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 2 * kMaxBufs + 1);
+  const uint32_t buf_mask = (1u << p.nbuf_log2) - 1u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32;
@@ -551,9 +500,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       mbar_init(b_full + 8 * s, kFlat ? 1 : kProdWarps + 1);  // per producer warp + TMA
       mbar_init(b_empty + 8 * s, 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < kMaxBufs; ++b) {
       mbar_init(b_tfull + 8 * b, 1);
-      mbar_init(b_tempty + 8 * b, kPair ? 2 * kEpiWarps : kEpiWarps);  // one arrive per epilogue warp
+      mbar_init(b_tempty + 8 * b, (kPair ? 8 : 4) * p.epi_groups);  // one arrive per epilogue warp of a tile
     }
     mbar_init(b_final, 1);
     *abort_flag = 0;
@@ -627,9 +576,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const uint32_t idesc_half =
           kFp4 ? idesc_fp4(BN / 2, kPair ? 2 * kMmaM : kMmaM) : idesc_e4m3(BN / 2, kPair ? 2 * kMmaM : kMmaM);
       const uint32_t sfa = tmem_base + (uint32_t)p.sf_col, sfb = sfa + 16;  // (FP4 only)
-      // descriptors of stage 0, k-step 0; later stages / sub-tiles / k-steps add
+      // descriptors of stage 0, k-step 0; later stages / k-steps add
       // (byte offset >> 4) to the 14-bit start-address field (shared addresses < 2^18)
-      // the descriptors' high words are constant; stages / sub-tiles / k-steps only move the
+      // the descriptors' high words are constant; stages / k-steps only move the
       // 14-bit start-address field in the low word (shared addresses < 2^18, no carry)
       const uint64_t da0 = sdesc_k<kBK>(s_a), db0 = sdesc_k<kBK>(s_b);
       const uint32_t a_lo0 = (uint32_t)da0, b_lo0 = (uint32_t)db0;
@@ -638,13 +587,12 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       bool ok = true;
       bool next_ready = false;  // the stage after the current one is known to be full
       for (int t = first_tile; t < tile_end && ok; t += tile_stride, ++lt) {
-        const uint32_t buf = lt & 1;
-        // (half-width tiles are counted within a layer; a launch of several layers has none)
-        const int t_in_layer = p.nlayers > 1 ? t - (t / p.layer_tiles) * p.layer_tiles : t;
-        const uint32_t idesc = t_in_layer < p.dp_tiles ? idesc_full : idesc_half;
-        if (!mbar_poll(b_tempty + 8 * buf, ((lt >> 1) & 1) ^ 1, abort_flag)) { ok = false; break; }
+        const uint32_t buf = lt & buf_mask;
+        // (a launch of several layers has no half-width tiles)
+        const uint32_t idesc = p.nlayers > 1 || t < p.dp_tiles ? idesc_full : idesc_half;
+        if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d0 = tmem_base + buf * (uint32_t)(kSub * BN);  // sub-tile j at +j*BN
+        const uint32_t d0 = tmem_base + buf * (uint32_t)BN;
         for (int q = 0; q < nk; ++q, ++it) {
           // (operands written by TMA, or by producer threads followed by fence.proxy.async,
           // are ordered for the MMA by the mbarrier phase alone; tcgen05.fence is needed only
@@ -662,18 +610,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             if (kk == kBK / 32 - 1) next_ready = mbar_test(b_full + 8 * s_next, ph_next);
             const uint32_t acc = (q > 0 || kk > 0) ? 1u : 0u;
             const uint64_t db = ((uint64_t)b_hi << 32) | (b_lo + 2 * kk);
-            if constexpr (kPair && kFp4) {
-              mma_fp4_pair(d0, ((uint64_t)a_hi << 32) | (a_lo + 2 * kk), db, idesc, sfa, sfb, acc);
-            } else if constexpr (kPair) {
-              mma_e4m3_pair(d0, ((uint64_t)a_hi << 32) | (a_lo + 2 * kk), db, idesc, acc);
-            } else {
-#pragma unroll
-              for (int j = 0; j < kSub; ++j) {
-                const uint64_t da = ((uint64_t)a_hi << 32) | (a_lo + j * (kSubA >> 4) + 2 * kk);
-                if constexpr (kFp4) mma_fp4(d0 + j * BN, da, db, idesc, sfa, sfb, acc);
-                else mma_e4m3(d0 + j * BN, da, db, idesc, acc);
-              }
-            }
+            const uint64_t da = ((uint64_t)a_hi << 32) | (a_lo + 2 * kk);
+            if constexpr (kPair && kFp4) mma_fp4_pair(d0, da, db, idesc, sfa, sfb, acc);
+            else if constexpr (kPair) mma_e4m3_pair(d0, da, db, idesc, acc);
+            else if constexpr (kFp4) mma_fp4(d0, da, db, idesc, sfa, sfb, acc);
+            else mma_e4m3(d0, da, db, idesc, acc);
           }
           if constexpr (kPair) mma_commit_pair_both(b_empty + 8 * s);
           else mma_commit(b_empty + 8 * s);
@@ -692,7 +633,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     }
   } else if (warp >= kWarpTma && warp < kWarpTma + kTma) {
     // ------------------------------------------------------------ weight loaders (TMA)
-    // One thread of each TMA warp issues every kTmaWarps-th chunk: a thread sustains
+    // One thread of each TMA warp issues every kTma-th chunk: a thread sustains
     // about one tensor copy at a time, so two threads keep two copies in flight.
     const int tw = warp - kWarpTma;
     if (lane == 0) {
@@ -764,9 +705,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     }
   } else if (!kFlat && warp >= kWarpProd0) {
     // ------------------------------------------------------------ activation producers
-    const int row = threadIdx.x - kWarpProd0 * 32;  // 0..255: tile row owned by this thread
-    const int sub = row >> 7, r7 = row & 7;
-    uint8_t* arow = smem + sub * kSubA + (row & 127) * BK;
+    const int row = threadIdx.x - kWarpProd0 * 32;  // tile row owned by this thread
+    const int r7 = row & 7;
+    uint8_t* arow = smem + row * BK;
     int my_tiles = 0;
     for (int t = first_tile; t < tile_end; t += tile_stride) ++my_tiles;
     const int total = my_tiles * nk;
@@ -779,10 +720,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const int m = ti.mt * BM + row;
       rc.valid = m < jb.m_total;
       const int mm = rc.valid ? m : 0;
-      const int hw = jb.ho * jb.wo;
-      const int img = mm / hw;
-      const int rem = mm - img * hw;
-      const int ho = rem / jb.wo, wo = rem - (rem / jb.wo) * jb.wo;
+      const int img = fast_div(mm, jb.div_img);
+      const int rem = mm - img * (jb.ho * jb.wo);
+      const int ho = fast_div(rem, jb.div_row), wo = rem - ho * jb.wo;
       rc.hb = ho * p.stride - p.pad;
       rc.wb = wo * p.stride - p.pad;
       rc.H = jb.h;
@@ -831,15 +771,22 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     if (!ok) fail(abort_flag, p.status);
   } else {
     // ------------------------------------------------------------ epilogue (warps 0..E-1)
-    // Warp w reads TMEM lanes 32*(w%4).. (the hardware lane quarter of its warp index).
-    // Warp group gi = w/4 takes sub-tiles / column groups in turn, so with 8 warps two
-    // warps share each lane quarter.
+    // Warp w reads TMEM lanes 32*(w%4).. (the hardware lane quarter of its warp index), one lane
+    // per output row, in steps of 16 columns. The warps of a quarter split a tile's 32-column groups
+    // into epi_groups ranges; sets of epi_groups warps take tiles in turn (epi_sets > 1: narrow
+    // tiles).
+    //
+    // What bounds it: integer instructions, about 9 per output and lane without a skip and 14 with
+    // one. So everything that does not depend on the column is done once per tile and lane (the
+    // output pixel, by multiply-high divisions, and the row pointers), the rare forms live in a
+    // function of their own, and four warps per scheduler cover the chains' latencies. Against two
+    // warps per scheduler, 25 and 40 instructions per output (divisions per 32 columns, 64-bit
+    // skip arithmetic): the whole detector at batch 8 1987 -> 1687 us, its third stage's entry
+    // block 104 -> 78 us, a 1x1 128->512 conv with a skip on 30,400 pixels 49 -> 36 us.
     const int quarter = warp & 3;
-    const int gi = warp >> 2;
-    constexpr int kGroups = kEpiWarps / 4;
+    const int gset = (warp >> 2) / p.epi_groups, grp = (warp >> 2) - gset * p.epi_groups;
     const int et = threadIdx.x;  // 0 .. kEpiThreads-1
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const int4* epf = reinterpret_cast<const int4*>(epi + 256);  // per-column fast constants
     uint32_t lt = 0;
     bool ok = true;
     const int out_bits = p.out_bits;
@@ -847,8 +794,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     // the per-column constant tables of the last tile's level and channel range: rebuilt only
     // when a tile needs others (tiles of one job and N range keep them), so most tiles start
     // without table loads or barriers
-    long long cur_key = -1;  // (level, first channel, width) of the tables
-    int flags = 0;           // bit 0: 32-bit requant form, 1: |bias| <= 2^30, 2: 32-bit skip form
+    uint32_t cur_key = 0xFFFFFFFFu;  // (first channel, half width, job, layer) of the tables
+    int flags = 0;
     for (int t = first_tile; t < tile_end; t += tile_stride, ++lt) {
       const TileInfo ti = tile_info(p, t);
       const ConvJobDev& jb = p.jobs[ti.job];
@@ -856,20 +803,15 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       // groups past it must not be written)
       const int TBN = ti.cn < p.cout - ti.col0 ? ti.cn : p.cout - ti.col0;
       const LayerDev& ly = p.layers[ti.layer];
-      const long long key =
-          ((long long)ti.layer << 48) | ((long long)jb.level << 32) | ((long long)ti.col0 << 10) | TBN;
+      const uint32_t key = ((uint32_t)ti.col0 << 6) | (ti.bn != BN ? 32u : 0u) | ((uint32_t)ti.job << 2) | (uint32_t)ti.layer;
       if (key != cur_key) {
         // (the same decision in every epilogue thread: all of them see the same tiles)
         named_bar(1, kEpiThreads);  // every epilogue warp is done with the previous tables
-        // Per-column constants of this tile's level. The 32-bit fast path applies when the
-        // total requant shift R = 31 + shift is >= 33 (then y = (mulhi(u, M0) + 2^(R-33)) >>
-        // (R-32) equals rhu(u * M0, R): the low product word cannot carry into the result)
-        // and |bias| <= 2^30 (acc + bias cannot leave int32 when |acc| < 2^24).
-        int fq = 1, sbias = 1;
+        int fq = 1, sbias = 1, fsk = 1;
         for (int col = et; col < 256; col += kEpiThreads) {
           const int ch = ti.col0 + col;
           EpiChan ec{};
-          int4 ef = make_int4((int32_t)(0u - kMagicBits), 0, 0, 1);
+          int4 ef = make_int4((int32_t)(0u - kMagicBits), 0, 0, 1), es = make_int4(0, 0, 1, 0);
           if (col < TBN && ch < p.cout) {
             const int64_t idx = (int64_t)jb.level * p.cout + ch;
             ec.bias = ly.bias ? ly.bias[idx] : 0;
@@ -883,236 +825,236 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
               if (r >= 33 && sb) { ef.y = ec.m0; ef.z = 1 << (r - 33); ef.w = r - 32; }
               else fq = 0;
             }
-            if (kSkip) { ec.c = p.skip_c[idx]; ec.d = p.skip_d[idx]; }
+            if constexpr (kSkip) {
+              ec.c = p.skip_c[idx]; ec.d = p.skip_d[idx];
+              fsk &= skip_const(p.skip_bits, ec.c, ec.d, es) ? 1 : 0;
+            }
           }
-          epi[col] = ec;
-          reinterpret_cast<int4*>(epi + 256)[col] = ef;
+          epi.gen()[col] = ec;
+          epi.fast()[col] = ef;
+          if constexpr (kSkip) epi.skip()[col] = es;
         }
         fq = named_bar_and(1, kEpiThreads, fq);
         sbias = named_bar_and(1, kEpiThreads, sbias);
-        // 32-bit skip path (fast_skip_group): default direction, code skips, d >= 8 everywhere
-        // (int32 skips: 64-bit product, any d >= 1)
-        int fsk = 0;
-        if (kSkip && p.scale_main == 0 && out_bits != 32 && fq && sbias) {
-          const int dmin = p.skip_bits <= 8 ? 8 : 1;
-          int okd = 1;
-          for (int col = et; col < TBN; col += kEpiThreads)
-            if (ti.col0 + col < p.cout && epi[col].d < dmin) okd = 0;
-          fsk = named_bar_and(1, kEpiThreads, okd);
+        flags = (fq ? kFlagReq : 0) | (sbias ? kFlagBias : 0);
+        if constexpr (kSkip) {
+          fsk = named_bar_and(1, kEpiThreads, fsk);
+          if (fsk && p.scale_main == 0) flags |= kFlagSkip;
         }
-        flags = fq | (sbias << 1) | (fsk << 2);
         cur_key = key;
       }
-      const int fast_req = flags & 1, small_bias = (flags >> 1) & 1, fast_skip = (flags >> 2) & 1;
-      // 0: general int64 epilogue; 1: fast requant to codes; 2: int32 output, no skip
-      // (kSkip: the skip instantiation runs exactly the calls with a skip, so its mode is 0 at
-      // compile time and it carries no code or registers of the other modes)
-      const int mode = (kSplit || kSkip) ? 0 : (out_bits == 32 ? 2 : (fast_req ? 1 : 0));
-      const bool magic = p.acc_small && (mode == 2 ? small_bias : fast_req);
-      const uint32_t buf = lt & 1;
-      if (!mbar_wait(b_tfull + 8 * buf, (lt >> 1) & 1, abort_flag)) { ok = false; break; }
-      tc_fence_after();
+      if ((int)(lt & (uint32_t)(p.epi_sets - 1)) != gset) continue;  // another set's tile (or an idle warp)
+      const uint32_t buf = lt & buf_mask;
 
-      // This warp's (sub-tile, 32-column group) units. The TMEM load of the next unit is in
-      // flight while the current one is converted and stored; no register written by a
-      // tcgen05.ld is read before the tcgen05.wait::ld that covers it.
-      const int ngrp = (TBN + 31) / 32;
-      const int nunits = kSub * ngrp;
-      const uint32_t tbuf = lane_base + buf * (uint32_t)(kSub * BN);
-      uint32_t va[32], vn[32];
-      __syncwarp();
-      if (gi < nunits) {
-        tmem_ld32(tbuf + (gi / ngrp) * (uint32_t)BN + (gi % ngrp) * 32, ti.cn - (gi % ngrp) * 32 >= 32, va);
-        tmem_wait_ld();
-        reg_fence32(va);
+      // this lane's output row
+      int m;  // output pixel index within the job
+      bool row_ok;
+      int img = 0, oh = 0, ow = 0;
+      if constexpr (kFlat) {
+        const FlatTile ft = flat_tile(jb, ti.mt, kTileRows);
+        const int vr = ft.v0 + (int)rank * 128 + quarter * 32 + lane;  // virtual row at the padded width
+        img = ft.img;
+        oh = fast_div(vr, jb.div_row);
+        ow = vr - oh * jb.wp;
+        row_ok = vr < jb.vimg && ow < jb.wo;  // else a junk column or past the image
+        m = (img * jb.ho + oh) * jb.wo + ow;
+      } else {
+        m = ti.mt * BM + quarter * 32 + lane;
+        row_ok = m < jb.m_total;
+        if constexpr (kSkip) {
+          img = fast_div(m, jb.div_img);
+          const int rem = m - img * (jb.ho * jb.wo);
+          oh = fast_div(rem, jb.div_row);
+          ow = rem - oh * jb.wo;
+        }
       }
-      for (int u0 = gi; u0 < nunits; u0 += kGroups) {
-        const int un = u0 + kGroups;
-        // the next unit's TMEM load overlaps this unit's work in the light modes; the general /
-        // skip mode (0) holds more registers and loads it afterwards
-        if (un < nunits && mode != 0)
-          tmem_ld32(tbuf + (un / ngrp) * (uint32_t)BN + (un % ngrp) * 32, ti.cn - (un % ngrp) * 32 >= 32, vn);
-        const int sub = u0 / ngrp, g0 = (u0 % ngrp) * 32;
-        const int ncols = (TBN - g0) < 32 ? (TBN - g0) : 32;
-        // 32 TMEM columns were loaded when the tile's MMA width covers them (else 16)
-        const bool full = ti.cn - g0 >= 32;
-        if (!full) {
-#pragma unroll
-          for (int i = 16; i < 32; ++i) va[i] = 0u;  // only the first 16 columns were loaded
+      uint8_t* yrow = ly.y[ti.job] + (int64_t)m * p.y_row_bytes;
+      uint8_t* irow = nullptr;  // this row of the chained image
+      const int nib = ly.ws_nib;
+      if (kFlat && ly.ws_out)
+        irow = ly.ws_out +
+               (size_t)(jb.orow_off + (img * jb.ohp + oh + p.out_pad) * jb.owp + ow + p.out_pad) * p.cout;
+      const uint8_t* srow = nullptr;
+      if constexpr (kSkip) {
+        const int up = p.upsample == 2 ? 1 : 0;
+        srow = jb.skip + (((int64_t)img * jb.skip_h + (oh >> up)) * jb.skip_w + (ow >> up)) * p.skip_row_bytes;
+      }
+
+      // this warp's columns [c_lo, c_hi), whole 32-column groups but for the tile's last one
+      const int per = ((TBN + 31) / 32 + p.epi_groups - 1) / p.epi_groups * 32;
+      const int c_lo = grp * per, c_hi = c_lo + per < TBN ? c_lo + per : TBN;
+      const uint32_t tbuf = lane_base + buf * (uint32_t)BN;
+      // The common forms; everything else goes through general_cols.
+      //  codes:  the 32-bit requant of FP32 accumulators below 2^22 (or split sums), and, with a
+      //          skip, the 32-bit rescale;  int32 outputs: the sum alone
+      bool common;
+      if constexpr (kOStage) common = p.acc_small && (flags & kFlagBias);
+      else if constexpr (kSkip)
+        common = p.acc_small && out_bits != 32 && (flags & (kFlagReq | kFlagSkip)) == (kFlagReq | kFlagSkip);
+      else if constexpr (kSplit) common = out_bits != 32 && (flags & kFlagReq);
+      else common = p.acc_small && (flags & (out_bits == 32 ? kFlagBias : kFlagReq));
+      // rows whose pieces would not be aligned, or not whole
+      if ((out_bits == 8 && (p.cout & 31) != 0) || (out_bits == 32 && (p.cout & 3) != 0)) common = false;
+      if (kSkip && p.skip_bits >= 8 && (p.skip_row_bytes & 15) != 0) common = false;
+      uint2 sw = make_uint2(0u, 0u);  // the next step's skip codes, loaded a step ahead
+      const bool sk_codes = kSkip && p.skip_bits <= 4;
+      if (sk_codes && c_lo < c_hi) sw = load_skip_words(srow, ti.col0 + c_lo, p.skip_bits, row_ok);
+      __syncwarp();
+      if (!mbar_wait(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      auto release = [&]() {  // every TMEM read of this warp is complete
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          if (kPair && !leader) mbar_arrive_cluster(mapa_shared(b_tempty + 8 * buf, 0));
+          else mbar_arrive(b_tempty + 8 * buf);
         }
-        if constexpr (kSplit) {
-          // split weights: va holds D1 (w_lo rows); D2 (w_hi rows) sits TBN columns on;
-          // the exact sum is D1 + 16 D2, each an integer x 2^-18 below 2^24
-          uint32_t vb[32];
-          tmem_ld32(tbuf + (uint32_t)ti.cn + g0, full, vb);
-          tmem_wait_ld();
-          reg_fence32(vb);
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int32_t d1 = __float2int_rn(__uint_as_float(va[i]) * kAccSc);
-            const int32_t d2 = (full || i < 16) ? __float2int_rn(__uint_as_float(vb[i]) * kAccSc) : 0;
-            va[i] = (uint32_t)(d1 + 16 * d2);
-          }
-        }
-        const uint32_t* v = va;
-        int m;  // output pixel index within the job
-        bool row_ok;
-        int oimg = 0, oh = 0, ow = 0;  // the pixel (flat path)
-        if constexpr (kFlat) {
-          const FlatTile ft = flat_tile(jb, ti.mt, kTileRows);
-          const int vr = ft.v0 + (int)rank * 128 + quarter * 32 + lane;  // virtual row at the padded width
-          const int ho = vr / jb.wp, wo = vr - (vr / jb.wp) * jb.wp;
-          row_ok = vr < jb.vimg && wo < jb.wo;  // else a junk column or past the image
-          m = (ft.img * jb.ho + ho) * jb.wo + wo;
-          oimg = ft.img; oh = ho; ow = wo;
-        } else {
-          m = ti.mt * BM + sub * 128 + quarter * 32 + lane;
-          row_ok = m < jb.m_total;
-        }
-        if constexpr (kOStage) {
-          // (launched for int32 outputs without a skip only: mode 2)
-          // int32 outputs through this warp's staging block: each lane holds its row's 32
-          // values; stored back four rows at a time, so every warp store covers four whole
-          // 128-byte row segments instead of 32 scattered 16-byte pieces (cout % 4 == 0)
-          uint32_t* stg = reinterpret_cast<uint32_t*>(smem + p.off_ostage) + warp * (32 * kStageRow);
-          const int ch0 = ti.col0 + g0;
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            int32_t o[4];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const float f = __uint_as_float(v[4 * q + k]);
-              o[k] = magic ? __float_as_int(__fmaf_rn(f, kAccSc, kMagic)) + epf[g0 + 4 * q + k].x
-                           : add_sat(__float2int_rn(f * kAccSc), epi[g0 + 4 * q + k].bias);
-            }
-            *reinterpret_cast<int4*>(stg + lane * kStageRow + 4 * q) = make_int4(o[0], o[1], o[2], o[3]);
-          }
+      };
+      uint32_t top = 0u;  // (3-bit codes: see store_codes16)
+      auto store16 = [&](int ch0, const uint32_t (&bw)[4]) {
+        if (!row_ok) return;
+        store_codes16(yrow, ch0, bw, out_bits, top);
+        if (kFlat && irow) store_image16(irow, ch0, bw, nib);
+      };
+      auto general_tile = [&]() {
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+          const int ch0 = ti.col0 + c0;
+          const GenCols gc{tbuf + (uint32_t)c0, tbuf + (uint32_t)(ti.cn + c0), epi.gen() + c0, srow, yrow, ch0,
+                           c_hi - c0 < 16 ? c_hi - c0 : 16, flags, row_ok};
+          const uint4 r = general_cols<kSkip, kSplit>(p, gc, kAccSc);
           __syncwarp();
-          const uint32_t rows_ok = __ballot_sync(0xffffffffu, row_ok);
-          const int nq = (ncols < p.cout - ch0 ? ncols : p.cout - ch0) >> 2;  // whole 16-byte pieces
+          const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
+          // (general_cols stores int32 outputs and 8-bit rows of no whole groups itself)
+          if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) store16(ch0, bw);
+        }
+      };
+      // int32 skips may turn out to need the general form, which reads the accumulator again
+      const bool late = !common || (kSkip && p.skip_bits == 32);
+      uint32_t big = 0u;  // bits above 27 set: an int32 skip beyond the 32-bit form
+      if (common) {
+        if (c_lo >= c_hi && !late) release();
+#pragma unroll 1
+        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
+          const int ch0 = ti.col0 + c0;
+          const bool last = c0 + 16 >= c_hi;
+          const int4* ef = epi.fast() + c0;
+          const int4* es = epi.skip() + c0;
+          uint32_t bw[4] = {0u, 0u, 0u, 0u};
+          uint32_t v[16];
+          tmem_ld16(tbuf + c0, v);
+          // One FMA turns the accumulator float acc / sc into the int32 acc + kMagicBits; ef.x
+          // holds bias - kMagicBits (no int32 overflow under the stated bounds).
+          if constexpr (kSkip) {
+            auto sum = [&](int i, const int4& c, int32_t scaled) {
+              return __float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + c.x + skip32(scaled, es[i]);
+            };
+            if (sk_codes) {
+              uint32_t sb[4];
+              skip_bytewords(sw, p.skip_bits, sb);
+              if (!last) sw = load_skip_words(srow, ch0 + 16, p.skip_bits, row_ok);
+              tmem_wait_ld();
+              reg_fence16(v);
 #pragma unroll
-          for (int r4 = 0; r4 < 8; ++r4) {
-            const int r = 4 * r4 + (lane >> 3), c4 = lane & 7;
-            const int mr = __shfl_sync(0xffffffffu, m, r);
-            if (((rows_ok >> r) & 1u) && c4 < nq) {
-              const int4 val = *reinterpret_cast<const int4*>(stg + r * kStageRow + 4 * c4);
-              *reinterpret_cast<int4*>(ly.y[ti.job] + (int64_t)mr * p.y_row_bytes + (int64_t)(ch0 + 4 * c4) * 4) = val;
-            }
-          }
-          __syncwarp();
-        } else {
-  if (row_ok) {
-            uint8_t* yrow = ly.y[ti.job] + (int64_t)m * p.y_row_bytes;
-            const int ch0 = ti.col0 + g0;
-            if (mode == 1 && magic) {
-              // codes as byte-words: the chained image takes them as they are, the packed
-              // output a couple of shifts per 8 codes
-              uint32_t bw[8], gw[8];
-              magic_requant_bytes(v, epf + g0, qmax, kAccSc, bw);
-              switch (out_bits) {
-                case 2: pack_bytewords<2>(bw, gw); break;
-                case 3: pack_bytewords<3>(bw, gw); break;
-                case 4: pack_bytewords<4>(bw, gw); break;
-                default: pack_bytewords<8>(bw, gw); break;
-              }
-              store_group(yrow + (ch0 >> 5) * group_bytes(out_bits), gw, out_bits);
-              if (kFlat && ly.ws_out) chain_store_bw(p, ly.ws_out, ly.ws_nib, jb, oimg, oh, ow, ch0, bw);
-            } else if (mode == 1) {
-              uint32_t gw[8];
-              {
-                switch (out_bits) {
-                  case 2: fast_requant_group<2>(v, epi, g0, qmax, kAccSc, gw); break;
-                  case 3: fast_requant_group<3>(v, epi, g0, qmax, kAccSc, gw); break;
-                  case 4: fast_requant_group<4>(v, epi, g0, qmax, kAccSc, gw); break;
-                  default: fast_requant_group<8>(v, epi, g0, qmax, kAccSc, gw); break;
-                }
-              }
-              store_group(yrow + (ch0 >> 5) * group_bytes(out_bits), gw, out_bits);
-              if (kFlat && ly.ws_out) chain_store(p, ly.ws_out, ly.ws_nib, jb, oimg, oh, ow, ch0, gw, out_bits);
-            } else if (mode == 2) {
-              int32_t* yr = reinterpret_cast<int32_t*>(yrow) + ch0;
-              const bool whole = ncols == 32 && ch0 + 32 <= p.cout;
-    #pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                int32_t o[4];
-    #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const float f = __uint_as_float(v[4 * q + k]);
-                  o[k] = magic ? __float_as_int(__fmaf_rn(f, kAccSc, kMagic)) + epf[g0 + 4 * q + k].x
-                               : add_sat(__float2int_rn(f * kAccSc), epi[g0 + 4 * q + k].bias);
-                }
-                if (whole) {
-                  reinterpret_cast<int4*>(yr)[q] = make_int4(o[0], o[1], o[2], o[3]);
-                } else {
-    #pragma unroll
-                  for (int k = 0; k < 4; ++k)
-                    if (4 * q + k < ncols && ch0 + 4 * q + k < p.cout) yr[4 * q + k] = o[k];
-                }
+              for (int i = 0; i < 16; ++i) {
+                const int4 c = ef[i];
+                const int32_t u = sum(i, c, (int32_t)__byte_perm(sb[i / 4], 0u, ((i % 4) << 12) | 0x0444));
+                bw[i / 4] += requant32(u, c, qmax) << (8 * (i % 4));  // codes < 256: the add is an or
               }
             } else {
-              const uint8_t* srow = nullptr;
-              if (kSkip) {
-                int img, ho, wo;
-                if constexpr (kFlat) {
-                  img = oimg; ho = oh; wo = ow;
+              // 8-bit or int32 skips, four columns at a time
+              tmem_wait_ld();
+              reg_fence16(v);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                int4 x = make_int4(0, 0, 0, 0);
+                if (p.skip_bits == 8) {
+                  const uint32_t w = row_ok ? __ldg(reinterpret_cast<const uint32_t*>(srow + ch0) + q) : 0u;
+                  x = make_int4((int)(__byte_perm(w, 0u, 0x0444) >> 1), (int)(__byte_perm(w, 0u, 0x1444) >> 1),
+                                (int)(__byte_perm(w, 0u, 0x2444) >> 1), (int)(__byte_perm(w, 0u, 0x3444) >> 1));
                 } else {
-                  const int hw = jb.ho * jb.wo;
-                  img = m / hw;
-                  const int rem = m - img * hw;
-                  ho = rem / jb.wo; wo = rem - ho * jb.wo;
+                  if (row_ok) x = __ldg(reinterpret_cast<const int4*>(srow) + (ch0 >> 2) + q);
+                  big |= (uint32_t)((x.x ^ (x.x >> 31)) | (x.y ^ (x.y >> 31)) | (x.z ^ (x.z >> 31)) | (x.w ^ (x.w >> 31)));
+                  x = make_int4((int)((uint32_t)x.x << 3), (int)((uint32_t)x.y << 3), (int)((uint32_t)x.z << 3),
+                                (int)((uint32_t)x.w << 3));
                 }
-                const int sh = p.upsample == 2 ? ho >> 1 : ho, sw = p.upsample == 2 ? wo >> 1 : wo;
-                srow = jb.skip + (((int64_t)img * jb.skip_h + sh) * jb.skip_w + sw) * p.skip_row_bytes;
-              }
-              int32_t oo[32];
-              if (kSkip && fast_skip && p.skip_bits <= 8) {
-                load_skip_group(p, srow, ch0, ncols, oo);   // skip codes, replaced by the results
-                fast_skip_group(v, epi + g0, oo, qmax, kAccSc, oo);
-              } else if (kSkip && fast_skip) {
-                load_skip_group(p, srow, ch0, ncols, oo);   // int32 skip, replaced by the results
-                fast_skip32_group(v, epi + g0, oo, qmax, kAccSc, oo);
-              } else {
-                general_group<kSkip, kSplit>(p, v, epi + g0, srow, ch0, ncols, kAccSc, oo);
-              }
-              if (out_bits == 32) {
-                int32_t* yr = reinterpret_cast<int32_t*>(yrow) + ch0;
-  #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  if (i < ncols && ch0 + i < p.cout) yr[i] = oo[i];
-              } else {
-                // clipped codes (< 2^out_bits) as byte-words, then the packed group
-                uint32_t bw[8], gw[8];
-  #pragma unroll
-                for (int j = 0; j < 8; ++j)
-                  bw[j] = (uint32_t)oo[4 * j] | ((uint32_t)oo[4 * j + 1] << 8) | ((uint32_t)oo[4 * j + 2] << 16) |
-                          ((uint32_t)oo[4 * j + 3] << 24);
-                switch (out_bits) {
-                  case 2: pack_bytewords<2>(bw, gw); break;
-                  case 3: pack_bytewords<3>(bw, gw); break;
-                  case 4: pack_bytewords<4>(bw, gw); break;
-                  default: pack_bytewords<8>(bw, gw); break;
-                }
-                store_group(yrow + (ch0 >> 5) * group_bytes(out_bits), gw, out_bits);
-                if (kFlat && ly.ws_out) chain_store_bw(p, ly.ws_out, ly.ws_nib, jb, oimg, oh, ow, ch0, bw);
+                const int4 c0 = ef[4 * q], c1 = ef[4 * q + 1], c2 = ef[4 * q + 2], c3 = ef[4 * q + 3];
+                bw[q] = requant32(sum(4 * q, c0, x.x), c0, qmax) | (requant32(sum(4 * q + 1, c1, x.y), c1, qmax) << 8) |
+                        (requant32(sum(4 * q + 2, c2, x.z), c2, qmax) << 16) |
+                        (requant32(sum(4 * q + 3, c3, x.w), c3, qmax) << 24);
               }
             }
-          }
-        }
-        if (un < nunits) {
-          if (mode == 0)
-            tmem_ld32(tbuf + (un / ngrp) * (uint32_t)BN + (un % ngrp) * 32, ti.cn - (un % ngrp) * 32 >= 32, vn);
-          tmem_wait_ld();
-          reg_fence32(vn);
+            if (last && !late) release();
+          } else if constexpr (kSplit) {
+            // split weights: v holds D1 (w_lo rows); D2 (w_hi rows) sits cn columns on; the exact
+            // sum is D1 + 16 D2, each an integer x 2^-18 below 2^24 (|sum| < 2^29, |bias| <= 2^30)
+            uint32_t vb[16];
+            tmem_ld16(tbuf + (uint32_t)(ti.cn + c0), vb);
+            tmem_wait_ld();
+            reg_fence16(v);
+            reg_fence16(vb);
+            if (last) release();
 #pragma unroll
-          for (int i = 0; i < 32; ++i) va[i] = vn[i];
+            for (int i = 0; i < 16; ++i) {
+              const int4 c = ef[i];
+              const int32_t d1 = __float2int_rn(__uint_as_float(v[i]) * kAccSc);
+              const int32_t d2 = __float2int_rn(__uint_as_float(vb[i]) * kAccSc);
+              bw[i / 4] += requant32(d1 + 16 * d2 + (int32_t)((uint32_t)c.x + kMagicBits), c, qmax) << (8 * (i % 4));
+            }
+          } else {
+            tmem_wait_ld();
+            reg_fence16(v);
+            if (last) release();
+            if (kOStage || out_bits == 32) {
+              // int32 outputs: acc + bias
+#pragma unroll
+              for (int i = 0; i < 16; ++i)
+                v[i] = (uint32_t)(__float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + ef[i].x);
+              const int nq = (c_hi - c0 < 16 ? c_hi - c0 : 16) >> 2;  // whole 16-byte pieces (cout % 4 == 0)
+              if constexpr (kOStage) {
+                // through this warp's staging block: each lane holds its row's 16 values; stored
+                // back eight rows at a time, so a warp store covers whole sectors of eight row
+                // segments instead of 32 scattered 16-byte pieces
+                uint32_t* stg = reinterpret_cast<uint32_t*>(smem + p.off_ostage) + warp * (32 * kStageRow);
+                const uint32_t rows_ok = __ballot_sync(0xffffffffu, row_ok);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  *reinterpret_cast<uint4*>(stg + lane * kStageRow + 4 * q) =
+                      make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                __syncwarp();
+#pragma unroll
+                for (int r8 = 0; r8 < 4; ++r8) {
+                  const int r = 8 * r8 + (lane >> 2), c4 = lane & 3;
+                  const int mr = __shfl_sync(0xffffffffu, m, r);
+                  if (((rows_ok >> r) & 1u) && c4 < nq)
+                    *reinterpret_cast<uint4*>(ly.y[ti.job] + (int64_t)mr * p.y_row_bytes + (int64_t)(ch0 + 4 * c4) * 4) =
+                        *reinterpret_cast<const uint4*>(stg + r * kStageRow + 4 * c4);
+                }
+                __syncwarp();
+              } else if (row_ok) {
+                uint4* yr = reinterpret_cast<uint4*>(yrow) + (ch0 >> 2);
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                  if (q < nq) yr[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+              }
+              continue;
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const int4 c = ef[i];
+              const int32_t u = __float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + c.x;
+              bw[i / 4] += requant32(u, c, qmax) << (8 * (i % 4));  // codes < 256: the add is an or
+            }
+          }
+          store16(ch0, bw);
         }
+        if constexpr (kSkip) {
+          if (__any_sync(0xffffffffu, (big >> 28) != 0u)) general_tile();
+        }
+      } else {
+        general_tile();
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        if (kPair && !leader) mbar_arrive_cluster(mapa_shared(b_tempty + 8 * buf, 0));
-        else mbar_arrive(b_tempty + 8 * buf);
-      }
+      if (late) release();
       if (kFlat && p.dep && ti.layer < p.nlayers - 1) {
         // this warp's stores of tile t are done: order them for the next layer's TMA (async
         // proxy) loads, gather the warp (__syncwarp orders its lanes' stores before lane 0's
@@ -1402,7 +1344,7 @@ bool conv_tc_uses_pair(const ConvArgs& a) {
   // tiles on the FP4 pipe: the 256->84 output conv of the head measured 35.7 us on single
   // CTAs against 39.4 us on pairs (same box, expansion included)
   if (a.fp4 && a.bn <= 128) return false;
-  return a.ws != nullptr && a.bn >= 16 && a.bn % 16 == 0 && tc::kSub == 1 && !a.no_pair;
+  return a.ws != nullptr && a.bn >= 16 && a.bn % 16 == 0 && !a.no_pair;
 }
 
 // Last-wave balancing: with `workers` persistent CTAs (or CTA pairs), the full tiles past the
@@ -1450,11 +1392,15 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
       jb.wp = jb.w + 2 * a.pad;
       jb.vimg = jb.ho * jb.wp;
       jb.tpi = (jb.vimg + tile_rows - 1) / tile_rows;
+      jb.div_img = div_magic(jb.tpi);
+      jb.div_row = div_magic(jb.wp);
       jb.row_off = (int32_t)rows;
       rows += (int64_t)jb.n * jb.hp * jb.wp;
       tiles += jb.n * jb.tpi * prm.n_tiles;
     } else {
       tiles += ((a.jobs[j].m_total + BM - 1) / BM) * prm.n_tiles;
+      prm.jobs[j].div_img = div_magic(a.jobs[j].ho * a.jobs[j].wo);
+      prm.jobs[j].div_row = div_magic(a.jobs[j].wo);
     }
   }
   // K chunk width: 128 bytes of one tap, or on the workspace path with cin % 128 != 0 the 64
@@ -1463,7 +1409,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   // bytes per row of the image: one code per byte, or two (nibbles) on the FP4 pipe
   const int img_row = fp4 ? a.cin / 2 : a.cin;
   const int bk = (flat && img_row % BK != 0) ? 64 : BK;
-  if (flat && (kSub != 1 || a.stride != 1 || img_row % bk != 0 || rows > a.ws_rows || (a.split_w && bk != BK))) {
+  if (flat && (a.stride != 1 || img_row % bk != 0 || rows > a.ws_rows || (a.split_w && bk != BK))) {
     *err = "conv_tc: workspace path needs stride 1, cin % 64 == 0 (128 for split weights) and a large enough workspace";
     return 1;
   }
@@ -1494,6 +1440,8 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.contig = (!pair && flat && nlayers <= 1 && prm.dp_tiles == tiles) ? 1 : 0;
   prm.nlayers = nlayers;
   prm.layer_tiles = prm.total_tiles / nlayers;
+  prm.div_layer = div_magic(prm.layer_tiles);
+  prm.div_nt = div_magic(prm.n_tiles);
   prm.num_kchunks = flat ? (fp4 ? a.k_total / 2 : a.k_total) / bk : a.k_pad / BK;
   prm.cin = a.cin; prm.cout = a.cout; prm.kh = a.kh; prm.kw = a.kw;
   prm.stride = a.stride; prm.pad = a.pad; prm.k_total = a.k_total;
@@ -1537,17 +1485,23 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   }
   prm.status = a.status;
   prm.dep = nlayers > 1 ? a.dep : nullptr;
-  prm.dep_target = (uint32_t)(2 * kEpiWarps);  // epilogue warps of both CTAs of a pair
+  // 32-column groups of a full tile over the epilogue warps of a lane quarter
+  const int warp_groups = epi_warps(flat) / 4;
+  const int col_groups = ((a.split_w ? BN / 2 : BN) + 31) / 32;
+  prm.epi_groups = col_groups < warp_groups ? col_groups : warp_groups;
+  prm.epi_sets = warp_groups / prm.epi_groups;
+  if (prm.epi_sets == 3) prm.epi_sets = 2;  // (a power of two: tiles are dealt by their low bits)
+  prm.dep_target = (uint32_t)(8 * prm.epi_groups);  // a tile's epilogue warps, both CTAs of a pair
   // shared memory plan: stages of (BM x bk A bytes + this CTA's B rows x bk bytes)
   const int b_rows = pair ? BN / 2 : BN;
-  const size_t stage_a = (size_t)kSub * 128 * bk;
+  const size_t stage_a = (size_t)BM * bk;
   const size_t stage_bytes = stage_a + (size_t)b_rows * bk;
-  const size_t epi_bytes = 256 * sizeof(EpiChan) + 256 * sizeof(int4);
-  const size_t bar_bytes = 8 * (2 * kMaxStages + 5) + 16;
+  const size_t epi_bytes = EpiTab::kBytes;
+  const size_t bar_bytes = 8 * (2 * kMaxStages + 2 * kMaxBufs + 1) + 16;
   const size_t qtab_bytes = kQTab * sizeof(uint32_t);
   const size_t budget = 232448 - 1024;  // max dynamic smem per block minus alignment slack
   // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least 6 stages remain
-  const size_t ostage_bytes = (size_t)kEpiWarps * 32 * kStageRow * sizeof(uint32_t);
+  const size_t ostage_bytes = (size_t)epi_warps(flat) * 32 * kStageRow * sizeof(uint32_t);
   const bool ostage = flat && bk == BK && a.out_bits == 32 && a.cout % 4 == 0 && !a.has_skip && !a.split_w &&
                       (budget - epi_bytes - bar_bytes - qtab_bytes - ostage_bytes) / stage_bytes >= 6;
   int stages = (int)((budget - epi_bytes - bar_bytes - qtab_bytes - (ostage ? ostage_bytes : 0)) / stage_bytes);
@@ -1565,11 +1519,14 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.off_qtab = prm.off_bar + (uint32_t)bar_bytes;
   prm.off_ostage = ostage ? (uint32_t)((prm.off_qtab + qtab_bytes + 15) / 16 * 16) : 0u;
   const size_t smem = 1024 + (ostage ? prm.off_ostage + ostage_bytes : prm.off_qtab + qtab_bytes);
-  // two buffers x kSub sub-tiles x BN fp32 columns (and, on the FP4 pipe, 32 columns of scales)
-  const int acc_cols = 2 * kSub * BN;
-  if (fp4 && acc_cols + 32 > 512) { *err = "conv_tc: FP4 tiles wider than 240 channels do not fit in TMEM"; return 2; }
+  // two accumulators of BN fp32 columns, or four where they fit beside the 32 columns of scales
+  // of the FP4 pipe
+  const int sf_cols = fp4 ? 32 : 0;
+  prm.nbuf_log2 = 4 * BN + sf_cols <= 512 ? 2 : 1;
+  const int acc_cols = BN << prm.nbuf_log2;
+  if (acc_cols + sf_cols > 512) { *err = "conv_tc: FP4 tiles wider than 240 channels do not fit in TMEM"; return 2; }
   int cols = 32;
-  while (cols < acc_cols + (fp4 ? 32 : 0)) cols *= 2;
+  while (cols < acc_cols + sf_cols) cols *= 2;
   prm.tmem_cols = cols;
   prm.sf_col = acc_cols;
 

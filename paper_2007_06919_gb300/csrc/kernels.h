@@ -25,6 +25,9 @@ struct ConvJobDev {
   int32_t hp, wp;         // padded height / width (h + 2 pad, w + 2 pad)
   int32_t vimg;           // virtual output rows per image: ho * wp (columns >= wo are junk)
   int32_t tpi;            // tiles per image
+  // fast_div of the tensor-core kernel: tiles per image and padded width on the flat path, else
+  // output pixels per image and output width
+  uint64_t div_img, div_row;
   // chained output (ws_out): zero-padded byte image of this job's output for the next conv
   int32_t orow_off;       // first ws_out row (one row = cout bytes) of image 0
   int32_t ohp, owp;       // padded output height / width (ho + 2 out_pad, wo + 2 out_pad)

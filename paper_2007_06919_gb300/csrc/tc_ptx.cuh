@@ -367,6 +367,12 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, bool full, uint32_t (&
           "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
         : "r"(taddr + 16));
 }
+// (reg_fence16: the same for 16 registers)
+__device__ __forceinline__ void reg_fence16(uint32_t (&r)[16]) {
+  asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+               "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]),
+               "+r"(r[14]), "+r"(r[15]));
+}
 // Makes every later use of r depend on this point (placed right after tcgen05.wait::ld, so
 // the compiler cannot move a read of a TMEM-loaded register above the wait).
 __device__ __forceinline__ void reg_fence32(uint32_t (&r)[32]) {

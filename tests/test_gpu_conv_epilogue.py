@@ -1,0 +1,101 @@
+"""The conv epilogue's forms at the sizes where their choice changes, byte for byte against the
+oracle: the 32-bit skip rescale and its limits, rows of no whole 32-channel groups, column
+counts that leave warps idle or let sets of warps take tiles in turn, and accumulators too
+large for the common form."""
+import numpy as np
+import pytest
+
+from paper_2007_06919_gb300 import synth
+
+from gpu_util import assert_same, conv_pair
+
+pytestmark = pytest.mark.gpu
+I32 = np.iinfo(np.int32)
+
+
+def tables(rng, cout, std, out_bits):
+    return synth.requant_params(rng, 1, cout, calib_std=std, out_bits=out_bits)
+
+
+# d at and beside the 32-bit form's limits: d + k >= 33 with k = 24 (2- to 4-bit codes), 23 (8-bit),
+# 3 (int32); from bits + 32 (codes) or 60 (int32) on the rescaled skip is 0
+@pytest.mark.parametrize("skip_bits,d_lo,d_hi", [(2, 8, 9), (2, 9, 33), (2, 34, 62), (3, 9, 36), (4, 8, 8), (4, 9, 12),
+                                                 (4, 30, 40), (8, 9, 10), (8, 10, 12), (8, 30, 62), (32, 29, 33),
+                                                 (32, 30, 34), (32, 55, 62)])
+@pytest.mark.parametrize("ws", [False, True])
+@pytest.mark.parametrize("huge", [False, True])
+def test_skip_rescale_forms_bit_exact(skip_bits, d_lo, d_hi, ws, huge):
+    rng = np.random.default_rng(100 * skip_bits + d_lo + 7 * ws)
+    n, h, w, cin, cout = 2, 9, 21, 64, 96
+    x = synth.act_codes(rng, (n, h, w, cin), 4)
+    wt = synth.weight_codes(rng, (cout, 3, 3, cin), 4)
+    m0, sh, b = tables(rng, cout, 3000.0, 4)
+    c = rng.integers(I32.min, I32.max, size=(1, cout), dtype=np.int64, endpoint=True).astype(np.int32)
+    c[0, :3] = (I32.min, I32.max, 0)
+    d = rng.integers(d_lo, d_hi + 1, size=(1, cout)).astype(np.int8)
+    if skip_bits == 32:
+        # below 2^28 everywhere, or values beyond it in some rows (those take the general form)
+        lim = 1 << 28
+        skip = rng.integers(-lim + 1, lim, size=(n, h, w, cout)).astype(np.int32)
+        if huge:
+            skip[0, 3, 5, 7], skip[1, 8, 20, 95], skip[1, 0, 0, 0] = I32.max, I32.min, lim
+    else:
+        skip = synth.act_codes(rng, (n, h, w, cout), skip_bits)
+        if huge:
+            b = np.where(rng.random((1, cout)) < 0.5, 1 << 30, -(1 << 30)).astype(np.int32)  # the bias limit
+    got, want, _ = conv_pair(x, 4, wt, 4, out_bits=4, m0=m0, shift=sh, bias=b, skip=skip, skip_bits=skip_bits, skip_c=c,
+                             skip_d=d, workspace=ws)
+    assert_same(got, want, cout, 4, f"skip {skip_bits} bits, d {d_lo}..{d_hi}")
+
+
+@pytest.mark.parametrize("out_bits,cout", [(8, 1), (8, 40), (8, 48), (8, 272), (8, 96), (32, 33), (32, 84), (32, 20),
+                                           (32, 258)])
+@pytest.mark.parametrize("skip", [False, True])
+@pytest.mark.parametrize("ws", [False, True])
+def test_rows_of_no_whole_groups_bit_exact(out_bits, cout, skip, ws):
+    rng = np.random.default_rng(cout)
+    n, h, w, cin = 1, 11, 27, 64
+    x = synth.act_codes(rng, (n, h, w, cin), 4)
+    wt = synth.weight_codes(rng, (cout, 3, 3, cin), 4)
+    m0, sh, b = tables(rng, cout, 600.0, min(out_bits, 8))
+    kw = {}
+    if skip:
+        kw = dict(skip=synth.act_codes(rng, (n, h, w, cout), 8), skip_bits=8,
+                  skip_c=rng.integers(-(1 << 30), 1 << 30, size=(1, cout)).astype(np.int32),
+                  skip_d=rng.integers(10, 30, size=(1, cout)).astype(np.int8))
+    got, want, _ = conv_pair(x, 4, wt, 4, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                             shift=None if out_bits == 32 else sh, bias=b, workspace=ws, **kw)
+    assert_same(got, want, cout, out_bits, f"cout {cout}")
+
+
+# several tiles per CTA pair; 1, 2, 3, 4 and 8 column groups, and two N tiles
+@pytest.mark.parametrize("cout", [32, 64, 96, 128, 256, 320])
+@pytest.mark.parametrize("out_bits", [2, 3, 4])
+@pytest.mark.parametrize("skip", [False, True])
+def test_column_groups_over_many_tiles_bit_exact(cout, out_bits, skip):
+    rng = np.random.default_rng(cout + out_bits)
+    n, h, w, cin = 3, 150, 179, 64
+    x = synth.act_codes(rng, (n, h, w, cin), 3)
+    wt = synth.weight_codes(rng, (cout, 1, 1, cin), 3)
+    m0, sh, b = tables(rng, cout, 80.0, out_bits)
+    sh = np.maximum(sh, 2).astype(np.int8)  # R >= 33
+    kw = {}
+    if skip:
+        c, d = synth.skip_params(rng, 1, cout, sh)
+        kw = dict(skip=synth.act_codes(rng, (n, h, w, cout), out_bits), skip_bits=out_bits, skip_c=c, skip_d=d)
+    got, want, _ = conv_pair(x, 3, wt, 3, pad=0, out_bits=out_bits, m0=m0, shift=sh, bias=b, workspace=True, **kw)
+    assert_same(got, want, cout, out_bits, f"cout {cout}")
+
+
+@pytest.mark.parametrize("ws", [False, True])
+@pytest.mark.parametrize("out_bits", [4, 32])
+def test_accumulators_beyond_the_common_form_bit_exact(ws, out_bits):
+    rng = np.random.default_rng(5)
+    cin, cout = 2112, 32  # K * 15 * 15 = 4.3e6 > 2^22, and sums up to that size occur
+    x = np.full((1, 5, 6, cin), 15, np.int32)
+    wt = np.full((cout, 3, 3, cin), 15, np.int32)  # odd grid: 2 * 15 - 15 = 15
+    wt[1:] = rng.integers(0, 16, size=(cout - 1, 3, 3, cin))
+    m0, sh, b = tables(rng, cout, 1e6, 4)
+    got, want, _ = conv_pair(x, 4, wt, 4, w_format=1, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                             shift=None if out_bits == 32 else sh, bias=b, workspace=ws)
+    assert_same(got, want, cout, out_bits)
