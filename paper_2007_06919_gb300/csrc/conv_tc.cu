@@ -906,8 +906,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
-          if (kPair && !leader) mbar_arrive_cluster(mapa_shared(b_tempty + 8 * buf, 0));
-          else mbar_arrive(b_tempty + 8 * buf);
+          if (kPair && !leader) mbar_arrive_cluster_relaxed(mapa_shared(b_tempty + 8 * buf, 0));
+          else mbar_arrive_relaxed(b_tempty + 8 * buf);
         }
       };
       uint32_t top = 0u;  // (3-bit codes: see store_codes16)

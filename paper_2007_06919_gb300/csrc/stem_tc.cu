@@ -398,7 +398,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(b_tempty + 8 * buf);
+      if (lane == 0) mbar_arrive_relaxed(b_tempty + 8 * buf);
     }
     if (!ok) fail(abort_flag, p.status);
   }
