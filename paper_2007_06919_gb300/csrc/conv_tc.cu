@@ -571,7 +571,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
 
   if (warp == kWarpMma) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0 && leader) {
+    if (leader && elect_one()) {
       const uint32_t idesc_full = kFp4 ? idesc_fp4(BN, kPair ? 2 * kMmaM : kMmaM) : idesc_e4m3(BN, kPair ? 2 * kMmaM : kMmaM);
       const uint32_t idesc_half =
           kFp4 ? idesc_fp4(BN / 2, kPair ? 2 * kMmaM : kMmaM) : idesc_e4m3(BN / 2, kPair ? 2 * kMmaM : kMmaM);
@@ -636,7 +636,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     // One thread of each TMA warp issues every kTma-th chunk: a thread sustains
     // about one tensor copy at a time, so two threads keep two copies in flight.
     const int tw = warp - kWarpTma;
-    if (lane == 0) {
+    if (elect_one()) {
       uint32_t it = 0, s = 0, ph = 0;
       bool ok = true;
       for (int t = first_tile; t < tile_end && ok; t += tile_stride) {

@@ -319,7 +319,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
   const int first = blockIdx.x, stride_t = gridDim.x;
   if (warp == kWarpMma) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t idesc = idesc_e4m3(p.n_pad);  // F16 has the same type code 0
       const uint64_t db0 = sdesc_noswz(s_b);
       uint32_t s = 0, ph = 0, lt = 0;

@@ -128,6 +128,19 @@ __device__ __forceinline__ void fail(volatile int* abort_flag, uint32_t* status)
   atomicCAS(status, 0u, (uint32_t)kStatusTimeout);
 }
 
+// One lane of a converged warp, by elect.sync: the compiler then knows that a single thread runs
+// the branch and issues its tensor-core and TMA instructions directly; under "lane == 0" it
+// wraps each in a loop over the active lanes (measured: 4 MMAs and their commit 650 cycles
+// against under 512, a TMA box about 650 cycles of its issuing thread).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t one;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.b32 %0, 1, 0, p;\n\t}"
+      : "=r"(one));
+  return one != 0;
+}
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
