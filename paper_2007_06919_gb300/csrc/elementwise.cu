@@ -1000,38 +1000,151 @@ __global__ void __launch_bounds__(kThreads, kBits == 2 ? 2 : 3)
   }
 }
 
-__global__ void __launch_bounds__(kThreads)
-pack_kernel(const int32_t* codes, int64_t rows, int c, int bits, int64_t row_bytes, uint8_t* out) {
-  const int groups = (c + 31) / 32;
-  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (t >= rows * groups) return;
-  const int64_t r = t / groups;
-  const int ch0 = (int)(t - r * groups) * 32;
-  int32_t v[32];
-#pragma unroll 4
-  for (int i = 0; i < 32; ++i) v[i] = (ch0 + i < c) ? codes[r * c + ch0 + i] : 0;
-  if (bits == 8) {
-    for (int i = 0; i < 32; ++i)
-      if (ch0 + i < c) out[r * row_bytes + ch0 + i] = (uint8_t)(v[i] & 0xFF);
-    return;
+// Packing and unpacking, bound by HBM: 4 bytes per int32 code on one side and bits / 8 on the other.
+// Rows are contiguous on both sides and a row is whole 32-channel groups (or, at 8 bits, plain
+// bytes), so the tensor is one run of codes. A warp takes blocks of 128 codes, lane l codes 4 l ..
+// 4 l + 3: 16 bytes per lane on the int32 side, 512 consecutive per warp, kPackUnroll blocks'
+// loads issued together. The four codes are one byte-word of the packed layout (channels 4 j .. 4 j
+// + 3 in bit field j of a word's bytes), so a packed word is the or of its lanes' shifted
+// byte-words. One thread per 32-channel group read its 128 bytes element by element, 32 lanes 128
+// bytes apart: 34M codes packed to 4 bits 494 -> 85 us, unpacked 172 -> 25 us.
+constexpr int kPackUnroll = 4;
+
+template <int kBits>
+__global__ void __launch_bounds__(kThreads) pack_run_kernel(const int32_t* __restrict__ codes, int64_t n,
+                                                            uint8_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
+  const int64_t blocks = (n + 127) / 128;
+  constexpr int kM = (1 << kBits) - 1;
+  for (int64_t b0 = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); b0 < blocks; b0 += warps * kPackUnroll) {
+    int4 v[kPackUnroll];
+    if ((b0 + (kPackUnroll - 1) * warps + 1) * 128 <= n) {  // (whole blocks: no branch between the loads)
+#pragma unroll
+      for (int u = 0; u < kPackUnroll; ++u)
+        v[u] = __ldcs(reinterpret_cast<const int4*>(codes + (b0 + u * warps) * 128) + lane);
+    } else {
+#pragma unroll
+      for (int u = 0; u < kPackUnroll; ++u) {
+        const int64_t e = (b0 + u * warps) * 128 + 4 * lane;
+        v[u] = make_int4(0, 0, 0, 0);
+        if (e + 4 <= n) v[u] = __ldcs(reinterpret_cast<const int4*>(codes + e));
+        else if (e < n) {  // (8 bits: a last run of 1 to 3 codes)
+          v[u].x = codes[e];
+          if (e + 1 < n) v[u].y = codes[e + 1];
+          if (e + 2 < n) v[u].z = codes[e + 2];
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPackUnroll; ++u) {
+      const int64_t e = (b0 + u * warps) * 128 + 4 * lane;  // this lane's first code
+      uint32_t w = (uint32_t)(v[u].x & kM) | ((uint32_t)(v[u].y & kM) << 8) | ((uint32_t)(v[u].z & kM) << 16) |
+                   ((uint32_t)(v[u].w & kM) << 24);
+      if constexpr (kBits == 8) {
+        if (e + 4 <= n) *reinterpret_cast<uint32_t*>(out + e) = w;
+        else
+          for (int k = 0; e + k < n; ++k) out[e + k] = (uint8_t)(w >> (8 * k));
+      } else if constexpr (kBits == 3) {
+        // words 0 and 1 of a group: the low bits of lanes 0..3 and 4..7; word 2: bit 2 of all eight
+        uint32_t lo = (w & 0x03030303u) << (2 * (lane & 3)), hi = ((w >> 2) & 0x01010101u) << (lane & 7);
+        lo |= __shfl_xor_sync(0xffffffffu, lo, 1);
+        hi |= __shfl_xor_sync(0xffffffffu, hi, 1);
+        lo |= __shfl_xor_sync(0xffffffffu, lo, 2);
+        hi |= __shfl_xor_sync(0xffffffffu, hi, 2);
+        hi |= __shfl_xor_sync(0xffffffffu, hi, 4);
+        const int64_t g = (e >> 5) * 3;
+        const int l8 = lane & 7;
+        if (e < n && (l8 == 0 || l8 == 4 || l8 == 1))
+          reinterpret_cast<uint32_t*>(out)[g + (l8 == 0 ? 0 : l8 == 4 ? 1 : 2)] = l8 == 1 ? hi : lo;
+      } else {
+        constexpr int kLanes = 8 / kBits;  // lanes per word
+        w <<= kBits * (lane & (kLanes - 1));
+#pragma unroll
+        for (int off = 1; off < kLanes; off <<= 1) w |= __shfl_xor_sync(0xffffffffu, w, off);
+        if (e < n && (lane & (kLanes - 1)) == 0) reinterpret_cast<uint32_t*>(out)[e * kBits / 32] = w;
+      }
+    }
   }
-  uint32_t g[8];
-  pack_group_vals(v, bits, g);
-  store_group(out + r * row_bytes + (ch0 >> 5) * group_bytes(bits), g, bits);
 }
 
+template <int kBits>
+__global__ void __launch_bounds__(kThreads) unpack_run_kernel(const uint8_t* __restrict__ packed, int64_t n,
+                                                              int is_signed, int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (kThreads / 32);
+  const int64_t blocks = (n + 127) / 128;
+  for (int64_t b0 = (int64_t)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); b0 < blocks; b0 += warps * kPackUnroll) {
+    uint32_t w[kPackUnroll], h[kPackUnroll];
+#pragma unroll
+    for (int u = 0; u < kPackUnroll; ++u) {
+      const int64_t e = (b0 + u * warps) * 128 + 4 * lane;
+      w[u] = h[u] = 0u;
+      if (e >= n) continue;
+      const uint32_t* p32 = reinterpret_cast<const uint32_t*>(packed);
+      if constexpr (kBits == 8) {
+        if (e + 4 <= n) w[u] = __ldg(p32 + e / 4);
+        else
+          for (int k = 0; e + k < n; ++k) w[u] |= (uint32_t)__ldg(packed + e + k) << (8 * k);
+      } else if constexpr (kBits == 3) {
+        w[u] = __ldg(p32 + (e >> 5) * 3 + ((lane >> 2) & 1));
+        h[u] = __ldg(p32 + (e >> 5) * 3 + 2);
+      } else {
+        w[u] = __ldg(p32 + e * kBits / 32);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kPackUnroll; ++u) {
+      const int64_t e = (b0 + u * warps) * 128 + 4 * lane;
+      if (e >= n) continue;
+      uint32_t b;  // byte-word
+      if constexpr (kBits == 8) b = w[u];
+      else if constexpr (kBits == 3)
+        b = ((w[u] >> (2 * (lane & 3))) & 0x03030303u) | (((h[u] >> (lane & 7)) & 0x01010101u) << 2);
+      else b = (w[u] >> (kBits * (lane & (8 / kBits - 1)))) & (((1u << kBits) - 1u) * 0x01010101u);
+      int32_t o[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        o[k] = (int32_t)((b >> (8 * k)) & 0xFFu);
+        if (is_signed) o[k] = (int32_t)((uint32_t)o[k] << (32 - kBits)) >> (32 - kBits);
+      }
+      if (e + 4 <= n) __stcs(reinterpret_cast<int4*>(out + e), make_int4(o[0], o[1], o[2], o[3]));
+      else
+        for (int k = 0; k < 4 && e + k < n; ++k) out[e + k] = o[k];
+    }
+  }
+}
+
+// The same code by code, for int32 or 8-bit runs at addresses that take no 16- or 4-byte accesses.
+template <int kBits>
 __global__ void __launch_bounds__(kThreads)
-unpack_kernel(const uint8_t* packed, int64_t rows, int c, int bits, int64_t row_bytes, int is_signed,
-              int32_t* out) {
-  const int groups = (c + 31) / 32;
+pack_kernel(const int32_t* codes, int64_t groups, uint8_t* out) {
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-  if (t >= rows * groups) return;
-  const int64_t r = t / groups;
-  const int ch0 = (int)(t - r * groups) * 32;
-  int32_t v[32];
-  load_vals(packed + r * row_bytes, bits, c, ch0, is_signed != 0, v);
-  for (int i = 0; i < 32; ++i)
-    if (ch0 + i < c) out[r * c + ch0 + i] = v[i];
+  if (t >= groups) return;
+  if constexpr (kBits == 8) {  // (one code per group)
+    out[t] = (uint8_t)(codes[t] & 0xFF);
+  } else {
+    int32_t v[32];
+#pragma unroll 4
+    for (int i = 0; i < 32; ++i) v[i] = codes[t * 32 + i];
+    uint32_t g[8];
+    pack_group_vals(v, kBits, g);
+    store_group(out + t * group_bytes(kBits), g, kBits);
+  }
+}
+
+template <int kBits>
+__global__ void __launch_bounds__(kThreads)
+unpack_kernel(const uint8_t* packed, int64_t groups, int is_signed, int32_t* out) {
+  const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+  if (t >= groups) return;
+  if constexpr (kBits == 8) {
+    out[t] = is_signed ? (int32_t)(int8_t)packed[t] : (int32_t)packed[t];
+  } else {
+    int32_t v[32];
+    unpack_group_vals(packed + t * group_bytes(kBits), kBits, is_signed != 0, v);
+    for (int i = 0; i < 32; ++i) out[t * 32 + i] = v[i];
+  }
 }
 
 // Prepared weights: E4M3 sign-magnitude bytes [cout_pad][k_pad] (zero padded; only when
@@ -1357,21 +1470,62 @@ int launch_maxpool_expand(const PoolArgs& a, uint8_t* ws, int32_t cpad, cudaStre
   return check_launch("maxpool_expand launch", err);
 }
 
+// Runs of n codes: whole 32-code groups at 2 to 4 bits, any length at 8. The run kernels read and
+// write 16 bytes of int32 and one word of codes per lane, so their pointers are aligned to that.
+template <int kBits>
+static void launch_pack_bits(const int32_t* codes, int64_t n, uint8_t* out, unsigned cap, cudaStream_t stream) {
+  if ((uintptr_t)codes % 16 == 0 && (uintptr_t)out % 4 == 0) {
+    const int64_t want = (n + 128 * 8 * elt::kPackUnroll - 1) / (128 * 8 * elt::kPackUnroll);
+    elt::pack_run_kernel<kBits><<<(unsigned)(want < cap ? want : cap), elt::kThreads, 0, stream>>>(codes, n, out);
+  } else {
+    const int64_t groups = kBits == 8 ? n : n / 32;
+    elt::pack_kernel<kBits><<<elt::blocks_for(groups), elt::kThreads, 0, stream>>>(codes, groups, out);
+  }
+}
+template <int kBits>
+static void launch_unpack_bits(const uint8_t* packed, int64_t n, int32_t is_signed, int32_t* out, unsigned cap,
+                               cudaStream_t stream) {
+  if ((uintptr_t)out % 16 == 0 && (uintptr_t)packed % 4 == 0) {
+    const int64_t want = (n + 128 * 8 * elt::kPackUnroll - 1) / (128 * 8 * elt::kPackUnroll);
+    elt::unpack_run_kernel<kBits><<<(unsigned)(want < cap ? want : cap), elt::kThreads, 0, stream>>>(packed, n, is_signed, out);
+  } else {
+    const int64_t groups = kBits == 8 ? n : n / 32;
+    elt::unpack_kernel<kBits><<<elt::blocks_for(groups), elt::kThreads, 0, stream>>>(packed, groups, is_signed, out);
+  }
+}
+// blocks of the run kernels: 8 per SM
+static unsigned run_cap() {
+  int dev = 0, sms = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return (unsigned)(sms > 0 ? sms : 152) * 8u;
+}
+
 int launch_pack(const int32_t* codes, int64_t rows, int32_t c, int32_t bits, uint8_t* out,
                 cudaStream_t stream, std::string* err) {
-  const int64_t total = rows * ((c + 31) / 32);
-  if (total == 0) return 0;
-  elt::pack_kernel<<<elt::blocks_for(total), elt::kThreads, 0, stream>>>(codes, rows, c, bits,
-                                                                          row_bytes_of(c, bits), out);
+  const int64_t n = rows * c;
+  if (n == 0) return 0;
+  const unsigned cap = run_cap();
+  switch (bits) {
+    case 2: launch_pack_bits<2>(codes, n, out, cap, stream); break;
+    case 3: launch_pack_bits<3>(codes, n, out, cap, stream); break;
+    case 4: launch_pack_bits<4>(codes, n, out, cap, stream); break;
+    default: launch_pack_bits<8>(codes, n, out, cap, stream); break;
+  }
   return check_launch("pack launch", err);
 }
 
 int launch_unpack(const uint8_t* packed, int64_t rows, int32_t c, int32_t bits, int32_t is_signed,
                   int32_t* out, cudaStream_t stream, std::string* err) {
-  const int64_t total = rows * ((c + 31) / 32);
-  if (total == 0) return 0;
-  elt::unpack_kernel<<<elt::blocks_for(total), elt::kThreads, 0, stream>>>(packed, rows, c, bits,
-                                                                            row_bytes_of(c, bits), is_signed, out);
+  const int64_t n = rows * c;
+  if (n == 0) return 0;
+  const unsigned cap = run_cap();
+  switch (bits) {
+    case 2: launch_unpack_bits<2>(packed, n, is_signed, out, cap, stream); break;
+    case 3: launch_unpack_bits<3>(packed, n, is_signed, out, cap, stream); break;
+    case 4: launch_unpack_bits<4>(packed, n, is_signed, out, cap, stream); break;
+    default: launch_unpack_bits<8>(packed, n, is_signed, out, cap, stream); break;
+  }
   return check_launch("unpack launch", err);
 }
 
