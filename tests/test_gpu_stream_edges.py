@@ -36,3 +36,34 @@ def test_pack_unpack_runs(bits, rows, c, offset):
         assert np.array_equal(out[1:-1].cpu().numpy(), want.reshape(-1))
         assert out[0] == 0xA5 and out[-1] == 0xA5
         assert np.array_equal(aqd.unpack_codes(out[1:-1].view(rows, c), c, 8).cpu().numpy(), codes)
+
+
+# both sides of 2^-20 and 2^20, a divisor of all ones, one just above a power of two, and values at
+# which a quotient under- or overflows
+@pytest.mark.parametrize("nu", [2.0 ** -21, 2.0 ** -20, np.float32(2.0 - 2.0 ** -23), np.float32(1.0 + 2.0 ** -23), 3.0, 0.1,
+                                2.0 ** 20, 2.0 ** 21, 1e30])
+@pytest.mark.parametrize("weight", [False, True])
+def test_fake_quant_divisors(nu, weight):
+    rng = np.random.default_rng(3)
+    nu = float(np.float32(nu))
+    n = 400_001
+    x = (rng.normal(0.0 if weight else 0.5, 0.8, size=n) * nu).astype(np.float32)
+    # rounding thresholds of 4-bit codes and their neighbours
+    t = ((np.arange(16) + 0.5) / 15.0 * (2.0 if weight else 1.0) - (1.0 if weight else 0.0)) * nu
+    x[:16] = t.astype(np.float32)
+    x[16:32] = np.nextafter(x[:16], np.float32(np.inf))
+    x[32:48] = np.nextafter(x[:16], np.float32(-np.inf))
+    x[48:60] = [0.0, -0.0, 1e-45, -1e-45, 1e-38, 3e-31, -3e-31, np.inf, -np.inf, 3e38, -3e38, np.nan]
+    gy = rng.normal(0.1, 1.0, size=n).astype(np.float32)
+    fwd, bwd = (ot.fake_quant_weight, ot.fake_quant_weight_backward) if weight else (ot.fake_quant_act, ot.fake_quant_act_backward)
+    with np.errstate(all="ignore"):
+        x1 = np.where(np.isnan(x), -np.float32(np.inf), x)  # a NaN counts as the lower side
+        want_y, want_c = fwd(x1, nu, 4)
+        want_gx, want_gnu = bwd(x1, gy, nu, 4)
+    y, codes = aqd.fake_quant(dev(x), nu, 4, weight=weight)
+    gx, gnu = aqd.fake_quant_backward(dev(x), dev(gy), nu, 4, weight=weight)
+    assert np.array_equal(codes.cpu().numpy(), want_c)
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), want_y.view(np.uint32))
+    assert np.array_equal(gx.cpu().numpy(), want_gx)
+    # float32 over runs of 16 vectors (64 products): 64 * 2^-24 of sum|gy dy/dnu| <= sum|gy|
+    assert abs(float(gnu.cpu()[0]) - want_gnu) <= 64 * 2.0 ** -24 * float(np.abs(gy.astype(np.float64)).sum())
