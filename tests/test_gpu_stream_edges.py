@@ -67,3 +67,25 @@ def test_fake_quant_divisors(nu, weight):
     assert np.array_equal(gx.cpu().numpy(), want_gx)
     # float32 over runs of 16 vectors (64 products): 64 * 2^-24 of sum|gy dy/dnu| <= sum|gy|
     assert abs(float(gnu.cpu()[0]) - want_gnu) <= 64 * 2.0 ** -24 * float(np.abs(gy.astype(np.float64)).sum())
+
+
+@pytest.mark.parametrize("c,offset", [(1, 0), (4, 0), (12, 0), (30, 0), (256, 0), (256, 1), (1028, 0), (1100, 0)])
+def test_bn_level_stats_channel_counts(c, offset):
+    rng = np.random.default_rng(c)
+    mean, sd = rng.normal(0, 1, c), rng.uniform(0.1, 3.0, c)
+    pix = [1, 700, 37, 0]
+    zs = [(rng.normal(0, 1, (p, c)) * sd + mean).astype(np.float32) for p in pix]
+    dz = []
+    for z in zs:
+        buf = torch.zeros(z.size + 1, dtype=torch.float32, device="cuda")
+        v = buf[offset:offset + z.size].view(z.shape)  # offset 1: no 16-byte reads
+        v.copy_(dev(z))
+        dz.append(v)
+    m, v = (t.cpu().numpy() for t in aqd.bn_level_stats(dz))
+    for l, z in enumerate(zs):
+        z64 = z.astype(np.float64)
+        wm = z64.mean(0) if len(z) else np.zeros(c)
+        wv = z64.var(0) if len(z) else np.zeros(c)
+        # sums of float32 runs of 32 shifted values: the bounds of test_gpu_train
+        assert np.all(np.abs(m[l] - wm) <= 1e-6 * (np.abs(wm) + sd))
+        assert np.all(np.abs(v[l] - wv) <= 1e-5 * wv + 1e-12)
