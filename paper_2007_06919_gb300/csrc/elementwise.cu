@@ -520,6 +520,7 @@ struct StageGeo {
   uint32_t s_bytes;      // bytes of one stage's skip rows (P * b_row_bytes, 0 without a skip)
   uint32_t stage_bytes;  // a_bytes + s_bytes rounded to 128
   uint32_t tab_bytes;    // skip table bytes rounded to 128
+  uint64_t div_hw, div_w;  // fast_div of the pixels per image and per row (kUp)
 };
 
 __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar,
@@ -572,7 +573,11 @@ __device__ __noinline__ void staged_general(const EltArgs& a, const int32_t* aro
   }
 }
 
-template <bool kSkip, int kOut, int kSkipBits, int kV>
+// kUp: the skip has another grid than the output (the FPN's nearest 2x up-read, or a larger map):
+// its rows are not one run per stage, so each lane loads its words of the warp's pixels of a stage
+// directly, before it waits for the stage. Against the lane kernel on 8x100x168x256 int32 plus a
+// 4-bit 8x50x84 map: 90 -> 47 us.
+template <bool kSkip, int kOut, int kSkipBits, int kV, bool kUp>
 __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip form: its table limits it to 2
     eltwise_staged_kernel(const EltArgs a, int64_t npix, const StageGeo sg, int tstride) {
   extern __shared__ __align__(128) uint8_t smem[];
@@ -634,11 +639,11 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
       const int64_t p0 = j * sg.P;
       const int np = (int)(npix - p0 < sg.P ? npix - p0 : sg.P);
       const uint32_t ab = (uint32_t)np * (uint32_t)a.c * 4u;
-      const uint32_t sb = kSkip ? (uint32_t)np * (uint32_t)a.b_row_bytes : 0u;
+      const uint32_t sb = kSkip && !kUp ? (uint32_t)np * (uint32_t)a.b_row_bytes : 0u;
       const uint32_t dst = tc::smem_u32(stage0 + (size_t)s * sg.stage_bytes);
       tc::mbar_arrive_expect_tx(full0 + 8 * s, ab + sb);
       bulk_g2s(dst, a.a + p0 * a.c * 4, ab, full0 + 8 * s, pol);
-      if constexpr (kSkip) bulk_g2s(dst + sg.a_bytes, a.b + p0 * a.b_row_bytes, sb, full0 + 8 * s, pol);
+      if constexpr (kSkip && !kUp) bulk_g2s(dst + sg.a_bytes, a.b + p0 * a.b_row_bytes, sb, full0 + 8 * s, pol);
     }
     // before leaving, the copies still in flight (the last `stages` chunks) land: bounded
     const int issued = it;
@@ -668,24 +673,68 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
   }
   const int sbase = kSkip ? code_pos<kSkip ? kSkipBits : 8>(i0) : 0;
   const int obase = kOut != 32 ? code_pos<kOut != 32 ? kOut : 8>(i0) : 0;
+  // kUp: the skip tensor's pixel under an output pixel
+  auto skip_pix = [&](int pix) {
+    const int img = fast_div(pix, sg.div_hw);
+    const int rem = pix - img * (a.h * a.w);
+    const int hh = fast_div(rem, sg.div_w), ww = rem - hh * a.w;
+    const int up = a.upsample == 2 ? 1 : 0;
+    return (img * a.b_h + (hh >> up)) * a.b_w + (ww >> up);
+  };
+  constexpr int kSkipWord = kSkip ? 32 / (kSkipBits > 0 ? kSkipBits : 32) : 1;  // channels per skip word
+  // pixels of a stage per warp: P c / (32 kV) blocks over 8 warps, P c <= 8192
+  constexpr int kPer = 32 / kV;
+  // kUp: this lane's words of the warp's pixels of stage chunk j; lane k finds pixel k's place
+  auto load_up = [&](int64_t j, uint32_t (&w)[kUp ? kPer : 1]) {
+    const int64_t p0 = j * sg.P;
+    const int np = (int)(npix - p0 < sg.P ? npix - p0 : sg.P);
+    const int mine = pg + (lane < kPer ? lane : 0) * pgs;
+    const int sp = skip_pix((int)p0 + (mine < np ? mine : 0));  // (pixel 0 of the chunk for those past its end)
+    const uint8_t* base = a.b + (ch0 >> 5) * group_bytes(kSkipBits) + 4 * (i0 / kSkipWord);
+#pragma unroll
+    for (int k = 0; k < (kUp ? kPer : 1); ++k)
+      w[k] = __ldg(reinterpret_cast<const uint32_t*>(base + (int64_t)__shfl_sync(0xffffffffu, sp, k) * a.b_row_bytes));
+  };
   int it = 0;
+  uint32_t up_w[kUp ? kPer : 1];
+  constexpr bool kAhead = kUp && kPer <= 8;  // the next stage's words beside this one's
+  if constexpr (kAhead) {
+    if ((int64_t)blockIdx.x < sg.nchunks) load_up(blockIdx.x, up_w);
+  }
   for (int64_t j = blockIdx.x; j < sg.nchunks; j += gridDim.x, ++it) {
     const int s = it % sg.stages;
+    const int64_t p0 = j * sg.P;
+    const int np = (int)(npix - p0 < sg.P ? npix - p0 : sg.P);
+    uint32_t up_n[kAhead ? kPer : 1];
+    if constexpr (kAhead) {
+      if (j + gridDim.x < sg.nchunks) {
+        load_up(j + gridDim.x, up_n);
+      } else {
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) up_n[k] = 0u;
+      }
+    } else if constexpr (kUp) {
+      load_up(j, up_w);
+    }
     if (!tc::mbar_wait(full0 + 8 * s, (it / sg.stages) & 1, &abort_flag)) {
       tc::fail(&abort_flag, a.status);
       return;
     }
-    const int64_t p0 = j * sg.P;
-    const int np = (int)(npix - p0 < sg.P ? npix - p0 : sg.P);
     const uint8_t* st = stage0 + (size_t)s * sg.stage_bytes;
     if (!ok) {
       for (int p = pg; p < np; p += pgs)
         staged_general<kSkip, kOut, kSkipBits, kV>(a, reinterpret_cast<const int32_t*>(st) + (size_t)p * a.c,
-                                                   st + sg.a_bytes + (size_t)p * a.b_row_bytes, ch0, lane, p0 + p);
+                                                   kUp ? a.b + (int64_t)skip_pix((int)(p0 + p)) * a.b_row_bytes
+                                                       : st + sg.a_bytes + (size_t)p * a.b_row_bytes,
+                                                   ch0, lane, p0 + p);
     } else {
       // two pixels per step (the second clamped to the last one and its store predicated off)
       // so their chains interleave
-      for (int p = pg; p < np; p += 2 * pgs) {
+      // (kUp: unrolled, so that the words loaded ahead stay in registers)
+#pragma unroll(kUp ? kPer / 2 : 1)
+      for (int k2 = 0; k2 < (kUp ? kPer / 2 : (sg.P / pgs + 1) / 2); ++k2) {
+        const int p = pg + 2 * k2 * pgs;
+        if (p >= np) break;
         const int pp[2] = {p, p + pgs < np ? p + pgs : np - 1};
         int32_t av[2][kV];
         uint32_t sw[2] = {0, 0};
@@ -701,7 +750,8 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
           } else {
             av[u][0] = arow[ch0];
           }
-          if constexpr (kSkip)
+          if constexpr (kUp) sw[u] = up_w[2 * k2 + u] >> sbase;
+          else if constexpr (kSkip)
             sw[u] = reinterpret_cast<const uint32_t*>(st + sg.a_bytes + pp[u] * (int)a.b_row_bytes +
                                                       (ch0 >> 5) * group_bytes(kSkipBits))[i0 / (32 / kSkipBits)] >> sbase;
         }
@@ -766,6 +816,10 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
     }
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(empty0 + 8 * s);
+    if constexpr (kAhead) {
+#pragma unroll
+      for (int k = 0; k < kPer; ++k) up_w[k] = up_n[k];
+    }
   }
 }
 
@@ -1283,9 +1337,9 @@ static bool launch_lane(const EltArgs& a, int sms, cudaStream_t stream) {
 }
 
 // The staged kernel: one wave of blocks, 2 stages of about 32 KB of int32 rows each.
-template <bool kSkip, int kOut, int kSkipBits, int kV>
+template <bool kSkip, int kOut, int kSkipBits, int kV, bool kUp>
 static void launch_staged_k(const EltArgs& a, int ts, int sms, cudaStream_t stream) {
-  auto kern = elt::eltwise_staged_kernel<kSkip, kOut, kSkipBits, kV>;
+  auto kern = elt::eltwise_staged_kernel<kSkip, kOut, kSkipBits, kV, kUp>;
   const int64_t npix = (int64_t)a.n * a.h * a.w;
   const int row = a.c * 4;
   elt::StageGeo g{};
@@ -1293,7 +1347,9 @@ static void launch_staged_k(const EltArgs& a, int ts, int sms, cudaStream_t stre
   g.stages = 2;
   g.nchunks = (npix + g.P - 1) / g.P;
   g.a_bytes = (uint32_t)g.P * (uint32_t)row;
-  g.s_bytes = kSkip ? (uint32_t)g.P * (uint32_t)a.b_row_bytes : 0u;
+  g.s_bytes = kSkip && !kUp ? (uint32_t)g.P * (uint32_t)a.b_row_bytes : 0u;
+  g.div_hw = div_magic((int64_t)a.h * a.w);
+  g.div_w = div_magic(a.w);
   g.stage_bytes = (g.a_bytes + g.s_bytes + 127u) / 128u * 128u;
   g.tab_bytes = ts > 0 ? (uint32_t)((((size_t)ts << kSkipBits) * sizeof(int32_t) + 127) / 128 * 128) : 0u;
   const size_t smem = g.tab_bytes + (size_t)g.stages * g.stage_bytes;
@@ -1314,19 +1370,20 @@ static void launch_staged_k(const EltArgs& a, int ts, int sms, cudaStream_t stre
   if (blocks > g.nchunks) blocks = g.nchunks;
   kern<<<(unsigned)blocks, elt::kThreads + 32, smem, stream>>>(a, npix, g, ts);
 }
-template <bool kSkip, int kSkipBits, int kV>
+static bool same_grid(const EltArgs& a) { return a.upsample == 1 && a.b_h == a.h && a.b_w == a.w; }
+template <bool kSkip, int kSkipBits, int kV, bool kUp>
 static bool launch_staged_v(const EltArgs& a, int ts, int sms, cudaStream_t stream) {
   switch (a.y_bits) {
-    case 2: launch_staged_k<kSkip, 2, kSkipBits, kV>(a, ts, sms, stream); return true;
-    case 4: launch_staged_k<kSkip, 4, kSkipBits, kV>(a, ts, sms, stream); return true;
-    case 8: launch_staged_k<kSkip, 8, kSkipBits, kV>(a, ts, sms, stream); return true;
-    case 32: launch_staged_k<kSkip, 32, kSkipBits, kV>(a, ts, sms, stream); return true;
+    case 2: launch_staged_k<kSkip, 2, kSkipBits, kV, kUp>(a, ts, sms, stream); return true;
+    case 4: launch_staged_k<kSkip, 4, kSkipBits, kV, kUp>(a, ts, sms, stream); return true;
+    case 8: launch_staged_k<kSkip, 8, kSkipBits, kV, kUp>(a, ts, sms, stream); return true;
+    case 32: launch_staged_k<kSkip, 32, kSkipBits, kV, kUp>(a, ts, sms, stream); return true;
     default: return false;
   }
 }
-// Whether the staged kernel takes these arguments: contiguous int32 rows (and skip rows on the
-// same grid, 2/4/8-bit, whole 16-byte rows) at 16-byte aligned addresses, and a channel-block
-// count that divides the 8 consumer warps.
+// Whether the staged kernel takes these arguments: contiguous int32 rows (and 2/4/8-bit skip rows;
+// on the same grid whole 16-byte rows) at 16-byte aligned addresses, and a channel-block count
+// that divides the 8 consumer warps.
 static bool staged_applies(const EltArgs& a) {
   if (a.a_bits != 32 || a.c % 32 != 0 || a.a_row_bytes != (int64_t)a.c * 4 || a.y_bits == 3) return false;
   if ((uintptr_t)a.a % 16 != 0) return false;
@@ -1335,8 +1392,8 @@ static bool staged_applies(const EltArgs& a) {
   if (cblocks != 1 && cblocks != 2 && cblocks != 4 && cblocks != 8) return false;
   if (a.has_skip) {
     if (a.b_bits != 2 && a.b_bits != 4 && a.b_bits != 8) return false;
-    if (!(a.upsample == 1 && a.b_h == a.h && a.b_w == a.w)) return false;
-    if (a.b_row_bytes % 16 != 0 || (uintptr_t)a.b % 16 != 0) return false;
+    // (another grid: word loads, and pixels counted in 31 bits, as the API checks)
+    if (same_grid(a) && (a.b_row_bytes % 16 != 0 || (uintptr_t)a.b % 16 != 0)) return false;
   }
   return true;
 }
@@ -1348,9 +1405,14 @@ static bool launch_staged(const EltArgs& a, int sms, cudaStream_t stream) {
     if (((size_t)ts << kSkipBits) * sizeof(int32_t) > 48 * 1024) ts = 0;
   }
   const int v = a.c % 128 == 0 ? 4 : (a.c % 64 == 0 ? 2 : 1);
-  if (v == 4) return launch_staged_v<kSkip, kSkipBits, 4>(a, ts, sms, stream);
-  if (v == 2) return launch_staged_v<kSkip, kSkipBits, 2>(a, ts, sms, stream);
-  return launch_staged_v<kSkip, kSkipBits, 1>(a, ts, sms, stream);
+  if (kSkip && !same_grid(a)) {
+    if (v == 4) return launch_staged_v<kSkip, kSkipBits, 4, kSkip>(a, ts, sms, stream);
+    if (v == 2) return launch_staged_v<kSkip, kSkipBits, 2, kSkip>(a, ts, sms, stream);
+    return launch_staged_v<kSkip, kSkipBits, 1, kSkip>(a, ts, sms, stream);
+  }
+  if (v == 4) return launch_staged_v<kSkip, kSkipBits, 4, false>(a, ts, sms, stream);
+  if (v == 2) return launch_staged_v<kSkip, kSkipBits, 2, false>(a, ts, sms, stream);
+  return launch_staged_v<kSkip, kSkipBits, 1, false>(a, ts, sms, stream);
 }
 
 int launch_elementwise(const EltArgs& a, cudaStream_t stream, std::string* err) {

@@ -1,4 +1,6 @@
-"""The streaming kernels at the edges of their dispatch, against the oracle."""
+"""The streaming kernels at the edges of their dispatch, against the oracle: packed runs with
+ragged ends and odd addresses, skips on another grid through the staged kernel, divisors at and
+past the limits of the known-divisor quotient, and batch statistics of odd channel counts."""
 import numpy as np
 import pytest
 import torch
@@ -36,6 +38,30 @@ def test_pack_unpack_runs(bits, rows, c, offset):
         assert np.array_equal(out[1:-1].cpu().numpy(), want.reshape(-1))
         assert out[0] == 0xA5 and out[-1] == 0xA5
         assert np.array_equal(aqd.unpack_codes(out[1:-1].view(rows, c), c, 8).cpu().numpy(), codes)
+
+
+@pytest.mark.parametrize("c", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("b_bits", [2, 4, 8])
+@pytest.mark.parametrize("shape", [(1, 1, 1), (2, 7, 11), (3, 37, 53)])
+@pytest.mark.parametrize("grid,wide", [("up", False), ("larger", False), ("up", True)])
+def test_skip_on_another_grid(c, b_bits, shape, grid, wide):
+    n, h, w = shape
+    rng = np.random.default_rng(c + b_bits + h)
+    up = 2 if grid == "up" else 1
+    bh, bw = ((h + 1) // 2 + 1, (w + 1) // 2) if up == 2 else (h + 2, w + 1)
+    a = rng.integers(-30000, 30000, size=(n, h, w, c)).astype(np.int32)
+    b = synth.act_codes(rng, (n, bh, bw, c), b_bits)
+    m0, sh, bias = synth.requant_params(rng, 1, c, calib_std=12000.0, out_bits=4)
+    cc, dd = synth.skip_params(rng, 1, c, sh)
+    if wide:
+        cc, dd = np.full_like(cc, 2 ** 31 - 1), np.zeros_like(dd)  # no 32-bit table: the int64 form
+    at, bt = oracle.CodeTensor.from_codes(a, 32), oracle.CodeTensor.from_codes(b, b_bits)
+    ref = oracle.residual_add(at, bt, cc, dd, upsample=up, scale_a=0, out_bits=4, m0=m0, shift=sh, bias=bias)
+    Y = aqd.DTensor.empty(n, h, w, c, 4)
+    Y.data.fill_(0xA5)
+    aqd.residual_add_int(to_device(at), to_device(bt), aqd.SkipParams.from_numpy(cc, dd, up), Y,
+                         rq=aqd.RequantParams.from_numpy(m0, sh, bias))
+    assert_same(Y.data.cpu().numpy().reshape(ref.packed.shape), ref.packed, c, 4, f"{grid} skip")
 
 
 # both sides of 2^-20 and 2^20, a divisor of all ones, one just above a power of two, and values at
