@@ -36,6 +36,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "epilogue.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
@@ -217,13 +218,6 @@ enum : int {
 constexpr float kMagic = 12582912.0f;
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
-// The 32-bit requant (every R = 31 + shift >= 33): rhu(u M0, R) = (mulhi(u, M0) + 2^(R-33)) >>
-// (R-32), as the low product word cannot carry into the rounded result; the clip of Eq. 2 is
-// one min.relu (max(min(x, qmax), 0)).
-__device__ __forceinline__ uint32_t requant32(int32_t u, const int4& f, int qmax) {
-  return (uint32_t)__vimin_s32_relu((__mulhi(u, f.y) + f.z) >> f.w, qmax);
-}
-
 // Eq. 7's rescaled skip rhu(s c, d) in 32-bit arithmetic: with s pre-scaled by 2^k so that
 // |s 2^k| < 2^31, rhu(s c, d) = (mulhi(s 2^k, c) + 2^(d+k-33)) >> (d+k-32) for d + k >= 33 (the
 // same identity as the requant's). k = 24 for 2- to 4-bit codes (the code in the top byte of a
@@ -244,30 +238,6 @@ __device__ __forceinline__ int32_t skip32(int32_t s_scaled, const int4& e) {
   return (__mulhi(s_scaled, e.x) + e.y) >> e.z;
 }
 
-// 16 codes < 2^bits as byte-words (word j: channels 4j..4j+3, one per byte) -> their place in the
-// packed row (the layout of common.cuh: word w of the 2/4/8-bit layout holds its channels 4k..4k+3
-// in bit field k of every byte; a 3-bit group of 32 channels is two 2-bit words of the low bits
-// and one word of bit 2, channel i at bit 8 (i%4) + i/4). ch: the first channel, a multiple of
-// 16; top: bit 2 of the group's first half (3-bit codes), kept for the second.
-__device__ __forceinline__ void store_codes16(uint8_t* yrow, int ch, const uint32_t (&bw)[4], int bits, uint32_t& top) {
-  if (bits == 4) {
-    *reinterpret_cast<uint2*>(yrow + (ch >> 1)) = make_uint2(bw[0] | (bw[1] << 4), bw[2] | (bw[3] << 4));
-  } else if (bits == 2) {
-    *reinterpret_cast<uint32_t*>(yrow + (ch >> 2)) = bw[0] | (bw[1] << 2) | (bw[2] << 4) | (bw[3] << 6);
-  } else if (bits == 8) {
-    *reinterpret_cast<uint4*>(yrow + ch) = make_uint4(bw[0], bw[1], bw[2], bw[3]);
-  } else {
-    const int half = (ch >> 4) & 1;
-    uint32_t* g = reinterpret_cast<uint32_t*>(yrow + (ch >> 5) * 12);
-    g[half] = (bw[0] & 0x03030303u) | ((bw[1] & 0x03030303u) << 2) | ((bw[2] & 0x03030303u) << 4) |
-              ((bw[3] & 0x03030303u) << 6);
-    uint32_t h = 0u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) h |= ((bw[j] >> 2) & 0x01010101u) << j;
-    if (half) g[2] = top | (h << 4);
-    else top = h;
-  }
-}
 // Chained output: the 16 codes at their place in the row of the zero-padded image that the next
 // stride-1 conv reads: one byte per code, or, when that conv runs on the FP4 pipe (nib), two
 // codes per byte (channel 2k in the low nibble of byte k) in the first half of the row.

@@ -19,10 +19,10 @@
 // apart, 8-row groups 2560 B apart).
 //
 // Per CTA (one per SM, persistent over tiles of 128 consecutive output pixels):
-//   warps 0..3   epilogue: tcgen05.ld (warp w reads TMEM lanes 32w.., every 32-column
-//                group in turn), Eq. 6 + Eq. 2, bit-pack, store
-//   warp  4      TMEM allocation + one thread issuing tcgen05.mma (M=128, N=cout, K=16)
-//   warps 5..12  im2col producers: two threads per tile row (kernel rows 0..3 / 4..6),
+//   warps 0..7   epilogue: tcgen05.ld (warp w reads TMEM lanes 32 (w % 4).., the two warps of a
+//                lane quarter every other 32-column group), Eq. 6 + Eq. 2, bit-pack, store
+//   warp  8      TMEM allocation + one thread issuing tcgen05.mma (M=128, N=cout, K=16)
+//   warps 9..16  im2col producers: two threads per tile row (kernel rows 0..3 / 4..6),
 //                word loads of the receptive field, PRMT to F16, 16-byte stores
 // The weights (cout x 160 F16) stay in shared memory for the whole launch. Every wait is
 // bounded: on expiry the CTA latches kStatusTimeout and unwinds.
@@ -33,6 +33,7 @@
 #include <mutex>
 
 #include "common.cuh"
+#include "epilogue.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
@@ -53,8 +54,10 @@ constexpr int kStageA = 128 * kK * 2;      // one tile's A operand
 constexpr int kSplitR = 4;                 // producer half 0: kernel rows [0, 4); half 1: [4, 7)
 static_assert((kSplitR * kLs) % 8 == 0, "the producer halves must meet on a core-matrix boundary");
 static_assert(kLs <= 24, "a receptive-field row must fit six realigned words");
-// 13 warps: at most 4 per SM sub-partition, so 128 registers per thread
-constexpr int kEpiWarps = 4, kWarpMma = 4, kWarpProd0 = 5, kProdWarps = 8;
+// 17 warps: at most 5 per SM sub-partition, so 96 registers per thread. (4 epilogue warps, one per
+// sub-partition, ran two 32-column groups each per tile as one chain of dependent instructions.
+// Now the producers bound it: they build a tile in 2.4k of its 2.8k cycles. Config 3's first conv, 8 x 400 x 672 x 64 outputs: 203 -> 173 us.)
+constexpr int kEpiWarps = 8, kWarpMma = kEpiWarps, kWarpProd0 = kEpiWarps + 1, kProdWarps = 8;
 constexpr int kThreads = (kWarpProd0 + kProdWarps) * 32;
 constexpr uint32_t kF16Pair1024 = 0x64006400u;
 
@@ -164,73 +167,18 @@ __device__ __forceinline__ void build_half(const StemParams& p, int mg, uint8_t*
     *reinterpret_cast<uint4*>(row_dst + (R0 * kLs / 8 + c) * kLBO) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
 }
 
-// Packs 32 k-bit codes into one group (the layout of common.cuh) and stores it at dst.
-template <int kOut>
-__device__ __forceinline__ void store_codes(uint8_t* dst, const uint32_t (&gw)[8]) {
-  uint32_t* d = reinterpret_cast<uint32_t*>(dst);
-  if constexpr (kOut == 2) {
-    *reinterpret_cast<uint2*>(d) = make_uint2(gw[0], gw[1]);
-  } else if constexpr (kOut == 3) {
-    d[0] = gw[0]; d[1] = gw[1]; d[2] = gw[2];
-  } else if constexpr (kOut == 4) {
-    *reinterpret_cast<uint4*>(d) = make_uint4(gw[0], gw[1], gw[2], gw[3]);
-  } else {
-    reinterpret_cast<uint4*>(d)[0] = make_uint4(gw[0], gw[1], gw[2], gw[3]);
-    reinterpret_cast<uint4*>(d)[1] = make_uint4(gw[4], gw[5], gw[6], gw[7]);
-  }
-}
-template <int kOut>
-__device__ __forceinline__ void put_code(uint32_t (&gw)[8], int i, uint32_t y) {
-  if constexpr (kOut == 3) {
-    gw[i / 16] |= (y & 3u) << (8 * (i % 4) + 2 * ((i % 16) / 4));
-    gw[2] |= (y >> 2) << (8 * (i % 4) + i / 4);
-  } else {
-    constexpr int q = 32 / kOut;
-    gw[i / q] |= y << (8 * (i % 4) + kOut * ((i % q) / 4));
-  }
-}
-
-// Epilogue of 32 accumulator columns [c0, c0 + ncols) of one tile row: Eq. 6 bias, Eq. 2
-// rescale + clip, packed into the k-bit group at column c0 (int32 out: stored in fours).
-// The 32-bit form (every R >= 33: rhu(u * M0, R) = (mulhi(u, M0) + 2^(R-33)) >> (R-32)) and
-// the int64 form are separate loops, so the common one runs as straight-line code.
-template <int kOut>
-__device__ __forceinline__ void epi_unit(const uint32_t (&v)[32], const int4* cst4, const EpiChan* cste, int c0,
-                                         int ncols, bool fast_req, int qmax, uint8_t* yrow, bool valid) {
-  if constexpr (kOut == 32) {
-    int32_t* y32 = reinterpret_cast<int32_t*>(yrow) + c0;
+// Eq. 6 -> Eq. 2 of 16 columns in int64, as the definition states them (some R < 33): byte-words of
+// the codes. Not inlined: its registers and code stay out of the common form.
+__device__ __noinline__ uint4 general_cols(uint32_t taddr, const EpiChan* c, int out_bits) {
+  uint32_t v[16];
+  tmem_ld16(taddr, v);
+  tmem_wait_ld();
+  reg_fence16(v);
+  uint32_t bw[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      int32_t o[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k)
-        o[k] = add_sat(__float2int_rn(__uint_as_float(v[4 * q + k])), cst4[c0 + 4 * q + k].x);
-      if (!valid) continue;
-      if (ncols == 32) {
-        reinterpret_cast<int4*>(y32)[q] = make_int4(o[0], o[1], o[2], o[3]);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          if (4 * q + k < ncols) y32[4 * q + k] = o[k];
-      }
-    }
-  } else {
-    uint32_t gw[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-    if (fast_req) {
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        const int4 c = cst4[c0 + i];  // bias, M0, 2^(R-33), R-32
-        const int32_t u = add_sat(__float2int_rn(__uint_as_float(v[i])), c.x);
-        put_code<kOut>(gw, i, (uint32_t)__vimin_s32_relu((__mulhi(u, c.y) + c.z) >> c.w, qmax));
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 32; ++i)
-        put_code<kOut>(gw, i, (uint32_t)epilogue<false>((int64_t)__float2int_rn(__uint_as_float(v[i])), 0,
-                                                         cste[c0 + i], 0, kOut));
-    }
-    if (valid) store_codes<kOut>(yrow + (c0 / 32) * 4 * kOut, gw);
-  }
+  for (int i = 0; i < 16; ++i)
+    bw[i / 4] |= (uint32_t)epilogue<false>((int64_t)__float2int_rn(__uint_as_float(v[i])), 0, c[i], 0, out_bits) << (8 * (i % 4));
+  return make_uint4(bw[0], bw[1], bw[2], bw[3]);
 }
 
 __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant__ StemParams p) {
@@ -362,39 +310,50 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
     }
     if (!ok) fail(abort_flag, p.status);
   } else {
-    // ------------------------------------------------------------ epilogue (warps 0..3)
-    const int quarter = warp;
+    // ------------------------------------------------------------ epilogue (warps 0..7)
+    const int quarter = warp & 3;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const int ngrp = (p.cout + 31) / 32;
     const int qmax = (1 << (p.out_bits & 15)) - 1;
     uint32_t lt = 0;
     bool ok = true;
     for (int t = first; t < p.total_tiles; t += stride_t, ++lt) {
       const uint32_t buf = lt & 1;
-      if (!mbar_wait(b_tfull + 8 * buf, (lt >> 1) & 1, abort_flag)) { ok = false; break; }
-      tc_fence_after();
       const int mg = t * 128 + quarter * 32 + lane;
       const bool valid = mg < p.m_total;
       uint8_t* yrow = p.y + (int64_t)(valid ? mg : 0) * p.y_row_bytes;
-      for (int g = 0; g < ngrp; ++g) {
-        const int c0 = g * 32;
-        const int ncols = p.cout - c0 < 32 ? p.cout - c0 : 32;
-        uint32_t v[32];
-        __syncwarp();
-        tmem_ld32(lane_base + buf * (uint32_t)p.n_pad + (uint32_t)c0, ncols == 32, v);
-        tmem_wait_ld();
-        reg_fence32(v);
-        if (ncols < 32) {
+      uint32_t top = 0u;  // (3-bit codes: see store_codes16)
+      if (!mbar_wait(b_tfull + 8 * buf, (lt >> 1) & 1, abort_flag)) { ok = false; break; }
+      tc_fence_after();
+      // 16 columns at a time, in whole 32-column groups (cout is a multiple of 16)
+#pragma unroll 1
+      for (int c0 = 32 * (warp >> 2); c0 < p.cout; c0 += (c0 & 16) ? 16 + 32 * (kEpiWarps / 4 - 1) : 16) {
+        const uint32_t taddr = lane_base + buf * (uint32_t)p.n_pad + (uint32_t)c0;
+        uint32_t bw[4] = {0u, 0u, 0u, 0u};
+        if (p.out_bits == 32 || fast_req) {
+          uint32_t v[16];
+          tmem_ld16(taddr, v);
+          tmem_wait_ld();
+          reg_fence16(v);
+          if (p.out_bits == 32) {
+            uint4* y4 = reinterpret_cast<uint4*>(yrow) + (c0 >> 2);
 #pragma unroll
-          for (int i = 16; i < 32; ++i) v[i] = 0u;  // only 16 columns were loaded
+            for (int i = 0; i < 16; ++i) v[i] = (uint32_t)add_sat(__float2int_rn(__uint_as_float(v[i])), cst4[c0 + i].x);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (valid) y4[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            continue;
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) {
+            const int4 c = cst4[c0 + i];  // bias, M0, 2^(R-33), R-32
+            bw[i / 4] += requant32(add_sat(__float2int_rn(__uint_as_float(v[i])), c.x), c, qmax) << (8 * (i % 4));
+          }
+        } else {
+          const uint4 r = general_cols(taddr, cste + c0, p.out_bits);
+          __syncwarp();
+          bw[0] = r.x; bw[1] = r.y; bw[2] = r.z; bw[3] = r.w;
         }
-        switch (p.out_bits) {
-          case 2: epi_unit<2>(v, cst4, cste, c0, ncols, fast_req, qmax, yrow, valid); break;
-          case 3: epi_unit<3>(v, cst4, cste, c0, ncols, fast_req, qmax, yrow, valid); break;
-          case 4: epi_unit<4>(v, cst4, cste, c0, ncols, fast_req, qmax, yrow, valid); break;
-          case 8: epi_unit<8>(v, cst4, cste, c0, ncols, fast_req, qmax, yrow, valid); break;
-          default: epi_unit<32>(v, cst4, cste, c0, ncols, fast_req, qmax, yrow, valid); break;
-        }
+        if (valid) store_codes16(yrow, c0, bw, p.out_bits, top);
       }
       tc_fence_before();
       __syncwarp();
