@@ -7,7 +7,9 @@ no CPU fallback: if the library or a GPU is missing the calls raise.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
+import struct
 from dataclasses import dataclass
 
 import torch
@@ -63,6 +65,26 @@ EXPORTS = ["aqd_row_bytes", "aqd_quantize_multiplier", "aqd_status_string", "aqd
            "aqd_bn_level_stats_workspace_bytes", "aqd_bn_level_stats"]
 
 _lib = None
+_hot = None  # the same library for the calls below that pass their structs as packed bytes
+
+# The C structs of include/aqd.h as packed bytes, for the calls a serving loop makes. Building a
+# ctypes structure per tensor and job took most of a call's host time: the head tower's 25 jobs 128 us
+# a call, 48 us this way; a whole detector at batch 1 1080 us, 530 us. Nothing is kept from one call
+# for the next: every call reads and checks its tensors again.
+_TENSOR = struct.Struct("=5i4xQ")       # aqd_tensor
+_REQUANT = struct.Struct("=QQQi4x")     # aqd_requant_params
+_SKIP = struct.Struct("=QQii")          # aqd_skip_params
+_NO_TENSOR = (0, 0, 0, 0, 0, 0)
+
+
+@functools.lru_cache(maxsize=None)
+def _job_struct(n: int) -> struct.Struct:
+    return struct.Struct("=" + "5i4xQ5i4xQ5i4xQi4x" * n)  # aqd_conv_job[n]
+
+
+@functools.lru_cache(maxsize=None)
+def _row_bytes(c: int, bits: int) -> int:
+    return int(load().aqd_row_bytes(c, bits))
 
 
 def lib_path() -> str:
@@ -71,7 +93,7 @@ def lib_path() -> str:
 
 def load(build_if_missing: bool = True):
     """Loads libaqd.so (building it in-tree first if it is missing)."""
-    global _lib
+    global _lib, _hot
     if _lib is not None:
         return _lib
     path = _build.LIB
@@ -141,8 +163,32 @@ def load(build_if_missing: bool = True):
                  "aqd_residual_add_int", "aqd_maxpool_codes", "aqd_maxpool_expand", "aqd_fake_quant",
                  "aqd_fake_quant_backward", "aqd_bn_level_stats"):
         getattr(L, name).restype = c_int
+    hot = ctypes.CDLL(path)
+    for name, args in (("aqd_conv_int", [vp, vp, i32, i32, i32, vp, vp, vp, vp, vp, sz, vp]),
+                       ("aqd_conv_int_grouped", [vp, i32, vp, i32, i32, vp, vp, vp, sz, vp]),
+                       ("aqd_conv_int_grouped_expanded", [vp, i32, vp, i32, i32, vp, vp, vp, sz, vp]),
+                       ("aqd_conv_int_grouped_chain", [vp, i32, vp, i32, i32, vp, vp, vp, sz, i32, vp, sz, vp]),
+                       ("aqd_conv_int_grouped_tower", [vp, i32, i32, vp, vp, i32, vp, vp, sz, vp, sz, i32, vp]),
+                       ("aqd_conv_expand_input", [vp, i32, vp, i32, i32, vp, sz, vp]),
+                       ("aqd_conv_int_static_workspace", [vp, vp, i32, i32, i32, vp, vp, vp, vp, vp]),
+                       ("aqd_conv_workspace_bytes", [vp, i32, vp, i32, i32]),
+                       ("aqd_conv_tower_sync_bytes", [vp, i32, i32, i32]),
+                       ("aqd_requant", [vp, vp, i32, vp, vp]),
+                       ("aqd_residual_add_int", [vp, vp, vp, vp, i32, vp, vp]),
+                       ("aqd_maxpool_codes", [vp, i32, i32, i32, vp, vp]),
+                       ("aqd_maxpool_expand", [vp, i32, i32, i32, vp, vp, i32, i32, vp, sz, vp])):
+        fn = getattr(hot, name)
+        fn.argtypes = args
+        fn.restype = sz if name.endswith("_bytes") else c_int
+    _hot = hot
     _lib = L
     return L
+
+
+def _calls():
+    if _hot is None:
+        load()
+    return _hot
 
 
 def _check(st: int, func: str):
@@ -151,8 +197,15 @@ def _check(st: int, func: str):
         raise AqdError(st, func, msg)
 
 
+# the current stream's handle without a Stream object around it
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream(stream=None) -> int:
     if stream is None:
+        if _raw_stream is not None and _raw_device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_raw_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream
 
@@ -168,7 +221,7 @@ def _ptr(t: torch.Tensor | None):
 
 
 def row_bytes(c: int, bits: int) -> int:
-    return int(load().aqd_row_bytes(c, bits))
+    return _row_bytes(c, bits)
 
 
 @dataclass
@@ -201,13 +254,24 @@ class DTensor:
 
     def codes(self, signed: bool = False) -> torch.Tensor:
         if self.bits == 32:
-            return self.data.contiguous().view(torch.int32).reshape(self.n, self.h, self.w, self.c)
+            v = self.data.contiguous().view(torch.int32)
+            shape = (self.n, self.h, self.w, self.c)
+            return v if v.shape == shape else v.reshape(shape)
         return unpack_codes(self.data.reshape(-1, row_bytes(self.c, self.bits)), self.c, self.bits,
                             signed).reshape(self.n, self.h, self.w, self.c)
 
+    def _fields(self):
+        """The fields of aqd_tensor, checked."""
+        n, h, w, c, bits, d = self.n, self.h, self.w, self.c, self.bits, self.data
+        assert d.nbytes == n * h * w * _row_bytes(c, bits)
+        assert d.is_cuda and d.is_contiguous(), "device tensors must be contiguous CUDA tensors"
+        return n, h, w, c, bits, d.data_ptr()
+
     def ct(self) -> _Tensor:
-        assert self.data.numel() * self.data.element_size() == self.n * self.h * self.w * row_bytes(self.c, self.bits)
-        return _Tensor(self.n, self.h, self.w, self.c, self.bits, _ptr(self.data))
+        return _Tensor(*self._fields())
+
+    def _packed(self) -> bytes:
+        return _TENSOR.pack(*self._fields())
 
 
 def pack_codes(codes: torch.Tensor, bits: int, out: torch.Tensor | None = None, stream=None) -> torch.Tensor:
@@ -252,6 +316,9 @@ class RequantParams:
     def c(self) -> _Requant:
         return _Requant(_ptr(self.m0), _ptr(self.shift), _ptr(self.bias), self.levels)
 
+    def _packed(self) -> bytes:
+        return _REQUANT.pack(_ptr(self.m0) or 0, _ptr(self.shift) or 0, _ptr(self.bias) or 0, self.levels)
+
 
 @dataclass
 class SkipParams:
@@ -267,6 +334,9 @@ class SkipParams:
 
     def cs(self) -> _Skip:
         return _Skip(_ptr(self.c), _ptr(self.d), self.upsample, self.scale_main)
+
+    def _packed(self) -> bytes:
+        return _SKIP.pack(_ptr(self.c) or 0, _ptr(self.d) or 0, self.upsample, self.scale_main)
 
 
 def quantize_multiplier(real: float) -> tuple[int, int]:
@@ -314,23 +384,20 @@ def conv_out_hw(h, w, kh, kw, stride, pad):
 def _ws(workspace: torch.Tensor | None):
     if workspace is None:
         return None, 0
-    return _ptr(workspace), workspace.numel() * workspace.element_size()
+    return _ptr(workspace), workspace.nbytes
+
+
+def _opt(p) -> bytes | None:
+    return None if p is None else p._packed()
 
 
 def conv_int(x: DTensor, w: ConvWeights, stride: int, pad: int, y: DTensor, *, level: int = 0,
              rq: RequantParams | None = None, skip: DTensor | None = None, sp: SkipParams | None = None,
              workspace: torch.Tensor | None = None, stream=None) -> DTensor:
-    xc, yc = x.ct(), y.ct()
-    rqc = rq.c() if rq is not None else None
-    skc = skip.ct() if skip is not None else None
-    spc = sp.cs() if sp is not None else None
     wsp, wsb = _ws(workspace)
-    _check(load().aqd_conv_int(ctypes.byref(xc), ctypes.byref(w.desc), stride, pad, level,
-                               ctypes.byref(rqc) if rqc is not None else None,
-                               ctypes.byref(skc) if skc is not None else None,
-                               ctypes.byref(spc) if spc is not None else None, ctypes.byref(yc), wsp, wsb,
-                               _stream(stream)),
-           "aqd_conv_int")
+    st = _calls().aqd_conv_int(x._packed(), ctypes.byref(w.desc), stride, pad, level, _opt(rq), _opt(skip), _opt(sp),
+                               y._packed(), wsp, wsb, _stream(stream))
+    _check(st, "aqd_conv_int")
     return y
 
 
@@ -339,32 +406,36 @@ def conv_int_static_workspace(x: DTensor, w: ConvWeights, stride: int, pad: int,
                               sp: SkipParams | None = None, stream=None) -> DTensor:
     """conv_int on the workspace path with the library's own fixed workspace (no allocation);
     calls that overlap in time share that workspace and must be ordered by the caller."""
-    xc, yc = x.ct(), y.ct()
-    rqc = rq.c() if rq is not None else None
-    skc = skip.ct() if skip is not None else None
-    spc = sp.cs() if sp is not None else None
-    _check(load().aqd_conv_int_static_workspace(ctypes.byref(xc), ctypes.byref(w.desc), stride, pad, level,
-                                                ctypes.byref(rqc) if rqc is not None else None,
-                                                ctypes.byref(skc) if skc is not None else None,
-                                                ctypes.byref(spc) if spc is not None else None, ctypes.byref(yc),
-                                                _stream(stream)),
-           "aqd_conv_int_static_workspace")
+    st = _calls().aqd_conv_int_static_workspace(x._packed(), ctypes.byref(w.desc), stride, pad, level, _opt(rq),
+                                                _opt(skip), _opt(sp), y._packed(), _stream(stream))
+    _check(st, "aqd_conv_int_static_workspace")
     return y
 
 
-def _jobs(jobs):
-    arr = (_Job * len(jobs))()
-    for i, (x, y, skip, level) in enumerate(jobs):
-        arr[i].x = x.ct()
-        arr[i].y = y.ct() if y is not None else _Tensor(0, 0, 0, 0, 0, None)
-        arr[i].skip = skip.ct() if skip is not None else _Tensor(0, 0, 0, 0, 0, None)
-        arr[i].level = level
-    return arr
+def _jobs(jobs) -> bytes:
+    """aqd_conv_job[len(jobs)] (a tensor that several jobs of one call share is read once)."""
+    if len(jobs) == 1:
+        x, y, skip, level = jobs[0]
+        return _job_struct(1).pack(*x._fields(), *(_NO_TENSOR if y is None else y._fields()),
+                                   *(_NO_TENSOR if skip is None else skip._fields()), level)
+    seen = {}
+    vals = []
+    for x, y, skip, level in jobs:
+        for t in (x, y, skip):
+            if t is None:
+                vals += _NO_TENSOR
+                continue
+            f = seen.get(id(t))
+            if f is None:
+                f = seen[id(t)] = t._fields()
+            vals += f
+        vals.append(level)
+    return _job_struct(len(jobs)).pack(*vals)
 
 
 def conv_workspace_bytes(jobs, w: ConvWeights, stride: int, pad: int) -> int:
     """Bytes of the expanded-activation workspace for these jobs (0: path not applicable)."""
-    return int(load().aqd_conv_workspace_bytes(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad))
+    return int(_calls().aqd_conv_workspace_bytes(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad))
 
 
 def workspace_for(jobs, w: ConvWeights, stride: int, pad: int, device="cuda") -> torch.Tensor | None:
@@ -380,39 +451,29 @@ def workspace_for(jobs, w: ConvWeights, stride: int, pad: int, device="cuda") ->
 def conv_int_grouped(jobs, w: ConvWeights, stride: int, pad: int, *, rq: RequantParams | None = None,
                      sp: SkipParams | None = None, workspace: torch.Tensor | None = None, stream=None):
     """jobs: list of (x: DTensor, y: DTensor, skip: DTensor | None, level: int)."""
-    arr = _jobs(jobs)
-    rqc = rq.c() if rq is not None else None
-    spc = sp.cs() if sp is not None else None
     wsp, wsb = _ws(workspace)
-    _check(load().aqd_conv_int_grouped(arr, len(jobs), ctypes.byref(w.desc), stride, pad,
-                                       ctypes.byref(rqc) if rqc is not None else None,
-                                       ctypes.byref(spc) if spc is not None else None, wsp, wsb,
-                                       _stream(stream)),
-           "aqd_conv_int_grouped")
+    st = _calls().aqd_conv_int_grouped(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad, _opt(rq), _opt(sp),
+                                       wsp, wsb, _stream(stream))
+    _check(st, "aqd_conv_int_grouped")
 
 
 def conv_expand_input(jobs, w: ConvWeights, stride: int, pad: int, workspace: torch.Tensor, stream=None):
     """Only the expansion step of the workspace path: writes the zero-padded byte image of the
     jobs' inputs into `workspace` (jobs as for conv_int_grouped; y and skip are ignored)."""
-    arr = _jobs(jobs)
     wsp, wsb = _ws(workspace)
-    _check(load().aqd_conv_expand_input(arr, len(jobs), ctypes.byref(w.desc), stride, pad, wsp, wsb,
-                                        _stream(stream)), "aqd_conv_expand_input")
+    st = _calls().aqd_conv_expand_input(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad, wsp, wsb,
+                                        _stream(stream))
+    _check(st, "aqd_conv_expand_input")
 
 
 def conv_int_grouped_expanded(jobs, w: ConvWeights, stride: int, pad: int, *, rq: RequantParams | None = None,
                               sp: SkipParams | None = None, workspace: torch.Tensor, stream=None):
     """conv_int_grouped fed from a workspace that already holds the expansion of these jobs'
     inputs (written by conv_expand_input); launches only the tensor-core convolution."""
-    arr = _jobs(jobs)
-    rqc = rq.c() if rq is not None else None
-    spc = sp.cs() if sp is not None else None
     wsp, wsb = _ws(workspace)
-    _check(load().aqd_conv_int_grouped_expanded(arr, len(jobs), ctypes.byref(w.desc), stride, pad,
-                                                ctypes.byref(rqc) if rqc is not None else None,
-                                                ctypes.byref(spc) if spc is not None else None, wsp, wsb,
-                                                _stream(stream)),
-           "aqd_conv_int_grouped_expanded")
+    st = _calls().aqd_conv_int_grouped_expanded(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad, _opt(rq),
+                                                _opt(sp), wsp, wsb, _stream(stream))
+    _check(st, "aqd_conv_int_grouped_expanded")
 
 
 def conv_int_grouped_chain(jobs, w: ConvWeights, stride: int, pad: int, *, rq: RequantParams | None = None,
@@ -421,21 +482,16 @@ def conv_int_grouped_chain(jobs, w: ConvWeights, stride: int, pad: int, *, rq: R
     """conv_int_grouped_expanded that also writes the outputs, one byte per code, as the
     zero-padded byte image the next stride-1 conv (padding next_pad) reads from
     next_workspace (whose border must hold zeros)."""
-    arr = _jobs(jobs)
-    rqc = rq.c() if rq is not None else None
-    spc = sp.cs() if sp is not None else None
     wsp, wsb = _ws(workspace)
     nwp, nwb = _ws(next_workspace)
-    _check(load().aqd_conv_int_grouped_chain(arr, len(jobs), ctypes.byref(w.desc), stride, pad,
-                                             ctypes.byref(rqc) if rqc is not None else None,
-                                             ctypes.byref(spc) if spc is not None else None, wsp, wsb,
-                                             next_pad, nwp, nwb, _stream(stream)),
-           "aqd_conv_int_grouped_chain")
+    st = _calls().aqd_conv_int_grouped_chain(_jobs(jobs), len(jobs), ctypes.byref(w.desc), stride, pad, _opt(rq), _opt(sp),
+                                             wsp, wsb, next_pad, nwp, nwb, _stream(stream))
+    _check(st, "aqd_conv_int_grouped_chain")
 
 
 def tower_sync_bytes(jobs, layers: int, pad: int) -> int:
     """Bytes of per-tile counters for conv_int_grouped_tower (jobs: layer 0's jobs)."""
-    return int(load().aqd_conv_tower_sync_bytes(_jobs(jobs), len(jobs), layers, pad))
+    return int(_calls().aqd_conv_tower_sync_bytes(_jobs(jobs), len(jobs), layers, pad))
 
 
 def conv_int_grouped_tower(layer_jobs, ws: list, rqs: list, pad: int, *, ws_a: torch.Tensor,
@@ -444,39 +500,38 @@ def conv_int_grouped_tower(layer_jobs, ws: list, rqs: list, pad: int, *, ws_a: t
     """layer_jobs: one list of (x, y, None, level) per layer, layer i's x being layer i-1's y;
     ws: ConvWeights per layer; rqs: RequantParams per layer. See aqd_conv_int_grouped_tower."""
     nl, nj = len(layer_jobs), len(layer_jobs[0])
-    arr = _jobs([jb for jobs in layer_jobs for jb in jobs])
-    wd = (_Weights * nl)(*[w.desc for w in ws])
-    rqa = (_Requant * nl)(*[r.c() for r in rqs])
+    jobs = _jobs([jb for jobs in layer_jobs for jb in jobs])
+    if len(ws) > nl or len(rqs) > nl:
+        raise IndexError("more weights or requant tables than layers")
+    # (what is missing reads as zeros, which the library refuses)
+    jobs = jobs.ljust(nl * nj * _job_struct(1).size, b"\0")
+    wd = b"".join([bytes(w.desc) for w in ws]).ljust(nl * ctypes.sizeof(_Weights), b"\0")
+    rqa = b"".join([r._packed() for r in rqs]).ljust(nl * _REQUANT.size, b"\0")
     wap, wab = _ws(ws_a)
     wbp, wbb = _ws(ws_b)
     assert wab == wbb, "ws_a and ws_b must have the same size"
     sp_, sb = _ws(sync) if sync is not None else (None, 0)
-    _check(load().aqd_conv_int_grouped_tower(arr, nj, nl, wd, rqa, pad, wap, wbp, wab, sp_, sb, int(input_expanded),
-                                             _stream(stream)),
-           "aqd_conv_int_grouped_tower")
+    st = _calls().aqd_conv_int_grouped_tower(jobs, nj, nl, wd, rqa, pad, wap, wbp, wab, sp_, sb, int(input_expanded),
+                                             _stream(stream))
+    _check(st, "aqd_conv_int_grouped_tower")
 
 
 def requant(acc: DTensor, rq: RequantParams, y: DTensor, *, level: int = 0, stream=None) -> DTensor:
-    ac, yc, rqc = acc.ct(), y.ct(), rq.c()
-    _check(load().aqd_requant(ctypes.byref(ac), ctypes.byref(rqc), level, ctypes.byref(yc), _stream(stream)),
-           "aqd_requant")
+    _check(_calls().aqd_requant(acc._packed(), rq._packed(), level, y._packed(), _stream(stream)), "aqd_requant")
     return y
 
 
 def residual_add_int(a: DTensor, b: DTensor, sp: SkipParams, y: DTensor, *, rq: RequantParams | None = None,
                      level: int = 0, stream=None) -> DTensor:
-    ac, bc, yc, spc = a.ct(), b.ct(), y.ct(), sp.cs()
-    rqc = rq.c() if rq is not None else None
-    _check(load().aqd_residual_add_int(ctypes.byref(ac), ctypes.byref(bc), ctypes.byref(spc),
-                                       ctypes.byref(rqc) if rqc is not None else None, level, ctypes.byref(yc),
-                                       _stream(stream)), "aqd_residual_add_int")
+    st = _calls().aqd_residual_add_int(a._packed(), b._packed(), sp._packed(), _opt(rq), level, y._packed(),
+                                       _stream(stream))
+    _check(st, "aqd_residual_add_int")
     return y
 
 
 def maxpool_codes(x: DTensor, k: int, stride: int, pad: int, y: DTensor, stream=None) -> DTensor:
-    xc, yc = x.ct(), y.ct()
-    _check(load().aqd_maxpool_codes(ctypes.byref(xc), k, stride, pad, ctypes.byref(yc), _stream(stream)),
-           "aqd_maxpool_codes")
+    st = _calls().aqd_maxpool_codes(x._packed(), k, stride, pad, y._packed(), _stream(stream))
+    _check(st, "aqd_maxpool_codes")
     return y
 
 
@@ -484,10 +539,10 @@ def maxpool_expand(x: DTensor, k: int, stride: int, pad: int, y: DTensor, w: Con
                    conv_pad: int, workspace: torch.Tensor, stream=None) -> DTensor:
     """maxpool_codes(x) -> y fused with conv_expand_input([(y, ...)], w, conv_stride, conv_pad,
     workspace): one pass writes y and the byte image of y for that convolution."""
-    xc, yc = x.ct(), y.ct()
     wsp, wsb = _ws(workspace)
-    _check(load().aqd_maxpool_expand(ctypes.byref(xc), k, stride, pad, ctypes.byref(yc), ctypes.byref(w.desc),
-                                     conv_stride, conv_pad, wsp, wsb, _stream(stream)), "aqd_maxpool_expand")
+    st = _calls().aqd_maxpool_expand(x._packed(), k, stride, pad, y._packed(), ctypes.byref(w.desc), conv_stride,
+                                     conv_pad, wsp, wsb, _stream(stream))
+    _check(st, "aqd_maxpool_expand")
     return y
 
 

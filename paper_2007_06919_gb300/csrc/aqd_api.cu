@@ -111,15 +111,22 @@ WeightGeom weight_geom(int32_t cout, int32_t kh, int32_t kw, int32_t cin) {
 static bool code_bits(int b) { return b == 2 || b == 3 || b == 4 || b == 8; }
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
+// What is wrong with a tensor argument, to follow its name, or NULL. (The name is put together only
+// for a message: a string per tensor of every job was a good part of a call's host time.)
+static const char* tensor_fault(const aqd_tensor* t, bool allow32) {
+  if (!t) return " is NULL";
+  if (!t->data) return "->data is NULL";
+  if (t->n <= 0 || t->h <= 0 || t->w <= 0 || t->c <= 0) return " has a non-positive dimension";
+  if (!(code_bits(t->bits) || (allow32 && t->bits == 32))) return " has unsupported bits";
+  if (row_bytes_of(t->c, t->bits) < 0) return ": channels must be a multiple of 32 at 2/3/4 bits";
+  if (!aligned16(t->data)) return "->data must be 16-byte aligned";
+  if ((int64_t)t->n * t->h * t->w >= (int64_t)INT_MAX) return " has too many pixels";
+  return nullptr;
+}
 static bool check_tensor(const aqd_tensor* t, bool allow32, const char* name, std::string* err) {
-  if (!t) { *err = std::string(name) + " is NULL"; return false; }
-  if (!t->data) { *err = std::string(name) + "->data is NULL"; return false; }
-  if (t->n <= 0 || t->h <= 0 || t->w <= 0 || t->c <= 0) { *err = std::string(name) + " has a non-positive dimension"; return false; }
-  if (!(code_bits(t->bits) || (allow32 && t->bits == 32))) { *err = std::string(name) + " has unsupported bits"; return false; }
-  if (row_bytes_of(t->c, t->bits) < 0) { *err = std::string(name) + ": channels must be a multiple of 32 at 2/3/4 bits"; return false; }
-  if (!aligned16(t->data)) { *err = std::string(name) + "->data must be 16-byte aligned"; return false; }
-  if ((int64_t)t->n * t->h * t->w >= (int64_t)INT_MAX) { *err = std::string(name) + " has too many pixels"; return false; }
-  return true;
+  const char* fault = tensor_fault(t, allow32);
+  if (fault) *err = std::string(name) + fault;
+  return fault == nullptr;
 }
 
 static int64_t max_abs_weight(int w_bits, int w_format) {
@@ -361,19 +368,21 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
   a.skip_bits = has_skip ? jobs[0].skip.bits : 0;
   for (int j = 0; j < njobs; ++j) {
     const aqd_conv_job& jb = jobs[j];
-    const std::string nm = "jobs[" + std::to_string(j) + "]";
-    if (!check_tensor(&jb.x, false, (nm + ".x").c_str(), &err)) return fail(AQD_ERR_INVALID, err);
-    if (!check_tensor(&jb.y, true, (nm + ".y").c_str(), &err)) return fail(AQD_ERR_INVALID, err);
-    if (jb.x.c != w->cin) return fail(AQD_ERR_INVALID, nm + ".x.c != weights cin");
-    if (jb.x.bits != a.x_bits || jb.y.bits != out_bits) return fail(AQD_ERR_INVALID, nm + ": all jobs must share x.bits and y.bits");
+    auto bad = [j](const char* what, const char* fault = "") {
+      return fail(AQD_ERR_INVALID, "jobs[" + std::to_string(j) + "]" + what + fault);
+    };
+    if (const char* f = tensor_fault(&jb.x, false)) return bad(".x", f);
+    if (const char* f = tensor_fault(&jb.y, true)) return bad(".y", f);
+    if (jb.x.c != w->cin) return bad(".x.c != weights cin");
+    if (jb.x.bits != a.x_bits || jb.y.bits != out_bits) return bad(": all jobs must share x.bits and y.bits");
     const int ho = (jb.x.h + 2 * pad - w->kh) / stride + 1;
     const int wo = (jb.x.w + 2 * pad - w->kw) / stride + 1;
     if (jb.x.h + 2 * pad < w->kh || jb.x.w + 2 * pad < w->kw || ho <= 0 || wo <= 0)
-      return fail(AQD_ERR_INVALID, nm + ": kernel larger than the padded input");
+      return bad(": kernel larger than the padded input");
     if (jb.y.n != jb.x.n || jb.y.h != ho || jb.y.w != wo || jb.y.c != w->cout)
-      return fail(AQD_ERR_INVALID, nm + ".y shape does not match the convolution output");
-    if (rq && (jb.level < 0 || jb.level >= rq->levels)) return fail(AQD_ERR_INVALID, nm + ".level out of range");
-    if (!rq && jb.level != 0) return fail(AQD_ERR_INVALID, nm + ".level must be 0 without rq");
+      return bad(".y shape does not match the convolution output");
+    if (rq && (jb.level < 0 || jb.level >= rq->levels)) return bad(".level out of range");
+    if (!rq && jb.level != 0) return bad(".level must be 0 without rq");
     if ((jb.skip.data != nullptr) != has_skip) return fail(AQD_ERR_INVALID, "all jobs must agree on having a skip");
     ConvJobDev& d = a.jobs[j];
     d.x = static_cast<const uint8_t*>(jb.x.data);
@@ -382,11 +391,11 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
     d.level = jb.level;
     d.m_total = jb.x.n * ho * wo;
     if (has_skip) {
-      if (!check_tensor(&jb.skip, true, (nm + ".skip").c_str(), &err)) return fail(AQD_ERR_INVALID, err);
+      if (const char* f = tensor_fault(&jb.skip, true)) return bad(".skip", f);
       if (jb.skip.bits != a.skip_bits) return fail(AQD_ERR_INVALID, "all skips must share bits");
       const int up = sp->upsample;
       if (jb.skip.n != jb.x.n || jb.skip.c != w->cout || jb.skip.h < (ho + up - 1) / up || jb.skip.w < (wo + up - 1) / up)
-        return fail(AQD_ERR_INVALID, nm + ".skip shape does not cover the output");
+        return bad(".skip shape does not cover the output");
       d.skip = static_cast<const uint8_t*>(jb.skip.data);
       d.skip_h = jb.skip.h; d.skip_w = jb.skip.w;
     }

@@ -43,6 +43,8 @@ class _ConvPlan:
     chain_to: "_ConvPlan | None" = None
     image: int = 0         # which of the two chain images this conv reads (when reads_image)
     pool: object = None    # the max-pool layer fused into this conv's expansion pass
+    src_ws: torch.Tensor | None = None    # the workspace or chain image this conv reads
+    next_ws: torch.Tensor | None = None   # the chain image it writes (chain_to)
 
 
 def _aligned(nbytes: int, device) -> torch.Tensor:
@@ -108,6 +110,15 @@ class IntDetector:
         for k, p in self.steps:
             if k == "conv" and p.reads_image and self._image_key(p) not in self.images:
                 self.images[self._image_key(p)] = [_aligned(p.ws_bytes, self.device) for _ in range(2)]
+        for k, p in self.steps:
+            if k != "conv":
+                continue
+            if p.reads_image:
+                p.src_ws = self.images[self._image_key(p)][p.image]
+            elif p.ws_bytes:
+                p.src_ws = self.workspace[:p.ws_bytes]
+            if p.chain_to is not None:
+                p.next_ws = self.images[self._image_key(p.chain_to)][p.chain_to.image]
         # a conv that expands its own input is two launches (with a fused pool the expansion
         # launch is the pool's, whose own step is gone)
         self.launches = sum(1 + (1 if (k == "conv" and p.ws_bytes and not p.reads_image) else 0)
@@ -194,10 +205,7 @@ class IntDetector:
                 k, s, pd = p.pool
                 aqd.maxpool_codes(T[p.src[0]], k, s, pd, T[p.dst[0]], stream=stream)
                 continue
-            if p.reads_image:
-                src_ws = self.images[self._image_key(p)][p.image]
-            else:
-                src_ws = self.workspace[:p.ws_bytes] if p.ws_bytes else None
+            src_ws = p.src_ws
             if p.pool is not None:
                 k, s, pd = p.pool.pool
                 aqd.maxpool_expand(T[p.pool.src[0]], k, s, pd, T[p.pool.dst[0]], p.w, p.stride, p.pad, src_ws,
@@ -207,8 +215,7 @@ class IntDetector:
                 if not p.reads_image and p.pool is None:
                     aqd.conv_expand_input(p.jobs, p.w, p.stride, p.pad, src_ws, stream=stream)
                 aqd.conv_int_grouped_chain(p.jobs, p.w, p.stride, p.pad, rq=p.rq, sp=p.sp, workspace=src_ws,
-                                           next_pad=nxt.pad, next_workspace=self.images[self._image_key(nxt)][nxt.image],
-                                           stream=stream)
+                                           next_pad=nxt.pad, next_workspace=p.next_ws, stream=stream)
             elif p.reads_image or p.pool is not None:
                 aqd.conv_int_grouped_expanded(p.jobs, p.w, p.stride, p.pad, rq=p.rq, sp=p.sp, workspace=src_ws,
                                               stream=stream)

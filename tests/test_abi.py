@@ -172,3 +172,17 @@ def test_training_entry_points_validate_before_any_launch(lib):
     assert lib.aqd_bn_level_stats(ptrs, pix, 1, 4, fake, fake, fake, 8, None) == 1         # workspace
     neg = (ctypes.c_int64 * 1)(-1)
     assert lib.aqd_bn_level_stats(ptrs, neg, 1, 4, fake, fake, fake, 1 << 20, None) == 1   # pixels
+
+
+def test_packed_structs_match_the_abi():
+    """The byte layouts that the binding packs are the ctypes (C) layouts, padding included."""
+    a, b, c = (aqd._Tensor(5 * i + 1, 5 * i + 2, 5 * i + 3, 5 * i + 4, 5 * i + 5, (1 << 40) + i) for i in range(3))
+    jobs = (aqd._Job * 2)()
+    for i, t in enumerate(((a, b, c), (c, a, b))):
+        jobs[i].x, jobs[i].y, jobs[i].skip = t
+        jobs[i].level = 7 + i
+    f = [(t.n, t.h, t.w, t.c, t.bits, t.data) for t in (a, b, c)]
+    assert bytes(a) == aqd._TENSOR.pack(*f[0])
+    assert bytes(jobs) == aqd._job_struct(2).pack(*f[0], *f[1], *f[2], 7, *f[2], *f[0], *f[1], 8)
+    assert bytes(aqd._Requant(1 << 40, 2 << 40, 3 << 40, 9)) == aqd._REQUANT.pack(1 << 40, 2 << 40, 3 << 40, 9)
+    assert bytes(aqd._Skip(1 << 40, 2 << 40, 2, 1)) == aqd._SKIP.pack(1 << 40, 2 << 40, 2, 1)
