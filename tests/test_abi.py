@@ -176,6 +176,7 @@ def test_training_entry_points_validate_before_any_launch(lib):
 
 def test_packed_structs_match_the_abi():
     """The byte layouts that the binding packs are the ctypes (C) layouts, padding included."""
+    from paper_2007_06919_gb300 import aqd
     a, b, c = (aqd._Tensor(5 * i + 1, 5 * i + 2, 5 * i + 3, 5 * i + 4, 5 * i + 5, (1 << 40) + i) for i in range(3))
     jobs = (aqd._Job * 2)()
     for i, t in enumerate(((a, b, c), (c, a, b))):
