@@ -412,6 +412,7 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
   const WeightGeom g = weight_geom(w->cout, w->kh, w->kw, w->cin);
   a.w_e4m3 = static_cast<const uint8_t*>(w->data);
   a.w_i16 = reinterpret_cast<const int16_t*>(static_cast<const uint8_t*>(w->data) + g.i16_offset);
+  a.w_f16 = w->w_bits == 8 ? 1 : 0;
   a.cout_pad = g.cout_pad; a.k_total = g.k_total; a.k_pad = g.k_pad; a.bn = g.bn;
   a.split_rows = g.split_rows;
   a.a_planes = 1;
@@ -451,6 +452,9 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
       a.ws_rows = (int64_t)(ws_bytes / ((size_t)planes * (size_t)w->cin));
       a.a_planes = planes;
       a.split_w = (!tc_ok && split_weights(w)) ? 1 : 0;
+      // both operands 8 bits wide: F16 holds either, so one product takes the place of the split
+      // form's four (the image has the two planes' bytes: one F16 value per code)
+      if (a.split_w && planes == 2) { a.f16 = 1; a.split_w = 0; a.a_planes = 1; }
     }
   }
   if (path == 1 && !tc_ok && !a.ws) path = 2;  // the split form exists only on the workspace path
@@ -477,7 +481,7 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
     const size_t need = (size_t)orows * (size_t)w->cout;
     if (chain->bytes < need) return fail(AQD_ERR_INVALID, "next_workspace is too small");
     const uintptr_t i0 = reinterpret_cast<uintptr_t>(workspace), o0 = reinterpret_cast<uintptr_t>(chain->ws);
-    const size_t in_need = (size_t)flat_rows(jobs, njobs, w, stride, pad) * (size_t)a.a_planes * (size_t)w->cin;
+    const size_t in_need = (size_t)flat_rows(jobs, njobs, w, stride, pad) * (size_t)(a.f16 ? 2 : a.a_planes) * (size_t)w->cin;
     if (i0 < o0 + need && o0 < i0 + in_need) return fail(AQD_ERR_INVALID, "workspace and next_workspace overlap");
     a.ws_out = static_cast<uint8_t*>(chain->ws);
     a.out_pad = chain->pad;
@@ -658,7 +662,7 @@ aqd_status aqd_conv_int_grouped_tower(const aqd_conv_job* jobs, int32_t njobs, i
              a.acc_bound == b.acc_bound;
     };
     auto fusable = [&](const ConvArgs& a) {
-      return conv_tc_uses_pair(a) && !a.split_w && a.a_planes <= 1 && a.bn == a.cout_pad && a.ws_out != nullptr;
+      return conv_tc_uses_pair(a) && !a.split_w && !a.f16 && a.a_planes <= 1 && a.bn == a.cout_pad && a.ws_out != nullptr;
     };
     while (fused < layers && fused < kMaxLayers && fusable(plans[fused - 1].a) && plans[fused].path == 1 &&
            same_shape(plans[0].a, plans[fused].a) && conv_tc_uses_pair(plans[fused].a))
@@ -806,7 +810,7 @@ aqd_status aqd_maxpool_expand(const aqd_tensor* x, int32_t k, int32_t stride, in
   const aqd_status s = plan_grouped(&job, 1, w, conv_stride, conv_pad, nullptr, nullptr, workspace, ws_bytes,
                                     kStageExpandOnly, nullptr, true, &plan);
   if (s != AQD_OK) return s;
-  if (plan.path != 1 || plan.a.a_planes != 1 || plan.a.fp4 || plan.a.cin != y->c || plan.a.jobs[0].row_off != 0)
+  if (plan.path != 1 || plan.a.a_planes != 1 || plan.a.f16 || plan.a.fp4 || plan.a.cin != y->c || plan.a.jobs[0].row_off != 0)
     return fail(AQD_ERR_UNSUPPORTED, "the convolution does not read a one-plane byte image");
   PoolArgs p{};
   p.x = static_cast<const uint8_t*>(x->data); p.y = static_cast<uint8_t*>(y->data);

@@ -6,6 +6,7 @@
 // multiple of 32 (the 3-channel image), and products too large for the exact FP32
 // accumulation bound. Each thread owns one output pixel and 32 output channels; the
 // block's 32 weight rows are staged in shared memory K-chunk by K-chunk.
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -56,7 +57,9 @@ conv_direct_kernel(const ConvArgs a, int job_index) {
     for (int i = threadIdx.x; i < kKC * 32; i += kThreads) {
       const int kk = i / 32, j = i % 32;
       const int co = co0 + j;
-      wsm[kk][j] = (kk < kc && co < a.cout) ? a.w_i16[(int64_t)co * a.k_total + k0 + kk] : (int16_t)0;
+      int16_t w = (kk < kc && co < a.cout) ? a.w_i16[(int64_t)co * a.k_total + k0 + kk] : (int16_t)0;
+      if (a.w_f16) w = (int16_t)__half2int_rn(__short_as_half(w));
+      wsm[kk][j] = w;
     }
     __syncthreads();
     int tap = k0 / a.cin;

@@ -17,6 +17,11 @@
 // nibble image keeps the byte image's row stride (cin bytes) and fills the first cin / 2
 // bytes of each row, so its zero border lies where a byte image's does in the same workspace.
 //
+// 8-bit codes with 8-bit weights on the F16 pipe (kF16): F16 holds either exactly, every product is
+// an integer below 2^15, and the FP32 accumulator is exact over 512 K elements (512 * 255 * 128 <
+// 2^24). K runs in segments of that length, each in its own TMEM accumulator; the epilogue warps
+// add the segments as int32 in registers. The image holds F16 values (2 cin bytes a row).
+//
 // Per CTA (one per SM, persistent over tiles of 128 output pixels x BN channels):
 //   warps 0..E-1  epilogue (E = 16, or 8 beside activation producers): tcgen05.ld of the
 //              accumulator, integer epilogue, bit-pack, store (warp w reads TMEM lanes
@@ -107,6 +112,7 @@ struct Params {
   uint32_t off_b, off_epi, off_bar, off_qtab;
   uint32_t off_ostage;  // int32 outputs: per-warp staging blocks for row-contiguous stores (0: none)
   int32_t out_pad;
+  int32_t seg_chunks; // kF16: K chunks per exact FP32 segment (512 K elements)
   int32_t a_planes;   // K runs over this many planes of the byte image (2: 8-bit activations)
   int32_t plane_rows; // workspace rows per plane
   int32_t split_w;    // weights in the split layout: a tile's bn B rows give bn/2 channels
@@ -298,22 +304,8 @@ struct GenCols {
 // and there is no skip (accumulators too large for the common form). Returns the codes as
 // byte-words; int32 outputs and 8-bit rows of no whole groups are stored here. Not inlined: its
 // registers and code stay out of the common forms.
-template <bool kSkip, bool kSplit>
-__device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, float sc) {
-  uint32_t v[16];
-  tmem_ld16(u.taddr, v);
-  tmem_wait_ld();
-  reg_fence16(v);
-  int32_t acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = __float2int_rn(__uint_as_float(v[i]) * sc);
-  if constexpr (kSplit) {
-    tmem_ld16(u.taddr_hi, v);
-    tmem_wait_ld();
-    reg_fence16(v);
-#pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
-  }
+template <bool kSkip>
+__device__ __noinline__ uint4 general_finish(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
   if (!u.row_ok) return make_uint4(0u, 0u, 0u, 0u);
   if (!kSkip && (u.flags & kFlagReq) && p.out_bits != 32) {
     const int qmax = (1 << p.out_bits) - 1;
@@ -349,6 +341,26 @@ __device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, fl
     bw[j] = (uint32_t)acc[4 * j] | ((uint32_t)acc[4 * j + 1] << 8) | ((uint32_t)acc[4 * j + 2] << 16) |
             ((uint32_t)acc[4 * j + 3] << 24);
   return make_uint4(bw[0], bw[1], bw[2], bw[3]);
+}
+
+// The same from the accumulators in TMEM.
+template <bool kSkip, bool kSplit>
+__device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, float sc) {
+  uint32_t v[16];
+  tmem_ld16(u.taddr, v);
+  tmem_wait_ld();
+  reg_fence16(v);
+  int32_t acc[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) acc[i] = __float2int_rn(__uint_as_float(v[i]) * sc);
+  if constexpr (kSplit) {
+    tmem_ld16(u.taddr_hi, v);
+    tmem_wait_ld();
+    reg_fence16(v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
+  }
+  return general_finish<kSkip>(p, u, acc);
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -422,6 +434,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   static_assert(!kPair || kFlat, "the CTA-pair form exists for the workspace path only");
   static_assert(kBK == BK || kFlat, "64-byte K chunks exist for the workspace path only");
   static_assert(!kFp4 || (kFlat && kBK == BK && !kSplit), "the FP4 pipe reads nibble images in 128-byte chunks");
+  constexpr bool kF16 = kXBits == 8;  // (flat kernels read images: kXBits names the pipe only here)
+  static_assert(!kF16 || (kFlat && kBK == BK && !kSplit && !kFp4 && !kSkip && !kOStage), "the F16 pipe's form");
   // the FP32 accumulator holds the integer sum / kAccSc
   constexpr float kAccSc = kFp4 ? 4.0f : 262144.0f;
   constexpr int kStA = BM * kBK;  // bytes of one stage's A operand
@@ -556,14 +570,19 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       uint32_t it = 0, lt = 0, s = 0, ph = 0;
       bool ok = true;
       bool next_ready = false;  // the stage after the current one is known to be full
-      for (int t = first_tile; t < tile_end && ok; t += tile_stride, ++lt) {
+      for (int t = first_tile; t < tile_end && ok; t += tile_stride) {
+       // (kF16: a tile's segments take accumulators in turn, as tiles do otherwise)
+       const int nseg = kF16 ? (nk + p.seg_chunks - 1) / p.seg_chunks : 1;
+       for (int sg = 0; sg < nseg && ok; ++sg, ++lt) {
         const uint32_t buf = lt & buf_mask;
         // (a launch of several layers has no half-width tiles)
         const uint32_t idesc = p.nlayers > 1 || t < p.dp_tiles ? idesc_full : idesc_half;
+        const int q_end = kF16 ? ((sg + 1) * p.seg_chunks < nk ? (sg + 1) * p.seg_chunks : nk) : nk;
+        const int q_0 = kF16 ? sg * p.seg_chunks : 0;
         if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + buf * (uint32_t)BN;
-        for (int q = 0; q < nk; ++q, ++it) {
+        for (int q = q_0; q < q_end; ++q, ++it) {
           // (operands written by TMA, or by producer threads followed by fence.proxy.async,
           // are ordered for the MMA by the mbarrier phase alone; tcgen05.fence is needed only
           // where TMEM changes hands, after the accumulator-empty wait above)
@@ -578,11 +597,13 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             // the previous MMA. Testing the next stage here, while the last MMAs of this
             // chunk run, lets the next chunk's first MMA follow this chunk's commit at once.
             if (kk == kBK / 32 - 1) next_ready = mbar_test(b_full + 8 * s_next, ph_next);
-            const uint32_t acc = (q > 0 || kk > 0) ? 1u : 0u;
+            const uint32_t acc = (q > q_0 || kk > 0) ? 1u : 0u;
             const uint64_t db = ((uint64_t)b_hi << 32) | (b_lo + 2 * kk);
             const uint64_t da = ((uint64_t)a_hi << 32) | (a_lo + 2 * kk);
             if constexpr (kPair && kFp4) mma_fp4_pair(d0, da, db, idesc, sfa, sfb, acc);
+            else if constexpr (kPair && kF16) mma_f16_pair(d0, da, db, idesc, acc);
             else if constexpr (kPair) mma_e4m3_pair(d0, da, db, idesc, acc);
+            else if constexpr (kF16) mma_f16(d0, da, db, idesc, acc);
             else if constexpr (kFp4) mma_fp4(d0, da, db, idesc, sfa, sfb, acc);
             else mma_e4m3(d0, da, db, idesc, acc);
           }
@@ -594,6 +615,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
           if constexpr (kPair) mma_commit_pair_both(b_tfull + 8 * buf);
           else mma_commit(b_tfull + 8 * buf);
         }
+       }
       }
       if (!ok) fail(abort_flag, p.status);
       // drain: every MMA issued above has completed once this barrier flips
@@ -814,6 +836,80 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         cur_key = key;
       }
       if ((int)(lt & (uint32_t)(p.epi_sets - 1)) != gset) continue;  // another set's tile (or an idle warp)
+      if constexpr (kF16) {
+        // this warp's columns: whole 32-column groups, at most 64 (one int32 sum each per lane)
+        const int per = ((TBN + 31) / 32 + p.epi_groups - 1) / p.epi_groups * 32;
+        const int c_lo = grp * per, c_hi = c_lo + per < TBN ? c_lo + per : TBN;
+        int32_t sum[64];
+#pragma unroll
+        for (int i = 0; i < 64; ++i) sum[i] = 0;
+        const int nseg = (nk + p.seg_chunks - 1) / p.seg_chunks;
+#pragma unroll 1
+        for (int sg = 0; sg < nseg; ++sg) {
+          const uint32_t un = lt * (uint32_t)nseg + (uint32_t)sg, b = un & buf_mask;
+          if (!mbar_wait(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          __syncwarp();
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            if (c_lo + 16 * j >= c_hi) break;
+            uint32_t v[16];
+            tmem_ld16(lane_base + b * (uint32_t)BN + (uint32_t)(c_lo + 16 * j), v);
+            tmem_wait_ld();
+            reg_fence16(v);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) sum[16 * j + i] += __float2int_rn(__uint_as_float(v[i]));
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            if (kPair && !leader) mbar_arrive_cluster_relaxed(mapa_shared(b_tempty + 8 * b, 0));
+            else mbar_arrive_relaxed(b_tempty + 8 * b);
+          }
+        }
+        if (!ok) break;
+        const FlatTile ft = flat_tile(jb, ti.mt, kTileRows);
+        const int vr = ft.v0 + (int)rank * 128 + quarter * 32 + lane;
+        const int oh = fast_div(vr, jb.div_row), ow = vr - oh * jb.wp;
+        if (vr < jb.vimg && ow < jb.wo) {  // else a junk column or past the image
+          uint8_t* yrow = ly.y[ti.job] + (int64_t)((ft.img * jb.ho + oh) * jb.wo + ow) * p.y_row_bytes;
+          uint8_t* irow = ly.ws_out ? ly.ws_out + (size_t)(jb.orow_off + (ft.img * jb.ohp + oh + p.out_pad) * jb.owp + ow +
+                                                           p.out_pad) * p.cout
+                                    : nullptr;
+          uint32_t top = 0u;
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int c0 = c_lo + 16 * j;
+            if (c0 >= c_hi) break;
+            const int ch0 = ti.col0 + c0, nc = c_hi - c0 < 16 ? c_hi - c0 : 16;
+            if (out_bits != 32 && (flags & kFlagReq) && (out_bits != 8 || (p.cout & 31) == 0)) {
+              // (|sum| < 2^28 and |bias| <= 2^30)
+              const int4* ef = epi.fast() + c0;
+              uint32_t bw[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+              for (int i = 0; i < 16; ++i) {
+                const int4 c = ef[i];
+                bw[i / 4] += requant32(sum[16 * j + i] + (int32_t)((uint32_t)c.x + kMagicBits), c, qmax) << (8 * (i % 4));
+              }
+              store_codes16(yrow, ch0, bw, out_bits, top);
+              if (irow) store_image16(irow, ch0, bw, ly.ws_nib);
+            } else {
+              int32_t one[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) one[i] = sum[16 * j + i];
+              const GenCols gc{0u, 0u, epi.gen() + c0, nullptr, yrow, ch0, nc, flags, true};
+              const uint4 r = general_finish<false>(p, gc, one);
+              const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
+              if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) {
+                store_codes16(yrow, ch0, bw, out_bits, top);
+                if (irow) store_image16(irow, ch0, bw, ly.ws_nib);
+              }
+            }
+          }
+        }
+        __syncwarp();
+        continue;
+      }
       const uint32_t buf = lt & buf_mask;
 
       // this lane's output row
@@ -1114,6 +1210,7 @@ __device__ __forceinline__ void expand_advance(const ExpandArgs& a, int d, Expan
   }
 }
 
+// kXBits = 16: 8-bit codes as F16 values (the F16 pipe's image), 8 codes per 16 bytes of the image.
 template <int kXBits>
 __global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ ExpandArgs a) {
   // The (row, 16-byte chunk) pairs of the workspace, row-major, are split into runs of
@@ -1128,7 +1225,9 @@ __global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ Exp
   if (threadIdx.x == 0) grid_dep_launch();
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < a.zero_words; i += blockDim.x) a.zero[i] = 0u;
-  const int chunks = a.cin >> 4;
+  constexpr bool kF16 = kXBits == 16;
+  const int chunks = kF16 ? a.cin >> 3 : a.cin >> 4;
+  const int row_bytes = kF16 ? 2 * a.cin : a.cin;
   const int total = (int)a.total_rows * chunks;
   const int lane = threadIdx.x & 31;
   const int e0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * (32 * kPerLane) + lane;
@@ -1137,7 +1236,7 @@ __global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ Exp
   ExpandPos ps;
   int q = e0 % chunks;
   expand_locate(a, e0 / chunks, ps);
-  uint32_t w[kPerLane][kXBits == 2 ? 1 : (kXBits == 8 ? 4 : 2)];
+  uint32_t w[kPerLane][kXBits == 2 ? 1 : (kXBits == 8 ? 4 : 2)];  // (16: 8 codes)
   uint8_t* dst[kPerLane];
   bool inside[kPerLane];
   int hsel[kPerLane];
@@ -1148,12 +1247,16 @@ __global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ Exp
     const ConvJobDev& jb = a.jobs[ps.job];
     const int hi = ps.hr - a.pad, wi = ps.wc - a.pad;
     inside[i] = live && hi >= 0 && hi < jb.h && wi >= 0 && wi < jb.w;
-    dst[i] = live ? a.ws + (size_t)ps.row * a.cin + q * 16 : nullptr;
+    dst[i] = live ? a.ws + (size_t)ps.row * row_bytes + q * 16 : nullptr;
     hsel[i] = q & 1;
     if (inside[i]) {
       const uint32_t* grp = reinterpret_cast<const uint32_t*>(
           jb.x + ((size_t)(ps.img * jb.h + hi) * jb.w + wi) * a.x_row_bytes + (q >> 1) * 4 * kXBits);
-      if constexpr (kXBits == 8) {
+      if constexpr (kF16) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(jb.x + ((size_t)(ps.img * jb.h + hi) * jb.w + wi) *
+                                                             a.x_row_bytes) + q);
+        w[i][0] = v.x; w[i][1] = v.y;
+      } else if constexpr (kXBits == 8) {
         // 16 one-byte codes: channels 16 q .. 16 q + 15
         const uint4 v = __ldg(reinterpret_cast<const uint4*>(jb.x + ((size_t)(ps.img * jb.h + hi) * jb.w + wi) *
                                                              a.x_row_bytes) + q);
@@ -1178,6 +1281,18 @@ __global__ void __launch_bounds__(256) expand_kernel(const __grid_constant__ Exp
   for (int i = 0; i < kPerLane; ++i) {
     if (!dst[i]) continue;
     uint32_t o[4] = {0u, 0u, 0u, 0u};
+    if constexpr (kF16) {
+      // the F16 bit pattern 0x6400 | x is 1024 + x; the subtraction of 1024 is exact
+      if (inside[i]) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t u = __byte_perm(w[i][k >> 1], 0x64646464u, (k & 1) ? 0x4342u : 0x4140u);
+          asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(o[k]) : "r"(u), "r"(0x64006400u));
+        }
+      }
+      *reinterpret_cast<uint4*>(dst[i]) = make_uint4(o[0], o[1], o[2], o[3]);
+      continue;
+    }
     if constexpr (kXBits == 8) {
       // plane 0: x_lo = x & 15 (raw byte); plane 1, total_rows rows on: 16 x_hi as E4M3
       uint32_t o1[4] = {0u, 0u, 0u, 0u};
@@ -1341,6 +1456,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   Params prm{};
   // split (8-bit) weights: tiles of 256 weight rows = 128 output channels
   const int BN = a.split_w ? 256 : a.bn;
+  const bool f16 = a.f16 != 0;
   const int w_rows = a.split_w ? a.split_rows : a.cout_pad;  // rows of the weight block
   prm.njobs = a.njobs;
   prm.n_tiles = w_rows / BN;
@@ -1377,7 +1493,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   // channels of one tap (cin % 64 == 0; 64-byte swizzled operand rows, two MMAs per chunk)
   const bool fp4 = a.fp4 != 0;
   // bytes per row of the image: one code per byte, or two (nibbles) on the FP4 pipe
-  const int img_row = fp4 ? a.cin / 2 : a.cin;
+  const int img_row = fp4 ? a.cin / 2 : (f16 ? 2 * a.cin : a.cin);
   const int bk = (flat && img_row % BK != 0) ? 64 : BK;
   if (flat && (a.stride != 1 || img_row % bk != 0 || rows > a.ws_rows || (a.split_w && bk != BK))) {
     *err = "conv_tc: workspace path needs stride 1, cin % 64 == 0 (128 for split weights) and a large enough workspace";
@@ -1412,7 +1528,8 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.layer_tiles = prm.total_tiles / nlayers;
   prm.div_layer = div_magic(prm.layer_tiles);
   prm.div_nt = div_magic(prm.n_tiles);
-  prm.num_kchunks = flat ? (fp4 ? a.k_total / 2 : a.k_total) / bk : a.k_pad / BK;
+  prm.num_kchunks = flat ? (fp4 ? a.k_total / 2 : (f16 ? 2 * a.k_total : a.k_total)) / bk : a.k_pad / BK;
+  prm.seg_chunks = 512 * 2 / BK;
   prm.cin = a.cin; prm.cout = a.cout; prm.kh = a.kh; prm.kw = a.kw;
   prm.stride = a.stride; prm.pad = a.pad; prm.k_total = a.k_total;
   prm.out_bits = a.out_bits; prm.skip_bits = a.skip_bits;
@@ -1472,7 +1589,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const size_t budget = 232448 - 1024;  // max dynamic smem per block minus alignment slack
   // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least 6 stages remain
   const size_t ostage_bytes = (size_t)epi_warps(flat) * 32 * kStageRow * sizeof(uint32_t);
-  const bool ostage = flat && bk == BK && a.out_bits == 32 && a.cout % 4 == 0 && !a.has_skip && !a.split_w &&
+  const bool ostage = flat && bk == BK && a.out_bits == 32 && a.cout % 4 == 0 && !a.has_skip && !a.split_w && !f16 &&
                       (budget - epi_bytes - bar_bytes - qtab_bytes - ostage_bytes) / stage_bytes >= 6;
   int stages = (int)((budget - epi_bytes - bar_bytes - qtab_bytes - (ostage ? ostage_bytes : 0)) / stage_bytes);
   if (stages > kMaxStages) stages = kMaxStages;
@@ -1504,14 +1621,16 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   if (!enc) return 3;
   Maps maps{};
   // weight rows: k_pad E4M3 bytes, or k_pad / 2 bytes of E2M1 nibbles on the FP4 pipe
-  const int w_row = fp4 ? a.k_pad / 2 : a.k_pad;
-  cuuint64_t gdim[2] = {(cuuint64_t)w_row, (cuuint64_t)w_rows};
+  // (F16: k_total values of 2 bytes, cout rows; a tile's rows past them read as zeros)
+  const int w_row = fp4 ? a.k_pad / 2 : (f16 ? 2 * a.k_total : a.k_pad);
+  cuuint64_t gdim[2] = {(cuuint64_t)w_row, (cuuint64_t)(f16 ? a.cout : w_rows)};
   cuuint64_t gstride[1] = {(cuuint64_t)w_row};
   cuuint32_t box[2] = {(cuuint32_t)bk, (cuuint32_t)b_rows};
   cuuint32_t estr[2] = {1, 1};
   const CUtensorMapSwizzle swz = bk == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
+  const uint8_t* w_src = fp4 ? a.w_fp4 : (f16 ? reinterpret_cast<const uint8_t*>(a.w_i16) : a.w_e4m3);
   for (int l = 0; l < nlayers; ++l) {
-    const uint8_t* wl = nlayers > 1 ? a.layer[l].w_e4m3 : (fp4 ? a.w_fp4 : a.w_e4m3);
+    const uint8_t* wl = nlayers > 1 ? a.layer[l].w_e4m3 : w_src;
     const CUresult r = enc(&maps.w[l], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void*)wl, gdim, gstride, box, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1521,7 +1640,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   maps.wh = maps.w[0];
   if (prm.dp_tiles < prm.layer_tiles) {
     cuuint32_t box_h[2] = {(cuuint32_t)bk, (cuuint32_t)(b_rows / 2)};
-    const CUresult r = enc(&maps.wh, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void*)(fp4 ? a.w_fp4 : a.w_e4m3), gdim,
+    const CUresult r = enc(&maps.wh, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void*)w_src, gdim,
                            gstride, box_h, estr,
                            CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1544,7 +1663,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
       ea.zero = a.zero_words > 0 ? a.zero : nullptr;
       ea.zero_words = a.zero_words;
       // one warp per run of 32 * 4 (row, 16-byte chunk) pairs, 8 warps per block
-      const int64_t pairs = ea.total_rows * (a.cin / 16);
+      const int64_t pairs = ea.total_rows * (a.cin / (f16 ? 8 : 16));
       const unsigned blocks = pairs > 0 ? (unsigned)((pairs + 1023) / 1024) : 1u;
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(blocks);
@@ -1566,7 +1685,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
         case 2: e = cudaLaunchKernelEx(&cfg, expand_kernel<2>, ea); break;
         case 3: e = cudaLaunchKernelEx(&cfg, expand_kernel<3>, ea); break;
         case 4: e = cudaLaunchKernelEx(&cfg, expand_kernel<4>, ea); break;
-        case 8: e = cudaLaunchKernelEx(&cfg, expand_kernel<8>, ea); break;
+        case 8: e = f16 ? cudaLaunchKernelEx(&cfg, expand_kernel<16>, ea) : cudaLaunchKernelEx(&cfg, expand_kernel<8>, ea); break;
         default: *err = "conv_tc: activation bits must be 2, 3 or 4"; return 2;
       }
       if (e == cudaSuccess) e = cudaGetLastError();
@@ -1577,7 +1696,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
     //    image) as [rows][cin] byte matrices with bk x 128 boxes
     // (a nibble image keeps the byte image's row stride: cin bytes, the first cin / 2 used)
     cuuint64_t gd[2] = {(cuuint64_t)img_row, (cuuint64_t)rows * (cuuint64_t)prm.a_planes};
-    cuuint64_t gs[1] = {(cuuint64_t)a.cin};
+    cuuint64_t gs[1] = {(cuuint64_t)(f16 ? 2 * a.cin : a.cin)};
     cuuint32_t bx[2] = {(cuuint32_t)bk, 128};
     for (int i = 0; i < (nlayers > 1 ? 2 : 1); ++i) {
       // (a nibble image row uses 128 of every 256 bytes: fetch 128-byte lines from DRAM)
@@ -1603,6 +1722,10 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
                           : launch_bits<2, true, true, true, false, false, 128, true>(prm, maps, grid, smem, stream, err);
       return a.has_skip ? launch_bits<2, true, true, false, true, false, 128, true>(prm, maps, grid, smem, stream, err)
                         : launch_bits<2, true, true, false, false, false, 128, true>(prm, maps, grid, smem, stream, err);
+    }
+    if (f16) {  // (no skip: the API keeps skips off the 8-bit forms)
+      if (pair) return launch_bits<8, true, true, true, false>(prm, maps, grid, smem, stream, err);
+      return launch_bits<8, true, true, false, false>(prm, maps, grid, smem, stream, err);
     }
     if (a.split_w) {  // (no skip: the API keeps skips off the split form)
       if (pair) return launch_bits<2, true, true, true, false, true>(prm, maps, grid, smem, stream, err);

@@ -8,6 +8,7 @@
 // pixel rows into shared memory, consumer warps with per-lane channel constants); other int32
 // inputs the lane kernel (kV channels per lane, direct loads); packed-code inputs the group
 // kernels (one thread per pixel's 32-channel group: whole packed groups per load and store).
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -1202,7 +1203,7 @@ unpack_kernel(const uint8_t* packed, int64_t groups, int is_signed, int32_t* out
 }
 
 // Prepared weights: E4M3 sign-magnitude bytes [cout_pad][k_pad] (zero padded; only when
-// every |w| <= 15) followed by int16 [cout][k_total].
+// every |w| <= 15) followed by int16 [cout][k_total] (F16 values for 8-bit weights).
 __global__ void __launch_bounds__(kThreads)
 prepare_weights_kernel(const uint8_t* wp, int w_bits, int w_format, WeightGeom g, int64_t w_row_bytes,
                        int make_e4m3, uint8_t* out) {
@@ -1248,7 +1249,9 @@ prepare_weights_kernel(const uint8_t* wp, int w_bits, int w_format, WeightGeom g
       out[t] = 0;
     }
   } else {
-    reinterpret_cast<int16_t*>(out + g.i16_offset)[t - n_e4] = (int16_t)w;
+    // (8-bit weights as F16, exact: the F16 pipe's operand and the stem's)
+    reinterpret_cast<int16_t*>(out + g.i16_offset)[t - n_e4] =
+        w_bits == 8 ? __half_as_short(__int2half_rn(w)) : (int16_t)w;
   }
 }
 

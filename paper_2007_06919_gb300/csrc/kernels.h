@@ -47,7 +47,8 @@ struct ConvArgs {
   int32_t upsample, scale_main, has_skip;
   // prepared weights
   const uint8_t* w_e4m3;  // [cout_pad][k_pad] E4M3 sign-magnitude bytes (|w| <= 15)
-  const int16_t* w_i16;   // [cout][k_total] signed integers
+  const int16_t* w_i16;   // [cout][k_total] signed integers (F16 values when w_f16)
+  int32_t w_f16;          // 8-bit weights: w_i16 holds F16 bit patterns
   int32_t cout_pad, k_total, k_pad, bn;
   int64_t acc_bound;      // K * max|x| * max|w|: bound on |accumulator|
   uint8_t* ws;            // expanded-activation workspace (NULL: in-kernel unpacking)
@@ -61,6 +62,7 @@ struct ConvArgs {
   int32_t a_planes;       // 1, or 2 for 8-bit activation codes
   int32_t split_w;        // weights in the split layout
   int32_t split_rows;     // weight rows of that layout (2 * round_up(cout, 128))
+  int32_t f16;            // 8-bit codes with 8-bit weights on the F16 pipe (the image holds F16 values)
   uint8_t* ws_out;        // chained output: also write the output codes as the next conv's byte image
   int32_t out_pad;        // padding of that next conv
   uint32_t* status;       // device status word

@@ -72,7 +72,7 @@ struct StemParams {
   const int32_t* m0;
   const int8_t* shift;
   const int32_t* bias;
-  const int16_t* w_i16;   // [cout][147], K order (r, s, c)
+  const int16_t* w_i16;   // [cout][147] F16 values, K order (r, s, c)
   uint32_t off_b, off_cst, off_bar;
   uint32_t* status;
 };
@@ -84,14 +84,6 @@ __device__ __forceinline__ uint64_t sdesc_noswz(uint32_t saddr) {
   d |= (uint64_t)(kSBO >> 4) << 32;
   d |= (uint64_t)1 << 46;  // descriptor version; swizzle field 0 = none
   return d;
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(d_tmem), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
 }
 
 // Two code bytes (bytes 0-1 or 2-3 of u) -> two F16 values: 1024 + x by a byte permute,
@@ -234,9 +226,9 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int r = (kk + h) / kLs, j = (kk + h) - r * kLs;
-      int16_t wv = 0;
-      if (n < p.cout && r < kKH && j < kSeg) wv = p.w_i16[(int64_t)n * (kKH * kSeg) + r * kSeg + j];
-      pr |= (uint32_t)__half_as_ushort(__short2half_rn(wv)) << (16 * h);
+      uint16_t wv = 0;  // (F16 zero)
+      if (n < p.cout && r < kKH && j < kSeg) wv = (uint16_t)p.w_i16[(int64_t)n * (kKH * kSeg) + r * kSeg + j];
+      pr |= (uint32_t)wv << (16 * h);
     }
     *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) = pr;
   }
@@ -373,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
 
 bool stem_applicable(const ConvArgs& a) {
   return a.njobs == 1 && a.x_bits == 8 && a.cin == stem::kC && a.kh == stem::kKH && a.kw == stem::kKW &&
-         !a.has_skip && a.cout % 16 == 0 && a.cout <= 256 && a.k_total == stem::kKH * stem::kSeg &&
+         a.w_f16 && !a.has_skip && a.cout % 16 == 0 && a.cout <= 256 && a.k_total == stem::kKH * stem::kSeg &&
          a.acc_bound < (1LL << 24);  // K * 255 * max|w|: the FP32 sum is exact
 }
 

@@ -99,3 +99,24 @@ def test_accumulators_beyond_the_common_form_bit_exact(ws, out_bits):
     got, want, _ = conv_pair(x, 4, wt, 4, w_format=1, out_bits=out_bits, m0=None if out_bits == 32 else m0,
                              shift=None if out_bits == 32 else sh, bias=b, workspace=ws)
     assert_same(got, want, cout, out_bits)
+
+
+# K below, at and past one exact segment of 512, a ragged last segment, several tiles per CTA pair,
+# narrow and no-whole-group rows
+@pytest.mark.parametrize("cin,k,cout,out_bits,shape", [(128, 1, 64, 8, (1, 7, 9)), (512, 1, 256, 4, (2, 31, 33)),
+                                                       (128, 3, 96, 3, (1, 20, 21)), (256, 3, 84, 32, (1, 13, 21)),
+                                                       (384, 3, 40, 8, (1, 9, 10)), (128, 3, 33, 32, (2, 5, 6)),
+                                                       (128, 3, 320, 2, (3, 90, 101)), (256, 1, 64, 8, (4, 100, 101))])
+@pytest.mark.parametrize("path", [0, 2, 3])
+def test_f16_pipe_bit_exact(cin, k, cout, out_bits, shape, path):
+    if path == 2 and cin * k * k * cout * np.prod(shape) > 1 << 31:
+        pytest.skip("the CUDA-core kernel takes seconds")
+    rng = np.random.default_rng(cin + cout)
+    x = synth.act_codes(rng, (*shape, cin), 8)
+    wt = rng.integers(-128, 128, size=(cout, k, k, cin)).astype(np.int32)
+    x[0, 0, :, :], wt[0], wt[1] = 255, -128, 127  # the largest sums of either sign
+    m0, sh, b = tables(rng, cout, 255 * 74 * np.sqrt(cin * k * k) / 2, min(out_bits, 8))
+    got, want, used = conv_pair(x, 8, wt, 8, pad=k // 2, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                                shift=None if out_bits == 32 else sh, bias=b, workspace=True, path=path)
+    assert used == {0: 4, 2: 2, 3: 3}[path]
+    assert_same(got, want, cout, out_bits, f"F16 pipe {cin}x{k}x{k} -> {cout}")
