@@ -106,10 +106,12 @@ struct Params {
   int32_t acc_small;  // |acc| < 2^22 guaranteed by K * max|x| * max|w|
   int32_t cin_chunks; // cin / 128 (flat path)
   int32_t dp_tiles;   // tiles [0, dp_tiles) are bn wide; later ones are the two bn/2 halves
+  int32_t tile_stride; // from one tile of a CTA (pair) to its next
   int32_t contig;     // each CTA takes one contiguous range of tiles (single CTAs, one layer,
                       // no half tiles) instead of every gridDim-th tile
                       // of the remaining full tiles (the last, partial wave)
   uint32_t off_b, off_epi, off_bar, off_qtab;
+  uint32_t off_sktab;   // table of 2- to 4-bit skip codes
   uint32_t off_ostage;  // int32 outputs: per-warp staging blocks for row-contiguous stores (0: none)
   int32_t out_pad;
   int32_t seg_chunks; // kF16: K chunks per exact FP32 segment (512 K elements)
@@ -226,12 +228,11 @@ constexpr uint32_t kMagicBits = 0x4B400000u;
 
 // Eq. 7's rescaled skip rhu(s c, d) in 32-bit arithmetic: with s pre-scaled by 2^k so that
 // |s 2^k| < 2^31, rhu(s c, d) = (mulhi(s 2^k, c) + 2^(d+k-33)) >> (d+k-32) for d + k >= 33 (the
-// same identity as the requant's). k = 24 for 2- to 4-bit codes (the code in the top byte of a
-// word: one byte permute), 23 for 8-bit codes, 3 for int32 skips below 2^28 in magnitude
-// (checked per value). A d so large that |s c| < 2^(d-1) for every s gives 0. The sum acc + bias
-// + rescaled skip then stays within int32 (|bias| <= 2^30, |acc| < 2^24, the skip term below
-// 2^29), so Eq. 7 needs no saturation.
-__device__ __forceinline__ int skip_prescale(int skip_bits) { return skip_bits == 32 ? 3 : (skip_bits == 8 ? 23 : 24); }
+// same identity as the requant's). k = 23 for 8-bit codes, 3 for int32 skips below 2^28 in
+// magnitude (checked per value). A d so large that |s c| < 2^(d-1) for every s gives 0. The sum
+// acc + bias + rescaled skip then stays within int32 (|bias| <= 2^30, |acc| < 2^24, the skip term
+// below 2^29), so Eq. 7 needs no saturation. (Narrower codes take a table, below.)
+__device__ __forceinline__ int skip_prescale(int skip_bits) { return skip_bits == 32 ? 3 : 23; }
 __device__ __forceinline__ bool skip_const(int skip_bits, int32_t c, int d, int4& o) {
   const int r = d + skip_prescale(skip_bits);
   if (r < 33) return false;
@@ -258,6 +259,16 @@ __device__ __forceinline__ void store_image16(uint8_t* irow, int ch, const uint3
   } else {
     *reinterpret_cast<uint4*>(irow + ch) = make_uint4(bw[0], bw[1], bw[2], bw[3]);
   }
+}
+
+// Skip codes of 2 to 4 bits: Eq. 6's bias and Eq. 7's rescaled skip together are one of 2^bits values per
+// column, bias + rhu(s c, d) - kMagicBits, kept in a shared-memory table (built in int64, any c and
+// d). Entry (s, col) at s kSkipStride + col words: the lanes of a warp, which look up one column
+// with their own codes, read different banks. The form holds where every entry's sum part is
+// within 2^30 (|acc| < 2^22 then cannot leave int32, so Eq. 7 needs no saturation).
+constexpr int kSkipStride = 257;
+__host__ __device__ constexpr size_t skip_tab_bytes(int skip_bits) {
+  return skip_bits >= 2 && skip_bits <= 4 ? (((size_t)1 << skip_bits) * kSkipStride * 4 + 15) / 16 * 16 : 0;
 }
 
 // The packed words of 16 skip codes of one row (2- to 4-bit codes: the layout needs cout % 32 ==
@@ -293,9 +304,9 @@ struct GenCols {
   uint32_t taddr;       // TMEM address of the first column
   uint32_t taddr_hi;    // split weights: of the w_hi accumulator
   const EpiChan* ep;    // the columns' constants
-  const uint8_t* srow;  // the skip's row (kSkip)
-  uint8_t* yrow;        // the output's row
-  int ch0, nc, flags;   // first channel, channels that exist
+  const uint8_t* srow;  // the skip's row (kSkip), at the tile's first channel
+  uint8_t* yrow;        // the output's row, likewise
+  int ch0, nc, flags;   // first channel from there, channels that exist
   bool row_ok;
 };
 
@@ -305,7 +316,7 @@ struct GenCols {
 // byte-words; int32 outputs and 8-bit rows of no whole groups are stored here. Not inlined: its
 // registers and code stay out of the common forms.
 template <bool kSkip>
-__device__ __noinline__ uint4 general_finish(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
+__device__ __forceinline__ uint4 general_finish(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
   if (!u.row_ok) return make_uint4(0u, 0u, 0u, 0u);
   if (!kSkip && (u.flags & kFlagReq) && p.out_bits != 32) {
     const int qmax = (1 << p.out_bits) - 1;
@@ -361,6 +372,10 @@ __device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, fl
     for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
   }
   return general_finish<kSkip>(p, u, acc);
+}
+// The same from sums in registers (kF16).
+__device__ __noinline__ uint4 general_sums(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
+  return general_finish<false>(p, u, acc);
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -542,16 +557,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   // This CTA's tiles: every tile_stride-th from first_tile, or (contig) the range
   // [first_tile, tile_end) of a balanced split of the tiles over the grid, so that a CTA's
   // consecutive tiles are neighbours (one level's table, adjacent rows in L2)
-  int first_tile = kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-  int tile_stride = kPair ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-  int tile_end = p.total_tiles;
-  if (!kPair && p.contig) {
-    const int q = p.total_tiles / (int)gridDim.x, r = p.total_tiles % (int)gridDim.x;
-    const int b = (int)blockIdx.x;
-    first_tile = b * q + (b < r ? b : r);
-    tile_end = first_tile + q + (b < r ? 1 : 0);
-    tile_stride = 1;
-  }
+  const bool contig = !kPair && p.contig;
+  const int share = contig ? p.total_tiles / (int)gridDim.x : 0, extra = contig ? p.total_tiles % (int)gridDim.x : 0;
+  const int bid = (int)blockIdx.x;
+  const int first_tile = kPair ? bid >> 1 : (contig ? bid * share + (bid < extra ? bid : extra) : bid);
+  const int tile_end = contig ? first_tile + share + (bid < extra ? 1 : 0) : p.total_tiles;
 
   if (warp == kWarpMma) {
     // ------------------------------------------------------------ MMA issuer
@@ -570,19 +580,18 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       uint32_t it = 0, lt = 0, s = 0, ph = 0;
       bool ok = true;
       bool next_ready = false;  // the stage after the current one is known to be full
-      for (int t = first_tile; t < tile_end && ok; t += tile_stride) {
-       // (kF16: a tile's segments take accumulators in turn, as tiles do otherwise)
-       const int nseg = kF16 ? (nk + p.seg_chunks - 1) / p.seg_chunks : 1;
-       for (int sg = 0; sg < nseg && ok; ++sg, ++lt) {
+      // (kF16: a tile's segments take accumulators in turn, as tiles do otherwise: q0 is the segment's
+      // first chunk, and t moves on after the last)
+      int q0 = 0;
+      for (int t = first_tile; t < tile_end && ok; ++lt) {
         const uint32_t buf = lt & buf_mask;
         // (a launch of several layers has no half-width tiles)
         const uint32_t idesc = p.nlayers > 1 || t < p.dp_tiles ? idesc_full : idesc_half;
-        const int q_end = kF16 ? ((sg + 1) * p.seg_chunks < nk ? (sg + 1) * p.seg_chunks : nk) : nk;
-        const int q_0 = kF16 ? sg * p.seg_chunks : 0;
+        const int q_end = kF16 && q0 + p.seg_chunks < nk ? q0 + p.seg_chunks : nk;
         if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d0 = tmem_base + buf * (uint32_t)BN;
-        for (int q = q_0; q < q_end; ++q, ++it) {
+        for (int q = q0; q < q_end; ++q, ++it) {
           // (operands written by TMA, or by producer threads followed by fence.proxy.async,
           // are ordered for the MMA by the mbarrier phase alone; tcgen05.fence is needed only
           // where TMEM changes hands, after the accumulator-empty wait above)
@@ -597,7 +606,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             // the previous MMA. Testing the next stage here, while the last MMAs of this
             // chunk run, lets the next chunk's first MMA follow this chunk's commit at once.
             if (kk == kBK / 32 - 1) next_ready = mbar_test(b_full + 8 * s_next, ph_next);
-            const uint32_t acc = (q > q_0 || kk > 0) ? 1u : 0u;
+            const uint32_t acc = (q > q0 || kk > 0) ? 1u : 0u;
             const uint64_t db = ((uint64_t)b_hi << 32) | (b_lo + 2 * kk);
             const uint64_t da = ((uint64_t)a_hi << 32) | (a_lo + 2 * kk);
             if constexpr (kPair && kFp4) mma_fp4_pair(d0, da, db, idesc, sfa, sfb, acc);
@@ -615,7 +624,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
           if constexpr (kPair) mma_commit_pair_both(b_tfull + 8 * buf);
           else mma_commit(b_tfull + 8 * buf);
         }
-       }
+        if (kF16 && q_end < nk) q0 = q_end;
+        else { q0 = 0; t += p.tile_stride; }
       }
       if (!ok) fail(abort_flag, p.status);
       // drain: every MMA issued above has completed once this barrier flips
@@ -631,7 +641,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     if (elect_one()) {
       uint32_t it = 0, s = 0, ph = 0;
       bool ok = true;
-      for (int t = first_tile; t < tile_end && ok; t += tile_stride) {
+      for (int t = first_tile; t < tile_end && ok; t += p.tile_stride) {
         const TileInfo ti = tile_info(p, t);
         // per tile: the first workspace row of this CTA's A rows (flat path) and the image width
         int row0 = 0, wp = 0;
@@ -701,7 +711,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     const int r7 = row & 7;
     uint8_t* arow = smem + row * BK;
     int my_tiles = 0;
-    for (int t = first_tile; t < tile_end; t += tile_stride) ++my_tiles;
+    for (int t = first_tile; t < tile_end; t += p.tile_stride) ++my_tiles;
     const int total = my_tiles * nk;
 
     RowCursor<kXBits> rc{};
@@ -725,7 +735,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     auto load_next = [&](uint32_t (&w)[4 * kXBits]) {
       if (l_q == 0) start_tile(l_tile);
       load_chunk<kXBits, kChunkInTap>(p, rc, l_q, w);
-      if (++l_q == nk) { l_q = 0; l_tile += tile_stride; }
+      if (++l_q == nk) { l_q = 0; l_tile += p.tile_stride; }
     };
     bool ok = true;
     auto consume = [&](int c, const uint32_t (&w)[4 * kXBits]) -> bool {
@@ -788,7 +798,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     // without table loads or barriers
     uint32_t cur_key = 0xFFFFFFFFu;  // (first channel, half width, job, layer) of the tables
     int flags = 0;
-    for (int t = first_tile; t < tile_end; t += tile_stride, ++lt) {
+    for (int t = first_tile; t < tile_end; t += p.tile_stride, ++lt) {
       const TileInfo ti = tile_info(p, t);
       const ConvJobDev& jb = p.jobs[ti.job];
       // this tile's output channels that exist (a last N tile may reach past cout; packed
@@ -819,12 +829,28 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             }
             if constexpr (kSkip) {
               ec.c = p.skip_c[idx]; ec.d = p.skip_d[idx];
-              fsk &= skip_const(p.skip_bits, ec.c, ec.d, es) ? 1 : 0;
+              if (p.skip_bits > 4) fsk &= skip_const(p.skip_bits, ec.c, ec.d, es) ? 1 : 0;
             }
           }
           epi.gen()[col] = ec;
           epi.fast()[col] = ef;
           if constexpr (kSkip) epi.skip()[col] = es;
+        }
+        if constexpr (kSkip) {
+          if (p.skip_bits <= 4) {
+            int32_t* tab = reinterpret_cast<int32_t*>(smem + p.off_sktab);
+            const int col = et & 255, ch = ti.col0 + col;
+            if (col < TBN && ch < p.cout) {
+              const int64_t idx = (int64_t)jb.level * p.cout + ch;
+              const int64_t bias = ly.bias ? ly.bias[idx] : 0, c = p.skip_c[idx];
+              const int dd = p.skip_d[idx];
+              for (int s = et >> 8; s < (1 << p.skip_bits); s += kEpiThreads / 256) {
+                const int64_t v = bias + rhu(s * c, dd);
+                fsk &= v >= -(1LL << 30) && v <= (1LL << 30);
+                tab[s * kSkipStride + col] = (int32_t)((uint32_t)v - kMagicBits);
+              }
+            }
+          }
         }
         fq = named_bar_and(1, kEpiThreads, fq);
         sbias = named_bar_and(1, kEpiThreads, sbias);
@@ -898,7 +924,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
 #pragma unroll
               for (int i = 0; i < 16; ++i) one[i] = sum[16 * j + i];
               const GenCols gc{0u, 0u, epi.gen() + c0, nullptr, yrow, ch0, nc, flags, true};
-              const uint4 r = general_finish<false>(p, gc, one);
+              const uint4 r = general_sums(p, gc, one);
               const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
               if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) {
                 store_codes16(yrow, ch0, bw, out_bits, top);
@@ -934,16 +960,20 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
           ow = rem - oh * jb.wo;
         }
       }
-      uint8_t* yrow = ly.y[ti.job] + (int64_t)m * p.y_row_bytes;
+      // the row pointers stand at the tile's first channel (a multiple of 32)
+      const int grp0 = ti.col0 >> 5;
+      uint8_t* yrow = ly.y[ti.job] + (int64_t)m * p.y_row_bytes + grp0 * group_bytes(out_bits);
       uint8_t* irow = nullptr;  // this row of the chained image
       const int nib = ly.ws_nib;
       if (kFlat && ly.ws_out)
         irow = ly.ws_out +
-               (size_t)(jb.orow_off + (img * jb.ohp + oh + p.out_pad) * jb.owp + ow + p.out_pad) * p.cout;
+               (size_t)(jb.orow_off + (img * jb.ohp + oh + p.out_pad) * jb.owp + ow + p.out_pad) * p.cout +
+               grp0 * (nib ? 16 : 32);
       const uint8_t* srow = nullptr;
       if constexpr (kSkip) {
         const int up = p.upsample == 2 ? 1 : 0;
-        srow = jb.skip + (((int64_t)img * jb.skip_h + (oh >> up)) * jb.skip_w + (ow >> up)) * p.skip_row_bytes;
+        srow = jb.skip + (((int64_t)img * jb.skip_h + (oh >> up)) * jb.skip_w + (ow >> up)) * p.skip_row_bytes +
+               grp0 * group_bytes(p.skip_bits);
       }
 
       // this warp's columns [c_lo, c_hi), whole 32-column groups but for the tile's last one
@@ -964,7 +994,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       if (kSkip && p.skip_bits >= 8 && (p.skip_row_bytes & 15) != 0) common = false;
       uint2 sw = make_uint2(0u, 0u);  // the next step's skip codes, loaded a step ahead
       const bool sk_codes = kSkip && p.skip_bits <= 4;
-      if (sk_codes && c_lo < c_hi) sw = load_skip_words(srow, ti.col0 + c_lo, p.skip_bits, row_ok);
+      if (sk_codes && c_lo < c_hi) sw = load_skip_words(srow, c_lo, p.skip_bits, row_ok);
       __syncwarp();
       if (!mbar_wait(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
@@ -977,22 +1007,21 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         }
       };
       uint32_t top = 0u;  // (3-bit codes: see store_codes16)
-      auto store16 = [&](int ch0, const uint32_t (&bw)[4]) {
+      auto store16 = [&](int c0, const uint32_t (&bw)[4]) {
         if (!row_ok) return;
-        store_codes16(yrow, ch0, bw, out_bits, top);
-        if (kFlat && irow) store_image16(irow, ch0, bw, nib);
+        store_codes16(yrow, c0, bw, out_bits, top);
+        if (kFlat && irow) store_image16(irow, c0, bw, nib);
       };
       auto general_tile = [&]() {
 #pragma unroll 1
         for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-          const int ch0 = ti.col0 + c0;
-          const GenCols gc{tbuf + (uint32_t)c0, tbuf + (uint32_t)(ti.cn + c0), epi.gen() + c0, srow, yrow, ch0,
+          const GenCols gc{tbuf + (uint32_t)c0, tbuf + (uint32_t)(ti.cn + c0), epi.gen() + c0, srow, yrow, c0,
                            c_hi - c0 < 16 ? c_hi - c0 : 16, flags, row_ok};
           const uint4 r = general_cols<kSkip, kSplit>(p, gc, kAccSc);
           __syncwarp();
           const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
           // (general_cols stores int32 outputs and 8-bit rows of no whole groups itself)
-          if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) store16(ch0, bw);
+          if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) store16(c0, bw);
         }
       };
       // int32 skips may turn out to need the general form, which reads the accumulator again
@@ -1002,7 +1031,6 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         if (c_lo >= c_hi && !late) release();
 #pragma unroll 1
         for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-          const int ch0 = ti.col0 + c0;
           const bool last = c0 + 16 >= c_hi;
           const int4* ef = epi.fast() + c0;
           const int4* es = epi.skip() + c0;
@@ -1018,14 +1046,15 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             if (sk_codes) {
               uint32_t sb[4];
               skip_bytewords(sw, p.skip_bits, sb);
-              if (!last) sw = load_skip_words(srow, ch0 + 16, p.skip_bits, row_ok);
+              if (!last) sw = load_skip_words(srow, c0 + 16, p.skip_bits, row_ok);
+              const int32_t* tab = reinterpret_cast<const int32_t*>(smem + p.off_sktab) + c0;
               tmem_wait_ld();
               reg_fence16(v);
 #pragma unroll
               for (int i = 0; i < 16; ++i) {
-                const int4 c = ef[i];
-                const int32_t u = sum(i, c, (int32_t)__byte_perm(sb[i / 4], 0u, ((i % 4) << 12) | 0x0444));
-                bw[i / 4] += requant32(u, c, qmax) << (8 * (i % 4));  // codes < 256: the add is an or
+                const int s = (int)((sb[i / 4] >> (8 * (i % 4))) & 0xFFu);
+                const int32_t u = __float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + tab[s * kSkipStride + i];
+                bw[i / 4] += requant32(u, ef[i], qmax) << (8 * (i % 4));  // codes < 256: the add is an or
               }
             } else {
               // 8-bit or int32 skips, four columns at a time
@@ -1035,17 +1064,17 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
               for (int q = 0; q < 4; ++q) {
                 int4 x = make_int4(0, 0, 0, 0);
                 if (p.skip_bits == 8) {
-                  const uint32_t w = row_ok ? __ldg(reinterpret_cast<const uint32_t*>(srow + ch0) + q) : 0u;
+                  const uint32_t w = row_ok ? __ldg(reinterpret_cast<const uint32_t*>(srow + c0) + q) : 0u;
                   x = make_int4((int)(__byte_perm(w, 0u, 0x0444) >> 1), (int)(__byte_perm(w, 0u, 0x1444) >> 1),
                                 (int)(__byte_perm(w, 0u, 0x2444) >> 1), (int)(__byte_perm(w, 0u, 0x3444) >> 1));
                 } else {
-                  if (row_ok) x = __ldg(reinterpret_cast<const int4*>(srow) + (ch0 >> 2) + q);
+                  if (row_ok) x = __ldg(reinterpret_cast<const int4*>(srow) + (c0 >> 2) + q);
                   big |= (uint32_t)((x.x ^ (x.x >> 31)) | (x.y ^ (x.y >> 31)) | (x.z ^ (x.z >> 31)) | (x.w ^ (x.w >> 31)));
                   x = make_int4((int)((uint32_t)x.x << 3), (int)((uint32_t)x.y << 3), (int)((uint32_t)x.z << 3),
                                 (int)((uint32_t)x.w << 3));
                 }
-                const int4 c0 = ef[4 * q], c1 = ef[4 * q + 1], c2 = ef[4 * q + 2], c3 = ef[4 * q + 3];
-                bw[q] = requant32(sum(4 * q, c0, x.x), c0, qmax) | (requant32(sum(4 * q + 1, c1, x.y), c1, qmax) << 8) |
+                const int4 k0 = ef[4 * q], c1 = ef[4 * q + 1], c2 = ef[4 * q + 2], c3 = ef[4 * q + 3];
+                bw[q] = requant32(sum(4 * q, k0, x.x), k0, qmax) | (requant32(sum(4 * q + 1, c1, x.y), c1, qmax) << 8) |
                         (requant32(sum(4 * q + 2, c2, x.z), c2, qmax) << 16) |
                         (requant32(sum(4 * q + 3, c3, x.w), c3, qmax) << 24);
               }
@@ -1093,12 +1122,12 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
                   const int r = 8 * r8 + (lane >> 2), c4 = lane & 3;
                   const int mr = __shfl_sync(0xffffffffu, m, r);
                   if (((rows_ok >> r) & 1u) && c4 < nq)
-                    *reinterpret_cast<uint4*>(ly.y[ti.job] + (int64_t)mr * p.y_row_bytes + (int64_t)(ch0 + 4 * c4) * 4) =
+                    *reinterpret_cast<uint4*>(ly.y[ti.job] + (int64_t)mr * p.y_row_bytes + (int64_t)(ti.col0 + c0 + 4 * c4) * 4) =
                         *reinterpret_cast<const uint4*>(stg + r * kStageRow + 4 * c4);
                 }
                 __syncwarp();
               } else if (row_ok) {
-                uint4* yr = reinterpret_cast<uint4*>(yrow) + (ch0 >> 2);
+                uint4* yr = reinterpret_cast<uint4*>(yrow) + (c0 >> 2);
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                   if (q < nq) yr[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -1112,7 +1141,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
               bw[i / 4] += requant32(u, c, qmax) << (8 * (i % 4));  // codes < 256: the add is an or
             }
           }
-          store16(ch0, bw);
+          store16(c0, bw);
         }
         if constexpr (kSkip) {
           if (__any_sync(0xffffffffu, (big >> 28) != 0u)) general_tile();
@@ -1121,7 +1150,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         general_tile();
       }
       if (late) release();
-      if (kFlat && p.dep && ti.layer < p.nlayers - 1) {
+      if (kFlat && p.dep && t < (p.nlayers - 1) * p.layer_tiles) {
         // this warp's stores of tile t are done: order them for the next layer's TMA (async
         // proxy) loads, gather the warp (__syncwarp orders its lanes' stores before lane 0's
         // next operations), and count the warp in with one release (cumulative over them)
@@ -1586,12 +1615,13 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const size_t epi_bytes = EpiTab::kBytes;
   const size_t bar_bytes = 8 * (2 * kMaxStages + 2 * kMaxBufs + 1) + 16;
   const size_t qtab_bytes = kQTab * sizeof(uint32_t);
+  const size_t sk_bytes = a.has_skip ? skip_tab_bytes(a.skip_bits) : 0;
   const size_t budget = 232448 - 1024;  // max dynamic smem per block minus alignment slack
   // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least 6 stages remain
   const size_t ostage_bytes = (size_t)epi_warps(flat) * 32 * kStageRow * sizeof(uint32_t);
   const bool ostage = flat && bk == BK && a.out_bits == 32 && a.cout % 4 == 0 && !a.has_skip && !a.split_w && !f16 &&
                       (budget - epi_bytes - bar_bytes - qtab_bytes - ostage_bytes) / stage_bytes >= 6;
-  int stages = (int)((budget - epi_bytes - bar_bytes - qtab_bytes - (ostage ? ostage_bytes : 0)) / stage_bytes);
+  int stages = (int)((budget - epi_bytes - bar_bytes - qtab_bytes - sk_bytes - 32 - (ostage ? ostage_bytes : 0)) / stage_bytes);
   if (stages > kMaxStages) stages = kMaxStages;
   if (stages < 2) { *err = "conv_tc: shared memory plan does not fit"; return 2; }
   // The TMA issuers take K chunks round-robin and each waits on its stage's "empty"
@@ -1604,8 +1634,10 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.off_epi = prm.off_b + (uint32_t)(stages * b_rows * bk);
   prm.off_bar = prm.off_epi + (uint32_t)epi_bytes;
   prm.off_qtab = prm.off_bar + (uint32_t)bar_bytes;
-  prm.off_ostage = ostage ? (uint32_t)((prm.off_qtab + qtab_bytes + 15) / 16 * 16) : 0u;
-  const size_t smem = 1024 + (ostage ? prm.off_ostage + ostage_bytes : prm.off_qtab + qtab_bytes);
+  // (a launch has a skip table or staging blocks, not both: staged outputs have no skip)
+  const uint32_t off_end = (uint32_t)((prm.off_qtab + qtab_bytes + 15) / 16 * 16);
+  prm.off_ostage = prm.off_sktab = off_end;
+  const size_t smem = 1024 + off_end + (ostage ? ostage_bytes : sk_bytes);
   // two accumulators of BN fp32 columns, or four where they fit beside the 32 columns of scales
   // of the FP4 pipe
   const int sf_cols = fp4 ? 32 : 0;
@@ -1650,6 +1682,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const int units = prm.total_tiles;
   int grid = units < sms ? units : sms;
   if (pair) grid = 2 * (units < sms / 2 ? units : sms / 2);
+  prm.tile_stride = pair ? grid / 2 : (prm.contig ? 1 : grid);
   const bool in_tap = (a.cin % BK) == 0;
   if (flat) {
     // 1) expand the packed codes of every job into the zero-padded byte workspace (unless
