@@ -271,6 +271,15 @@ __host__ __device__ constexpr size_t skip_tab_bytes(int skip_bits) {
   return skip_bits >= 2 && skip_bits <= 4 ? (((size_t)1 << skip_bits) * kSkipStride * 4 + 15) / 16 * 16 : 0;
 }
 
+// int32 skips: each warp stages the next 16 columns of its 32 rows (64 bytes a row) in shared memory
+// by cp.async, two steps in flight. A lane that reads its own row takes 16 bytes of 32 different rows
+// per load; four lanes per row take whole 64-byte pieces. The 16-byte pieces of a row are
+// rotated by its index, so that both the copies and the row reads are conflict-free.
+constexpr int kSkipStage = 32 * 64;  // bytes of one step of one warp
+__device__ __forceinline__ uint32_t skip_stage_off(int row, int piece) {
+  return (uint32_t)(row * 64 + ((piece ^ (row >> 1)) & 3) * 16);
+}
+
 // The packed words of 16 skip codes of one row (2- to 4-bit codes: the layout needs cout % 32 ==
 // 0, so they all exist) from channel ch on, and their byte-words.
 __device__ __forceinline__ uint2 load_skip_words(const uint8_t* srow, int ch, int sb, bool ok) {
@@ -992,11 +1001,39 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       // rows whose pieces would not be aligned, or not whole
       if ((out_bits == 8 && (p.cout & 31) != 0) || (out_bits == 32 && (p.cout & 3) != 0)) common = false;
       if (kSkip && p.skip_bits >= 8 && (p.skip_row_bytes & 15) != 0) common = false;
+      // int32 skips: the skip pixels of the four rows whose pieces this lane copies (-1: none)
+      [[maybe_unused]] int sp4[4] = {-1, -1, -1, -1};
+      [[maybe_unused]] const uint32_t sk_stage = sbase + p.off_sktab + (uint32_t)warp * (2 * kSkipStage);
+      auto copy_skip32 = [&](int c0, int step) {  // columns c0 .. c0 + 15 (none past the end)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const bool on = sp4[k] >= 0 && c0 < c_hi;
+          const uint8_t* src = jb.skip;
+          if (on) src += (int64_t)sp4[k] * p.skip_row_bytes + (int64_t)(ti.col0 + c0) * 4 + (lane & 3) * 16;
+          cp_async<16>(sk_stage + (uint32_t)(step & 1) * kSkipStage + skip_stage_off(8 * k + (lane >> 2), lane & 3), src, on);
+        }
+        cp_async_commit();
+      };
+      const bool sk_int = kSkip && p.skip_bits == 32 && common;
+      if constexpr (kSkip) {
+        if (sk_int) {
+          const int up = p.upsample == 2 ? 1 : 0;
+          const int sp = row_ok ? (img * jb.skip_h + (oh >> up)) * jb.skip_w + (ow >> up) : -1;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) sp4[k] = __shfl_sync(0xffffffffu, sp, 8 * k + (lane >> 2));
+          copy_skip32(c_lo, 0);
+          copy_skip32(c_lo + 16, 1);
+        }
+      }
       uint2 sw = make_uint2(0u, 0u);  // the next step's skip codes, loaded a step ahead
       const bool sk_codes = kSkip && p.skip_bits <= 4;
       if (sk_codes && c_lo < c_hi) sw = load_skip_words(srow, c_lo, p.skip_bits, row_ok);
       __syncwarp();
-      if (!mbar_wait(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) { ok = false; break; }
+      if (!mbar_wait(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) {
+        if constexpr (kSkip) cp_async_wait<0>();  // (no copy outlives the block)
+        ok = false;
+        break;
+      }
       tc_fence_after();
       auto release = [&]() {  // every TMEM read of this warp is complete
         tc_fence_before();
@@ -1060,6 +1097,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
               // 8-bit or int32 skips, four columns at a time
               tmem_wait_ld();
               reg_fence16(v);
+              const int step = (c0 - c_lo) >> 4;
+              if (p.skip_bits == 32) {
+                cp_async_wait<1>();  // this step's copies (the next step's may be in flight)
+                __syncwarp();
+              }
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
                 int4 x = make_int4(0, 0, 0, 0);
@@ -1068,7 +1110,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
                   x = make_int4((int)(__byte_perm(w, 0u, 0x0444) >> 1), (int)(__byte_perm(w, 0u, 0x1444) >> 1),
                                 (int)(__byte_perm(w, 0u, 0x2444) >> 1), (int)(__byte_perm(w, 0u, 0x3444) >> 1));
                 } else {
-                  if (row_ok) x = __ldg(reinterpret_cast<const int4*>(srow) + (c0 >> 2) + q);
+                  x = *reinterpret_cast<const int4*>(smem + (sk_stage - sbase) + (step & 1) * kSkipStage + skip_stage_off(lane, q));
                   big |= (uint32_t)((x.x ^ (x.x >> 31)) | (x.y ^ (x.y >> 31)) | (x.z ^ (x.z >> 31)) | (x.w ^ (x.w >> 31)));
                   x = make_int4((int)((uint32_t)x.x << 3), (int)((uint32_t)x.y << 3), (int)((uint32_t)x.z << 3),
                                 (int)((uint32_t)x.w << 3));
@@ -1077,6 +1119,10 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
                 bw[q] = requant32(sum(4 * q, k0, x.x), k0, qmax) | (requant32(sum(4 * q + 1, c1, x.y), c1, qmax) << 8) |
                         (requant32(sum(4 * q + 2, c2, x.z), c2, qmax) << 16) |
                         (requant32(sum(4 * q + 3, c3, x.w), c3, qmax) << 24);
+              }
+              if (p.skip_bits == 32) {
+                __syncwarp();  // every lane has read its row
+                copy_skip32(c0 + 32, step);
               }
             }
             if (last && !late) release();
@@ -1615,7 +1661,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const size_t epi_bytes = EpiTab::kBytes;
   const size_t bar_bytes = 8 * (2 * kMaxStages + 2 * kMaxBufs + 1) + 16;
   const size_t qtab_bytes = kQTab * sizeof(uint32_t);
-  const size_t sk_bytes = a.has_skip ? skip_tab_bytes(a.skip_bits) : 0;
+  const size_t sk_bytes = !a.has_skip ? 0 : (a.skip_bits == 32 ? (size_t)epi_warps(flat) * 2 * kSkipStage : skip_tab_bytes(a.skip_bits));
   const size_t budget = 232448 - 1024;  // max dynamic smem per block minus alignment slack
   // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least 6 stages remain
   const size_t ostage_bytes = (size_t)epi_warps(flat) * 32 * kStageRow * sizeof(uint32_t);
