@@ -39,6 +39,7 @@
 
 #include <cstdio>
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 #include "epilogue.cuh"
@@ -56,9 +57,18 @@ constexpr int BK = 128;            // K bytes per stage
 // latencies. The in-kernel-unpack variant keeps 8: its producer warps need the registers.
 __host__ __device__ constexpr int epi_warps(bool flat) { return flat ? 16 : 8; }
 constexpr int kProdWarps = 4;  // one thread per tile row
-// The expanded-activation ("flat") variant has no producer warps: TMA loads both operands,
-// two boxes per K chunk. One issuing thread sustains about one box per ~700 cycles
-// (measured), so that variant spreads the chunks over kTmaWarpsFlat threads.
+// The expanded-activation ("flat") variant has no producer warps: TMA loads both operands, one
+// thread the activations and two the weights.
+//
+// Activations come in slabs: the 128 + kw - 1 image rows that the kw taps of one kernel row read,
+// once, and the tap s multiplies the 128 rows from row s of the slab on. The swizzle of an operand
+// row depends on its address alone, so a later first row is only a later start address in the
+// MMA's descriptor. Weights stay in shared memory for the whole launch where all of them fit, and
+// come per tap otherwise. L2 delivers about 70 bytes per clock to each SM, and a 128 x 128-byte
+// piece of each operand per 4 MMAs needed all of that: a 3x3 layer's 32 KB per tap are 21.7 KB this
+// way, and with 64 channels and resident weights 2.9 KB instead of 10. Together with the MMA
+// thread's loop below, at batch 8: 64-channel layer 58 -> 49 us, 256-channel tower layer 72 -> 68, the
+// whole detector 1397 -> 1343 (slabs alone, with the loop as it was: 64 and 68 us, 1399).
 constexpr int kTmaWarpsFlat = 3;
 __host__ __device__ constexpr int tma_warps(bool flat) { return flat ? kTmaWarpsFlat : 1; }
 __host__ __device__ constexpr int threads_for(bool flat) {
@@ -67,7 +77,6 @@ __host__ __device__ constexpr int threads_for(bool flat) {
 constexpr int kMaxBufs = 4;    // TMEM accumulators
 constexpr int kMaxStages = 16;
 constexpr int kStageRow = 20;  // words per row of an int32 staging block: 16 and a pad (conflict-free)
-constexpr int kQTab = 256;  // K-chunk table entries (larger K falls back to division)
 
 // One layer of a launch: its per-channel tables, the packed output of each job and the
 // zero-padded byte image its epilogue writes for the next layer (NULL: none).
@@ -107,10 +116,16 @@ struct Params {
   int32_t cin_chunks; // cin / 128 (flat path)
   int32_t dp_tiles;   // tiles [0, dp_tiles) are bn wide; later ones are the two bn/2 halves
   int32_t tile_stride; // from one tile of a CTA (pair) to its next
+  int32_t share, extra; // contig: tiles per CTA, CTAs with one more
   int32_t contig;     // each CTA takes one contiguous range of tiles (single CTAs, one layer,
                       // no half tiles) instead of every gridDim-th tile
                       // of the remaining full tiles (the last, partial wave)
-  uint32_t off_b, off_epi, off_bar, off_qtab;
+  // flat path: a ring of `stages` activation slabs and one of stages_b weight tiles (resident: all
+  // weight tiles, loaded once)
+  int32_t stages_b, resident;
+  uint32_t slab_bytes;
+  int32_t taps;        // taps that share a slab: kw, or 1 for kernels too wide for that
+  uint32_t off_b, off_epi, off_bar;
   uint32_t off_sktab;   // table of 2- to 4-bit skip codes
   uint32_t off_ostage;  // int32 outputs: per-warp staging blocks for row-contiguous stores (0: none)
   int32_t out_pad;
@@ -480,14 +495,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   const uint32_t s_b = sbase + p.off_b;
   const EpiTab epi{smem + p.off_epi};
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
-  // barrier slots: full[0..S), empty[0..S), tfull[nbuf], tempty[nbuf], final (kMaxBufs each)
-  const int S = p.stages;
-  const uint32_t b_full = smem_u32(bars);
-  const uint32_t b_empty = b_full + 8 * S;
-  const uint32_t b_tfull = b_empty + 8 * S;
-  const uint32_t b_tempty = b_tfull + 8 * kMaxBufs;
-  const uint32_t b_final = b_tempty + 8 * kMaxBufs;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 2 * kMaxBufs + 1);
+  // barrier slots: tfull[nbuf], tempty[nbuf] (kMaxBufs each), final, then full[0..S), empty[0..S), on
+  // the flat path of the slabs, and of the weight tiles wfull[0..SB), wempty[0..SB)
+  const uint32_t b_tfull = smem_u32(bars), b_tempty = b_tfull + 8 * kMaxBufs;
+  const uint32_t b_final = b_tempty + 8 * kMaxBufs, b_full = b_final + 8;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kMaxBufs + 1 + 4 * kMaxStages);
   const uint32_t buf_mask = (1u << p.nbuf_log2) - 1u;
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -496,17 +508,23 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   const int BN = p.bn;
   const uint32_t stage_b_bytes = (uint32_t)(kPair ? BN / 2 : BN) * kBK;  // this CTA's rows of B
 
-  // K chunk q -> (tap row r, tap column sx, 128-channel block cb), for the TMA issuers
-  uint32_t* qtab = reinterpret_cast<uint32_t*>(smem + p.off_qtab);
-  for (int q = threadIdx.x; q < p.num_kchunks && q < kQTab; q += blockDim.x) {
-    const int tap = q / p.cin_chunks, cb = q - tap * p.cin_chunks;
-    const int r = tap / p.kw, sx = tap - r * p.kw;
-    qtab[q] = ((uint32_t)r << 24) | ((uint32_t)sx << 16) | (uint32_t)cb;
-  }
+  // (the roles that use them work these out for themselves: the epilogue has no register to spare)
+  auto slots = [&](uint32_t& empty, uint32_t& wfull, uint32_t& wempty) {
+    empty = b_full + 8 * p.stages;
+    wfull = empty + 8 * p.stages;
+    wempty = wfull + 8 * (kFlat ? p.stages_b : 0);
+  };
   if (threadIdx.x == 0) {
+    const int S = p.stages, SB = kFlat ? p.stages_b : 0;
+    uint32_t b_empty, b_wfull, b_wempty;
+    slots(b_empty, b_wfull, b_wempty);
     for (int s = 0; s < S; ++s) {
       mbar_init(b_full + 8 * s, kFlat ? 1 : kProdWarps + 1);  // per producer warp + TMA
       mbar_init(b_empty + 8 * s, 1);
+    }
+    for (int s = 0; s < SB; ++s) {
+      mbar_init(b_wfull + 8 * s, 1);
+      mbar_init(b_wempty + 8 * s, 1);
     }
     for (int b = 0; b < kMaxBufs; ++b) {
       mbar_init(b_tfull + 8 * b, 1);
@@ -566,15 +584,18 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   // This CTA's tiles: every tile_stride-th from first_tile, or (contig) the range
   // [first_tile, tile_end) of a balanced split of the tiles over the grid, so that a CTA's
   // consecutive tiles are neighbours (one level's table, adjacent rows in L2)
-  const bool contig = !kPair && p.contig;
-  const int share = contig ? p.total_tiles / (int)gridDim.x : 0, extra = contig ? p.total_tiles % (int)gridDim.x : 0;
+  // (contig: share tiles each, one more for the first `extra` CTAs)
   const int bid = (int)blockIdx.x;
-  const int first_tile = kPair ? bid >> 1 : (contig ? bid * share + (bid < extra ? bid : extra) : bid);
-  const int tile_end = contig ? first_tile + share + (bid < extra ? 1 : 0) : p.total_tiles;
+  const bool contig = !kPair && p.contig;
+  const int first_tile = kPair ? bid >> 1 : (contig ? bid * p.share + (bid < p.extra ? bid : p.extra) : bid);
+  const int tile_end = contig ? first_tile + p.share + (bid < p.extra ? 1 : 0) : p.total_tiles;
 
   if (warp == kWarpMma) {
     // ------------------------------------------------------------ MMA issuer
     if (leader && elect_one()) {
+      const int S = p.stages, SB = kFlat ? p.stages_b : 0;
+      uint32_t b_empty, b_wfull, b_wempty;
+      slots(b_empty, b_wfull, b_wempty);
       const uint32_t idesc_full = kFp4 ? idesc_fp4(BN, kPair ? 2 * kMmaM : kMmaM) : idesc_e4m3(BN, kPair ? 2 * kMmaM : kMmaM);
       const uint32_t idesc_half =
           kFp4 ? idesc_fp4(BN / 2, kPair ? 2 * kMmaM : kMmaM) : idesc_e4m3(BN / 2, kPair ? 2 * kMmaM : kMmaM);
@@ -586,55 +607,120 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const uint64_t da0 = sdesc_k<kBK>(s_a), db0 = sdesc_k<kBK>(s_b);
       const uint32_t a_lo0 = (uint32_t)da0, b_lo0 = (uint32_t)db0;
       const uint32_t a_hi = (uint32_t)(da0 >> 32), b_hi = (uint32_t)(db0 >> 32);
-      uint32_t it = 0, lt = 0, s = 0, ph = 0;
+      // one instruction of K = 32 bytes: operand rows at da, db
+      auto mma = [&](uint32_t d0, uint32_t a_lo, uint32_t b_lo, uint32_t idesc, uint32_t acc) {
+        const uint64_t da = ((uint64_t)a_hi << 32) | a_lo, db = ((uint64_t)b_hi << 32) | b_lo;
+        if constexpr (kPair && kFp4) mma_fp4_pair(d0, da, db, idesc, sfa, sfb, acc);
+        else if constexpr (kPair && kF16) mma_f16_pair(d0, da, db, idesc, acc);
+        else if constexpr (kPair) mma_e4m3_pair(d0, da, db, idesc, acc);
+        else if constexpr (kF16) mma_f16(d0, da, db, idesc, acc);
+        else if constexpr (kFp4) mma_fp4(d0, da, db, idesc, sfa, sfb, acc);
+        else mma_e4m3(d0, da, db, idesc, acc);
+      };
+      auto commit = [&](uint32_t bar) {
+        if constexpr (kPair) mma_commit_pair_both(bar);
+        else mma_commit(bar);
+      };
+      uint32_t lt = 0;
       bool ok = true;
-      bool next_ready = false;  // the stage after the current one is known to be full
-      // (kF16: a tile's segments take accumulators in turn, as tiles do otherwise: q0 is the segment's
-      // first chunk, and t moves on after the last)
-      int q0 = 0;
-      for (int t = first_tile; t < tile_end && ok; ++lt) {
-        const uint32_t buf = lt & buf_mask;
-        // (a launch of several layers has no half-width tiles)
-        const uint32_t idesc = p.nlayers > 1 || t < p.dp_tiles ? idesc_full : idesc_half;
-        const int q_end = kF16 && q0 + p.seg_chunks < nk ? q0 + p.seg_chunks : nk;
-        if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d0 = tmem_base + buf * (uint32_t)BN;
-        for (int q = q0; q < q_end; ++q, ++it) {
-          // (operands written by TMA, or by producer threads followed by fence.proxy.async,
-          // are ordered for the MMA by the mbarrier phase alone; tcgen05.fence is needed only
-          // where TMEM changes hands, after the accumulator-empty wait above)
-          if (!next_ready && !mbar_poll(b_full + 8 * s, ph, abort_flag)) { ok = false; break; }
-          const uint32_t a_lo = a_lo0 + ((s * kStA) >> 4);
-          const uint32_t b_lo = b_lo0 + ((s * stage_b_bytes) >> 4);
-          const uint32_t s_next = s + 1 == (uint32_t)S ? 0u : s + 1;
-          const uint32_t ph_next = s_next == 0 ? ph ^ 1u : ph;
+      // (operands written by TMA, or by producer threads followed by fence.proxy.async, are ordered
+      // for the MMA by the mbarrier phase alone; tcgen05.fence is needed only where TMEM changes
+      // hands, after the accumulator-empty wait)
+      if constexpr (kFlat) {
+        // The issuing thread runs one instruction at a time between the epilogue's warps, about 10
+        // cycles each, while the MMAs queue behind it: with narrow tiles its bookkeeping, not the
+        // tensor pipe, set the pace (330 of 450 cycles per chunk). So addresses advance by additions,
+        // the taps of a slab are unrolled (1 and 3 of them), and a barrier is tested once, where
+        // it is needed: the queued MMAs cover that.
+        const bool resident = p.resident != 0;
+        if (resident && !mbar_poll(b_wfull, 0, abort_flag)) ok = false;
+        uint32_t sa = 0, pa = 0, a_cur = a_lo0;              // slab stage, its phase, its descriptor
+        uint32_t fw = b_wfull, pw = 0, w_cur = b_lo0;        // weight barrier, its phase, descriptor
+        const uint32_t a_step = p.slab_bytes >> 4, w_step = stage_b_bytes >> 4;
+        const uint32_t w_end = b_lo0 + (uint32_t)SB * w_step, w_empty = b_wempty - b_wfull;
+        uint32_t buf = 0, d0 = 0, acc = 0;
+        int sq = 0;  // kF16: chunks of this accumulator
+        auto open = [&]() {  // the next accumulator
+          buf = lt & buf_mask;
+          if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) return false;
+          tc_fence_after();
+          d0 = tmem_base + buf * (uint32_t)BN;
+          acc = 0;
+          sq = 0;
+          return true;
+        };
+        // the MMAs of one slab: false if a wait ran out
+        auto slab = [&](auto taps_c, uint32_t idesc) {
+          constexpr int kTaps = decltype(taps_c)::value;  // 0: p.taps
+          if (!mbar_poll(b_full + 8 * sa, pa, abort_flag)) return false;
+          const int taps = kTaps > 0 ? kTaps : p.taps;
+#pragma unroll(kTaps > 0 ? kTaps : 1)
+          for (int tap = 0; tap < taps; ++tap) {
+            if (kF16 && sq == p.seg_chunks) {  // (a tile's segments take accumulators in turn)
+              commit(b_tfull + 8 * buf);
+              ++lt;
+              if (!open()) return false;
+            }
+            if (!resident && !mbar_poll(fw, pw, abort_flag)) return false;
 #pragma unroll
-          for (int kk = 0; kk < kBK / 32; ++kk) {
-            // The tensor pipe takes about one instruction at a time, so each issue waits for
-            // the previous MMA. Testing the next stage here, while the last MMAs of this
-            // chunk run, lets the next chunk's first MMA follow this chunk's commit at once.
-            if (kk == kBK / 32 - 1) next_ready = mbar_test(b_full + 8 * s_next, ph_next);
-            const uint32_t acc = (q > q0 || kk > 0) ? 1u : 0u;
-            const uint64_t db = ((uint64_t)b_hi << 32) | (b_lo + 2 * kk);
-            const uint64_t da = ((uint64_t)a_hi << 32) | (a_lo + 2 * kk);
-            if constexpr (kPair && kFp4) mma_fp4_pair(d0, da, db, idesc, sfa, sfb, acc);
-            else if constexpr (kPair && kF16) mma_f16_pair(d0, da, db, idesc, acc);
-            else if constexpr (kPair) mma_e4m3_pair(d0, da, db, idesc, acc);
-            else if constexpr (kF16) mma_f16(d0, da, db, idesc, acc);
-            else if constexpr (kFp4) mma_fp4(d0, da, db, idesc, sfa, sfb, acc);
-            else mma_e4m3(d0, da, db, idesc, acc);
+            for (int kk = 0; kk < kBK / 32; ++kk) {
+              mma(d0, a_cur + (uint32_t)(tap * (kBK >> 4) + 2 * kk), w_cur + 2 * kk, idesc, acc);
+              acc = 1;
+            }
+            w_cur += w_step;
+            if (!resident) {
+              commit(fw + w_empty);
+              fw += 8;
+              if (w_cur == w_end) { w_cur = b_lo0; fw = b_wfull; pw ^= 1; }
+            }
+            if constexpr (kF16) ++sq;
           }
-          if constexpr (kPair) mma_commit_pair_both(b_empty + 8 * s);
-          else mma_commit(b_empty + 8 * s);
-          if (++s == (uint32_t)S) { s = 0; ph ^= 1; }
+          commit(b_empty + 8 * sa);
+          a_cur += a_step;
+          if (++sa == (uint32_t)S) { sa = 0; a_cur = a_lo0; pa ^= 1; }
+          return true;
+        };
+        for (int t = first_tile; t < tile_end && ok; t += p.tile_stride, ++lt) {
+          // (a launch of several layers has no half-width tiles)
+          const uint32_t idesc = p.nlayers > 1 || t < p.dp_tiles ? idesc_full : idesc_half;
+          if (!open()) { ok = false; break; }
+          for (int plane = 0; plane < p.a_planes && ok; ++plane) {
+            // resident weights: the tiles of this N range (a second plane meets the same ones)
+            if (resident)
+              w_cur = b_lo0 + (p.n_tiles > 1 ? (uint32_t)(tile_info(p, t).brow / BN * p.num_kchunks) * w_step : 0u);
+            for (int q = 0; q < p.num_kchunks && ok; q += p.taps)
+              ok = p.taps == 3 ? slab(std::integral_constant<int, 3>{}, idesc)
+                               : p.taps == 1 ? slab(std::integral_constant<int, 1>{}, idesc)
+                                             : slab(std::integral_constant<int, 0>{}, idesc);
+          }
+          if (ok) commit(b_tfull + 8 * buf);
         }
-        if (ok) {
-          if constexpr (kPair) mma_commit_pair_both(b_tfull + 8 * buf);
-          else mma_commit(b_tfull + 8 * buf);
+      } else {
+        uint32_t s = 0, ph = 0;
+        bool next_ready = false;  // the stage after the current one is known to be full
+        for (int t = first_tile; t < tile_end && ok; t += p.tile_stride, ++lt) {
+          const uint32_t buf = lt & buf_mask;
+          const uint32_t idesc = t < p.dp_tiles ? idesc_full : idesc_half;
+          if (!mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t d0 = tmem_base + buf * (uint32_t)BN;
+          for (int q = 0; q < nk; ++q) {
+            if (!next_ready && !mbar_poll(b_full + 8 * s, ph, abort_flag)) { ok = false; break; }
+            const uint32_t a_lo = a_lo0 + ((s * kStA) >> 4);
+            const uint32_t b_lo = b_lo0 + ((s * stage_b_bytes) >> 4);
+            const uint32_t s_next = s + 1 == (uint32_t)S ? 0u : s + 1;
+            const uint32_t ph_next = s_next == 0 ? ph ^ 1u : ph;
+#pragma unroll
+            for (int kk = 0; kk < kBK / 32; ++kk) {
+              if (kk == kBK / 32 - 1) next_ready = mbar_test(b_full + 8 * s_next, ph_next);
+              mma(d0, a_lo + 2 * kk, b_lo + 2 * kk, idesc, (q > 0 || kk > 0) ? 1u : 0u);
+            }
+            commit(b_empty + 8 * s);
+            s = s_next;
+            ph = ph_next;
+          }
+          if (ok) commit(b_tfull + 8 * buf);
         }
-        if (kF16 && q_end < nk) q0 = q_end;
-        else { q0 = 0; t += p.tile_stride; }
       }
       if (!ok) fail(abort_flag, p.status);
       // drain: every MMA issued above has completed once this barrier flips
@@ -643,73 +729,84 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       if (!mbar_wait(b_final, 0, abort_flag)) fail(abort_flag, p.status);
     }
   } else if (warp >= kWarpTma && warp < kWarpTma + kTma) {
-    // ------------------------------------------------------------ weight loaders (TMA)
-    // One thread of each TMA warp issues every kTma-th chunk: a thread sustains
-    // about one tensor copy at a time, so two threads keep two copies in flight.
+    // ------------------------------------------------------------ operand loaders (TMA)
     const int tw = warp - kWarpTma;
     if (elect_one()) {
-      uint32_t it = 0, s = 0, ph = 0;
+      const int S = p.stages, SB = kFlat ? p.stages_b : 0;
+      uint32_t b_empty, b_wfull, b_wempty;
+      slots(b_empty, b_wfull, b_wempty);
       bool ok = true;
-      for (int t = first_tile; t < tile_end && ok; t += p.tile_stride) {
-        const TileInfo ti = tile_info(p, t);
-        // per tile: the first workspace row of this CTA's A rows (flat path) and the image width
-        int row0 = 0, wp = 0;
-        if constexpr (kFlat) {
+      // arms a barrier of this CTA, or of a pair's leader, which counts both CTAs' copies, and loads
+      // one box into this CTA's shared memory
+      auto load = [&](uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar, uint32_t bytes) {
+        if (leader) {
+          if (bytes > 0) mbar_arrive_expect_tx(bar, (kPair ? 2u : 1u) * bytes);
+          tma_load_2d(dst, map, x, y, bar);
+        } else {
+          tma_load_2d_pair(dst, map, x, y, mapa_shared(bar, 0));
+        }
+      };
+      if constexpr (!kFlat) {
+        uint32_t s = 0, ph = 0;
+        for (int t = first_tile; t < tile_end && ok; t += p.tile_stride) {
+          const TileInfo ti = tile_info(p, t);
+          const CUtensorMap* wm = ti.bn == BN ? &maps.w[0] : &maps.wh;
+          for (int q = 0; q < nk; ++q, s = (s + 1 == (uint32_t)S) ? 0 : s + 1, ph ^= (s == 0)) {
+            if (!mbar_wait(b_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+            load(s_b + s * stage_b_bytes, wm, q * kBK, ti.brow, b_full + 8 * s, (uint32_t)ti.bn * kBK);
+          }
+        }
+      } else if (tw == 0) {
+        // slabs: the rows that the taps of kernel row r (p.taps at a time) read of channel block cb, for
+        // each plane of the image (8-bit activations in two planes: x_lo, then 16 x_hi)
+        const uint32_t bytes = (uint32_t)(BM + p.taps - 1) * kBK;
+        uint32_t s = 0, ph = 0;
+        for (int t = first_tile; t < tile_end && ok; t += p.tile_stride) {
+          const TileInfo ti = tile_info(p, t);
           const ConvJobDev& jb = p.jobs[ti.job];
           const FlatTile ft = flat_tile(jb, ti.mt, kTileRows);
-          row0 = jb.row_off + ft.img * jb.hp * jb.wp + ft.v0 + (int)rank * 128;
-          wp = jb.wp;
+          const int row0 = jb.row_off + ft.img * jb.hp * jb.wp + ft.v0 + (int)rank * 128;
+          const CUtensorMap* am = &maps.a[ti.layer & 1];  // layers read the two images in turn
+          // the previous layer's tiles that this tile reads (and that read what it writes)
+          if (ti.layer > 0 && !wait_dep_tiles<kTileRows>(p, ti.layer, ti.job, ti.mt, abort_flag)) { ok = false; break; }
+          for (int pr = 0; pr < p.a_planes * p.kh && ok; ++pr) {
+            const int plane = pr >= p.kh ? 1 : 0;
+            const int row = row0 + plane * p.plane_rows + (pr - plane * p.kh) * jb.wp;
+            for (int cb = 0; cb < p.cin_chunks && ok; ++cb)
+              for (int sx = 0; sx < p.kw; sx += p.taps, s = (s + 1 == (uint32_t)S) ? 0 : s + 1, ph ^= (s == 0)) {
+                if (!mbar_wait(b_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+                load(s_a + s * p.slab_bytes, am, cb * kBK, row + sx, b_full + 8 * s, bytes);
+              }
+          }
         }
-        const CUtensorMap* wm = ti.bn == BN ? &maps.w[ti.layer] : &maps.wh;
-        const CUtensorMap* am = &maps.a[ti.layer & 1];  // layers read the two images in turn
-        bool deps_ready = !kFlat || ti.layer == 0;
-        for (int q2 = 0; q2 < nk; ++q2, ++it, s = (s + 1 == (uint32_t)S) ? 0 : s + 1, ph ^= (s == 0)) {
-          if ((int)(it % kTma) != tw) continue;
-          if (!deps_ready) {
-            // the previous layer's tiles that this tile reads (and that read what it writes)
-            if (!wait_dep_tiles<kTileRows>(p, ti.layer, ti.job, ti.mt, abort_flag)) { ok = false; break; }
-            deps_ready = true;
+      } else if (p.resident) {
+        // all weight tiles, once, by one thread; their barrier counts them all
+        if (tw == 1) {
+          for (int nt = 0, i = 0; nt < p.n_tiles; ++nt)
+            for (int r = 0; r < p.kh; ++r)
+              for (int cb = 0; cb < p.cin_chunks; ++cb)
+                for (int sx = 0; sx < p.kw; ++sx, ++i)
+                  load(s_b + i * stage_b_bytes, &maps.w[0], ((r * p.kw + sx) * p.cin_chunks + cb) * kBK,
+                       nt * BN + (int)rank * (BN / 2), b_wfull,
+                       i == 0 ? (uint32_t)(p.n_tiles * p.num_kchunks) * stage_b_bytes : 0u);
+        }
+      } else {
+        // weight tiles in the MMA's order (r, cb, s), the two threads taking every other one
+        uint32_t it = 0, s = 0, ph = 0;
+        for (int t = first_tile; t < tile_end && ok; t += p.tile_stride) {
+          const TileInfo ti = tile_info(p, t);
+          const CUtensorMap* wm = ti.bn == BN ? &maps.w[ti.layer] : &maps.wh;
+          const int rows = kPair ? ti.bn / 2 : ti.bn, brow = ti.brow + (int)rank * rows;
+          for (int pr = 0; pr < p.a_planes * p.kh && ok; ++pr) {
+            const int r = pr >= p.kh ? pr - p.kh : pr;
+            for (int cb = 0; cb < p.cin_chunks && ok; ++cb)
+              for (int sx = 0; sx < p.kw; ++sx, ++it, s = (s + 1 == (uint32_t)SB) ? 0 : s + 1, ph ^= (s == 0)) {
+                if ((int)(it & 1) != tw - 1) continue;
+                if (!mbar_wait(b_wempty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
+                load(s_b + s * stage_b_bytes, wm, ((r * p.kw + sx) * p.cin_chunks + cb) * kBK, brow, b_wfull + 8 * s,
+                     (uint32_t)rows * kBK);
+              }
           }
-          if (!mbar_wait(b_empty + 8 * s, ph ^ 1, abort_flag)) { ok = false; break; }
-          // plane of the byte image (8-bit activations: x_lo, then 16 x_hi) and K chunk in it
-          const int plane = q2 >= p.num_kchunks ? 1 : 0;
-          const int q = q2 - plane * p.num_kchunks;
-          const int prow = plane * p.plane_rows;
-          int r, sx, cb;
-          if (q < kQTab) {
-            const uint32_t e = qtab[q];
-            r = (int)(e >> 24); sx = (int)((e >> 16) & 255u); cb = (int)(e & 0xFFFFu);
-          } else {
-            const int tap = q / p.cin_chunks;
-            cb = q - tap * p.cin_chunks;
-            r = tap / p.kw; sx = tap - r * p.kw;
-          }
-          if constexpr (kPair) {
-            // this CTA's 128 rows of A and its half of B; both CTAs' copies complete on the
-            // leader's "full" barrier, which the leader arms with the bytes of all four
-            const int row = row0 + prow + r * wp + sx;
-            const int brow = ti.brow + (int)rank * (ti.bn / 2);
-            const uint32_t b_bytes = (uint32_t)(ti.bn / 2) * kBK;
-            if (leader) {
-              mbar_arrive_expect_tx(b_full + 8 * s, 2 * (b_bytes + kStA));
-              tma_load_2d(s_a + s * kStA, am, cb * kBK, row, b_full + 8 * s);
-              tma_load_2d(s_b + s * stage_b_bytes, wm, q * kBK, brow, b_full + 8 * s);
-            } else {
-              const uint32_t fb = mapa_shared(b_full + 8 * s, 0);
-              tma_load_2d_pair(s_a + s * kStA, am, cb * kBK, row, fb);
-              tma_load_2d_pair(s_b + s * stage_b_bytes, wm, q * kBK, brow, fb);
-            }
-            continue;
-          } else if constexpr (kFlat) {
-            // A: 128 consecutive rows of the padded byte image, shifted by the tap (r, s)
-            const int row = row0 + prow + r * wp + sx;
-            mbar_arrive_expect_tx(b_full + 8 * s, (uint32_t)ti.bn * kBK + kStA);
-            tma_load_2d(s_a + s * kStA, am, cb * kBK, row, b_full + 8 * s);
-          } else {
-            (void)r; (void)sx; (void)cb;
-            mbar_arrive_expect_tx(b_full + 8 * s, (uint32_t)ti.bn * kBK);
-          }
-          tma_load_2d(s_b + s * stage_b_bytes, wm, q * kBK, ti.brow, b_full + 8 * s);
         }
       }
       if (!ok) fail(abort_flag, p.status);
@@ -747,6 +844,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       if (++l_q == nk) { l_q = 0; l_tile += p.tile_stride; }
     };
     bool ok = true;
+    const int S = p.stages;
+    uint32_t b_empty, b_wfull, b_wempty;
+    slots(b_empty, b_wfull, b_wempty);
     auto consume = [&](int c, const uint32_t (&w)[4 * kXBits]) -> bool {
       const uint32_t s = c % S, ph = (c / S) & 1;
       if (!mbar_wait(b_empty + 8 * s, ph ^ 1, abort_flag)) return false;
@@ -807,7 +907,16 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     // without table loads or barriers
     uint32_t cur_key = 0xFFFFFFFFu;  // (first channel, half width, job, layer) of the tables
     int flags = 0;
-    for (int t = first_tile; t < tile_end; t += p.tile_stride, ++lt) {
+    for (;; ++lt) {
+      // (worked out anew for every tile: no register to spare for the range)
+      int t = (kPair ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) + (int)lt * p.tile_stride;
+      if (!kPair && p.contig) {
+        const int b = (int)blockIdx.x;
+        t = b * p.share + (b < p.extra ? b : p.extra) + (int)lt;
+        if ((int)lt >= p.share + (b < p.extra ? 1 : 0)) break;
+      } else if (t >= p.total_tiles) {
+        break;
+      }
       const TileInfo ti = tile_info(p, t);
       const ConvJobDev& jb = p.jobs[ti.job];
       // this tile's output channels that exist (a last N tile may reach past cout; packed
@@ -1029,7 +1138,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const bool sk_codes = kSkip && p.skip_bits <= 4;
       if (sk_codes && c_lo < c_hi) sw = load_skip_words(srow, c_lo, p.skip_bits, row_ok);
       __syncwarp();
-      if (!mbar_wait(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) {
+      if (!mbar_wait_inline(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) {
         if constexpr (kSkip) cp_async_wait<0>();  // (no copy outlives the block)
         ok = false;
         break;
@@ -1654,34 +1763,57 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.epi_sets = warp_groups / prm.epi_groups;
   if (prm.epi_sets == 3) prm.epi_sets = 2;  // (a power of two: tiles are dealt by their low bits)
   prm.dep_target = (uint32_t)(8 * prm.epi_groups);  // a tile's epilogue warps, both CTAs of a pair
-  // shared memory plan: stages of (BM x bk A bytes + this CTA's B rows x bk bytes)
+  // shared memory plan. Flat path: a ring of activation slabs and one of weight tiles (this CTA's B
+  // rows x bk bytes), or all weight tiles resident. Otherwise stages of both operands.
   const int b_rows = pair ? BN / 2 : BN;
-  const size_t stage_a = (size_t)BM * bk;
-  const size_t stage_bytes = stage_a + (size_t)b_rows * bk;
+  const size_t b_tile = (size_t)b_rows * bk;
+  prm.taps = a.kw <= 16 ? a.kw : 1;
+  const size_t slab = flat ? ((size_t)(BM + prm.taps - 1) * bk + 1023) / 1024 * 1024 : (size_t)BM * bk;
   const size_t epi_bytes = EpiTab::kBytes;
-  const size_t bar_bytes = 8 * (2 * kMaxStages + 2 * kMaxBufs + 1) + 16;
-  const size_t qtab_bytes = kQTab * sizeof(uint32_t);
+  const size_t bar_bytes = 8 * (4 * kMaxStages + 2 * kMaxBufs + 1) + 16;
   const size_t sk_bytes = !a.has_skip ? 0 : (a.skip_bits == 32 ? (size_t)epi_warps(flat) * 2 * kSkipStage : skip_tab_bytes(a.skip_bits));
   const size_t budget = 232448 - 1024;  // max dynamic smem per block minus alignment slack
-  // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least 6 stages remain
+  const size_t fixed = epi_bytes + bar_bytes + sk_bytes + 32;
+  // int32 outputs with cout % 4 == 0: per-warp staging blocks when at least two slabs and their weight
+  // tiles remain
   const size_t ostage_bytes = (size_t)epi_warps(flat) * 32 * kStageRow * sizeof(uint32_t);
   const bool ostage = flat && bk == BK && a.out_bits == 32 && a.cout % 4 == 0 && !a.has_skip && !a.split_w && !f16 &&
-                      (budget - epi_bytes - bar_bytes - qtab_bytes - ostage_bytes) / stage_bytes >= 6;
-  int stages = (int)((budget - epi_bytes - bar_bytes - qtab_bytes - sk_bytes - 32 - (ostage ? ostage_bytes : 0)) / stage_bytes);
-  if (stages > kMaxStages) stages = kMaxStages;
-  if (stages < 2) { *err = "conv_tc: shared memory plan does not fit"; return 2; }
-  // The TMA issuers take K chunks round-robin and each waits on its stage's "empty"
-  // barrier by phase parity. That parity is unambiguous only while no issuer can run more
-  // than one phase ahead of the last completed one, which holds when the issuers are at
-  // most as many as the stages.
-  if (stages < tma_warps(flat)) { *err = "conv_tc: fewer pipeline stages than TMA issuers"; return 2; }
+                      budget >= fixed + ostage_bytes + 2 * (slab + (size_t)prm.taps * b_tile);
+  const size_t avail = budget - fixed - (ostage ? ostage_bytes : 0);
+  int stages = 0, stages_b = 0;
+  if (flat) {
+    // Resident weights: every N tile's, where they leave at least 3 slabs and a third of the room. (A
+    // half-width tile takes other rows per CTA of a pair: a launch with such tiles streams.)
+    const size_t all_w = (size_t)prm.n_tiles * prm.num_kchunks * b_tile;
+    prm.resident = nlayers <= 1 && prm.dp_tiles == tiles && all_w * 3 <= avail * 2 && all_w + 3 * slab <= avail;
+    if (prm.resident) {
+      stages = (int)((avail - all_w) / slab);
+      stages_b = 1;
+    } else {
+      stages = (int)(avail / (slab + (size_t)prm.taps * b_tile));
+      if (stages < 2) stages = 2;
+      if (stages > kMaxStages) stages = kMaxStages;
+      if (avail < stages * slab + 2 * b_tile) { *err = "conv_tc: shared memory plan does not fit"; return 2; }
+      stages_b = (int)((avail - stages * slab) / b_tile);
+      if (stages_b > kMaxStages) stages_b = kMaxStages;
+    }
+    if (stages > kMaxStages) stages = kMaxStages;
+  } else {
+    stages = (int)(avail / (slab + b_tile));
+    if (stages > kMaxStages) stages = kMaxStages;
+    if (stages < 2) { *err = "conv_tc: shared memory plan does not fit"; return 2; }
+  }
+  // (The weight issuers take tiles round-robin and wait on their stage's "empty" barrier by phase
+  // parity, which is unambiguous while there are at least as many stages as issuers: two.)
   prm.stages = stages;
-  prm.off_b = (uint32_t)(stages * stage_a);
-  prm.off_epi = prm.off_b + (uint32_t)(stages * b_rows * bk);
+  prm.stages_b = stages_b;
+  prm.slab_bytes = (uint32_t)slab;
+  prm.off_b = (uint32_t)(stages * slab);
+  const size_t b_all = flat ? (prm.resident ? (size_t)prm.n_tiles * prm.num_kchunks : (size_t)stages_b) * b_tile : stages * b_tile;
+  prm.off_epi = (uint32_t)((prm.off_b + b_all + 15) / 16 * 16);
   prm.off_bar = prm.off_epi + (uint32_t)epi_bytes;
-  prm.off_qtab = prm.off_bar + (uint32_t)bar_bytes;
   // (a launch has a skip table or staging blocks, not both: staged outputs have no skip)
-  const uint32_t off_end = (uint32_t)((prm.off_qtab + qtab_bytes + 15) / 16 * 16);
+  const uint32_t off_end = (uint32_t)((prm.off_bar + bar_bytes + 15) / 16 * 16);
   prm.off_ostage = prm.off_sktab = off_end;
   const size_t smem = 1024 + off_end + (ostage ? ostage_bytes : sk_bytes);
   // two accumulators of BN fp32 columns, or four where they fit beside the 32 columns of scales
@@ -1728,6 +1860,8 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const int units = prm.total_tiles;
   int grid = units < sms ? units : sms;
   if (pair) grid = 2 * (units < sms / 2 ? units : sms / 2);
+  prm.share = prm.total_tiles / grid;
+  prm.extra = prm.total_tiles % grid;
   prm.tile_stride = pair ? grid / 2 : (prm.contig ? 1 : grid);
   const bool in_tap = (a.cin % BK) == 0;
   if (flat) {
@@ -1772,11 +1906,11 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
     }
     if (a.expand_only) return 0;
     // 2) tensor maps over the workspace (and, for chained layers in one launch, the second
-    //    image) as [rows][cin] byte matrices with bk x 128 boxes
+    //    image) as [rows][cin] byte matrices with boxes of a slab
     // (a nibble image keeps the byte image's row stride: cin bytes, the first cin / 2 used)
     cuuint64_t gd[2] = {(cuuint64_t)img_row, (cuuint64_t)rows * (cuuint64_t)prm.a_planes};
     cuuint64_t gs[1] = {(cuuint64_t)(f16 ? 2 * a.cin : a.cin)};
-    cuuint32_t bx[2] = {(cuuint32_t)bk, 128};
+    cuuint32_t bx[2] = {(cuuint32_t)bk, (cuuint32_t)(BM + prm.taps - 1)};
     for (int i = 0; i < (nlayers > 1 ? 2 : 1); ++i) {
       // (a nibble image row uses 128 of every 256 bytes: fetch 128-byte lines from DRAM)
       const CUresult r2 = enc(&maps.a[i], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void*)(i == 0 ? a.ws : a.ws2), gd, gs, bx,

@@ -107,7 +107,7 @@ __device__ __forceinline__ bool mbar_poll(uint32_t bar, uint32_t parity, volatil
 // Bounded wait: false if the deadline (kLimitNs after the call) passed or another role
 // aborted. The kernels use the 1 s limit; the wait self-test instantiates a short one.
 template <uint64_t kLimitNs = kTimeoutNs>
-static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+__device__ __forceinline__ bool mbar_wait_loop(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   const uint64_t deadline = globaltimer() + kLimitNs;
   for (uint32_t spin = 1;; ++spin) {
     if (AQD_WAIT_HINT_NS > 0 ? mbar_try_sleep(bar, parity, AQD_WAIT_HINT_NS) : mbar_try(bar, parity)) return true;
@@ -117,10 +117,18 @@ static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity
     }
   }
 }
+template <uint64_t kLimitNs = kTimeoutNs>
+static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return mbar_wait_loop<kLimitNs>(bar, parity, abort_flag);
+}
 
 template <uint64_t kLimitNs = kTimeoutNs>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   return mbar_try(bar, parity) || mbar_wait_slow<kLimitNs>(bar, parity, abort_flag);
+}
+// The same without a call, where the caller has no registers to keep across one.
+__device__ __forceinline__ bool mbar_wait_inline(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+  return mbar_try(bar, parity) || mbar_wait_loop<kTimeoutNs>(bar, parity, abort_flag);
 }
 
 __device__ __forceinline__ void fail(volatile int* abort_flag, uint32_t* status) {

@@ -1,5 +1,5 @@
-"""The conv epilogue's forms at the sizes where their choice changes, byte for byte against the
-oracle: the 32-bit skip rescale and its limits, rows of no whole 32-channel groups, column
+"""The conv kernel's forms at the sizes where their choice changes, byte for byte against the
+oracle: slabs shared by the taps of a kernel row, the skip forms and their limits, rows of no whole 32-channel groups, column
 counts that leave warps idle or let sets of warps take tiles in turn, and accumulators too
 large for the common form."""
 import numpy as np
@@ -120,3 +120,21 @@ def test_f16_pipe_bit_exact(cin, k, cout, out_bits, shape, path):
                                 shift=None if out_bits == 32 else sh, bias=b, workspace=True, path=path)
     assert used == {0: 4, 2: 2, 3: 3}[path]
     assert_same(got, want, cout, out_bits, f"F16 pipe {cin}x{k}x{k} -> {cout}")
+
+
+# taps per slab 1, 2, 3, 5, 7 and 16, kernels too wide for one (17); resident weights with one and two
+# N tiles and with two planes of an 8-bit image; weights streamed beside half-width tiles
+@pytest.mark.parametrize("kh,kw,pad,cin,cout,bits", [(1, 1, 0, 128, 512, 4), (2, 2, 0, 64, 128, 3), (3, 3, 1, 64, 512, 4),
+                                                     (3, 3, 1, 128, 64, 8), (3, 3, 1, 256, 256, 2), (5, 5, 2, 64, 96, 4),
+                                                     (7, 7, 3, 64, 64, 2), (1, 16, 0, 64, 32, 4), (3, 17, 1, 128, 64, 4),
+                                                     (1, 17, 0, 64, 272, 2), (17, 1, 0, 64, 64, 4)])
+@pytest.mark.parametrize("path", [0, 3])
+def test_slabs_bit_exact(kh, kw, pad, cin, cout, bits, path):
+    rng = np.random.default_rng(kh * 31 + kw + cin)
+    x = synth.act_codes(rng, (2, 41, 83, cin), bits)
+    wb = min(bits, 4)
+    wt = synth.weight_codes(rng, (cout, kh, kw, cin), wb)
+    m0, sh, b = tables(rng, cout, 3.0 * (1 << bits) * np.sqrt(kh * kw * cin) / 4, 4)
+    got, want, used = conv_pair(x, bits, wt, wb, pad=pad, out_bits=4, m0=m0, shift=sh, bias=b, workspace=True, path=path)
+    assert used == (6 if bits == 2 and cin == 256 and cout <= 240 else 4 if path == 0 else 3)
+    assert_same(got, want, cout, 4, f"{kh}x{kw} {cin}->{cout}")
