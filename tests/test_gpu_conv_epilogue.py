@@ -127,7 +127,7 @@ def test_f16_pipe_bit_exact(cin, k, cout, out_bits, shape, path):
 @pytest.mark.parametrize("kh,kw,pad,cin,cout,bits", [(1, 1, 0, 128, 512, 4), (2, 2, 0, 64, 128, 3), (3, 3, 1, 64, 512, 4),
                                                      (3, 3, 1, 128, 64, 8), (3, 3, 1, 256, 256, 2), (5, 5, 2, 64, 96, 4),
                                                      (7, 7, 3, 64, 64, 2), (1, 16, 0, 64, 32, 4), (3, 17, 1, 128, 64, 4),
-                                                     (1, 17, 0, 64, 272, 2), (17, 1, 0, 64, 64, 4)])
+                                                     (1, 17, 0, 64, 288, 2), (17, 1, 0, 64, 64, 4)])
 @pytest.mark.parametrize("path", [0, 3])
 def test_slabs_bit_exact(kh, kw, pad, cin, cout, bits, path):
     rng = np.random.default_rng(kh * 31 + kw + cin)
