@@ -68,6 +68,7 @@ struct StemParams {
   int32_t n, h, w, ho, wo, stride, pad;
   int32_t m_total, hw_out; // n * ho * wo (< 2^31, checked on the host), ho * wo
   int32_t cout, n_pad, out_bits, level, total_tiles, stages, tmem_cols;
+  int32_t strips, nbuf_log2;  // (rows kernel) strips of 128 output columns, accumulators
   int64_t y_row_bytes;
   const int32_t* m0;
   const int8_t* shift;
@@ -173,6 +174,108 @@ __device__ __noinline__ uint4 general_cols(uint32_t taddr, const EpiChan* c, int
   return make_uint4(bw[0], bw[1], bw[2], bw[3]);
 }
 
+// int32 outputs of 16 columns: sum + bias, saturating.
+__device__ __noinline__ void sums_int32(uint32_t taddr, const EpiChan* c, uint4* y, bool valid) {
+  uint32_t v[16];
+  tmem_ld16(taddr, v);
+  tmem_wait_ld();
+  reg_fence16(v);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = (uint32_t)add_sat(__float2int_rn(__uint_as_float(v[i])), c[i].bias);
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (valid) y[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+  __syncwarp();
+}
+
+// One float add turns an exact sum v, |v| < 2^22, into the int32 v + kMagicBits: the mantissa of
+// 1.5 x 2^23 + v. (The conversion instruction runs at a sixteenth of the add's rate.)
+constexpr float kMagic = 12582912.0f;
+constexpr uint32_t kMagicBits = 0x4B400000u;
+
+// Per-channel constants of the launch's level: {bias - kMagicBits, M0, 2^(R-33), R-32} and the int64
+// form. The 32-bit form holds (and 1 stays in *s_fast) where every R >= 33, |bias| <= 2^30, and
+// every |sum| < 2^22 (weights_small).
+__device__ __forceinline__ void load_channels(const StemParams& p, int4* cst4, EpiChan* cste, int* s_fast) {
+  int fast = 1;
+  for (int n = threadIdx.x; n < p.n_pad; n += blockDim.x) {
+    EpiChan ec{};
+    int4 c4 = make_int4(0, 0, 0, 0);
+    if (n < p.cout) {
+      const int64_t idx = (int64_t)p.level * p.cout + n;
+      ec.bias = p.bias ? p.bias[idx] : 0;
+      if (p.out_bits != 32) {
+        ec.m0 = p.m0[idx];
+        const int r = 31 + p.shift[idx];
+        ec.r = (int8_t)r;
+        if (r >= 33 && ec.bias >= -(1 << 30) && ec.bias <= (1 << 30))
+          c4 = make_int4((int)((uint32_t)ec.bias - kMagicBits), ec.m0, 1 << (r - 33), r - 32);
+        else fast = 0;
+      }
+    }
+    cst4[n] = c4;
+    cste[n] = ec;
+  }
+  if (!fast) atomicAnd(s_fast, 0);
+}
+
+__device__ __forceinline__ uint32_t abs_f16(uint16_t w) {
+  return (uint32_t)__half2int_rn(__ushort_as_half(w & 0x7FFFu));
+}
+// a channel's sum of |w| (the warp's lanes each hold a part): every |sum of products| < 2^22
+__device__ __forceinline__ bool weights_small(uint32_t part) { return __reduce_add_sync(0xffffffffu, part) * 255u < (1u << 22); }
+
+// kTiles accumulators' columns of one output pixel each: the 32-column groups 0, 2, .. (odd = 0)
+// or 1, 3, .. (odd = 1), 16 columns at a time (cout is a multiple of 16). Constants are read from
+// shared memory once for all tiles; release() hands the accumulators back after the last read.
+template <int kTiles, class Release>
+__device__ __forceinline__ void drain_pixels(const StemParams& p, const uint32_t (&tbase)[kTiles], uint8_t* const (&yrow)[kTiles],
+                                             const bool (&valid)[kTiles], int odd, bool fast, const int4* cst4,
+                                             const EpiChan* cste, Release&& release) {
+  const int qmax = (1 << (p.out_bits & 15)) - 1;
+  uint32_t top[kTiles] = {};  // (3-bit codes: see store_codes16)
+  if (fast && p.out_bits != 32) {
+    if (32 * odd >= p.cout) release();
+#pragma unroll 1
+    for (int c0 = 32 * odd, next; c0 < p.cout; c0 = next) {
+      next = c0 + ((c0 & 16) ? 48 : 16);
+      uint32_t v[kTiles][16], bw[kTiles][4] = {};
+#pragma unroll
+      for (int k = 0; k < kTiles; ++k) tmem_ld16(tbase[k] + (uint32_t)c0, v[k]);
+      tmem_wait_ld();
+#pragma unroll
+      for (int k = 0; k < kTiles; ++k) reg_fence16(v[k]);
+      if (next >= p.cout) release();
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int4 c = cst4[c0 + i];
+#pragma unroll
+        for (int k = 0; k < kTiles; ++k)
+          bw[k][i / 4] += requant32(__float_as_int(__uint_as_float(v[k][i]) + kMagic) + c.x, c, qmax) << (8 * (i % 4));
+      }
+#pragma unroll
+      for (int k = 0; k < kTiles; ++k)
+        if (valid[k]) store_codes16(yrow[k], c0, bw[k], p.out_bits, top[k]);
+    }
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < kTiles; ++k) {
+#pragma unroll 1
+    for (int c0 = 32 * odd; c0 < p.cout; c0 += (c0 & 16) ? 48 : 16) {
+      if (p.out_bits == 32) {
+        sums_int32(tbase[k] + (uint32_t)c0, cste + c0, reinterpret_cast<uint4*>(yrow[k]) + (c0 >> 2), valid[k]);
+      } else {
+        const uint4 r = general_cols(tbase[k] + (uint32_t)c0, cste + c0, p.out_bits);
+        __syncwarp();
+        const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
+        if (valid[k]) store_codes16(yrow[k], c0, bw, p.out_bits, top[k]);
+      }
+    }
+  }
+  release();
+}
+
 __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant__ StemParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -232,29 +335,15 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
     }
     *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) = pr;
   }
-  int fast = 1;
-  for (int n = threadIdx.x; n < p.n_pad; n += blockDim.x) {
-    EpiChan ec{};
-    int4 c4 = make_int4(0, 0, 0, 0);
-    if (n < p.cout) {
-      const int64_t idx = (int64_t)p.level * p.cout + n;
-      ec.bias = p.bias ? p.bias[idx] : 0;
-      c4.x = ec.bias;
-      if (p.out_bits != 32) {
-        ec.m0 = p.m0[idx];
-        const int r = 31 + p.shift[idx];
-        ec.r = (int8_t)r;
-        if (r >= 33) c4 = make_int4(ec.bias, ec.m0, 1 << (r - 33), r - 32);
-        else fast = 0;
-      }
-    }
-    cst4[n] = c4;
-    cste[n] = ec;
+  load_channels(p, cst4, cste, s_fast);
+  for (int n = warp; n < p.cout; n += kThreads / 32) {
+    uint32_t part = 0;
+    for (int k = lane; k < kKH * kSeg; k += 32) part += abs_f16((uint16_t)p.w_i16[(int64_t)n * (kKH * kSeg) + k]);
+    if (!weights_small(part) && lane == 0) atomicAnd(s_fast, 0);
   }
-  if (!fast) atomicAnd(s_fast, 0);
   fence_proxy_async();  // generic-proxy stores of B -> visible to the MMA
   __syncthreads();
-  const bool fast_req = *s_fast != 0;
+  const bool fast = *s_fast != 0;
 
   const int first = blockIdx.x, stride_t = gridDim.x;
   if (warp == kWarpMma) {
@@ -305,7 +394,6 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
     // ------------------------------------------------------------ epilogue (warps 0..7)
     const int quarter = warp & 3;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
-    const int qmax = (1 << (p.out_bits & 15)) - 1;
     uint32_t lt = 0;
     bool ok = true;
     for (int t = first; t < p.total_tiles; t += stride_t, ++lt) {
@@ -313,49 +401,312 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       const int mg = t * 128 + quarter * 32 + lane;
       const bool valid = mg < p.m_total;
       uint8_t* yrow = p.y + (int64_t)(valid ? mg : 0) * p.y_row_bytes;
-      uint32_t top = 0u;  // (3-bit codes: see store_codes16)
       if (!mbar_wait(b_tfull + 8 * buf, (lt >> 1) & 1, abort_flag)) { ok = false; break; }
       tc_fence_after();
-      // 16 columns at a time, in whole 32-column groups (cout is a multiple of 16)
-#pragma unroll 1
-      for (int c0 = 32 * (warp >> 2); c0 < p.cout; c0 += (c0 & 16) ? 16 + 32 * (kEpiWarps / 4 - 1) : 16) {
-        const uint32_t taddr = lane_base + buf * (uint32_t)p.n_pad + (uint32_t)c0;
-        uint32_t bw[4] = {0u, 0u, 0u, 0u};
-        if (p.out_bits == 32 || fast_req) {
-          uint32_t v[16];
-          tmem_ld16(taddr, v);
-          tmem_wait_ld();
-          reg_fence16(v);
-          if (p.out_bits == 32) {
-            uint4* y4 = reinterpret_cast<uint4*>(yrow) + (c0 >> 2);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = (uint32_t)add_sat(__float2int_rn(__uint_as_float(v[i])), cst4[c0 + i].x);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              if (valid) y4[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-            continue;
-          }
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int4 c = cst4[c0 + i];  // bias, M0, 2^(R-33), R-32
-            bw[i / 4] += requant32(add_sat(__float2int_rn(__uint_as_float(v[i])), c.x), c, qmax) << (8 * (i % 4));
-          }
-        } else {
-          const uint4 r = general_cols(taddr, cste + c0, p.out_bits);
-          __syncwarp();
-          bw[0] = r.x; bw[1] = r.y; bw[2] = r.z; bw[3] = r.w;
-        }
-        if (valid) store_codes16(yrow, c0, bw, p.out_bits, top);
-      }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive_relaxed(b_tempty + 8 * buf);
+      const uint32_t tbase[1] = {lane_base + buf * (uint32_t)p.n_pad};
+      uint8_t* const yrows[1] = {yrow};
+      const bool valids[1] = {valid};
+      drain_pixels<1>(p, tbase, yrows, valids, warp >> 2, fast, cst4, cste, [&] {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_relaxed(b_tempty + 8 * buf);
+      });
     }
     if (!ok) fail(abort_flag, p.status);
   }
   tc_fence_before();
   __syncthreads();
   if (warp == kWarpMma) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
+  }
+}
+
+// ------------------------------------------------------------------ stride 2: no im2col
+// With 4 channels per pixel (the fourth 0) in F16 a pixel is 8 bytes, so at stride 2 the receptive
+// fields of neighbouring output pixels start 16 bytes apart in an image row: one core-matrix row.
+// The image row itself is then the A operand of one kernel row: 8 output pixels are 128 contiguous
+// bytes, the next 16 bytes of K lie 16 bytes further (leading offset 16: core matrices overlap), the
+// next 8 pixels 128. Seven pixels and an eighth with zero weights are K = 32 per kernel row, 224 in
+// all. An image pixel is converted once per tile row pair instead of 12 times, and a CTA's tiles
+// go down the rows of a strip of 128 output columns, so that each tile brings two new image rows.
+//   warps 0..7    epilogue, two tiles at a time
+//   warp  8       TMEM allocation + one thread issuing tcgen05.mma (M=128, N=cout, 14 of K=16)
+//   warps 9..18   producers: two sets of 5 take row pairs in turn, 4 pixels per thread, the words
+//                 of the next pair loaded before this one is written
+constexpr int kRK = 32 * kKH;                // K
+constexpr int kRSBO = (kRK / 8) * 128;       // 8-row groups of the weights
+constexpr int kRowUnits = 132;               // 2-pixel units of a strip's row: 127 + 4, and one to make groups whole
+constexpr int kRowBytes = kRowUnits * 16;
+constexpr int kPairBytes = 2 * kRowBytes;
+constexpr int kPairs = 16;                   // ring of row pairs (a tile reads 4)
+constexpr int kRowGroups = kRowUnits / 2;    // 4-pixel groups
+constexpr int kRSets = 2, kRSetWarps = (2 * kRowGroups + 31) / 32;
+constexpr int kREpiWarps = 8, kRWarpMma = kREpiWarps, kRWarpProd0 = kREpiWarps + 1;
+constexpr int kRThreads = (kRWarpProd0 + kRSets * kRSetWarps) * 32;
+constexpr int kMaxBufs = 4;
+static_assert((kPairs & (kPairs - 1)) == 0 && kPairs > 4, "ring");
+
+// A CTA's contiguous tiles [t, end), numbered (image, strip, output row), as runs down one strip.
+struct Run {
+  int t, end, img, strip, h0, len;
+  __device__ __forceinline__ Run(const StemParams& p, int t0, int t1) : t(t0), end(t1) {
+    const int col = t / p.ho;
+    h0 = t - col * p.ho;
+    img = col / p.strips;
+    strip = col - img * p.strips;
+    len = min(p.ho - h0, end - t);
+  }
+  __device__ __forceinline__ bool done() const { return t >= end; }
+  __device__ __forceinline__ void next(const StemParams& p) {
+    t += len;
+    h0 = 0;
+    if (++strip == p.strips) { strip = 0; ++img; }
+    len = min(p.ho, end - t);
+  }
+};
+
+// 12 code bytes of 4 pixels as loaded: aligned words and the shift that realigns them, and the bytes to keep.
+struct Group {
+  uint32_t w[4];
+  uint32_t shr, keep;  // keep: bit i = pixel i lies inside the image
+};
+
+__device__ __forceinline__ Group load_group(const StemParams& p, int img, int hi, int wi) {
+  Group g{};
+  if (hi < 0 || hi >= p.h || wi <= -4 || wi >= p.w) return g;
+  const int64_t a = (((int64_t)img * p.h + hi) * p.w + wi) * kC;
+  const int64_t a4 = a & ~(int64_t)3;
+  g.shr = 8u * (uint32_t)(a & 3);
+  g.keep = 15u;
+  if (wi < 0) g.keep &= 15u << -wi;
+  if (wi + 4 > p.w) g.keep &= 15u >> (wi + 4 - p.w);
+  if (a4 >= 0 && a4 + 16 <= p.x_bytes) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(p.x + a4);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) g.w[i] = __ldg(src + i);
+  } else {  // the first and last bytes of the tensor
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (a4 + i >= 0 && a4 + i < p.x_bytes) g.w[i / 4] |= (uint32_t)__ldg(p.x + a4 + i) << (8 * (i % 4));
+  }
+  return g;
+}
+
+__device__ __forceinline__ uint32_t f16_bytes(uint32_t a, uint32_t sel) {  // 1024 + x, minus 1024
+  uint32_t r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(__byte_perm(a, kF16Pair1024, sel)), "r"(kF16Pair1024));
+  return r;
+}
+
+__device__ __forceinline__ void store_group(const Group& g, uint8_t* dst) {
+  uint32_t b[4];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) b[i] = __funnelshift_r(g.w[i], g.w[i + 1], g.shr);
+  b[3] = b[2] >> 8;                              // pixel 3
+  b[2] = __funnelshift_r(b[1], b[2], 16);        // pixel 2
+  b[1] = __funnelshift_r(b[0], b[1], 24);        // pixel 1
+#pragma unroll
+  for (int i = 0; i < 4; ++i) b[i] = (g.keep >> i) & 1u ? b[i] : 0u;
+  // {x0, x1}, {x2, 0}: bytes of the permute are x, 0x64 and, for the fourth channel, 0x00, 0x64
+  *reinterpret_cast<uint4*>(dst) = make_uint4(f16_bytes(b[0], 0x5150u), f16_bytes(b[0], 0x5452u),
+                                              f16_bytes(b[1], 0x5150u), f16_bytes(b[1], 0x5452u));
+  *reinterpret_cast<uint4*>(dst + 16) = make_uint4(f16_bytes(b[2], 0x5150u), f16_bytes(b[2], 0x5452u),
+                                                   f16_bytes(b[3], 0x5150u), f16_bytes(b[3], 0x5452u));
+}
+
+__device__ __forceinline__ uint64_t sdesc_offsets(uint32_t saddr, int lbo, int sbo) {
+  uint64_t d = (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)(lbo >> 4) << 16;
+  d |= (uint64_t)(sbo >> 4) << 32;
+  d |= (uint64_t)1 << 46;  // descriptor version; swizzle field 0 = none
+  return d;
+}
+
+__global__ void __launch_bounds__(kRThreads, 1) stem_rows_kernel(const __grid_constant__ StemParams p) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t s_a = smem_u32(smem);
+  const uint32_t s_b = s_a + p.off_b;
+  int4* cst4 = reinterpret_cast<int4*>(smem + p.off_cst);
+  EpiChan* cste = reinterpret_cast<EpiChan*>(smem + p.off_cst + 256 * sizeof(int4));
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
+  const uint32_t b_full = smem_u32(bars);
+  const uint32_t b_empty = b_full + 8 * kPairs;
+  const uint32_t b_tfull = b_empty + 8 * kPairs;
+  const uint32_t b_tempty = b_tfull + 8 * kMaxBufs;
+  const uint32_t b_final = b_tempty + 8 * kMaxBufs;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kPairs + 2 * kMaxBufs + 1);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  int* s_fast = reinterpret_cast<int*>(tmem_slot + 2);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kPairs; ++s) {
+      mbar_init(b_full + 8 * s, kRSetWarps);
+      mbar_init(b_empty + 8 * s, 1);
+    }
+    for (int b = 0; b < kMaxBufs; ++b) {
+      mbar_init(b_tfull + 8 * b, 1);
+      mbar_init(b_tempty + 8 * b, kREpiWarps);
+    }
+    mbar_init(b_final, 1);
+    *abort_flag = 0;
+    *s_fast = 1;
+    fence_barrier_init();
+  }
+  if (warp == kRWarpMma) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(smem_u32(tmem_slot)), "r"(p.tmem_cols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  grid_dep_wait();
+  if (threadIdx.x == 0) grid_dep_launch();
+
+  // weights -> F16 B operand (n_pad rows x 224): kk = 32 r + 4 s + c, zero at s = 7 and c = 3; a
+  // warp per channel
+  for (int n = warp; n < p.n_pad; n += kRThreads / 32) {
+    uint32_t part = 0;
+#pragma unroll
+    for (int j = 0; j < (kRK / 2 + 31) / 32; ++j) {
+      const int kk = 2 * (lane + 32 * j);
+      const int r = kk / 32, s = (kk % 32) / 4, c = kk % 4;  // (c is 0 or 2)
+      uint16_t w0 = 0, w1 = 0;
+      if (n < p.cout && kk < kRK && s < kKW) {
+        const int16_t* w = p.w_i16 + (int64_t)n * (kKH * kSeg) + r * kSeg + s * kC + c;
+        w0 = (uint16_t)w[0];
+        if (c == 0) w1 = (uint16_t)w[1];
+      }
+      part += abs_f16(w0) + abs_f16(w1);
+      if (kk < kRK)
+        *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kRSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) =
+            (uint32_t)w0 | ((uint32_t)w1 << 16);
+    }
+    if (!weights_small(part) && lane == 0) atomicAnd(s_fast, 0);
+  }
+  load_channels(p, cst4, cste, s_fast);
+  fence_proxy_async();  // generic-proxy stores of B -> visible to the MMA
+  __syncthreads();
+  const bool fast = *s_fast != 0;
+
+  const int share = p.total_tiles / gridDim.x, extra = p.total_tiles - share * gridDim.x;
+  const int first = blockIdx.x * share + min((int)blockIdx.x, extra);
+  Run run(p, first, first + share + ((int)blockIdx.x < extra));
+  bool ok = true;
+  if (warp == kRWarpMma) {
+    // ------------------------------------------------------------ MMA issuer
+    if (elect_one()) {
+      const uint32_t idesc = idesc_e4m3(p.n_pad);  // F16 has the same type code 0
+      const uint64_t da0 = sdesc_offsets(s_a, 16, 128);
+      const uint64_t db0 = sdesc_offsets(s_b, kLBO, kRSBO);
+      const uint32_t buf_mask = (1u << p.nbuf_log2) - 1u;
+      uint32_t pair = 0, lt = 0;  // first row pair of the tile, tiles done
+      for (; !run.done() && ok; run.next(p)) {
+        for (uint32_t i = 0; i < 3 && ok; ++i)  // the run's first tile reads four new pairs
+          ok = mbar_poll(b_full + 8 * ((pair + i) % kPairs), ((pair + i) / kPairs) & 1, abort_flag);
+        for (int i = 0; i < run.len && ok; ++i, ++pair, ++lt) {
+          const uint32_t buf = lt & buf_mask;
+          ok = mbar_poll(b_tempty + 8 * buf, ((lt >> p.nbuf_log2) & 1) ^ 1, abort_flag) &&
+               mbar_poll(b_full + 8 * ((pair + 3) % kPairs), ((pair + 3) / kPairs) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t d = tmem_base + buf * (uint32_t)p.n_pad;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const uint64_t da = da0 + ((pair + q) % kPairs) * (kPairBytes >> 4);
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {  // (row, K half) of the pair
+              const int r = 2 * q + h / 2;
+              if (r < kKH)
+                mma_f16(d, da + (uint64_t)(((h / 2) * kRowBytes + (h & 1) * 32) >> 4),
+                        db0 + (uint64_t)((4 * r + 2 * (h & 1)) * kLBO >> 4), idesc, q + h > 0 ? 1u : 0u);
+            }
+          }
+          mma_commit(b_tfull + 8 * buf);
+          mma_commit(b_empty + 8 * (pair % kPairs));
+        }
+        for (int i = 0; i < 3 && ok; ++i, ++pair) mma_commit(b_empty + 8 * (pair % kPairs));
+      }
+      if (!ok) fail(abort_flag, p.status);
+      mma_commit(b_final);
+      if (!mbar_wait(b_final, 0, abort_flag)) fail(abort_flag, p.status);
+    }
+  } else if (warp >= kRWarpProd0) {
+    // ------------------------------------------------------------ producers
+    const int set = (warp - kRWarpProd0) / kRSetWarps;
+    const int item = (warp - kRWarpProd0 - set * kRSetWarps) * 32 + lane;
+    const bool busy = item < 2 * kRowGroups;
+    const int row = item >= kRowGroups, grp = item - row * kRowGroups;
+    uint8_t* dst = smem + row * kRowBytes + grp * 32;
+    int i = set;  // pair of the run
+    auto settle = [&] {  // to the run that holds pair i
+      while (!run.done() && i >= run.len + 3) { i -= run.len + 3; run.next(p); }
+    };
+    auto load = [&] {
+      return busy && !run.done()
+                 ? load_group(p, run.img, 2 * (run.h0 + i) + row - p.pad, 256 * run.strip - p.pad + 4 * grp)
+                 : Group{};
+    };
+    settle();
+    Group cur = load();
+    for (uint32_t pair = set; !run.done(); pair += kRSets) {
+      i += kRSets;
+      settle();
+      const Group nxt = load();
+      const uint32_t s = pair % kPairs;
+      if (!mbar_wait(b_empty + 8 * s, ((pair / kPairs) & 1) ^ 1, abort_flag)) { ok = false; break; }
+      if (busy) store_group(cur, dst + s * kPairBytes);
+      fence_proxy_async();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(b_full + 8 * s);
+      cur = nxt;
+    }
+    if (!ok) fail(abort_flag, p.status);
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int quarter = warp & 3;
+    const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t buf_mask = (1u << p.nbuf_log2) - 1u;
+    const int col = quarter * 32 + lane, total = run.end - run.t;
+    int i = 0;  // tile of the run
+    uint8_t* yrow[2];
+    bool valid[2];
+    auto take = [&](int k) {  // the next tile's output row of this lane
+      valid[k] = false;
+      yrow[k] = p.y;
+      if (run.done()) return;
+      const int wo = run.strip * 128 + col;
+      valid[k] = wo < p.wo;
+      if (valid[k]) yrow[k] += (((int64_t)run.img * p.ho + run.h0 + i) * p.wo + wo) * p.y_row_bytes;
+      if (++i == run.len) { i = 0; run.next(p); }
+    };
+    for (int lt = 0; lt < total; lt += 2) {
+      const uint32_t b0 = lt & buf_mask, b1 = (lt + 1) & buf_mask;
+      const bool two = lt + 1 < total;
+      take(0);
+      take(1);
+      if (!mbar_wait(b_tfull + 8 * b0, (lt >> p.nbuf_log2) & 1, abort_flag) ||
+          (two && !mbar_wait(b_tfull + 8 * b1, ((lt + 1) >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
+      tc_fence_after();
+      const uint32_t tbase[2] = {lane_base + b0 * (uint32_t)p.n_pad, lane_base + b1 * (uint32_t)p.n_pad};
+      drain_pixels<2>(p, tbase, yrow, valid, warp >> 2, fast, cst4, cste, [&] {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) {
+          mbar_arrive_relaxed(b_tempty + 8 * b0);
+          if (two) mbar_arrive_relaxed(b_tempty + 8 * b1);
+        }
+      });
+    }
+    if (!ok) fail(abort_flag, p.status);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kRWarpMma) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(p.tmem_cols) : "memory");
   }
@@ -390,32 +741,43 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   if (m_total + 128 >= (1LL << 31)) { *err = "stem conv: more than 2^31 output pixels"; return 2; }
   p.m_total = (int32_t)m_total;
   p.hw_out = jb.ho * jb.wo;
-  p.total_tiles = (int32_t)((m_total + 127) / 128);
-  if (p.total_tiles == 0) return 0;
-  int cols = 32;
-  while (cols < 2 * p.n_pad) cols *= 2;
-  p.tmem_cols = cols;
+  if (m_total == 0) return 0;
   int dev = 0, sms = 0, max_smem = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  const uint32_t b_bytes = (uint32_t)p.n_pad * kK * 2;
   const uint32_t cst_bytes = (uint32_t)(256 * (sizeof(int4) + sizeof(EpiChan)));
-  int stages = 4;
+  const uint32_t bar_rest = 16 + 1024;  // TMEM slot + 2 flags, alignment
+  const bool rows = a.stride == 2;
   uint32_t total = 0;
-  for (; stages >= 2; --stages) {
-    p.off_b = (uint32_t)stages * kStageA;
-    p.off_cst = p.off_b + b_bytes;
+  p.strips = (jb.wo + 127) / 128;
+  if (rows) {
+    p.total_tiles = (int32_t)((int64_t)jb.n * p.strips * jb.ho);
+    p.nbuf_log2 = 4 * p.n_pad <= 512 ? 2 : 1;
+    p.off_b = kPairs * kPairBytes;
+    p.off_cst = p.off_b + (uint32_t)p.n_pad * kRK * 2;
     p.off_bar = (p.off_cst + cst_bytes + 15) / 16 * 16;
-    total = p.off_bar + 8 * (2 * stages + 5) + 16 + 1024;  // barriers, TMEM slot + 2 flags, alignment
-    if ((int)total <= max_smem) break;
+    total = p.off_bar + 8 * (2 * kPairs + 2 * kMaxBufs + 1) + bar_rest;
+  } else {
+    p.total_tiles = (int32_t)((m_total + 127) / 128);
+    p.nbuf_log2 = 1;
+    for (p.stages = 4; p.stages >= 2; --p.stages) {
+      p.off_b = (uint32_t)p.stages * kStageA;
+      p.off_cst = p.off_b + (uint32_t)p.n_pad * kK * 2;
+      p.off_bar = (p.off_cst + cst_bytes + 15) / 16 * 16;
+      total = p.off_bar + 8 * (2 * p.stages + 5) + bar_rest;
+      if ((int)total <= max_smem) break;
+    }
   }
-  if (stages < 2) { *err = "stem conv: shared memory too small"; return 2; }
-  p.stages = stages;
+  if ((int)total > max_smem) { *err = "stem conv: shared memory too small"; return 2; }
+  p.tmem_cols = 32;
+  while (p.tmem_cols < (p.n_pad << p.nbuf_log2)) p.tmem_cols *= 2;
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(attr_once, [&] {
     attr_err = cudaFuncSetAttribute(stem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    if (attr_err == cudaSuccess)
+      attr_err = cudaFuncSetAttribute(stem_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   });
   if (attr_err != cudaSuccess) {
     *err = std::string("stem conv: shared-memory attribute: ") + cudaGetErrorString(attr_err);
@@ -424,7 +786,7 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const int grid = (int)(p.total_tiles < sms ? p.total_tiles : sms);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kThreads);
+  cfg.blockDim = dim3(rows ? kRThreads : kThreads);
   cfg.dynamicSmemBytes = total;
   cfg.stream = stream;
   cudaLaunchAttribute attr[1];
@@ -432,7 +794,7 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, stem_kernel, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, rows ? stem_rows_kernel : stem_kernel, p);
   if (e != cudaSuccess) {
     *err = std::string("stem conv launch: ") + cudaGetErrorString(e);
     return 3;

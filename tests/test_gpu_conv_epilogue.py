@@ -138,3 +138,20 @@ def test_slabs_bit_exact(kh, kw, pad, cin, cout, bits, path):
     got, want, used = conv_pair(x, bits, wt, wb, pad=pad, out_bits=4, m0=m0, shift=sh, bias=b, workspace=True, path=path)
     assert used == (6 if bits == 2 and cin == 256 and cout <= 240 else 4 if path == 0 else 3)
     assert_same(got, want, cout, 4, f"{kh}x{kw} {cin}->{cout}")
+
+
+# the first conv at stride 2 (image rows as the operand): strips of 128 output columns and their edges, runs of
+# tiles that cross strips and images, more row pairs than the ring holds, images smaller than the kernel, wide padding
+@pytest.mark.parametrize("shape,pad,cout,out_bits", [((1, 7, 7), 0, 16, 8), ((1, 1, 1), 3, 64, 4), ((2, 3, 5), 6, 32, 3),
+                                                     ((1, 5, 259), 3, 64, 2), ((3, 61, 255), 3, 64, 4), ((1, 9, 257), 3, 96, 32),
+                                                     ((2, 211, 262), 0, 48, 8), ((1, 30, 1031), 2, 256, 4),
+                                                     ((40, 37, 20), 3, 64, 4), ((2, 1200, 517), 3, 64, 4)])
+def test_first_conv_rows_bit_exact(shape, pad, cout, out_bits):
+    rng = np.random.default_rng(shape[1] * 7 + shape[2])
+    x = synth.act_codes(rng, (*shape, 3), 8)
+    wt = rng.integers(-7, 8, size=(cout, 7, 7, 3)).astype(np.int32)
+    m0, sh, b = tables(rng, cout, 255 * 2.6 * 12, min(out_bits, 8))
+    got, want, used = conv_pair(x, 8, wt, 8, stride=2, pad=pad, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                                shift=None if out_bits == 32 else sh, bias=b)
+    assert used == 5
+    assert_same(got, want, cout, out_bits, f"first conv {shape}")
