@@ -28,7 +28,7 @@
 //              32*(w%4)..; the E / 4 warps of a lane quarter split the columns)
 //   warp  E    TMEM allocation + one thread issuing tcgen05.mma (kind::f8f6f4, M=128)
 //   warp  E+1.. one thread each loading operands with TMA (cp.async.bulk.tensor, SW128)
-//   then 4 warps of activation producers (in-kernel variant): im2col gather of packed k-bit codes
+//   then 8 warps of activation producers (in-kernel variant): im2col gather of packed k-bit codes
 //              (zero-fill = the padding code 0), unpack to E4M3 bytes, store into the
 //              128B-swizzled K-major operand layout, signal an mbarrier
 // Stages of 128 K-bytes (one 128B swizzle atom) circulate between producers and the MMA
@@ -56,7 +56,11 @@ constexpr int BK = 128;            // K bytes per stage
 // scheduler that holds two such warps issued in a third of its cycles; with four it covers the
 // latencies. The in-kernel-unpack variant keeps 8: its producer warps need the registers.
 __host__ __device__ constexpr int epi_warps(bool flat) { return flat ? 16 : 8; }
-constexpr int kProdWarps = 4;  // one thread per tile row
+// Producers of the in-kernel-unpack variant: two threads per tile row, each 64 channels of a K chunk, with
+// four chunks in flight. (One thread per row and a 128-channel chunk was a chain of 150 instructions on one
+// warp per scheduler: ragged 3-bit conv 10.4 -> 9.4 us, small 2-bit conv 11.1 -> 9.6, the 3x3 stride-2 64 -> 128
+// conv at batch 8 34 -> 30.)
+constexpr int kProdWarps = 8;
 // The expanded-activation ("flat") variant has no producer warps: TMA loads both operands, one
 // thread the activations and two the weights.
 //
@@ -404,9 +408,9 @@ __device__ __noinline__ uint4 general_sums(const Params& p, const GenCols& u, in
 
 // ---------------------------------------------------------------- the kernel
 
-// Loads the packed codes of one 128-channel K chunk of one output row into registers
-// (4 * kXBits words; group g = channels 32g..32g+31 of the chunk at words [g*kXBits, ...)).
-// Taps outside the image (and rows past the end of the job) read zeros = code 0.
+// Loads the packed codes of half (64 channels) of a 128-channel K chunk of one output row into
+// registers (2 * kXBits words; group g = 32 channels at words [g * kXBits, ...)). Taps outside the
+// image (and rows past the end of the job) read zeros = code 0.
 template <int kXBits>
 struct RowCursor {
   const uint8_t* xbase;  // image base of this row's pixel
@@ -415,35 +419,46 @@ struct RowCursor {
   int tr, ts, tc0;       // tap (r, s) and channel offset of the next 32-channel group
 };
 
+template <int kXBits>
+__device__ __forceinline__ void skip_groups(const Params& p, RowCursor<kXBits>& rc, int n) {
+  for (int g = 0; g < n; ++g) {
+    rc.tc0 += 32;
+    if (rc.tc0 == p.cin) { rc.tc0 = 0; if (++rc.ts == p.kw) { rc.ts = 0; ++rc.tr; } }
+  }
+}
+
+// The cursor stands at this half's first group of chunk q, and is left at that of chunk q + 1.
 template <int kXBits, bool kChunkInTap>
-__device__ __forceinline__ void load_chunk(const Params& p, RowCursor<kXBits>& rc, int q, uint32_t (&w)[4 * kXBits]) {
+__device__ __forceinline__ void load_half(const Params& p, RowCursor<kXBits>& rc, int q, int half, uint32_t (&w)[2 * kXBits]) {
   constexpr int kGB = 4 * kXBits;
   if constexpr (kChunkInTap) {
     // cin % 128 == 0: the chunk is 128 consecutive channels of one tap
     const int hi = rc.hb + rc.tr, wi = rc.wb + rc.ts;
     const bool ok = rc.valid && hi >= 0 && hi < rc.H && wi >= 0 && wi < rc.W;
-    const uint4* src = reinterpret_cast<const uint4*>(rc.xbase + ((int64_t)hi * rc.W + wi) * p.x_row_bytes +
-                                                      (rc.tc0 >> 5) * kGB);
+    // (3-bit halves are 24 bytes: 8-byte pieces)
+    using Piece = std::conditional_t<kXBits == 3, uint2, uint4>;
+    constexpr int kPieces = 2 * kGB / (int)sizeof(Piece), kPw = (int)sizeof(Piece) / 4;
+    const Piece* src = reinterpret_cast<const Piece*>(rc.xbase + ((int64_t)hi * rc.W + wi) * p.x_row_bytes + (rc.tc0 >> 5) * kGB);
 #pragma unroll
-    for (int i = 0; i < kXBits; ++i) {
-      uint4 v = make_uint4(0, 0, 0, 0);
+    for (int i = 0; i < kPieces; ++i) {
+      Piece v{};
       if (ok) v = __ldg(src + i);
-      w[4 * i] = v.x; w[4 * i + 1] = v.y; w[4 * i + 2] = v.z; w[4 * i + 3] = v.w;
+      w[kPw * i] = v.x; w[kPw * i + 1] = v.y;
+      if constexpr (kPw == 4) { w[kPw * i + 2] = v.z; w[kPw * i + 3] = v.w; }
     }
     rc.tc0 += 128;
-    if (rc.tc0 == p.cin) { rc.tc0 = 0; if (++rc.ts == p.kw) { rc.ts = 0; ++rc.tr; } }
+    if (rc.tc0 >= p.cin) { rc.tc0 -= p.cin; if (++rc.ts == p.kw) { rc.ts = 0; ++rc.tr; } }
   } else {
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const int k0 = q * BK + 32 * g;
+    for (int g = 0; g < 2; ++g) {
+      const int k0 = q * BK + 64 * half + 32 * g;
       bool ok = false;
       const uint8_t* src = rc.xbase;
       if (k0 < p.k_total) {
         const int hi = rc.hb + rc.tr, wi = rc.wb + rc.ts;
         ok = rc.valid && hi >= 0 && hi < rc.H && wi >= 0 && wi < rc.W;
         src = rc.xbase + ((int64_t)hi * rc.W + wi) * p.x_row_bytes + (rc.tc0 >> 5) * kGB;
-        rc.tc0 += 32;
-        if (rc.tc0 == p.cin) { rc.tc0 = 0; if (++rc.ts == p.kw) { rc.ts = 0; ++rc.tr; } }
+        skip_groups(p, rc, 1);
       }
       if constexpr (kXBits == 2) {
         uint2 v = make_uint2(0, 0);
@@ -458,6 +473,7 @@ __device__ __forceinline__ void load_chunk(const Params& p, RowCursor<kXBits>& r
         for (int i = 0; i < 3; ++i) w[3 * g + i] = ok ? __ldg(reinterpret_cast<const uint32_t*>(src) + i) : 0u;
       }
     }
+    skip_groups(p, rc, 2);  // (the other half's)
   }
 }
 
@@ -813,7 +829,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     }
   } else if (!kFlat && warp >= kWarpProd0) {
     // ------------------------------------------------------------ activation producers
-    const int row = threadIdx.x - kWarpProd0 * 32;  // tile row owned by this thread
+    const int row = (threadIdx.x - kWarpProd0 * 32) & (BM - 1);  // tile row of this thread,
+    const int half = (warp - kWarpProd0) / (BM / 32);             // and its half of every K chunk
     const int r7 = row & 7;
     uint8_t* arow = smem + row * BK;
     int my_tiles = 0;
@@ -821,7 +838,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     const int total = my_tiles * nk;
 
     RowCursor<kXBits> rc{};
-    int l_tile = first_tile, l_q = 0;  // load cursor (runs kDepth chunks ahead)
+    int l_tile = first_tile, l_q = 0;  // load cursor (runs four chunks ahead)
     auto start_tile = [&](int t) {
       const TileInfo ti = tile_info(p, t);
       const ConvJobDev& jb = p.jobs[ti.job];
@@ -837,46 +854,46 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       rc.W = jb.w;
       rc.xbase = jb.x + (int64_t)img * jb.h * jb.w * p.x_row_bytes;
       rc.tr = 0; rc.ts = 0; rc.tc0 = 0;
+      if constexpr (kChunkInTap) rc.tc0 = 64 * half;
+      else skip_groups(p, rc, 2 * half);
     };
-    auto load_next = [&](uint32_t (&w)[4 * kXBits]) {
+    auto load_next = [&](uint32_t (&w)[2 * kXBits]) {
       if (l_q == 0) start_tile(l_tile);
-      load_chunk<kXBits, kChunkInTap>(p, rc, l_q, w);
+      load_half<kXBits, kChunkInTap>(p, rc, l_q, half, w);
       if (++l_q == nk) { l_q = 0; l_tile += p.tile_stride; }
     };
     bool ok = true;
     const int S = p.stages;
     uint32_t b_empty, b_wfull, b_wempty;
     slots(b_empty, b_wfull, b_wempty);
-    auto consume = [&](int c, const uint32_t (&w)[4 * kXBits]) -> bool {
-      const uint32_t s = c % S, ph = (c / S) & 1;
+    uint32_t s = 0, ph = 0;
+    auto consume = [&](const uint32_t (&w)[2 * kXBits]) -> bool {
       if (!mbar_wait(b_empty + 8 * s, ph ^ 1, abort_flag)) return false;
       uint8_t* dst = arow + (size_t)s * kStageA;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < 2; ++g) {
         uint32_t o[8];
         unpack_group_bytes<kXBits>(w + g * kXBits, o);  // raw E4M3 byte = code
-        *reinterpret_cast<uint4*>(dst + 16 * ((2 * g) ^ r7)) = make_uint4(o[0], o[1], o[2], o[3]);
-        *reinterpret_cast<uint4*>(dst + 16 * ((2 * g + 1) ^ r7)) = make_uint4(o[4], o[5], o[6], o[7]);
+        const int c16 = 4 * half + 2 * g;               // 16-byte column of the operand row
+        *reinterpret_cast<uint4*>(dst + 16 * (c16 ^ r7)) = make_uint4(o[0], o[1], o[2], o[3]);
+        *reinterpret_cast<uint4*>(dst + 16 * ((c16 + 1) ^ r7)) = make_uint4(o[4], o[5], o[6], o[7]);
       }
       fence_proxy_async();  // this thread's generic-proxy stores -> visible to the MMA
       __syncwarp();
       if (lane == 0) mbar_arrive(b_full + 8 * s);
+      if (++s == (uint32_t)S) { s = 0; ph ^= 1; }
       return true;
     };
-    uint32_t w0[4 * kXBits], w1[4 * kXBits], w2[4 * kXBits];
-    if (total > 0) load_next(w0);
-    if (total > 1) load_next(w1);
-    if (total > 2) load_next(w2);
-    for (int c = 0; c < total && ok; c += 3) {
-      if (!consume(c, w0)) { ok = false; break; }
-      if (c + 3 < total) load_next(w0);
-      if (c + 1 < total) {
-        if (!consume(c + 1, w1)) { ok = false; break; }
-        if (c + 4 < total) load_next(w1);
-      }
-      if (c + 2 < total) {
-        if (!consume(c + 2, w2)) { ok = false; break; }
-        if (c + 5 < total) load_next(w2);
+    uint32_t w[4][2 * kXBits];  // chunks in flight
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < total) load_next(w[i]);
+    for (int c = 0; c < total && ok; c += 4) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (c + i >= total) break;
+        if (!consume(w[i])) { ok = false; break; }
+        if (c + i + 4 < total) load_next(w[i]);
       }
     }
     if (!ok) fail(abort_flag, p.status);

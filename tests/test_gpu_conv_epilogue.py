@@ -155,3 +155,19 @@ def test_first_conv_rows_bit_exact(shape, pad, cout, out_bits):
                                 shift=None if out_bits == 32 else sh, bias=b)
     assert used == 5
     assert_same(got, want, cout, out_bits, f"first conv {shape}")
+
+
+# the in-kernel unpack's two threads per row: K tails of 1 to 4 groups of 32 (whole and empty second halves), chunks
+# that cross taps, chunks of one tap (cin % 128 == 0), fewer and more chunks than are held in flight
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("cin,k,stride,shape", [(32, 1, 1, (1, 9, 15)), (64, 1, 2, (1, 9, 15)), (96, 1, 1, (1, 5, 7)),
+                                                (32, 3, 2, (1, 20, 21)), (160, 3, 1, (1, 6, 7)), (96, 5, 2, (1, 11, 13)),
+                                                (128, 1, 2, (1, 17, 19)), (128, 3, 2, (2, 13, 15)), (384, 3, 2, (1, 9, 9))])
+def test_unpack_halves_bit_exact(cin, k, stride, shape, bits):
+    rng = np.random.default_rng(cin * k + bits)
+    x = synth.act_codes(rng, (*shape, cin), bits)
+    wt = synth.weight_codes(rng, (64, k, k, cin), bits)
+    m0, sh, b = tables(rng, 64, 3.0 * (1 << bits) * np.sqrt(k * k * cin) / 4, 4)
+    got, want, used = conv_pair(x, bits, wt, bits, stride=stride, pad=k // 2, out_bits=4, m0=m0, shift=sh, bias=b)
+    assert used == 1
+    assert_same(got, want, 64, 4, f"in-kernel unpack {cin}x{k}x{k}")
