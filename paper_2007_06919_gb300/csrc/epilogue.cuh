@@ -41,5 +41,30 @@ __device__ __forceinline__ void store_codes16(uint8_t* yrow, int ch, const uint3
     else top = h;
   }
 }
+
+// 32 bytes of a row, 32-byte aligned: one store of a whole sector
+__device__ __forceinline__ void store_sector(uint8_t* p, const uint32_t (&a)[4], const uint32_t (&b)[4]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a[0]), "r"(a[1]), "r"(a[2]),
+               "r"(a[3]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3])
+               : "memory");
+}
+// A whole 32-channel group: the byte-words of its halves to their place in the packed row (see
+// store_codes16)
+__device__ __forceinline__ void store_codes32(uint8_t* yrow, int ch, const uint32_t (&a)[4], const uint32_t (&b)[4], int bits) {
+  if (bits == 4) {
+    *reinterpret_cast<uint4*>(yrow + (ch >> 1)) =
+        make_uint4(a[0] | (a[1] << 4), a[2] | (a[3] << 4), b[0] | (b[1] << 4), b[2] | (b[3] << 4));
+  } else if (bits == 2) {
+    *reinterpret_cast<uint2*>(yrow + (ch >> 2)) =
+        make_uint2(a[0] | (a[1] << 2) | (a[2] << 4) | (a[3] << 6), b[0] | (b[1] << 2) | (b[2] << 4) | (b[3] << 6));
+  } else if (bits == 8) {
+    *reinterpret_cast<uint4*>(yrow + ch) = make_uint4(a[0], a[1], a[2], a[3]);
+    *reinterpret_cast<uint4*>(yrow + ch + 16) = make_uint4(b[0], b[1], b[2], b[3]);
+  } else {
+    uint32_t top = 0u;
+    store_codes16(yrow, ch, a, bits, top);
+    store_codes16(yrow, ch + 16, b, bits, top);
+  }
+}
 }  // namespace tc
 }  // namespace aqd
