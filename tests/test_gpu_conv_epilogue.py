@@ -171,3 +171,18 @@ def test_unpack_halves_bit_exact(cin, k, stride, shape, bits):
     got, want, used = conv_pair(x, bits, wt, bits, stride=stride, pad=k // 2, out_bits=4, m0=m0, shift=sh, bias=b)
     assert used == 1
     assert_same(got, want, 64, 4, f"in-kernel unpack {cin}x{k}x{k}")
+
+
+# int32 outputs of the in-kernel variant through the staging blocks: whole and partial 16- and 32-column steps, several N
+# tiles, a last row group that is not whole; cout % 4 != 0 stays with the general form
+@pytest.mark.parametrize("cin,k,cout,shape", [(64, 1, 4, (1, 3, 5)), (64, 1, 36, (1, 20, 21)), (32, 3, 128, (2, 13, 15)),
+                                              (128, 1, 260, (1, 9, 31)), (128, 3, 516, (1, 7, 9)), (64, 1, 30, (1, 9, 9))])
+@pytest.mark.parametrize("bits", [2, 3, 4])
+def test_unpack_int32_outputs_bit_exact(cin, k, cout, shape, bits):
+    rng = np.random.default_rng(cout + bits)
+    x = synth.act_codes(rng, (*shape, cin), bits)
+    wt = synth.weight_codes(rng, (cout, k, k, cin), bits)
+    b = rng.integers(-(1 << 29), 1 << 29, size=(1, cout)).astype(np.int32)
+    got, want, used = conv_pair(x, bits, wt, bits, stride=2, pad=k // 2, out_bits=32, m0=None, shift=None, bias=b)
+    assert used == 1
+    assert_same(got, want, cout, 32, f"int32 {cin}x{k}x{k} -> {cout}")
