@@ -921,8 +921,9 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
     // into epi_groups ranges; sets of epi_groups warps take tiles in turn (epi_sets > 1: narrow
     // tiles).
     //
-    // What bounds it: integer instructions, about 9 per output and lane without a skip and 14 with
-    // one. So everything that does not depend on the column is done once per tile and lane (the
+    // What bounds it: for 256-channel tiles, stores to rows that lie apart (see store16 below); then the
+    // issue of dependent integer instructions, about 9 per output and lane without a skip and 14 with
+    // one, in about half of the cycles. So everything that does not depend on the column is done once per tile and lane (the
     // output pixel, by multiply-high divisions, and the row pointers), the rare forms live in a
     // function of their own, and four warps per scheduler cover the chains' latencies. Against two
     // warps per scheduler, 25 and 40 instructions per output (divisions per 32 columns, 64-bit

@@ -18,7 +18,10 @@
 // no-swizzle K-major layout of 8-row x 16-byte core matrices (K-adjacent core matrices 128 B
 // apart, 8-row groups 2560 B apart).
 //
-// Per CTA (one per SM, persistent over tiles of 128 consecutive output pixels):
+// Two kernels: stem_rows_kernel for stride 2 (a network's first conv), whose operand is the image
+// row itself, and stem_kernel for every other stride, which builds each pixel's receptive field.
+//
+// stem_kernel, per CTA (one per SM, persistent over tiles of 128 consecutive output pixels):
 //   warps 0..7   epilogue: tcgen05.ld (warp w reads TMEM lanes 32 (w % 4).., the two warps of a
 //                lane quarter every other 32-column group), Eq. 6 + Eq. 2, bit-pack, store
 //   warp  8      TMEM allocation + one thread issuing tcgen05.mma (M=128, N=cout, K=16)
@@ -55,8 +58,8 @@ constexpr int kSplitR = 4;                 // producer half 0: kernel rows [0, 4
 static_assert((kSplitR * kLs) % 8 == 0, "the producer halves must meet on a core-matrix boundary");
 static_assert(kLs <= 24, "a receptive-field row must fit six realigned words");
 // 17 warps: at most 5 per SM sub-partition, so 96 registers per thread. (4 epilogue warps, one per
-// sub-partition, ran two 32-column groups each per tile as one chain of dependent instructions.
-// Now the producers bound it: they build a tile in 2.4k of its 2.8k cycles. Config 3's first conv, 8 x 400 x 672 x 64 outputs: 203 -> 173 us.)
+// sub-partition, ran two 32-column groups each per tile as one chain of dependent instructions:
+// 8 x 400 x 672 x 64 outputs 203 -> 173 us.)
 constexpr int kEpiWarps = 8, kWarpMma = kEpiWarps, kWarpProd0 = kEpiWarps + 1, kProdWarps = 8;
 constexpr int kThreads = (kWarpProd0 + kProdWarps) * 32;
 constexpr uint32_t kF16Pair1024 = 0x64006400u;
@@ -430,6 +433,10 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
 // next 8 pixels 128. Seven pixels and an eighth with zero weights are K = 32 per kernel row, 224 in
 // all. An image pixel is converted once per tile row pair instead of 12 times, and a CTA's tiles
 // go down the rows of a strip of 128 output columns, so that each tile brings two new image rows.
+// What bounds it is the epilogue: a sum was converted by F2I (a sixteenth of the add's rate) and added
+// with saturation, and 16 bytes of constants were read per output. Two tiles now share each read, and
+// one float add converts. 8 x 400 x 672 x 64 4-bit outputs 171 -> 130 us (HBM alone 14); 16 epilogue
+// warps in two sets take 141. With the requant left out 93 remain: no one pipe, the issue of its 19 warps.
 //   warps 0..7    epilogue, two tiles at a time
 //   warp  8       TMEM allocation + one thread issuing tcgen05.mma (M=128, N=cout, 14 of K=16)
 //   warps 9..18   producers: two sets of 5 take row pairs in turn, 4 pixels per thread, the words
