@@ -731,11 +731,7 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
     } else {
       // two pixels per step (the second clamped to the last one and its store predicated off)
       // so their chains interleave
-      // (kUp: unrolled, so that the words loaded ahead stay in registers)
-#pragma unroll(kUp ? kPer / 2 : 1)
-      for (int k2 = 0; k2 < (kUp ? kPer / 2 : (sg.P / pgs + 1) / 2); ++k2) {
-        const int p = pg + 2 * k2 * pgs;
-        if (p >= np) break;
+      auto step = [&](int p, [[maybe_unused]] int k2) {
         const int pp[2] = {p, p + pgs < np ? p + pgs : np - 1};
         int32_t av[2][kV];
         uint32_t sw[2] = {0, 0};
@@ -813,6 +809,14 @@ __global__ void __launch_bounds__(kThreads + 32, kSkip ? 2 : 3)  // the skip for
               reinterpret_cast<uint32_t*>(yrow + (ch0 >> 5) * group_bytes(kOut))[i0 / q] = v;
           }
         }
+      };
+      if constexpr (kUp) {
+        // unrolled, so that the words loaded ahead stay in registers
+#pragma unroll
+        for (int k2 = 0; k2 < kPer / 2; ++k2)
+          if (pg + 2 * k2 * pgs < np) step(pg + 2 * k2 * pgs, k2);
+      } else {
+        for (int p = pg; p < np; p += 2 * pgs) step(p, 0);
       }
     }
     __syncwarp();
