@@ -19,7 +19,8 @@
 // apart, 8-row groups 2560 B apart).
 //
 // Two kernels: stem_rows_kernel for stride 2 (a network's first conv), whose operand is the image
-// row itself, and stem_kernel for every other stride, which builds each pixel's receptive field.
+// row itself, and stem_kernel for other strides and narrow outputs, which builds each pixel's
+// receptive field.
 //
 // stem_kernel, per CTA (one per SM, persistent over tiles of 128 consecutive output pixels):
 //   warps 0..7   epilogue: tcgen05.ld (warp w reads TMEM lanes 32 (w % 4).., the two warps of a
@@ -755,9 +756,14 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   const uint32_t cst_bytes = (uint32_t)(256 * (sizeof(int4) + sizeof(EpiChan)));
   const uint32_t bar_rest = 16 + 1024;  // TMEM slot + 2 flags, alignment
-  const bool rows = a.stride == 2;
-  uint32_t total = 0;
   p.strips = (jb.wo + 127) / 128;
+  // Stride 2: image rows as the operand, unless the strips of 128 columns are mostly empty and there
+  // is more than one tile per SM. A tile of a strip costs 0.6 of a built one whatever its columns: 64
+  // images of 32 x 32 outputs 21.7 us against 17.1 built, of 32 x 48 21.9 / 20.9, of 64 x 64 35.2 /
+  // 37.3, 32 of 64 x 80 21.9 / 25.0, of 64 x 128 21.9 / 37.8, of 64 x 136 (two strips) 35.2 / 33.7; one
+  // image of 16 x 16 9.6 / 11.2.
+  const bool rows = a.stride == 2 && (jb.wo >= 72 * p.strips || (int64_t)jb.n * p.strips * jb.ho <= sms);
+  uint32_t total = 0;
   if (rows) {
     p.total_tiles = (int32_t)((int64_t)jb.n * p.strips * jb.ho);
     p.nbuf_log2 = 4 * p.n_pad <= 512 ? 2 : 1;

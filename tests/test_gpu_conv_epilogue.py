@@ -145,7 +145,8 @@ def test_slabs_bit_exact(kh, kw, pad, cin, cout, bits, path):
 @pytest.mark.parametrize("shape,pad,cout,out_bits", [((1, 7, 7), 0, 16, 8), ((1, 1, 1), 3, 64, 4), ((2, 3, 5), 6, 32, 3),
                                                      ((1, 5, 259), 3, 64, 2), ((3, 61, 255), 3, 64, 4), ((1, 9, 257), 3, 96, 32),
                                                      ((2, 211, 262), 0, 48, 8), ((1, 30, 1031), 2, 256, 4),
-                                                     ((40, 37, 20), 3, 64, 4), ((2, 1200, 517), 3, 64, 4)])
+                                                     ((40, 37, 20), 3, 64, 4), ((2, 1200, 517), 3, 64, 4),
+                                                     ((30, 21, 141), 3, 64, 4), ((30, 21, 143), 3, 64, 4)])
 def test_first_conv_rows_bit_exact(shape, pad, cout, out_bits):
     rng = np.random.default_rng(shape[1] * 7 + shape[2])
     x = synth.act_codes(rng, (*shape, 3), 8)
