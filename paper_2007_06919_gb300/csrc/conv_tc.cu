@@ -1814,8 +1814,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const int warp_groups = epi_warps(flat) / 4;
   const int col_groups = ((a.split_w ? BN / 2 : BN) + 31) / 32;
   prm.epi_groups = col_groups < warp_groups ? col_groups : warp_groups;
-  prm.epi_sets = warp_groups / prm.epi_groups;
-  if (prm.epi_sets == 3) prm.epi_sets = 2;  // (a power of two: tiles are dealt by their low bits)
+  prm.epi_sets = warp_groups / prm.epi_groups;  // 1, 2 or 4: tiles are dealt by their low bits
   prm.dep_target = (uint32_t)(8 * prm.epi_groups);  // a tile's epilogue warps, both CTAs of a pair
   // shared memory plan. Flat path: a ring of activation slabs and one of weight tiles (this CTA's B
   // rows x bk bytes), or all weight tiles resident. Otherwise stages of both operands.
@@ -1874,6 +1873,13 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   // of the FP4 pipe
   const int sf_cols = fp4 ? 32 : 0;
   prm.nbuf_log2 = 4 * BN + sf_cols <= 512 ? 2 : 1;
+  // A set that takes every epi_sets-th tile waits for an accumulator by phase parity, having last seen
+  // the end of its previous tile complete: the use that its wait could mistake for its own, one ring
+  // of accumulators earlier, must be among those. A tile uses nseg accumulators in turn, so that is
+  // (epi_sets - 1) nseg < accumulators; it bounds the sets only on the F16 pipe (elsewhere nseg is 1 and
+  // more than one set means four accumulators).
+  const int nseg = f16 ? (prm.num_kchunks + prm.seg_chunks - 1) / prm.seg_chunks : 1;
+  while ((prm.epi_sets - 1) * nseg >= 1 << prm.nbuf_log2) prm.epi_sets /= 2;
   const int acc_cols = BN << prm.nbuf_log2;
   if (acc_cols + sf_cols > 512) { *err = "conv_tc: FP4 tiles wider than 240 channels do not fit in TMEM"; return 2; }
   int cols = 32;

@@ -5,9 +5,10 @@ large for the common form."""
 import numpy as np
 import pytest
 
-from paper_2007_06919_gb300 import synth
+import oracle
+from paper_2007_06919_gb300 import aqd, synth
 
-from gpu_util import assert_same, conv_pair
+from gpu_util import assert_same, conv_pair, to_device, weights
 
 pytestmark = pytest.mark.gpu
 I32 = np.iinfo(np.int32)
@@ -120,6 +121,46 @@ def test_f16_pipe_bit_exact(cin, k, cout, out_bits, shape, path):
                                 shift=None if out_bits == 32 else sh, bias=b, workspace=True, path=path)
     assert used == {0: 4, 2: 2, 3: 3}[path]
     assert_same(got, want, cout, out_bits, f"F16 pipe {cin}x{k}x{k} -> {cout}")
+
+
+# narrow outputs of 2 to 8 segments with four tiles or more per CTA (pair): the sets of epilogue warps that take
+# tiles in turn, each tile's segments in the four accumulators in turn
+@pytest.mark.parametrize("cin,kh,kw,cout,out_bits", [(1024, 1, 1, 64, 8), (128, 3, 3, 64, 4), (128, 4, 4, 64, 3), (256, 3, 3, 64, 32),
+                                                     (256, 3, 3, 36, 32), (384, 3, 3, 36, 8), (640, 1, 1, 32, 2),
+                                                     (128, 3, 3, 32, 4), (128, 4, 4, 16, 8), (128, 4, 8, 4, 32)])
+@pytest.mark.parametrize("path", [0, 3])
+def test_f16_pipe_sets_of_warps_bit_exact(cin, kh, kw, cout, out_bits, path):
+    rng = np.random.default_rng(cin + kw + cout)
+    x = synth.act_codes(rng, (1, 281, 289, cin), 8)
+    wt = rng.integers(-128, 128, size=(cout, kh, kw, cin)).astype(np.int32)
+    m0, sh, b = tables(rng, cout, 255 * 74 * np.sqrt(cin * kh * kw) / 2, min(out_bits, 8))
+    got, want, used = conv_pair(x, 8, wt, 8, pad=kh // 2, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                                shift=None if out_bits == 32 else sh, bias=b, workspace=True, path=path)
+    assert used == {0: 4, 3: 3}[path]
+    assert_same(got, want, cout, out_bits, f"F16 pipe {kh}x{kw} {cin}->{cout}")
+
+
+# the same over three levels of their own tables, which the sets rebuild together
+@pytest.mark.parametrize("path", [0, 3])
+def test_f16_pipe_sets_of_warps_over_levels_bit_exact(path):
+    rng = np.random.default_rng(36)
+    cin, cout, lv = 256, 36, [(1, 200, 203), (2, 100, 102), (3, 51, 50)]
+    wt = rng.integers(-128, 128, size=(cout, 3, 3, cin)).astype(np.int32)
+    b = rng.integers(-(1 << 20), 1 << 20, size=(len(lv), cout)).astype(np.int32)
+    W, wp = weights(wt, 8)
+    xs = [synth.act_codes(rng, (n, h, w, cin), 8) for n, h, w in lv]
+    xt = [oracle.CodeTensor.from_codes(x, 8) for x in xs]
+    jobs = [(to_device(x), aqd.DTensor.empty(n, h, w, cout, 32), None, l) for l, (x, (n, h, w)) in enumerate(zip(xt, lv))]
+    old = aqd.set_conv_path(path)
+    try:
+        aqd.conv_int_grouped(jobs, W, 1, 1, rq=aqd.RequantParams.from_numpy(None, None, b),
+                             workspace=aqd.workspace_for(jobs, W, 1, 1))
+    finally:
+        aqd.set_conv_path(old)
+    assert aqd.device_status() == 0
+    for l, x in enumerate(xt):
+        ref = oracle.conv_int(x, wp, 8, 0, 3, 3, 1, 1, cout, level=l, bias=b, levels=len(lv), out_bits=32)
+        assert_same(jobs[l][1].data.cpu().numpy().reshape(ref.packed.shape), ref.packed, cout, 32, f"level {l}")
 
 
 # taps per slab 1, 2, 3, 5, 7 and 16, kernels too wide for one (17); resident weights with one and two
