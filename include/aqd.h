@@ -160,7 +160,8 @@ int32_t aqd_last_conv_path(void);
  * shared abort flag. out: 5 int64 in device memory, written by the kernel:
  * [0] 1 if the short wait expired, [1] its duration in ns, [2] 1 if the second wait
  * returned without its phase, [3] its duration in ns, [4] 1 if a control barrier whose
- * phase completed was seen as complete. The next aqd_device_status() returns
+ * phase completed was seen as complete, and two sets of warps that take a loop's tiles in
+ * turn, one of which loses a wait, met at every barrier of that loop. The next aqd_device_status() returns
  * AQD_ERR_TIMEOUT once and clears it. */
 aqd_status aqd_selftest_wait_timeout(int64_t* out, aqd_stream_t stream);
 

@@ -1018,7 +1018,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         }
         cur_key = key;
       }
-      if ((int)(lt & (uint32_t)(p.epi_sets - 1)) != gset) continue;  // another set's tile (or an idle warp)
+      if (!takes_tile(ok, lt, p.epi_sets, gset)) continue;  // another set's tile (or an idle warp, or a wait ran out)
+      // (below, a warp's lanes give up on a wait together: they go on to warp-wide instructions and barriers)
       if constexpr (kF16) {
         // this warp's columns: whole 32-column groups, at most 64 (one int32 sum each per lane)
         const int per = ((TBN + 31) / 32 + p.epi_groups - 1) / p.epi_groups * 32;
@@ -1030,9 +1031,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
 #pragma unroll 1
         for (int sg = 0; sg < nseg; ++sg) {
           const uint32_t un = lt * (uint32_t)nseg + (uint32_t)sg, b = un & buf_mask;
-          if (!mbar_wait(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag)) { ok = false; break; }
+          if (!__all_sync(0xffffffffu, mbar_wait(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
           tc_fence_after();
-          __syncwarp();
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
             if (c_lo + 16 * j >= c_hi) break;
@@ -1050,7 +1050,10 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             else mbar_arrive_relaxed(b_tempty + 8 * b);
           }
         }
-        if (!ok) break;
+        if (!ok) {
+          fail(abort_flag, p.status);
+          continue;
+        }
         const FlatTile ft = flat_tile(jb, ti.mt, kTileRows);
         const int vr = ft.v0 + (int)rank * 128 + quarter * 32 + lane;
         const int oh = fast_div(vr, jb.div_row), ow = vr - oh * jb.wp;
@@ -1177,10 +1180,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const bool sk_codes = kSkip && p.skip_bits <= 4;
       if (sk_codes && c_lo < c_hi) sw = load_skip_group(srow, c_lo, p.skip_bits, row_ok);
       __syncwarp();
-      if (!mbar_wait_inline(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag)) {
+      if (!__all_sync(0xffffffffu, mbar_wait_inline(b_tfull + 8 * buf, (lt >> p.nbuf_log2) & 1, abort_flag))) {
         if constexpr (kSkip) cp_async_wait<0>();  // (no copy outlives the block)
         ok = false;
-        break;
+        fail(abort_flag, p.status);
+        continue;
       }
       tc_fence_after();
       auto release = [&]() {  // every TMEM read of this warp is complete
@@ -1369,7 +1373,6 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         if (lane == 0) red_release_gpu_add(p.dep + tile, 1u);
       }
     }
-    if (!ok) fail(abort_flag, p.status);
   }
 
   tc_fence_before();

@@ -187,6 +187,13 @@ static __device__ __noinline__ bool counters_wait(const uint32_t* c, int n, uint
 __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
+// Whether a set of epilogue warps does the work of a loop's tile lt: sets of warps take tiles in turn
+// (sets is a power of two), and all of them meet at the named barriers of some tiles, which have no limit.
+// So a set whose wait ran out (ok is false) stays in the loop to its end and meets the others at those
+// barriers, without waiting or storing; if it left, a set that had run ahead would wait there for ever.
+__device__ __forceinline__ bool takes_tile(bool ok, uint32_t lt, int sets, int set) {
+  return ok && (int)(lt & (uint32_t)(sets - 1)) == set;
+}
 __device__ __forceinline__ void named_bar(int id, int n) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
