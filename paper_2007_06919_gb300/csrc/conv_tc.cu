@@ -260,6 +260,7 @@ __device__ __forceinline__ bool skip_const(int skip_bits, int32_t c, int d, int4
   else o = make_int4(c, 1 << (r - 33), r - 32, 0);
   return true;
 }
+__device__ __forceinline__ uint32_t magnitude(int32_t s) { return s < 0 ? 0u - (uint32_t)s : (uint32_t)s; }
 __device__ __forceinline__ int32_t skip32(int32_t s_scaled, const int4& e) {
   return (__mulhi(s_scaled, e.x) + e.y) >> e.z;
 }
@@ -1277,7 +1278,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
                                 (int)(__byte_perm(w, 0u, 0x2444) >> 1), (int)(__byte_perm(w, 0u, 0x3444) >> 1));
                 } else {
                   x = *reinterpret_cast<const int4*>(smem + (sk_stage - sbase) + (step & 1) * kSkipStage + skip_stage_off(lane, q));
-                  big |= (uint32_t)((x.x ^ (x.x >> 31)) | (x.y ^ (x.y >> 31)) | (x.z ^ (x.z >> 31)) | (x.w ^ (x.w >> 31)));
+                  big |= magnitude(x.x) | magnitude(x.y) | magnitude(x.z) | magnitude(x.w);
                   x = make_int4((int)((uint32_t)x.x << 3), (int)((uint32_t)x.y << 3), (int)((uint32_t)x.z << 3),
                                 (int)((uint32_t)x.w << 3));
                 }

@@ -49,6 +49,24 @@ def test_skip_rescale_forms_bit_exact(skip_bits, d_lo, d_hi, ws, huge):
     assert_same(got, want, cout, 4, f"skip {skip_bits} bits, d {d_lo}..{d_hi}")
 
 
+# int32 skips at the 32-bit form's limit of 2^28 in magnitude: the one product of the largest multiplier that a shift of
+# 60 does not round to 0 is that of -2^28 itself (beside it, and at 59, both forms agree)
+@pytest.mark.parametrize("s", [-(1 << 28), -(1 << 28) + 1, (1 << 28) - 1, 1 << 28])
+@pytest.mark.parametrize("d", [59, 60])
+@pytest.mark.parametrize("ws", [False, True])
+def test_int32_skip_at_the_limit_bit_exact(s, d, ws):
+    n, h, w, cin, cout = 1, 6, 21, 64, 96
+    x, wt = np.zeros((n, h, w, cin), np.int32), np.ones((cout, 1, 1, cin), np.int32)
+    skip = np.zeros((n, h, w, cout), np.int32)
+    skip[0, 1, 5], skip[0, 4, 20, ::7] = s, s
+    full = lambda v, t: np.full((1, cout), v, t)
+    # a quarter of bias + rescaled skip: 2 is code 0, 3 is code 1
+    got, want, _ = conv_pair(x, 4, wt, 4, pad=0, out_bits=4, m0=full(I32.max, np.int32), shift=full(2, np.int8),
+                             bias=full(2, np.int32), skip=skip, skip_bits=32, skip_c=full(I32.min, np.int32),
+                             skip_d=full(d, np.int8), workspace=ws)
+    assert_same(got, want, cout, 4, f"skip {s}, d {d}")
+
+
 @pytest.mark.parametrize("out_bits,cout", [(8, 1), (8, 40), (8, 48), (8, 272), (8, 96), (32, 33), (32, 84), (32, 20),
                                            (32, 258)])
 @pytest.mark.parametrize("skip", [False, True])
