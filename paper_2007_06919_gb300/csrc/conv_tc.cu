@@ -1156,13 +1156,17 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       // int32 skips: the skip pixels of the four rows whose pieces this lane copies (-1: none)
       [[maybe_unused]] int sp4[4] = {-1, -1, -1, -1};
       [[maybe_unused]] const uint32_t sk_stage = sbase + p.off_sktab + (uint32_t)warp * (2 * kSkipStage);
-      auto copy_skip32 = [&](int c0, int step) {  // columns c0 .. c0 + 15 (none past the end)
+      // Columns c0 .. c0 + 15, or an empty group past the end: the wait of the last step then completes
+      // every copy, before the next tile's copies (which nothing would order against them) go to the same places.
+      auto copy_skip32 = [&](int c0, int step) {
+        if (c0 < c_hi) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const bool on = sp4[k] >= 0 && c0 < c_hi;
-          const uint8_t* src = jb.skip;
-          if (on) src += (int64_t)sp4[k] * p.skip_row_bytes + (int64_t)(ti.col0 + c0) * 4 + (lane & 3) * 16;
-          cp_async<16>(sk_stage + (uint32_t)(step & 1) * kSkipStage + skip_stage_off(8 * k + (lane >> 2), lane & 3), src, on);
+          for (int k = 0; k < 4; ++k) {
+            const bool on = sp4[k] >= 0;
+            const uint8_t* src = jb.skip;
+            if (on) src += (int64_t)sp4[k] * p.skip_row_bytes + (int64_t)(ti.col0 + c0) * 4 + (lane & 3) * 16;
+            cp_async<16>(sk_stage + (uint32_t)(step & 1) * kSkipStage + skip_stage_off(8 * k + (lane >> 2), lane & 3), src, on);
+          }
         }
         cp_async_commit();
       };

@@ -106,6 +106,23 @@ def test_column_groups_over_many_tiles_bit_exact(cout, out_bits, skip):
     assert_same(got, want, cout, out_bits, f"cout {cout}")
 
 
+# int32 skips through their staging slots over many tiles per warp: the last step's copies of a tile and the first
+# of the next go to the same places; 1, 2, 3 and 8 column groups, a tile's last group beside idle warps, and two N tiles
+@pytest.mark.parametrize("cout", [32, 64, 96, 256, 320])
+@pytest.mark.parametrize("ws", [False, True])
+def test_int32_skips_over_many_tiles_bit_exact(cout, ws):
+    rng = np.random.default_rng(cout + ws)
+    n, h, w, cin = 3, 150, 179, 64
+    x = synth.act_codes(rng, (n, h, w, cin), 3)
+    wt = synth.weight_codes(rng, (cout, 1, 1, cin), 3)
+    m0, sh, b = tables(rng, cout, 80.0, 4)
+    c, d = synth.skip_params_acc(rng, 1, cout)
+    skip = rng.integers(-4000, 4000, size=(n, h, w, cout)).astype(np.int32)
+    got, want, _ = conv_pair(x, 3, wt, 3, pad=0, out_bits=4, m0=m0, shift=np.maximum(sh, 2).astype(np.int8), bias=b,
+                             skip=skip, skip_bits=32, skip_c=c, skip_d=d, workspace=ws)
+    assert_same(got, want, cout, 4, f"cout {cout}")
+
+
 @pytest.mark.parametrize("ws", [False, True])
 @pytest.mark.parametrize("out_bits", [4, 32])
 def test_accumulators_beyond_the_common_form_bit_exact(ws, out_bits):
