@@ -346,18 +346,19 @@ __global__ void __launch_bounds__(kThreads) bn_stats_partial4_kernel(const Stats
 }
 
 // mean = k + S1 / N, var = S2 / N - (S1 / N)^2 (biased, as batch normalization's training
-// statistics), in float64 from the blocks' partials. Block (l, g) finishes channels 8 g .. of level
-// l: thread (r, ch), r < 32, adds the partials of blocks r, r + 32, ..., then one thread per channel
-// the 32 sums, both in a fixed order. One thread per channel over all partials was a serial chain of
-// about 600 loads and double additions on five SMs: 120 -> 17 us.
+// statistics), in float64 from the blocks' partials. Block (g, l) finishes channels 8 g .. of level
+// l (channels along x: y takes 65,535 blocks, 524,280 channels): thread (r, ch), r < 32, adds the
+// partials of blocks r, r + 32, ..., then one thread per channel the 32 sums, both in a fixed order.
+// One thread per channel over all partials was a serial chain of about 600 loads and double additions
+// on five SMs: 120 -> 17 us.
 constexpr int kFinCh = 8;
 __global__ void __launch_bounds__(kThreads) bn_stats_final_kernel(const StatsArgs a, const double* __restrict__ s1,
                                                                   const double* __restrict__ s2,
                                                                   double* __restrict__ mean, double* __restrict__ var) {
   constexpr int kR = kThreads / kFinCh;
   __shared__ double r1[kR][kFinCh], r2[kR][kFinCh];
-  const int l = blockIdx.x, c8 = threadIdx.x % kFinCh, r = threadIdx.x / kFinCh;
-  const int ch = kFinCh * (int)blockIdx.y + c8;
+  const int l = blockIdx.y, c8 = threadIdx.x % kFinCh, r = threadIdx.x / kFinCh;
+  const int64_t ch = (int64_t)kFinCh * blockIdx.x + c8;
   const int64_t P = a.pixels[l];
   double t1 = 0.0, t2 = 0.0;
   if (ch < a.c) {
@@ -474,7 +475,7 @@ int launch_bn_level_stats(const float* const* z, const int64_t* pixels, int32_t 
   double* s2 = work + (size_t)cap * c;
   if (v4) trn::bn_stats_partial4_kernel<<<(unsigned)total, trn::kThreads, 0, stream>>>(a, s1, s2);
   else trn::bn_stats_partial_kernel<<<(unsigned)total, trn::kThreads, 0, stream>>>(a, s1, s2);
-  const dim3 fin((unsigned)levels, (unsigned)((c + trn::kFinCh - 1) / trn::kFinCh));
+  const dim3 fin(((unsigned)c + trn::kFinCh - 1) / trn::kFinCh, (unsigned)levels);
   trn::bn_stats_final_kernel<<<fin, trn::kThreads, 0, stream>>>(a, s1, s2, mean, var);
   return check_launch_t("bn_level_stats launch", err);
 }

@@ -109,6 +109,17 @@ def test_bn_level_stats_matches_oracle(batch, c):
     assert np.all(v[4] == 0) and np.all(m[4] == 3.25)
 
 
+@pytest.mark.parametrize("c", [524_289, 524_296])  # more channels than 65,535 blocks of 8
+def test_bn_level_stats_of_many_channels(c):
+    rng = np.random.default_rng(c)
+    zs = [rng.normal(2, 3, size=(1, 1, p, c)).astype(np.float32) for p in (3, 2)]
+    want_m, want_v = ot.bn_level_stats(zs)
+    m, v = (t.cpu().numpy() for t in aqd.bn_level_stats([_cuda(z) for z in zs]))
+    assert np.all(np.abs(m - want_m) <= 1e-6 * (np.abs(want_m) + np.sqrt(want_v)) + 1e-12)
+    # (over three pixels the sum of the squares, rounded to 2^-23 of itself, is at most nine variances)
+    assert np.all(np.abs(v - want_v) <= 1e-5 * want_v + 1e-12)
+
+
 def test_training_argument_errors():
     x = torch.zeros(16, dtype=torch.float32, device="cuda")
     for bad in (dict(nu=0.0, bits=2), dict(nu=float("inf"), bits=2), dict(nu=1.0, bits=9), dict(nu=1.0, bits=0)):
