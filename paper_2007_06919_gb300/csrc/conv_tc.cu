@@ -1080,6 +1080,15 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
               }
               store_codes16(yrow, ch0, bw, out_bits, top);
               if (irow) store_image16(irow, ch0, bw, ly.ws_nib);
+            } else if (out_bits == 32 && (flags & kFlagBias) && (p.cout & 3) == 0) {
+              // int32 outputs: sum + bias in whole 16-byte pieces (likewise without saturation)
+              const int4* ef = epi.fast() + c0;
+              uint4* yr = reinterpret_cast<uint4*>(yrow) + (ch0 >> 2);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                auto out = [&](int i) { return (uint32_t)sum[16 * j + i] + (uint32_t)ef[i].x + kMagicBits; };
+                if (4 * q < nc) yr[q] = make_uint4(out(4 * q), out(4 * q + 1), out(4 * q + 2), out(4 * q + 3));
+              }
             } else {
               int32_t one[16];
 #pragma unroll

@@ -198,6 +198,21 @@ def test_f16_pipe_sets_of_warps_over_levels_bit_exact(path):
         assert_same(jobs[l][1].data.cpu().numpy().reshape(ref.packed.shape), ref.packed, cout, 32, f"level {l}")
 
 
+# int32 outputs of the F16 pipe: 16-byte pieces where rows are whole ones and the biases stay within 2^30, else the
+# general form (which saturates)
+@pytest.mark.parametrize("cout", [4, 36, 64, 70, 256, 300])
+@pytest.mark.parametrize("bias", [1 << 30, -(1 << 30), (1 << 30) + 1, I32.max, I32.min])
+def test_f16_pipe_int32_outputs_bit_exact(cout, bias):
+    rng = np.random.default_rng(cout)
+    x = synth.act_codes(rng, (1, 19, 31, 128), 8)
+    wt = rng.integers(-128, 128, size=(cout, 3, 3, 128)).astype(np.int32)
+    b = rng.integers(-1000, 1000, size=(1, cout)).astype(np.int32)
+    b[0, cout // 2] = bias
+    got, want, used = conv_pair(x, 8, wt, 8, out_bits=32, bias=b, workspace=True)
+    assert used == 4
+    assert_same(got, want, cout, 32, f"bias {bias}")
+
+
 # taps per slab 1, 2, 3, 5, 7 and 16, kernels too wide for one (17); resident weights with one and two
 # N tiles and with two planes of an 8-bit image; weights streamed beside half-width tiles
 @pytest.mark.parametrize("kh,kw,pad,cin,cout,bits", [(1, 1, 0, 128, 512, 4), (2, 2, 0, 64, 128, 3), (3, 3, 1, 64, 512, 4),
