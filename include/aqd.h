@@ -205,8 +205,8 @@ aqd_status aqd_conv_int_grouped(const aqd_conv_job* jobs, int32_t njobs,
                                 void* workspace, size_t ws_bytes, aqd_stream_t stream);
 
 /* Workspace that lets a convolution expand its packed input codes once into a zero-padded
- * byte image (one byte per code: sum over jobs of n*(h+2*pad)*(w+2*pad)*cin bytes) and feed
- * the tensor cores from it with TMA tile loads, instead of unpacking every code once per
+ * byte image (one byte per code, two per 8-bit code: sum over jobs of
+ * n*(h+2*pad)*(w+2*pad)*cin bytes, twice that at 8 bits) and feed the tensor cores from it with TMA tile loads, instead of unpacking every code once per
  * kernel tap inside the convolution. Returns 0 when this path does not apply (stride != 1,
  * cin % 64 != 0, codes or weights wider than 4 bits with cin % 128 != 0, K * 3825 >= 2^24
  * with 8-bit codes or weights); a NULL or smaller workspace passed
@@ -220,7 +220,8 @@ size_t aqd_conv_workspace_bytes(const aqd_conv_job* jobs, int32_t njobs,
  * each job is read; y, skip and level are ignored). aqd_conv_int_grouped_expanded is
  * aqd_conv_int_grouped reading that image: `workspace` must hold the expansion of exactly
  * these jobs' inputs, for the same weights' geometry, stride and pad, written by an
- * earlier aqd_conv_expand_input on this stream. Both need the workspace path to apply
+ * earlier aqd_conv_expand_input on this stream. That image does not depend on the weights' bits or
+ * format: weights of any width may read it. Both need the workspace path to apply
  * (aqd_conv_workspace_bytes > 0) and a large enough workspace: otherwise AQD_ERR_INVALID,
  * or AQD_ERR_UNSUPPORTED when the tensor-core kernel does not take the convolution. */
 aqd_status aqd_conv_expand_input(const aqd_conv_job* jobs, int32_t njobs, const aqd_conv_weights* w,

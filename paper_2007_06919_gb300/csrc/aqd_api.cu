@@ -101,8 +101,8 @@ WeightGeom weight_geom(int32_t cout, int32_t kh, int32_t kw, int32_t cin) {
   // |w| <= 15, or, for 8-bit weights, per 128 output channels 128 rows of w_lo = w & 15 then
   // 128 rows of w_hi = w >> 4 (floor), so it is sized for the larger of the two
   g.e4m3_bytes = (size_t)(g.cout_pad > g.split_rows ? g.cout_pad : g.split_rows) * g.k_pad;
-  g.i16_offset = (g.e4m3_bytes + 255) / 256 * 256;
-  g.fp4_offset = (g.i16_offset + 2 * (size_t)cout * g.k_total + 255) / 256 * 256;
+  g.f16_offset = (g.e4m3_bytes + 255) / 256 * 256;
+  g.fp4_offset = (g.f16_offset + 2 * (size_t)cout * g.k_total + 255) / 256 * 256;
   g.fp4_bytes = (size_t)g.cout_pad * (size_t)(g.k_pad / 2);
   g.total_bytes = g.fp4_offset + g.fp4_bytes;
   return g;
@@ -265,14 +265,14 @@ aqd_status aqd_conv_prepare_weights(const void* w_packed, const aqd_conv_weights
   return st ? fail((aqd_status)st, err) : AQD_OK;
 }
 
-// Rows (of cin bytes) of the expanded-activation workspace, or 0 if that path does not apply.
-// Whether 8-bit operands go through the split form on the tensor cores (see ConvArgs).
+// Whether the tensor-core weight block holds the split layout (see ConvArgs).
 static bool split_weights(const aqd_conv_weights* w) { return w->w_bits == 8 && w->w_format == AQD_W_TWOS; }
 
-// Rows (of cin bytes, per plane) of the expanded-activation workspace, or 0 if that path does
-// not apply. 8-bit activations take two planes; 8-bit two's-complement weights the split
-// layout. Every partial sum of the FP32 accumulator stays exact while K * 3825 < 2^24
-// (x_lo * w_lo + 16 x_hi * w_lo <= 15 * 255 per term, w_hi likewise smaller).
+// Rows of the expanded-activation workspace, or 0 if that path does not apply; a row takes
+// *planes * cin bytes (8-bit codes: two bytes each, as an F16 value or in two planes).
+// With 8-bit operands K * 3825 < 2^24 (K <= 4386): the planes' FP32 sum of x_lo * w + 16 x_hi * w, at
+// most 255 * 15 per term, stays exact, the split sums (225 K) and the F16 segments do beyond it, and
+// every |sum| < 2^28, as the F16 epilogue needs.
 static int64_t flat_rows(const aqd_conv_job* jobs, int32_t njobs, const aqd_conv_weights* w, int32_t stride,
                          int32_t pad, int32_t* planes = nullptr) {
   if (!jobs || njobs <= 0 || njobs > kMaxJobs || !w) return 0;
@@ -411,8 +411,7 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
   else { a.upsample = 1; }
   const WeightGeom g = weight_geom(w->cout, w->kh, w->kw, w->cin);
   a.w_e4m3 = static_cast<const uint8_t*>(w->data);
-  a.w_i16 = reinterpret_cast<const int16_t*>(static_cast<const uint8_t*>(w->data) + g.i16_offset);
-  a.w_f16 = w->w_bits == 8 ? 1 : 0;
+  a.w_f16 = reinterpret_cast<const uint16_t*>(static_cast<const uint8_t*>(w->data) + g.f16_offset);
   a.cout_pad = g.cout_pad; a.k_total = g.k_total; a.k_pad = g.k_pad; a.bn = g.bn;
   a.split_rows = g.split_rows;
   a.a_planes = 1;
@@ -426,7 +425,7 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
   a.acc_bound = bound;
   const bool tc_ok = a.x_bits <= 4 && max_w <= 15 && (a.cin % 32) == 0 && bound < (1LL << 24);
   const bool direct_ok = bound < (1LL << 31);
-  // 8-bit operands go to the tensor cores in split form, on the workspace path, without a skip
+  // 8-bit operands go to the tensor cores on the workspace path, without a skip
   int32_t wide_planes = 1;
   bool wide_ok = false;
   if (!tc_ok && workspace && !has_skip && (a.x_bits == 8 || split_weights(w))) {
@@ -450,14 +449,18 @@ static aqd_status plan_grouped(const aqd_conv_job* jobs, int32_t njobs, const aq
     if (rows > 0 && (size_t)rows * (size_t)planes * (size_t)w->cin <= ws_bytes) {
       a.ws = static_cast<uint8_t*>(workspace);
       a.ws_rows = (int64_t)(ws_bytes / ((size_t)planes * (size_t)w->cin));
-      a.a_planes = planes;
-      a.split_w = (!tc_ok && split_weights(w)) ? 1 : 0;
-      // both operands 8 bits wide: F16 holds either, so one product takes the place of the split
-      // form's four (the image has the two planes' bytes: one F16 value per code)
-      if (a.split_w && planes == 2) { a.f16 = 1; a.split_w = 0; a.a_planes = 1; }
+      // 8-bit codes: F16 with 8-bit weights (one product instead of the four of halves). With narrower
+      // weights two planes take as many products at the E4M3 rate, but only where this call expands its
+      // input: an image that one call expands and others read is F16 for weights of every width.
+      // (Neither is better everywhere. One call, 4-bit weights, two 100 x 168 maps, planes / F16: 3x3 384 -> 512
+      // 81 / 74 us, 1x1 128 -> 64 14.1 / 11.7, 1x1 512 -> 512 35 / 38; 3x3 128 -> 32 at 32 x 32 9.0 / 10.0.)
+      const bool own_image = stage == kStageBoth || stage == kStageBothChain;
+      a.f16 = planes == 2 && (split_weights(w) || !own_image) ? 1 : 0;
+      a.a_planes = a.f16 ? 1 : planes;
+      a.split_w = (!tc_ok && !a.f16 && split_weights(w)) ? 1 : 0;
     }
   }
-  if (path == 1 && !tc_ok && !a.ws) path = 2;  // the split form exists only on the workspace path
+  if (path == 1 && !tc_ok && !a.ws) path = 2;  // 8-bit operands run only on the workspace path
   if (path == 2 && !direct_ok) return fail(AQD_ERR_UNSUPPORTED, "accumulator bound exceeds int32");
   // a caller that gave the library's own workspace wants the workspace path or nothing
   if (require_ws && (path != 1 || !a.ws))

@@ -57,9 +57,8 @@ conv_direct_kernel(const ConvArgs a, int job_index) {
     for (int i = threadIdx.x; i < kKC * 32; i += kThreads) {
       const int kk = i / 32, j = i % 32;
       const int co = co0 + j;
-      int16_t w = (kk < kc && co < a.cout) ? a.w_i16[(int64_t)co * a.k_total + k0 + kk] : (int16_t)0;
-      if (a.w_f16) w = (int16_t)__half2int_rn(__short_as_half(w));
-      wsm[kk][j] = w;
+      const uint16_t w = (kk < kc && co < a.cout) ? a.w_f16[(int64_t)co * a.k_total + k0 + kk] : (uint16_t)0;
+      wsm[kk][j] = (int16_t)__half2int_rn(__ushort_as_half(w));
     }
     __syncthreads();
     int tap = k0 / a.cin;

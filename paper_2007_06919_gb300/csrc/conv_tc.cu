@@ -17,10 +17,11 @@
 // nibble image keeps the byte image's row stride (cin bytes) and fills the first cin / 2
 // bytes of each row, so its zero border lies where a byte image's does in the same workspace.
 //
-// 8-bit codes with 8-bit weights on the F16 pipe (kF16): F16 holds either exactly, every product is
-// an integer below 2^15, and the FP32 accumulator is exact over 512 K elements (512 * 255 * 128 <
+// 8-bit codes on the F16 pipe (kF16): F16 holds them and weights of any width exactly, every product is an
+// integer, and with 8-bit weights the FP32 accumulator is exact over 512 K elements (512 * 255 * 128 <
 // 2^24). K runs in segments of that length, each in its own TMEM accumulator; the epilogue warps
-// add the segments as int32 in registers. The image holds F16 values (2 cin bytes a row).
+// add the segments as int32 in registers. (With narrower weights one segment holds all of K.) The image
+// holds F16 values (2 cin bytes a row).
 //
 // Per CTA (one per SM, persistent over tiles of 128 output pixels x BN channels):
 //   warps 0..E-1  epilogue (E = 16, or 8 beside activation producers): tcgen05.ld of the
@@ -133,8 +134,8 @@ struct Params {
   uint32_t off_sktab;   // table of 2- to 4-bit skip codes
   uint32_t off_ostage;  // int32 outputs: per-warp staging blocks for row-contiguous stores (0: none)
   int32_t out_pad;
-  int32_t seg_chunks; // kF16: K chunks per exact FP32 segment (512 K elements)
-  int32_t a_planes;   // K runs over this many planes of the byte image (2: 8-bit activations)
+  int32_t seg_chunks; // kF16: K chunks per exact FP32 segment
+  int32_t a_planes;   // K runs over this many planes of the byte image (2: 8-bit codes in halves)
   int32_t plane_rows; // workspace rows per plane
   int32_t split_w;    // weights in the split layout: a tile's bn B rows give bn/2 channels
   uint32_t* status;
@@ -1784,7 +1785,8 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   prm.div_layer = div_magic(prm.layer_tiles);
   prm.div_nt = div_magic(prm.n_tiles);
   prm.num_kchunks = flat ? (fp4 ? a.k_total / 2 : (f16 ? 2 * a.k_total : a.k_total)) / bk : a.k_pad / BK;
-  prm.seg_chunks = 512 * 2 / BK;
+  // (64 K elements per chunk; acc_bound / k_total bounds one product)
+  prm.seg_chunks = f16 ? (int)(((1LL << 24) - 1) / (a.acc_bound / a.k_total) / 64) : 0;
   prm.cin = a.cin; prm.cout = a.cout; prm.kh = a.kh; prm.kw = a.kw;
   prm.stride = a.stride; prm.pad = a.pad; prm.k_total = a.k_total;
   prm.out_bits = a.out_bits; prm.skip_bits = a.skip_bits;
@@ -1915,7 +1917,7 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   cuuint32_t box[2] = {(cuuint32_t)bk, (cuuint32_t)b_rows};
   cuuint32_t estr[2] = {1, 1};
   const CUtensorMapSwizzle swz = bk == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
-  const uint8_t* w_src = fp4 ? a.w_fp4 : (f16 ? reinterpret_cast<const uint8_t*>(a.w_i16) : a.w_e4m3);
+  const uint8_t* w_src = fp4 ? a.w_fp4 : (f16 ? reinterpret_cast<const uint8_t*>(a.w_f16) : a.w_e4m3);
   for (int l = 0; l < nlayers; ++l) {
     const uint8_t* wl = nlayers > 1 ? a.layer[l].w_e4m3 : w_src;
     const CUresult r = enc(&maps.w[l], CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, (void*)wl, gdim, gstride, box, estr,

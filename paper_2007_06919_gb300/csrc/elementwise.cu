@@ -1207,7 +1207,8 @@ unpack_kernel(const uint8_t* packed, int64_t groups, int is_signed, int32_t* out
 }
 
 // Prepared weights: E4M3 sign-magnitude bytes [cout_pad][k_pad] (zero padded; only when
-// every |w| <= 15) followed by int16 [cout][k_total] (F16 values for 8-bit weights).
+// every |w| <= 15) followed by F16 [cout][k_total] (every width is exact in F16: the operand of 8-bit
+// codes, of the first conv and of the CUDA-core kernel).
 __global__ void __launch_bounds__(kThreads)
 prepare_weights_kernel(const uint8_t* wp, int w_bits, int w_format, WeightGeom g, int64_t w_row_bytes,
                        int make_e4m3, uint8_t* out) {
@@ -1216,8 +1217,8 @@ prepare_weights_kernel(const uint8_t* wp, int w_bits, int w_format, WeightGeom g
   const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
   const int64_t e4_rows = make_e4m3 == 2 ? g.split_rows : g.cout_pad;
   const int64_t n_e4 = e4_rows * g.k_pad;
-  const int64_t n_i16 = (int64_t)g.cout * g.k_total;
-  if (t >= n_e4 + n_i16) return;
+  const int64_t n_f16 = (int64_t)g.cout * g.k_total;
+  if (t >= n_e4 + n_f16) return;
   int64_t co, k;
   int part = 0;  // split layout: 0 = w_lo, 1 = w_hi
   if (t < n_e4) {
@@ -1253,9 +1254,7 @@ prepare_weights_kernel(const uint8_t* wp, int w_bits, int w_format, WeightGeom g
       out[t] = 0;
     }
   } else {
-    // (8-bit weights as F16, exact: the F16 pipe's operand and the stem's)
-    reinterpret_cast<int16_t*>(out + g.i16_offset)[t - n_e4] =
-        w_bits == 8 ? __half_as_short(__int2half_rn(w)) : (int16_t)w;
+    reinterpret_cast<__half*>(out + g.f16_offset)[t - n_e4] = __int2half_rn(w);
   }
 }
 

@@ -47,8 +47,7 @@ struct ConvArgs {
   int32_t upsample, scale_main, has_skip;
   // prepared weights
   const uint8_t* w_e4m3;  // [cout_pad][k_pad] E4M3 sign-magnitude bytes (|w| <= 15)
-  const int16_t* w_i16;   // [cout][k_total] signed integers (F16 values when w_f16)
-  int32_t w_f16;          // 8-bit weights: w_i16 holds F16 bit patterns
+  const uint16_t* w_f16;  // [cout][k_total] the same weights, of any width, as F16 values
   int32_t cout_pad, k_total, k_pad, bn;
   int64_t acc_bound;      // K * max|x| * max|w|: bound on |accumulator|
   uint8_t* ws;            // expanded-activation workspace (NULL: in-kernel unpacking)
@@ -56,13 +55,14 @@ struct ConvArgs {
   int32_t skip_expand;    // workspace already holds the expansion: launch only the conv
   int32_t expand_only;    // launch only the expansion into the workspace
   int32_t no_pair;        // workspace path: use the one-CTA kernel even for 256-wide N tiles
-  // 8-bit operands on the tensor cores (workspace path): activations as two planes of
-  // 4-bit halves (x_lo, 16 x_hi) over which K runs twice; weights, when wider than 15, as
-  // two row blocks per 128 output channels (w_lo, w_hi) whose accumulators combine as D1 + 16 D2
-  int32_t a_planes;       // 1, or 2 for 8-bit activation codes
+  // 8-bit operands on the tensor cores (workspace path). 8-bit codes: the F16 pipe (the image holds F16
+  // values), or, where one call expands them for 2- to 4-bit weights, two planes of 4-bit halves (x_lo,
+  // 16 x_hi) over which K runs twice. 8-bit weights of narrower codes: two row blocks per 128 output
+  // channels (w_lo, w_hi) whose accumulators combine as D1 + 16 D2.
+  int32_t f16;            // the F16 pipe
+  int32_t a_planes;       // 1, or 2
   int32_t split_w;        // weights in the split layout
   int32_t split_rows;     // weight rows of that layout (2 * round_up(cout, 128))
-  int32_t f16;            // 8-bit codes with 8-bit weights on the F16 pipe (the image holds F16 values)
   uint8_t* ws_out;        // chained output: also write the output codes as the next conv's byte image
   int32_t out_pad;        // padding of that next conv
   uint32_t* status;       // device status word
@@ -99,7 +99,7 @@ struct WeightGeom {
   int32_t cout, kh, kw, cin;
   int32_t k_total, k_pad, bn, cout_pad;
   int32_t split_rows;     // 2 * round_up(cout, 128): rows of the split (8-bit) weight layout
-  size_t e4m3_bytes, i16_offset;
+  size_t e4m3_bytes, f16_offset;
   // [cout_pad][k_pad / 2] E2M1 nibbles (weight w as the value w / 2, |w| <= 4; weight k of a
   // row in the low nibble of byte k / 2 for even k): the FP4 tensor-core B operand
   size_t fp4_offset, fp4_bytes;

@@ -77,7 +77,7 @@ struct StemParams {
   const int32_t* m0;
   const int8_t* shift;
   const int32_t* bias;
-  const int16_t* w_i16;   // [cout][147] F16 values, K order (r, s, c)
+  const uint16_t* w_f16;  // [cout][147] F16 values, K order (r, s, c)
   uint32_t off_b, off_cst, off_bar;
   uint32_t* status;
 };
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
     for (int h = 0; h < 2; ++h) {
       const int r = (kk + h) / kLs, j = (kk + h) - r * kLs;
       uint16_t wv = 0;  // (F16 zero)
-      if (n < p.cout && r < kKH && j < kSeg) wv = (uint16_t)p.w_i16[(int64_t)n * (kKH * kSeg) + r * kSeg + j];
+      if (n < p.cout && r < kKH && j < kSeg) wv = p.w_f16[(int64_t)n * (kKH * kSeg) + r * kSeg + j];
       pr |= (uint32_t)wv << (16 * h);
     }
     *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) = pr;
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
   load_channels(p, cst4, cste, s_fast);
   for (int n = warp; n < p.cout; n += kThreads / 32) {
     uint32_t part = 0;
-    for (int k = lane; k < kKH * kSeg; k += 32) part += abs_f16((uint16_t)p.w_i16[(int64_t)n * (kKH * kSeg) + k]);
+    for (int k = lane; k < kKH * kSeg; k += 32) part += abs_f16(p.w_f16[(int64_t)n * (kKH * kSeg) + k]);
     if (!weights_small(part) && lane == 0) atomicAnd(s_fast, 0);
   }
   fence_proxy_async();  // generic-proxy stores of B -> visible to the MMA
@@ -585,9 +585,9 @@ __global__ void __launch_bounds__(kRThreads, 1) stem_rows_kernel(const __grid_co
       const int r = kk / 32, s = (kk % 32) / 4, c = kk % 4;  // (c is 0 or 2)
       uint16_t w0 = 0, w1 = 0;
       if (n < p.cout && kk < kRK && s < kKW) {
-        const int16_t* w = p.w_i16 + (int64_t)n * (kKH * kSeg) + r * kSeg + s * kC + c;
-        w0 = (uint16_t)w[0];
-        if (c == 0) w1 = (uint16_t)w[1];
+        const uint16_t* w = p.w_f16 + (int64_t)n * (kKH * kSeg) + r * kSeg + s * kC + c;
+        w0 = w[0];
+        if (c == 0) w1 = w[1];
       }
       part += abs_f16(w0) + abs_f16(w1);
       if (kk < kRK)
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(kRThreads, 1) stem_rows_kernel(const __grid_co
 
 bool stem_applicable(const ConvArgs& a) {
   return a.njobs == 1 && a.x_bits == 8 && a.cin == stem::kC && a.kh == stem::kKH && a.kw == stem::kKW &&
-         a.w_f16 && !a.has_skip && a.cout % 16 == 0 && a.cout <= 256 && a.k_total == stem::kKH * stem::kSeg &&
+         !a.has_skip && a.cout % 16 == 0 && a.cout <= 256 && a.k_total == stem::kKH * stem::kSeg &&
          a.acc_bound < (1LL << 24);  // K * 255 * max|w|: the FP32 sum is exact
 }
 
@@ -743,7 +743,7 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   p.level = jb.level;
   p.y_row_bytes = a.y_row_bytes;
   p.m0 = a.m0; p.shift = a.shift; p.bias = a.bias;
-  p.w_i16 = a.w_i16;
+  p.w_f16 = a.w_f16;
   p.status = a.status;
   const int64_t m_total = (int64_t)jb.n * jb.ho * jb.wo;
   if (m_total + 128 >= (1LL << 31)) { *err = "stem conv: more than 2^31 output pixels"; return 2; }

@@ -3,8 +3,9 @@ CPU oracle: bit-exact on every output byte, through the C ABI, for both kernels.
 import numpy as np
 import pytest
 
-from gpu_util import assert_same, conv_pair, weights
-from paper_2007_06919_gb300 import synth
+import oracle
+from gpu_util import assert_same, conv_pair, to_device, weights
+from paper_2007_06919_gb300 import aqd, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -302,11 +303,11 @@ def oracle_unpack(packed, c, bits):
     return oracle.unpack(packed, c, bits)
 
 
-# (x_bits, w_bits, n, h, w, cin, cout, out_bits): 8-bit operands on the tensor cores, split
-# into 4-bit halves (activation planes x_lo, 16 x_hi; weight rows w_lo, w_hi)
+# (x_bits, w_bits, n, h, w, cin, cout, out_bits): 8-bit operands on the tensor cores: on the F16 pipe, or split
+# into 4-bit halves beside narrower ones (activation planes x_lo, 16 x_hi; weight rows w_lo, w_hi)
 WIDE_CASES = [
     (8, 4, 2, 11, 13, 128, 64, 4),     # 8-bit activations, 4-bit weights: two planes
-    (8, 8, 1, 9, 17, 256, 256, 8),     # both 8-bit: two planes, split weights
+    (8, 8, 1, 9, 17, 256, 256, 8),     # both 8-bit: segments of 512
     (2, 8, 2, 7, 9, 128, 96, 2),       # 8-bit weights only
     (4, 8, 1, 12, 10, 256, 80, 32),    # int32 output
     (8, 8, 3, 5, 6, 128, 384, 4),      # three 128-channel output blocks
@@ -329,8 +330,8 @@ def test_wide_operands_on_tensor_cores_bit_exact(case, pairs):
 
 
 def test_wide_operands_exact_at_the_bound():
-    """Every code 255 and every weight -128 or 127 (signs mixed per channel), K = 3456 (the
-    FP32 partial sums D1 <= 3825 K stay below 2^24): int32 outputs equal the oracle's."""
+    """Every code 255 and every weight -128 or 127 (signs mixed per channel), K = 3456 in
+    segments whose FP32 sums stay just below 2^24: int32 outputs equal the oracle's."""
     cin = 384
     x = np.full((1, 4, 5, cin), 255, np.int32)
     w = np.full((64, 3, 3, cin), -128, np.int32)
@@ -341,6 +342,58 @@ def test_wide_operands_exact_at_the_bound():
     assert used == 4
     assert_same(got, want, 64, 32, "wide exactness")
     assert np.abs(want.view(np.int32)).max() > (1 << 26)
+
+
+# the largest K of the workspace path with 8-bit operands (4352 of at most 4386): 8-bit codes with 4-bit weights, whose
+# planes' FP32 sum reaches 3825 K, and 8-bit weights split as D1 + 16 D2 beside 4-bit codes
+@pytest.mark.parametrize("xb,wb,w_format", [(8, 4, 0), (8, 4, 1), (4, 8, 0)])
+@pytest.mark.parametrize("pairs", [True, False])
+def test_one_sided_wide_operands_exact_at_the_bound(xb, wb, w_format, pairs):
+    cin, kh, kw = 128, 2, 17
+    x = np.full((1, 5, 30, cin), (1 << xb) - 1, np.int32)
+    if w_format:  # stored codes 0 and 15 of the odd grid: -15 and 15
+        lo, hi = 0, 15
+    else:
+        lo, hi = -(1 << (wb - 1)), (1 << (wb - 1)) - 1
+    w = np.full((64, kh, kw, cin), lo, np.int32)
+    w[1::2] = hi
+    w[3, :, :, ::2] = lo
+    w[5] = np.random.default_rng(5).integers(lo, hi + 1, size=(kh, kw, cin))
+    got, want, used = conv_pair(x, xb, w, wb, w_format=w_format, pad=0, out_bits=32, bias=np.zeros((1, 64), np.int32),
+                                path=TC if pairs else TC_NO_PAIR, workspace=True)
+    assert used == (4 if pairs else 3)
+    assert_same(got, want, 64, 32, f"{xb}-bit codes, {wb}-bit weights")
+    if xb == 8:  # and as separate calls, one F16 segment of all of K
+        X, (W, _) = to_device(oracle.CodeTensor.from_codes(x, xb)), weights(w, wb, w_format)
+        jobs = [(X, aqd.DTensor.empty(1, 4, 14, 64, 32), None, 0)]
+        ws = aqd.workspace_for(jobs, W, 1, 0)
+        aqd.conv_expand_input(jobs, W, 1, 0, ws)
+        aqd.conv_int_grouped_expanded(jobs, W, 1, 0, workspace=ws)
+        assert_same(jobs[0][1].data.cpu().numpy().reshape(want.shape), want, 64, 32, f"separate calls, {wb}-bit weights")
+
+
+# one expansion of 8-bit codes read by convs of every weight width, expanded for one of them or for another
+@pytest.mark.parametrize("expand_for", [8, 4, 2])
+@pytest.mark.parametrize("cout,k", [(256, 3), (64, 1)])
+def test_one_expansion_read_by_several_weight_widths(expand_for, cout, k):
+    rng = np.random.default_rng(expand_for + cout)
+    cin, shape = 256, (2, 19, 23)
+    xt = oracle.CodeTensor.from_codes(synth.act_codes(rng, (*shape, cin), 8), 8)
+    X = to_device(xt)
+    W = {wb: weights(rng.integers(-(1 << (wb - 1)), 1 << (wb - 1), size=(cout, k, k, cin)).astype(np.int32), wb)
+         for wb in (2, 3, 4, 8)}
+    jobs = [(X, aqd.DTensor.empty(*shape, cout, 32), None, 0)]
+    size = {aqd.conv_workspace_bytes(jobs, w, 1, k // 2) for w, _ in W.values()}
+    assert len(size) == 1
+    ws = aqd.workspace_for(jobs, W[expand_for][0], 1, k // 2)
+    ws.fill_(0x5A)
+    aqd.conv_expand_input(jobs, W[expand_for][0], 1, k // 2, ws)
+    for wb in (8, 4, 3, 2, 8):
+        aqd.conv_int_grouped_expanded(jobs, W[wb][0], 1, k // 2, workspace=ws)
+        want = oracle.conv_int(xt, W[wb][1], wb, 0, k, k, 1, k // 2, cout, out_bits=32)
+        got = jobs[0][1].data.cpu().numpy().reshape(want.packed.shape)
+        assert_same(got, want.packed, cout, 32, f"expanded for {expand_for}-bit weights, read by {wb}-bit ones")
+    assert aqd.device_status() == 0
 
 
 @pytest.mark.parametrize("neg_m0", [False, True])
