@@ -38,6 +38,7 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdio>
 #include <mutex>
 #include <type_traits>
@@ -346,52 +347,136 @@ __device__ __forceinline__ void skip_bytewords(const uint2& g, int sb, uint32_t 
   }
 }
 
-// 16 columns of one row in the general form.
-struct GenCols {
-  uint32_t taddr;       // TMEM address of the first column
-  uint32_t taddr_hi;    // split weights: of the w_hi accumulator
-  const EpiChan* ep;    // the columns' constants
-  const uint8_t* srow;  // the skip's row (kSkip), at the tile's first channel
-  uint8_t* yrow;        // the output's row, likewise
-  int ch0, nc, flags;   // first channel from there, channels that exist
-  bool row_ok;
-};
+// ---- the general form: any shift, any skip direction and width, any row size, int32 outputs with a skip, biases
+// beyond 2^30. Eq. 6 -> Eq. 7 -> Eq. 2 as the definition states them, in int64 where a value needs it. Functions
+// of their own, not inlined: their registers and code stay out of the common forms. Skips are loaded and int32
+// outputs stored in whole pieces where rows allow it. Against element by element, on two 100 x 168 maps: 3x3 256 ->
+// 256 with a 4-bit skip and R = 32 151 -> 52 us, 1x1 64 -> 256 with a 4-bit skip and int32 outputs 156 -> 44.
 
-// Eq. 6 -> Eq. 7 -> Eq. 2 as the definition states them, element by element in int64 (any shift,
-// any skip direction and width, any row size), with the 32-bit requant where the tables allow it
-// and there is no skip (accumulators too large for the common form). Returns the codes as
-// byte-words; int32 outputs and 8-bit rows of no whole groups are stored here. Not inlined: its
-// registers and code stay out of the common forms.
+// A column's constants (EpiChan) from their shared-memory address
+struct ColConst {
+  int32_t bias, m0, c;
+  int r, d;
+};
+__device__ __forceinline__ ColConst col_const(uint32_t addr) {
+  int32_t w;
+  ColConst k;
+  asm volatile("ld.shared.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(k.bias), "=r"(k.m0), "=r"(k.c), "=r"(w) : "r"(addr));
+  k.r = w & 0xFF;
+  k.d = (w >> 8) & 0xFF;
+  return k;
+}
+static_assert(sizeof(EpiChan) == 16 && offsetof(EpiChan, r) == 12 && offsetof(EpiChan, d) == 13, "col_const");
+
+// rhu in one variable shift: floor((v + 2^(r-1)) / 2^r) = floor((floor(v / 2^(r-1)) + 1) / 2)
+__device__ __forceinline__ int64_t rhu1(int64_t v, int r) { return r > 0 ? ((v >> (r - 1)) + 1) >> 1 : v; }
+__device__ __forceinline__ int32_t sat_s32(int64_t v) { return (int32_t)sat32(v); }
+
+// The row's skip values of nc columns from channel ch on.
+__device__ __forceinline__ void general_skip(const Params& p, const uint8_t* srow, int ch, int nc, int32_t (&sk)[16]) {
+  const int sb = p.skip_bits;
+  const bool whole = (p.skip_row_bytes & 15) == 0;  // (then nc is a multiple of 4, and 16 with 8-bit codes)
+#pragma unroll
+  for (int i = 0; i < 16; ++i) sk[i] = 0;
+  if (sb == 32 && whole) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      int4 v = make_int4(0, 0, 0, 0);
+      if (4 * q < nc) v = __ldg(reinterpret_cast<const int4*>(srow) + (ch >> 2) + q);
+      sk[4 * q] = v.x; sk[4 * q + 1] = v.y; sk[4 * q + 2] = v.z; sk[4 * q + 3] = v.w;
+    }
+  } else if (sb == 32) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < nc) sk[i] = __ldg(reinterpret_cast<const int32_t*>(srow) + ch + i);
+  } else if (sb == 8 && !whole) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      if (i < nc) sk[i] = __ldg(srow + ch + i);
+  } else {
+    uint32_t b[4];
+    if (sb == 8) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(srow + ch));
+      b[0] = v.x; b[1] = v.y; b[2] = v.z; b[3] = v.w;
+    } else {
+      // (2- to 4-bit codes: whole groups, of which these are a half)
+      uint2 g = make_uint2(0u, 0u);
+      if (sb == 4) g = __ldg(reinterpret_cast<const uint2*>(srow + (ch >> 1)));
+      else if (sb == 2) g.x = __ldg(reinterpret_cast<const uint32_t*>(srow + (ch >> 2)));
+      else {
+        const uint32_t* g3 = reinterpret_cast<const uint32_t*>(srow + (ch >> 5) * 12);
+        const int half = (ch >> 4) & 1;
+        g = make_uint2(__ldg(g3 + half), __ldg(g3 + 2) >> (4 * half));
+      }
+      skip_bytewords(g, sb, b);
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) sk[i] = (int32_t)((b[i / 4] >> (8 * (i % 4))) & 0xFFu);
+  }
+}
+
+// nc columns (at most 16) of one row from channel ch on (srow and yrow stand at the tile's first channel; ep: the
+// columns' constants): the codes as byte-words, or the outputs of int32 rows and of 8-bit rows of no whole groups
+// stored here.
 template <bool kSkip>
-__device__ __forceinline__ uint4 general_finish(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
-  if (!u.row_ok) return make_uint4(0u, 0u, 0u, 0u);
-  if (!kSkip && (u.flags & kFlagReq) && p.out_bits != 32) {
-    const int qmax = (1 << p.out_bits) - 1;
+__device__ __forceinline__ uint4 general_finish(const Params& p, uint32_t ep, const uint8_t* srow, uint8_t* yrow, int ch,
+                                                int nc, int flags, int32_t (&acc)[16]) {
+  const int out_bits = p.out_bits;
+  const int32_t qmax = (1 << (out_bits & 15)) - 1;
+  const auto at = [ep](int i) { return ep + (uint32_t)(i * sizeof(EpiChan)); };
+  auto requant = [qmax](int32_t u, const ColConst& k) {
+    const int64_t v = rhu1((int64_t)u * k.m0, k.r);
+    return v < 0 ? 0 : (v > qmax ? qmax : (int32_t)v);
+  };
+  if constexpr (kSkip) {
+    int32_t sk[16];
+    general_skip(p, srow, ch, nc, sk);
+    if (p.scale_main == 0) {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const ColConst k = col_const(at(i));
+        acc[i] = sat_s32((int64_t)acc[i] + k.bias + rhu1((int64_t)sk[i] * k.c, k.d));
+        if (out_bits != 32) acc[i] = requant(acc[i], k);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const ColConst k = col_const(at(i));
+        acc[i] = sat_s32(rhu1((int64_t)add_sat(acc[i], k.bias) * k.c, k.d) + sk[i]);
+        if (out_bits != 32) acc[i] = requant(acc[i], k);
+      }
+    }
+  } else if (out_bits == 32) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = add_sat(acc[i], col_const(at(i)).bias);
+  } else if (flags & kFlagReq) {
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      const EpiChan c = u.ep[i];
-      acc[i] = i < u.nc ? __vimin_s32_relu((__mulhi(add_sat(acc[i], c.bias), c.m0) + (1 << (c.r - 33))) >> (c.r - 32), qmax) : 0;
+      const ColConst k = col_const(at(i));
+      acc[i] = __vimin_s32_relu((__mulhi(add_sat(acc[i], k.bias), k.m0) + (1 << (k.r - 33))) >> (k.r - 32), qmax);
     }
   } else {
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
-      if (i < u.nc) {
-        const int32_t s = kSkip ? read_code(u.srow, u.ch0 + i, p.skip_bits, false) : 0;
-        acc[i] = epilogue<kSkip>(acc[i], s, u.ep[i], p.scale_main, p.out_bits);
-      } else {
-        acc[i] = 0;
-      }
+      const ColConst k = col_const(at(i));
+      acc[i] = requant(add_sat(acc[i], k.bias), k);
     }
   }
-  if (p.out_bits == 32) {
-    int32_t* yr = reinterpret_cast<int32_t*>(u.yrow) + u.ch0;
+  if (out_bits == 32) {
+    int32_t* yr = reinterpret_cast<int32_t*>(yrow) + ch;
+    if ((p.cout & 3) == 0) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (4 * q < nc) reinterpret_cast<int4*>(yr)[q] = make_int4(acc[4 * q], acc[4 * q + 1], acc[4 * q + 2], acc[4 * q + 3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        if (i < nc) yr[i] = acc[i];
+    }
+  } else if (out_bits == 8 && (p.cout & 31) != 0) {
 #pragma unroll
     for (int i = 0; i < 16; ++i)
-      if (i < u.nc) yr[i] = acc[i];
-  } else if (p.out_bits == 8 && (p.cout & 31) != 0) {
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      if (i < u.nc) u.yrow[u.ch0 + i] = (uint8_t)acc[i];
+      if (i < nc) yrow[ch + i] = (uint8_t)acc[i];
   }
   uint32_t bw[4];
 #pragma unroll
@@ -401,28 +486,58 @@ __device__ __forceinline__ uint4 general_finish(const Params& p, const GenCols& 
   return make_uint4(bw[0], bw[1], bw[2], bw[3]);
 }
 
-// The same from the accumulators in TMEM.
+// A warp's columns of a tile in the general form. (In memory: as arguments they would be registers of the caller.)
+struct GenTile {
+  uint32_t taddr;       // TMEM address of the tile's first column
+  int cn;               // split weights: columns from there to the w_hi accumulator
+  uint32_t ep;          // shared address of the first column's constants
+  int c_lo, c_hi, flags, nib;
+  const uint8_t* srow;  // the lane's row of the skip (kSkip), of the output (NULL: none) and of the chained image, at the
+  uint8_t *yrow, *irow; // tile's first channel
+};
+template <bool kSkip>
+__device__ __forceinline__ void general_step(const Params& p, const GenTile& g, int c0, int32_t (&acc)[16], uint32_t& top) {
+  const uint4 r = general_finish<kSkip>(p, g.ep + (uint32_t)(c0 * sizeof(EpiChan)), g.srow, g.yrow, c0,
+                                        g.c_hi - c0 < 16 ? g.c_hi - c0 : 16, g.flags, acc);
+  if (p.out_bits == 32 || (p.out_bits == 8 && (p.cout & 31) != 0)) return;  // (stored by general_finish)
+  const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
+  store_codes16(g.yrow, c0, bw, p.out_bits, top);
+  if (g.irow) store_image16(g.irow, c0, bw, g.nib);
+}
+// From the accumulators in TMEM, which hold the integer sum / sc.
 template <bool kSkip, bool kSplit>
-__device__ __noinline__ uint4 general_cols(const Params& p, const GenCols& u, float sc) {
-  uint32_t v[16];
-  tmem_ld16(u.taddr, v);
-  tmem_wait_ld();
-  reg_fence16(v);
-  int32_t acc[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) acc[i] = __float2int_rn(__uint_as_float(v[i]) * sc);
-  if constexpr (kSplit) {
-    tmem_ld16(u.taddr_hi, v);
+__device__ __noinline__ void general_tile(const Params& p, const GenTile& g, float sc) {
+  uint32_t top = 0u;  // (3-bit codes: see store_codes16)
+#pragma unroll 1
+  for (int c0 = g.c_lo; c0 < g.c_hi; c0 += 16) {
+    uint32_t v[16];
+    tmem_ld16(g.taddr + (uint32_t)c0, v);
     tmem_wait_ld();
     reg_fence16(v);
+    int32_t acc[16];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
+    for (int i = 0; i < 16; ++i) acc[i] = __float2int_rn(__uint_as_float(v[i]) * sc);
+    if constexpr (kSplit) {
+      tmem_ld16(g.taddr + (uint32_t)(g.cn + c0), v);
+      tmem_wait_ld();
+      reg_fence16(v);
+#pragma unroll
+      for (int i = 0; i < 16; ++i) acc[i] += 16 * __float2int_rn(__uint_as_float(v[i]) * sc);
+    }
+    if (g.yrow) general_step<kSkip>(p, g, c0, acc, top);
+    __syncwarp();
   }
-  return general_finish<kSkip>(p, u, acc);
 }
-// The same from sums in registers (kF16).
-__device__ __noinline__ uint4 general_sums(const Params& p, const GenCols& u, int32_t (&acc)[16]) {
-  return general_finish<false>(p, u, acc);
+// From a lane's sums of the columns from c_lo on (kF16).
+__device__ __noinline__ void general_sums(const Params& p, const GenTile& g, const int32_t* sums) {
+  uint32_t top = 0u;
+#pragma unroll 1
+  for (int c0 = g.c_lo; c0 < g.c_hi; c0 += 16, sums += 16) {
+    int32_t acc[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = sums[i];
+    general_step<false>(p, g, c0, acc, top);
+  }
 }
 
 // ---------------------------------------------------------------- the kernel
@@ -499,8 +614,8 @@ __device__ __forceinline__ void load_half(const Params& p, RowCursor<kXBits>& rc
 // kSkip: the instantiation that handles a skip tensor (Eq. 7); the others carry no skip code,
 // which keeps the common path's registers free.
 // kSplit: the 8-bit split form (split weights combined as D1 + 16 D2 in the epilogue).
-// kOStage: int32 outputs go through per-warp shared-memory staging blocks (an instantiation of
-// its own, so that the other forms keep their registers)
+// kOStage: int32 outputs, through per-warp shared-memory staging blocks, or on the F16 pipe stored as they are
+// (an instantiation of its own, so that the other forms keep their registers)
 template <int kXBits, bool kChunkInTap, bool kFlat, bool kPair, bool kSkip, bool kSplit, int kBK, bool kFp4,
           bool kOStage>
 __global__ void __launch_bounds__(threads_for(kFlat), 1)
@@ -509,7 +624,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
   static_assert(kBK == BK || kFlat, "64-byte K chunks exist for the workspace path only");
   static_assert(!kFp4 || (kFlat && kBK == BK && !kSplit), "the FP4 pipe reads nibble images in 128-byte chunks");
   constexpr bool kF16 = kXBits == 8;  // (flat kernels read images: kXBits names the pipe only here)
-  static_assert(!kF16 || (kFlat && kBK == BK && !kSplit && !kFp4 && !kSkip && !kOStage), "the F16 pipe's form");
+  static_assert(!kF16 || (kFlat && kBK == BK && !kSplit && !kFp4 && !kSkip), "the F16 pipe's form");
   // the FP32 accumulator holds the integer sum / kAccSc
   constexpr float kAccSc = kFp4 ? 4.0f : 262144.0f;
   constexpr int kStA = BM * kBK;  // bytes of one stage's A operand
@@ -1060,48 +1175,41 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         const int vr = ft.v0 + (int)rank * 128 + quarter * 32 + lane;
         const int oh = fast_div(vr, jb.div_row), ow = vr - oh * jb.wp;
         if (vr < jb.vimg && ow < jb.wo) {  // else a junk column or past the image
-          uint8_t* yrow = ly.y[ti.job] + (int64_t)((ft.img * jb.ho + oh) * jb.wo + ow) * p.y_row_bytes;
+          // (the row pointers stand at the tile's first channel, a multiple of 32)
+          const int grp0 = ti.col0 >> 5, nib = ly.ws_nib;
+          uint8_t* yrow = ly.y[ti.job] + (int64_t)((ft.img * jb.ho + oh) * jb.wo + ow) * p.y_row_bytes + grp0 * group_bytes(out_bits);
           uint8_t* irow = ly.ws_out ? ly.ws_out + (size_t)(jb.orow_off + (ft.img * jb.ohp + oh + p.out_pad) * jb.owp + ow +
-                                                           p.out_pad) * p.cout
+                                                           p.out_pad) * p.cout + grp0 * (nib ? 16 : 32)
                                     : nullptr;
-          uint32_t top = 0u;
+          const bool lean = kOStage ? (flags & kFlagBias) && (p.cout & 3) == 0
+                                    : (flags & kFlagReq) && (out_bits != 8 || (p.cout & 31) == 0);
+          if (lean) {
+            // (|sum| < 2^28 and |bias| <= 2^30)
+            uint32_t top = 0u;
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int c0 = c_lo + 16 * j;
-            if (c0 >= c_hi) break;
-            const int ch0 = ti.col0 + c0, nc = c_hi - c0 < 16 ? c_hi - c0 : 16;
-            if (out_bits != 32 && (flags & kFlagReq) && (out_bits != 8 || (p.cout & 31) == 0)) {
-              // (|sum| < 2^28 and |bias| <= 2^30)
+            for (int j = 0; j < 4; ++j) {
+              const int c0 = c_lo + 16 * j;
+              if (c0 >= c_hi) break;
               const int4* ef = epi.fast() + c0;
-              uint32_t bw[4] = {0u, 0u, 0u, 0u};
+              auto biased = [&](int i) { return sum[16 * j + i] + (int32_t)((uint32_t)ef[i].x + kMagicBits); };
+              if constexpr (kOStage) {  // sum + bias in whole 16-byte pieces
+                int4* yr = reinterpret_cast<int4*>(yrow) + (c0 >> 2);
 #pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const int4 c = ef[i];
-                bw[i / 4] += requant32(sum[16 * j + i] + (int32_t)((uint32_t)c.x + kMagicBits), c, qmax) << (8 * (i % 4));
-              }
-              store_codes16(yrow, ch0, bw, out_bits, top);
-              if (irow) store_image16(irow, ch0, bw, ly.ws_nib);
-            } else if (out_bits == 32 && (flags & kFlagBias) && (p.cout & 3) == 0) {
-              // int32 outputs: sum + bias in whole 16-byte pieces (likewise without saturation)
-              const int4* ef = epi.fast() + c0;
-              uint4* yr = reinterpret_cast<uint4*>(yrow) + (ch0 >> 2);
+                for (int q = 0; q < 4; ++q)
+                  if (c0 + 4 * q < c_hi) yr[q] = make_int4(biased(4 * q), biased(4 * q + 1), biased(4 * q + 2), biased(4 * q + 3));
+              } else {
+                uint32_t bw[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                auto out = [&](int i) { return (uint32_t)sum[16 * j + i] + (uint32_t)ef[i].x + kMagicBits; };
-                if (4 * q < nc) yr[q] = make_uint4(out(4 * q), out(4 * q + 1), out(4 * q + 2), out(4 * q + 3));
-              }
-            } else {
-              int32_t one[16];
-#pragma unroll
-              for (int i = 0; i < 16; ++i) one[i] = sum[16 * j + i];
-              const GenCols gc{0u, 0u, epi.gen() + c0, nullptr, yrow, ch0, nc, flags, true};
-              const uint4 r = general_sums(p, gc, one);
-              const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
-              if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0)) {
-                store_codes16(yrow, ch0, bw, out_bits, top);
-                if (irow) store_image16(irow, ch0, bw, ly.ws_nib);
+                for (int i = 0; i < 16; ++i) bw[i / 4] += requant32(biased(i), ef[i], qmax) << (8 * (i % 4));
+                store_codes16(yrow, c0, bw, out_bits, top);
+                if (irow) store_image16(irow, c0, bw, nib);
               }
             }
+          } else {
+            int32_t all[64];
+#pragma unroll
+            for (int i = 0; i < 64; ++i) all[i] = sum[i];
+            general_sums(p, GenTile{0u, 0, smem_u32(epi.gen()), c_lo, c_hi, flags, nib, nullptr, yrow, irow}, all);
           }
         }
         __syncwarp();
@@ -1151,11 +1259,12 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
       const int per = ((TBN + 31) / 32 + p.epi_groups - 1) / p.epi_groups * 32;
       const int c_lo = grp * per, c_hi = c_lo + per < TBN ? c_lo + per : TBN;
       const uint32_t tbuf = lane_base() + buf * (uint32_t)BN;
-      // The common forms; everything else goes through general_cols.
+      // The common forms; everything else goes through general_tile.
       //  codes:  the 32-bit requant of FP32 accumulators below 2^22 (or split sums), and, with a
       //          skip, the 32-bit rescale;  int32 outputs: the sum alone
       bool common;
-      if constexpr (kOStage) common = p.acc_small && (flags & kFlagBias);
+      [[maybe_unused]] const bool lean32 = p.acc_small && (flags & kFlagBias);  // int32 outputs without saturation
+      if constexpr (kOStage) common = true;
       else if constexpr (kSkip)
         common = p.acc_small && out_bits != 32 && (flags & (kFlagReq | kFlagSkip)) == (kFlagReq | kFlagSkip);
       else if constexpr (kSplit) common = out_bits != 32 && (flags & kFlagReq);
@@ -1224,22 +1333,6 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
         if (!row_ok) return;
         store_codes32(yrow, c0 - 16, first, bw, out_bits);
         if (kFlat && irow) store_image32(irow, c0 - 16, first, bw, nib);
-      };
-      auto general_tile = [&]() {
-        uint32_t top = 0u;  // (3-bit codes: see store_codes16)
-#pragma unroll 1
-        for (int c0 = c_lo; c0 < c_hi; c0 += 16) {
-          const GenCols gc{tbuf + (uint32_t)c0, tbuf + (uint32_t)(ti.cn + c0), epi.gen() + c0, srow, yrow, c0,
-                           c_hi - c0 < 16 ? c_hi - c0 : 16, flags, row_ok};
-          const uint4 r = general_cols<kSkip, kSplit>(p, gc, kAccSc);
-          __syncwarp();
-          const uint32_t bw[4] = {r.x, r.y, r.z, r.w};
-          // (general_cols stores int32 outputs and 8-bit rows of no whole groups itself)
-          if (out_bits != 32 && (out_bits != 8 || (p.cout & 31) == 0) && row_ok) {
-            store_codes16(yrow, c0, bw, out_bits, top);
-            if (kFlat && irow) store_image16(irow, c0, bw, nib);
-          }
-        }
       };
       // int32 skips may turn out to need the general form, which reads the accumulator again
       const bool late = !common || (kSkip && p.skip_bits == 32);
@@ -1329,9 +1422,15 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
             if (last) release();
             if (kOStage || out_bits == 32) {
               // int32 outputs: acc + bias
+              if (!kOStage || lean32) {
 #pragma unroll
-              for (int i = 0; i < 16; ++i)
-                v[i] = (uint32_t)(__float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + ef[i].x);
+                for (int i = 0; i < 16; ++i)
+                  v[i] = (uint32_t)(__float_as_int(__fmaf_rn(__uint_as_float(v[i]), kAccSc, kMagic)) + ef[i].x);
+              } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                  v[i] = (uint32_t)add_sat(__float2int_rn(__uint_as_float(v[i]) * kAccSc), (int32_t)((uint32_t)ef[i].x + kMagicBits));
+              }
               const int nq = (c_hi - c0 < 16 ? c_hi - c0 : 16) >> 2;  // whole 16-byte pieces (cout % 4 == 0)
               if constexpr (kOStage) {
                 // through this warp's staging block: each lane holds its row's 16 values; stored
@@ -1370,11 +1469,11 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
           }
           store16(c0, bw);
         }
-        if constexpr (kSkip) {
-          if (__any_sync(0xffffffffu, (big >> 28) != 0u)) general_tile();
-        }
-      } else {
-        general_tile();
+        if constexpr (kSkip) common = !__any_sync(0xffffffffu, (big >> 28) != 0u);
+      }
+      if (!common) {
+        const GenTile g{tbuf, ti.cn, smem_u32(epi.gen()), c_lo, c_hi, flags, nib, srow, row_ok ? yrow : nullptr, irow};
+        general_tile<kSkip, kSplit>(p, g, kAccSc);
       }
       if (late) release();
       const int tile = (int)(blockIdx.x >> 1) + (int)lt * p.tile_stride;  // (t, worked out again)
@@ -2016,8 +2115,11 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
                         : launch_bits<2, true, true, false, false, false, 128, true>(prm, maps, grid, smem, stream, err);
     }
     if (f16) {  // (no skip: the API keeps skips off the 8-bit forms)
-      if (pair) return launch_bits<8, true, true, true, false>(prm, maps, grid, smem, stream, err);
-      return launch_bits<8, true, true, false, false>(prm, maps, grid, smem, stream, err);
+      if (a.out_bits == 32)
+        return pair ? launch_bits<8, true, true, true, false, false, 128, false, true>(prm, maps, grid, smem, stream, err)
+                    : launch_bits<8, true, true, false, false, false, 128, false, true>(prm, maps, grid, smem, stream, err);
+      return pair ? launch_bits<8, true, true, true, false>(prm, maps, grid, smem, stream, err)
+                  : launch_bits<8, true, true, false, false>(prm, maps, grid, smem, stream, err);
     }
     if (a.split_w) {  // (no skip: the API keeps skips off the split form)
       if (pair) return launch_bits<2, true, true, true, false, true>(prm, maps, grid, smem, stream, err);

@@ -67,6 +67,39 @@ def test_int32_skip_at_the_limit_bit_exact(s, d, ws):
     assert_same(got, want, cout, 4, f"skip {s}, d {d}")
 
 
+# the general form: shifts below the 32-bit requant's (R = 0, 1, 31, 32), both skip directions with every d down to 0,
+# every skip width, saturating biases, int32 outputs with a skip
+# (8-bit operands with a skip run on CUDA cores)
+@pytest.mark.parametrize("xb,wb,ws,skip_bits,scale_main",
+                         [(4, 4, ws, sb, sm) for ws in (False, True) for sb in (2, 3, 4, 8, 32) for sm in (0, 1)] +
+                         [(xb, wb, ws, 0, 0) for xb, wb, ws in ((4, 4, False), (4, 4, True), (8, 8, True), (4, 8, True))])
+@pytest.mark.parametrize("out_bits", [2, 3, 4, 8, 32])
+def test_general_form_bit_exact(xb, wb, ws, skip_bits, scale_main, out_bits):
+    rng = np.random.default_rng(skip_bits + 7 * out_bits + scale_main)
+    n, h, w, cin, cout = 2, 7, 19, 128, 96
+    x = synth.act_codes(rng, (n, h, w, cin), xb)
+    wt = synth.weight_codes(rng, (cout, 1, 1, cin), wb)
+    m0 = rng.integers(1, 1 << 31, size=(1, cout), dtype=np.int64).astype(np.int32)
+    sh = rng.integers(-31, 13, size=(1, cout)).astype(np.int8)
+    sh[0, :4], m0[0, :4] = (-31, -30, 0, 1), (3, -5, I32.max, I32.min)
+    m0[0, 4::3] >>= rng.integers(0, 31, size=m0[0, 4::3].shape)
+    b = rng.integers(-3000, 3000, size=(1, cout)).astype(np.int32)
+    b[0, ::9], b[0, 1::9] = I32.max, I32.min
+    kw = {}
+    if skip_bits:
+        c = rng.integers(I32.min, I32.max, size=(1, cout), dtype=np.int64, endpoint=True).astype(np.int32)
+        c[0, 3::4] >>= 24
+        skip = rng.integers(I32.min, I32.max, size=(n, h, w, cout), dtype=np.int64, endpoint=True).astype(np.int32)
+        skip[:, ::2] >>= 16
+        d = rng.integers(0, 63, size=(1, cout)).astype(np.int8)
+        skip[0, 2, :, :2], c[0, :2], d[0, :2] = I32.min, I32.min, (0, 62)  # the largest product, 2^62
+        kw = dict(skip=skip if skip_bits == 32 else synth.act_codes(rng, (n, h, w, cout), skip_bits), skip_bits=skip_bits,
+                  skip_c=c, skip_d=d, scale_main=scale_main)
+    got, want, _ = conv_pair(x, xb, wt, wb, pad=0, out_bits=out_bits, m0=None if out_bits == 32 else m0,
+                             shift=None if out_bits == 32 else sh, bias=b, workspace=ws, **kw)
+    assert_same(got, want, cout, out_bits, f"skip {skip_bits}, out {out_bits}, scale_main {scale_main}")
+
+
 @pytest.mark.parametrize("out_bits,cout", [(8, 1), (8, 40), (8, 48), (8, 272), (8, 96), (32, 33), (32, 84), (32, 20),
                                            (32, 258)])
 @pytest.mark.parametrize("skip", [False, True])
