@@ -368,8 +368,6 @@ __device__ __forceinline__ ColConst col_const(uint32_t addr) {
 }
 static_assert(sizeof(EpiChan) == 16 && offsetof(EpiChan, r) == 12 && offsetof(EpiChan, d) == 13, "col_const");
 
-// rhu in one variable shift: floor((v + 2^(r-1)) / 2^r) = floor((floor(v / 2^(r-1)) + 1) / 2)
-__device__ __forceinline__ int64_t rhu1(int64_t v, int r) { return r > 0 ? ((v >> (r - 1)) + 1) >> 1 : v; }
 __device__ __forceinline__ int32_t sat_s32(int64_t v) { return (int32_t)sat32(v); }
 
 // The row's skip values of nc columns from channel ch on.
@@ -424,10 +422,7 @@ __device__ __forceinline__ uint4 general_finish(const Params& p, uint32_t ep, co
   const int out_bits = p.out_bits;
   const int32_t qmax = (1 << (out_bits & 15)) - 1;
   const auto at = [ep](int i) { return ep + (uint32_t)(i * sizeof(EpiChan)); };
-  auto requant = [qmax](int32_t u, const ColConst& k) {
-    const int64_t v = rhu1((int64_t)u * k.m0, k.r);
-    return v < 0 ? 0 : (v > qmax ? qmax : (int32_t)v);
-  };
+  auto requant = [qmax](int32_t u, const ColConst& k) { return requant64(u, k.m0, k.r, qmax); };
   if constexpr (kSkip) {
     int32_t sk[16];
     general_skip(p, srow, ch, nc, sk);

@@ -17,6 +17,13 @@ __device__ __forceinline__ uint32_t requant32(int32_t u, const int4& f, int qmax
   return (uint32_t)__vimin_s32_relu((__mulhi(u, f.y) + f.z) >> f.w, qmax);
 }
 
+// The same for any R: rhu in one variable shift, floor((v + 2^(r-1)) / 2^r) = floor((floor(v / 2^(r-1)) + 1) / 2)
+__device__ __forceinline__ int64_t rhu1(int64_t v, int r) { return r > 0 ? ((v >> (r - 1)) + 1) >> 1 : v; }
+__device__ __forceinline__ int32_t requant64(int32_t u, int32_t m0, int r, int32_t qmax) {
+  const int64_t v = rhu1((int64_t)u * m0, r);
+  return v < 0 ? 0 : (v > qmax ? qmax : (int32_t)v);
+}
+
 // 16 codes < 2^bits as byte-words (word j: channels 4j..4j+3, one per byte) -> their place in the
 // packed row (the layout of common.cuh: word w of the 2/4/8-bit layout holds its channels 4k..4k+3
 // in bit field k of every byte; a 3-bit group of 32 channels is two 2-bit words of the low bits
@@ -46,6 +53,11 @@ __device__ __forceinline__ void store_codes16(uint8_t* yrow, int ch, const uint3
 __device__ __forceinline__ void store_sector(uint8_t* p, const uint32_t (&a)[4], const uint32_t (&b)[4]) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a[0]), "r"(a[1]), "r"(a[2]),
                "r"(a[3]), "r"(b[0]), "r"(b[1]), "r"(b[2]), "r"(b[3])
+               : "memory");
+}
+__device__ __forceinline__ void store_words8(uint8_t* p, const uint32_t* w) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+               "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
                : "memory");
 }
 // A whole 32-channel group: the byte-words of its halves to their place in the packed row (see

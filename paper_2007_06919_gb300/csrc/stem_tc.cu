@@ -164,8 +164,7 @@ __device__ __forceinline__ void build_half(const StemParams& p, int mg, uint8_t*
     *reinterpret_cast<uint4*>(row_dst + (R0 * kLs / 8 + c) * kLBO) = make_uint4(o[4 * c], o[4 * c + 1], o[4 * c + 2], o[4 * c + 3]);
 }
 
-// Eq. 6 -> Eq. 2 of 16 columns in int64, as the definition states them (some R < 33): byte-words of
-// the codes. Not inlined: its registers and code stay out of the common form.
+// Eq. 6 -> Eq. 2 of 16 columns as the definition states them (some R < 33): byte-words of the codes. Not inlined: its registers and code stay out of the common form.
 __device__ __noinline__ uint4 general_cols(uint32_t taddr, const EpiChan* c, int out_bits) {
   uint32_t v[16];
   tmem_ld16(taddr, v);
@@ -174,7 +173,8 @@ __device__ __noinline__ uint4 general_cols(uint32_t taddr, const EpiChan* c, int
   uint32_t bw[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
   for (int i = 0; i < 16; ++i)
-    bw[i / 4] |= (uint32_t)epilogue<false>((int64_t)__float2int_rn(__uint_as_float(v[i])), 0, c[i], 0, out_bits) << (8 * (i % 4));
+    bw[i / 4] |= (uint32_t)requant64(add_sat(__float2int_rn(__uint_as_float(v[i])), c[i].bias), c[i].m0, c[i].r,
+                                     (1 << out_bits) - 1) << (8 * (i % 4));
   return make_uint4(bw[0], bw[1], bw[2], bw[3]);
 }
 
@@ -198,8 +198,8 @@ constexpr float kMagic = 12582912.0f;
 constexpr uint32_t kMagicBits = 0x4B400000u;
 
 // Per-channel constants of the launch's level: {bias - kMagicBits, M0, 2^(R-33), R-32} and the int64
-// form. The 32-bit form holds (and 1 stays in *s_fast) where every R >= 33, |bias| <= 2^30, and
-// every |sum| < 2^22 (weights_small).
+// form. The 32-bit form holds (and 1 stays in *s_fast) where every R >= 33 (code outputs), |bias| <= 2^30, and
+// every |sum| < 2^22 (weights_small); int32 outputs then need no saturation either.
 __device__ __forceinline__ void load_channels(const StemParams& p, int4* cst4, EpiChan* cste, int* s_fast) {
   int fast = 1;
   for (int n = threadIdx.x; n < p.n_pad; n += blockDim.x) {
@@ -208,12 +208,13 @@ __device__ __forceinline__ void load_channels(const StemParams& p, int4* cst4, E
     if (n < p.cout) {
       const int64_t idx = (int64_t)p.level * p.cout + n;
       ec.bias = p.bias ? p.bias[idx] : 0;
+      if (ec.bias < -(1 << 30) || ec.bias > (1 << 30)) fast = 0;
+      c4.x = (int)((uint32_t)ec.bias - kMagicBits);
       if (p.out_bits != 32) {
         ec.m0 = p.m0[idx];
         const int r = 31 + p.shift[idx];
         ec.r = (int8_t)r;
-        if (r >= 33 && ec.bias >= -(1 << 30) && ec.bias <= (1 << 30))
-          c4 = make_int4((int)((uint32_t)ec.bias - kMagicBits), ec.m0, 1 << (r - 33), r - 32);
+        if (r >= 33) c4 = make_int4(c4.x, ec.m0, 1 << (r - 33), r - 32);
         else fast = 0;
       }
     }
@@ -232,13 +233,15 @@ __device__ __forceinline__ bool weights_small(uint32_t part) { return __reduce_a
 // kTiles accumulators' columns of one output pixel each: the 32-column groups 0, 2, .. (odd = 0)
 // or 1, 3, .. (odd = 1), 16 columns at a time (cout is a multiple of 16). Constants are read from
 // shared memory once for all tiles; release() hands the accumulators back after the last read.
-template <int kTiles, class Release>
+// kInt: int32 outputs (an instantiation of its own: beside the codes' form in one loop, codes took 2 to 9% longer).
+template <int kTiles, bool kInt, class Release>
 __device__ __forceinline__ void drain_pixels(const StemParams& p, const uint32_t (&tbase)[kTiles], uint8_t* const (&yrow)[kTiles],
                                              const bool (&valid)[kTiles], int odd, bool fast, const int4* cst4,
                                              const EpiChan* cste, Release&& release) {
   const int qmax = (1 << (p.out_bits & 15)) - 1;
   uint32_t top[kTiles] = {};  // (3-bit codes: see store_codes16)
-  if (fast && p.out_bits != 32) {
+  [[maybe_unused]] const bool sectors = (reinterpret_cast<uintptr_t>(p.y) & 31) == 0;  // (int32 rows are multiples of 64 bytes)
+  if (fast) {
     if (32 * odd >= p.cout) release();
 #pragma unroll 1
     for (int c0 = 32 * odd, next; c0 < p.cout; c0 = next) {
@@ -250,16 +253,36 @@ __device__ __forceinline__ void drain_pixels(const StemParams& p, const uint32_t
 #pragma unroll
       for (int k = 0; k < kTiles; ++k) reg_fence16(v[k]);
       if (next >= p.cout) release();
+      if constexpr (kInt) {
+        // (a tile's row at a time, whole sectors where the rows allow it: the two tiles' 16-byte pieces in turn
+        // left half-written sectors behind, 256 channels of 4 x 240 x 320 outputs 230 us against 112)
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int4 c = cst4[c0 + i];
+        for (int k = 0; k < kTiles; ++k) {
+#pragma unroll
+          for (int i = 0; i < 16; ++i) v[k][i] = (uint32_t)(__float_as_int(__uint_as_float(v[k][i]) + kMagic) + cst4[c0 + i].x);
+          if (!valid[k]) continue;
+          uint8_t* row = yrow[k] + 4 * c0;
+          if (sectors) {
+            store_words8(row, &v[k][0]);
+            store_words8(row + 32, &v[k][8]);
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              reinterpret_cast<uint4*>(row)[q] = make_uint4(v[k][4 * q], v[k][4 * q + 1], v[k][4 * q + 2], v[k][4 * q + 3]);
+          }
+        }
+      } else {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int4 c = cst4[c0 + i];
+#pragma unroll
+          for (int k = 0; k < kTiles; ++k)
+            bw[k][i / 4] += requant32(__float_as_int(__uint_as_float(v[k][i]) + kMagic) + c.x, c, qmax) << (8 * (i % 4));
+        }
 #pragma unroll
         for (int k = 0; k < kTiles; ++k)
-          bw[k][i / 4] += requant32(__float_as_int(__uint_as_float(v[k][i]) + kMagic) + c.x, c, qmax) << (8 * (i % 4));
+          if (valid[k]) store_codes16(yrow[k], c0, bw[k], p.out_bits, top[k]);
       }
-#pragma unroll
-      for (int k = 0; k < kTiles; ++k)
-        if (valid[k]) store_codes16(yrow[k], c0, bw[k], p.out_bits, top[k]);
     }
     return;
   }
@@ -267,7 +290,7 @@ __device__ __forceinline__ void drain_pixels(const StemParams& p, const uint32_t
   for (int k = 0; k < kTiles; ++k) {
 #pragma unroll 1
     for (int c0 = 32 * odd; c0 < p.cout; c0 += (c0 & 16) ? 48 : 16) {
-      if (p.out_bits == 32) {
+      if constexpr (kInt) {
         sums_int32(tbase[k] + (uint32_t)c0, cste + c0, reinterpret_cast<uint4*>(yrow[k]) + (c0 >> 2), valid[k]);
       } else {
         const uint4 r = general_cols(tbase[k] + (uint32_t)c0, cste + c0, p.out_bits);
@@ -280,6 +303,7 @@ __device__ __forceinline__ void drain_pixels(const StemParams& p, const uint32_t
   release();
 }
 
+template <bool kInt>
 __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant__ StemParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -326,25 +350,30 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
   grid_dep_wait();
   if (threadIdx.x == 0) grid_dep_launch();
 
-  // weights -> F16 B operand (n_pad rows x 160, core-matrix layout); per-channel constants
-  for (int e = threadIdx.x; e < p.n_pad * (kK / 2); e += blockDim.x) {
-    const int n = e / (kK / 2), kk = 2 * (e - n * (kK / 2));
-    uint32_t pr = 0u;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = (kk + h) / kLs, j = (kk + h) - r * kLs;
-      uint16_t wv = 0;  // (F16 zero)
-      if (n < p.cout && r < kKH && j < kSeg) wv = p.w_f16[(int64_t)n * (kKH * kSeg) + r * kSeg + j];
-      pr |= (uint32_t)wv << (16 * h);
-    }
-    *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) = pr;
-  }
-  load_channels(p, cst4, cste, s_fast);
-  for (int n = warp; n < p.cout; n += kThreads / 32) {
+  // weights -> F16 B operand (n_pad rows x 160, core-matrix layout), a warp per channel with all its loads
+  // issued together (element by element over the block, and the sums of |w| in a pass of their own, a call of 256
+  // channels and 32 x 32 outputs took 30 us, now 16)
+#pragma unroll 2
+  for (int n = warp; n < p.n_pad; n += kThreads / 32) {
     uint32_t part = 0;
-    for (int k = lane; k < kKH * kSeg; k += 32) part += abs_f16(p.w_f16[(int64_t)n * (kKH * kSeg) + k]);
+#pragma unroll
+    for (int q = 0; q < (kK / 2 + 31) / 32; ++q) {
+      const int kk = 2 * (lane + 32 * q);  // (kLs is even: a pair lies in one kernel row)
+      const int r = kk / kLs, j = kk - r * kLs;
+      uint16_t w0 = 0, w1 = 0;  // (F16 zero)
+      if (n < p.cout && r < kKH) {
+        const uint16_t* w = p.w_f16 + (int64_t)n * (kKH * kSeg) + r * kSeg + j;
+        w0 = w[0];
+        if (j + 1 < kSeg) w1 = w[1];
+      }
+      part += abs_f16(w0) + abs_f16(w1);
+      if (kk < kK)
+        *reinterpret_cast<uint32_t*>(smem + p.off_b + (n / 8) * kSBO + (kk / 8) * kLBO + (n % 8) * 16 + (kk % 8) * 2) =
+            (uint32_t)w0 | ((uint32_t)w1 << 16);
+    }
     if (!weights_small(part) && lane == 0) atomicAnd(s_fast, 0);
   }
+  load_channels(p, cst4, cste, s_fast);
   fence_proxy_async();  // generic-proxy stores of B -> visible to the MMA
   __syncthreads();
   const bool fast = *s_fast != 0;
@@ -410,7 +439,7 @@ __global__ void __launch_bounds__(kThreads, 1) stem_kernel(const __grid_constant
       const uint32_t tbase[1] = {lane_base + buf * (uint32_t)p.n_pad};
       uint8_t* const yrows[1] = {yrow};
       const bool valids[1] = {valid};
-      drain_pixels<1>(p, tbase, yrows, valids, warp >> 2, fast, cst4, cste, [&] {
+      drain_pixels<1, kInt>(p, tbase, yrows, valids, warp >> 2, fast, cst4, cste, [&] {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_relaxed(b_tempty + 8 * buf);
@@ -531,6 +560,7 @@ __device__ __forceinline__ uint64_t sdesc_offsets(uint32_t saddr, int lbo, int s
   return d;
 }
 
+template <bool kInt>
 __global__ void __launch_bounds__(kRThreads, 1) stem_rows_kernel(const __grid_constant__ StemParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -701,7 +731,7 @@ __global__ void __launch_bounds__(kRThreads, 1) stem_rows_kernel(const __grid_co
           (two && !mbar_wait(b_tfull + 8 * b1, ((lt + 1) >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
       tc_fence_after();
       const uint32_t tbase[2] = {lane_base + b0 * (uint32_t)p.n_pad, lane_base + b1 * (uint32_t)p.n_pad};
-      drain_pixels<2>(p, tbase, yrow, valid, warp >> 2, fast, cst4, cste, [&] {
+      drain_pixels<2, kInt>(p, tbase, yrow, valid, warp >> 2, fast, cst4, cste, [&] {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
@@ -785,12 +815,13 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   if ((int)total > max_smem) { *err = "stem conv: shared memory too small"; return 2; }
   p.tmem_cols = 32;
   while (p.tmem_cols < (p.n_pad << p.nbuf_log2)) p.tmem_cols *= 2;
+  const auto kern = rows ? (a.out_bits == 32 ? stem_rows_kernel<true> : stem_rows_kernel<false>)
+                         : (a.out_bits == 32 ? stem_kernel<true> : stem_kernel<false>);
   static std::once_flag attr_once;
   static cudaError_t attr_err = cudaSuccess;
   std::call_once(attr_once, [&] {
-    attr_err = cudaFuncSetAttribute(stem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-    if (attr_err == cudaSuccess)
-      attr_err = cudaFuncSetAttribute(stem_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    for (auto k : {stem_rows_kernel<true>, stem_rows_kernel<false>, stem_kernel<true>, stem_kernel<false>})
+      if (attr_err == cudaSuccess) attr_err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
   });
   if (attr_err != cudaSuccess) {
     *err = std::string("stem conv: shared-memory attribute: ") + cudaGetErrorString(attr_err);
@@ -807,7 +838,7 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, rows ? stem_rows_kernel : stem_kernel, p);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, p);
   if (e != cudaSuccess) {
     *err = std::string("stem conv launch: ") + cudaGetErrorString(e);
     return 3;

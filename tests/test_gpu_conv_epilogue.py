@@ -4,6 +4,7 @@ counts that leave warps idle or let sets of warps take tiles in turn, and accumu
 large for the common form."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2007_06919_gb300 import aqd, synth
@@ -280,6 +281,30 @@ def test_first_conv_rows_bit_exact(shape, pad, cout, out_bits):
                                 shift=None if out_bits == 32 else sh, bias=b)
     assert used == 5
     assert_same(got, want, cout, out_bits, f"first conv {shape}")
+
+
+# its int32 outputs: whole sectors or, at an address of 16 bytes, 16-byte pieces; sums or biases beyond the lean form
+@pytest.mark.parametrize("stride,cout", [(1, 16), (1, 96), (2, 64), (2, 256)])
+@pytest.mark.parametrize("offset", [0, 16])
+@pytest.mark.parametrize("wide", ["", "weights", "bias"])
+def test_first_conv_int32_outputs_bit_exact(stride, cout, offset, wide):
+    rng = np.random.default_rng(stride + cout)
+    x = synth.act_codes(rng, (2, 37, 141, 3), 8)
+    lim = 128 if wide == "weights" else 8
+    wt = rng.integers(-lim, lim, size=(cout, 7, 7, 3)).astype(np.int32)
+    x[0, :9, :9], wt[0] = 255, -lim
+    b = rng.integers(-1000, 1000, size=(1, cout)).astype(np.int32)
+    if wide == "bias":
+        b[0, 1], b[0, cout - 1] = I32.max, I32.min
+    W, wp = weights(wt, 8)
+    xt = oracle.CodeTensor.from_codes(x, 8)
+    want = oracle.conv_int(xt, wp, 8, 0, 7, 7, stride, 3, cout, bias=b, out_bits=32)
+    buf = torch.full((want.packed.size + 32,), 0xA5, dtype=torch.uint8, device="cuda")
+    y = aqd.DTensor(buf[offset:offset + want.packed.size], want.n, want.h, want.w, cout, 32)
+    aqd.conv_int(to_device(xt), W, stride, 3, y, rq=aqd.RequantParams.from_numpy(None, None, b))
+    assert aqd.last_conv_path() == 5 and aqd.device_status() == 0
+    assert_same(y.data.cpu().numpy().reshape(want.packed.shape), want.packed, cout, 32, f"stride {stride}, {wide}")
+    assert bool((buf[:offset] == 0xA5).all()) and bool((buf[offset + want.packed.size:] == 0xA5).all())
 
 
 # the in-kernel unpack's two threads per row: K tails of 1 to 4 groups of 32 (whole and empty second halves), chunks
