@@ -1387,10 +1387,20 @@ static bool launch_staged_v(const EltArgs& a, int ts, int sms, cudaStream_t stre
     default: return false;
   }
 }
+// Words from one code to the next of the staged kernel's skip table (at most 48 KB), 0 for none.
+static int table_stride(const EltArgs& a) {
+  const int ts = (a.c + a.c / 32 + 31) / 32 * 32;
+  return a.scale_main == 0 && ((size_t)ts << a.b_bits) * sizeof(int32_t) <= 48 * 1024 ? ts : 0;
+}
 // Whether the staged kernel takes these arguments: contiguous int32 rows (and 2/4/8-bit skip rows;
 // on the same grid whole 16-byte rows) at 16-byte aligned addresses, and a channel-block count
-// that divides the 8 consumer warps.
-static bool staged_applies(const EltArgs& a) {
+// that divides the 8 consumer warps. With a skip on another grid also enough stages of 32 KB for the
+// SMs: a block takes a stage's time at least, while the lane kernel spreads small maps over the chip.
+// Without the skip table (8-bit codes, scale_main, wide rows) a stage takes 9 us (256 channels) to 20 (32).
+// Measured, lane / staged in us, codes out: with a table 32 channels 17 / 7 at 262 stages, 11.5 / 8.6 at
+// 131, 128 channels 6.8 / 4.9 at 66, 256 channels 5.9 / 5.1 at 32 and 4.7 / 4.9 at 8; without one 32 channels
+// 30.5 / 25.8 at 262 and 17.6 / 19.5 at 131, 128 channels 10.2 / 12.5 at 66, 256 channels 6.1 / 12.1 at 8.
+static bool staged_applies(const EltArgs& a, int sms) {
   if (a.a_bits != 32 || a.c % 32 != 0 || a.a_row_bytes != (int64_t)a.c * 4 || a.y_bits == 3) return false;
   if ((uintptr_t)a.a % 16 != 0) return false;
   const int v = a.c % 128 == 0 ? 4 : (a.c % 64 == 0 ? 2 : 1);
@@ -1399,17 +1409,17 @@ static bool staged_applies(const EltArgs& a) {
   if (a.has_skip) {
     if (a.b_bits != 2 && a.b_bits != 4 && a.b_bits != 8) return false;
     // (another grid: word loads, and pixels counted in 31 bits, as the API checks)
-    if (same_grid(a) && (a.b_row_bytes % 16 != 0 || (uintptr_t)a.b % 16 != 0)) return false;
+    if (same_grid(a)) return a.b_row_bytes % 16 == 0 && (uintptr_t)a.b % 16 == 0;
+    const int64_t stages = (int64_t)a.n * a.h * a.w * a.c * 4 / 32768;
+    const int need = table_stride(a) > 0 ? (a.c >= 128 ? sms / 6 : (a.c >= 64 || a.y_bits == 32 ? sms / 4 : sms / 2))
+                                         : (a.c >= 128 ? sms * 3 / 4 : sms * 3 / 2);
+    if (stages < need) return false;
   }
   return true;
 }
 template <bool kSkip, int kSkipBits>
 static bool launch_staged(const EltArgs& a, int sms, cudaStream_t stream) {
-  int ts = 0;
-  if (kSkip && a.scale_main == 0) {
-    ts = (a.c + a.c / 32 + 31) / 32 * 32;
-    if (((size_t)ts << kSkipBits) * sizeof(int32_t) > 48 * 1024) ts = 0;
-  }
+  const int ts = kSkip ? table_stride(a) : 0;
   const int v = a.c % 128 == 0 ? 4 : (a.c % 64 == 0 ? 2 : 1);
   if (kSkip && !same_grid(a)) {
     if (v == 4) return launch_staged_v<kSkip, kSkipBits, 4, kSkip>(a, ts, sms, stream);
@@ -1432,7 +1442,7 @@ int launch_elementwise(const EltArgs& a, cudaStream_t stream, std::string* err) 
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 152;
     bool ok = false;
-    if (staged_applies(a)) {
+    if (staged_applies(a, sms)) {
       if (!a.has_skip) ok = launch_staged<false, 0>(a, sms, stream);
       else if (a.b_bits == 2) ok = launch_staged<true, 2>(a, sms, stream);
       else if (a.b_bits == 4) ok = launch_staged<true, 4>(a, sms, stream);

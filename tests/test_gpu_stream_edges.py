@@ -45,6 +45,20 @@ def test_pack_unpack_runs(bits, rows, c, offset):
 @pytest.mark.parametrize("shape", [(1, 1, 1), (2, 7, 11), (3, 37, 53)])
 @pytest.mark.parametrize("grid,wide", [("up", False), ("larger", False), ("up", True)])
 def test_skip_on_another_grid(c, b_bits, shape, grid, wide):
+    check_skip_on_another_grid(c, b_bits, shape, grid, wide)
+
+
+# maps on either side of the sizes from which the staged kernel takes them
+@pytest.mark.parametrize("c,shape", [(32, (1, 83, 127)), (32, (3, 97, 131)), (32, (5, 97, 131)), (64, (1, 83, 127)),
+                                     (64, (3, 97, 131)), (128, (1, 41, 127)), (128, (1, 83, 127)), (256, (1, 41, 67)),
+                                     (256, (1, 83, 127))])
+@pytest.mark.parametrize("b_bits", [2, 4, 8])
+@pytest.mark.parametrize("grid,wide", [("up", False), ("larger", False), ("up", True)])
+def test_skip_on_another_grid_of_larger_maps(c, b_bits, shape, grid, wide):
+    check_skip_on_another_grid(c, b_bits, shape, grid, wide)
+
+
+def check_skip_on_another_grid(c, b_bits, shape, grid, wide):
     n, h, w = shape
     rng = np.random.default_rng(c + b_bits + h)
     up = 2 if grid == "up" else 1
