@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -73,38 +74,73 @@ __device__ __forceinline__ float quant_one(float x, const Quant& k, uint32_t& et
   }
 }
 
-// Streaming passes, bound by HBM. Each thread takes kUnroll vectors a grid apart per step with all
-// their loads issued first: one vector per step left too few bytes in flight. Measured on
-// 16x100x168x256 values: forward 113 -> 91 us (9 bytes a value), backward 240 -> 120 us (12).
-constexpr int kUnroll = 4;
+// Streaming passes, bound by HBM. Each thread takes kUnroll units a grid apart per step with all their
+// loads issued first: one at a time left too few bytes in flight. A unit is four values, or one where
+// an address is not a multiple of 16. Measured on 16x100x168x256 values: forward 113 -> 91 us (9 bytes a
+// value), backward 240 -> 120 us (12), backward at odd addresses 387 -> 170.
+// kStream: evict-first accesses, for tensors larger than L2 together (33M values 50.5 -> 49.4 us); smaller
+// ones are left for what reads them next (8M values read and written again from L2 11.7 -> 9.8).
+template <int kVec>
+struct Unit;
+template <>
+struct Unit<4> {
+  using F = float4;
+  using C = uint32_t;
+  static constexpr int kUnroll = 4;
+};
+template <>
+struct Unit<1> {
+  using F = float;
+  using C = uint8_t;
+  static constexpr int kUnroll = 8;
+};
+template <bool kStream, class T>
+__device__ __forceinline__ T load(const T* p) {
+  if constexpr (kStream) return __ldcs(p);
+  else return __ldg(p);
+}
+template <bool kStream, class T>
+__device__ __forceinline__ void store(T* p, T v) {
+  if constexpr (kStream) __stcs(p, v);
+  else *p = v;
+}
 
-template <bool kWeight, bool kKnown, int kVec>
+template <bool kWeight, bool kKnown>
+__device__ __forceinline__ float quant_unit(float v, const Quant& k, uint8_t& code) {
+  uint32_t e;
+  const float o = quant_one<kWeight, kKnown>(v, k, e);
+  code = (uint8_t)e;
+  return o;
+}
+template <bool kWeight, bool kKnown>
+__device__ __forceinline__ float4 quant_unit(const float4& v, const Quant& k, uint32_t& codes) {
+  uint32_t e0, e1, e2, e3;
+  const float4 o = make_float4(quant_one<kWeight, kKnown>(v.x, k, e0), quant_one<kWeight, kKnown>(v.y, k, e1),
+                               quant_one<kWeight, kKnown>(v.z, k, e2), quant_one<kWeight, kKnown>(v.w, k, e3));
+  codes = e0 | (e1 << 8) | (e2 << 16) | (e3 << 24);
+  return o;
+}
+
+template <bool kWeight, bool kKnown, int kVec, bool kStream>
 __global__ void __launch_bounds__(kThreads) fake_quant_kernel(const float* __restrict__ x, int64_t n, const Quant k,
                                                               float* __restrict__ y, uint8_t* __restrict__ codes) {
+  using F = typename Unit<kVec>::F;
+  using C = typename Unit<kVec>::C;
+  constexpr int kUnroll = Unit<kVec>::kUnroll;
   const int64_t units = n / kVec, step = (int64_t)gridDim.x * kThreads;
-  if constexpr (kVec == 4) {
-    for (int64_t u0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; u0 < units; u0 += step * kUnroll) {
-      float4 v[kUnroll];
+  for (int64_t u0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; u0 < units; u0 += step * kUnroll) {
+    F v[kUnroll];
 #pragma unroll
-      for (int j = 0; j < kUnroll; ++j)
-        if (u0 + j * step < units) v[j] = __ldcs(reinterpret_cast<const float4*>(x) + u0 + j * step);
+    for (int j = 0; j < kUnroll; ++j)
+      if (u0 + j * step < units) v[j] = load<kStream>(reinterpret_cast<const F*>(x) + u0 + j * step);
 #pragma unroll
-      for (int j = 0; j < kUnroll; ++j) {
-        const int64_t u = u0 + j * step;
-        if (u >= units) break;
-        uint32_t e0, e1, e2, e3;
-        const float4 o = make_float4(quant_one<kWeight, kKnown>(v[j].x, k, e0), quant_one<kWeight, kKnown>(v[j].y, k, e1),
-                                     quant_one<kWeight, kKnown>(v[j].z, k, e2), quant_one<kWeight, kKnown>(v[j].w, k, e3));
-        if (y) __stcs(reinterpret_cast<float4*>(y) + u, o);
-        if (codes) __stcs(reinterpret_cast<uint32_t*>(codes) + u, e0 | (e1 << 8) | (e2 << 16) | (e3 << 24));
-      }
-    }
-  } else {
-    for (int64_t u = (int64_t)blockIdx.x * kThreads + threadIdx.x; u < units; u += step) {
-      uint32_t e;
-      const float o = quant_one<kWeight, kKnown>(__ldg(x + u), k, e);
-      if (y) y[u] = o;
-      if (codes) codes[u] = (uint8_t)e;
+    for (int j = 0; j < kUnroll; ++j) {
+      const int64_t u = u0 + j * step;
+      if (u >= units) break;
+      C c;
+      const F o = quant_unit<kWeight, kKnown>(v[j], k, c);
+      if (y) store<kStream>(reinterpret_cast<F*>(y) + u, o);
+      if (codes) store<kStream>(reinterpret_cast<C*>(codes) + u, c);
     }
   }
   // the tail past the last whole vector (kVec = 4: at most 3 elements), by block 0
@@ -139,51 +175,55 @@ __device__ __forceinline__ float dquant_one(float x, float gy, const Quant& k, f
   return inside ? gy : 0.0f;
 }
 
-// gx (STE) and one float64 partial of sum(gy * dy/dnu) per block: float32 over runs of 16 vectors
+template <bool kWeight, bool kKnown>
+__device__ __forceinline__ float dquant_unit(float x, float g, const Quant& k, float& acc) {
+  float d;
+  const float o = dquant_one<kWeight, kKnown>(x, g, k, d);
+  acc = __fadd_rn(acc, __fmul_rn(g, d));
+  return o;
+}
+template <bool kWeight, bool kKnown>
+__device__ __forceinline__ float4 dquant_unit(const float4& x, const float4& g, const Quant& k, float& acc) {
+  float d0, d1, d2, d3;
+  const float4 o = make_float4(dquant_one<kWeight, kKnown>(x.x, g.x, k, d0), dquant_one<kWeight, kKnown>(x.y, g.y, k, d1),
+                               dquant_one<kWeight, kKnown>(x.z, g.z, k, d2), dquant_one<kWeight, kKnown>(x.w, g.w, k, d3));
+  acc = __fadd_rn(acc, __fadd_rn(__fadd_rn(__fmul_rn(g.x, d0), __fmul_rn(g.y, d1)),
+                                 __fadd_rn(__fmul_rn(g.z, d2), __fmul_rn(g.w, d3))));
+  return o;
+}
+
+// gx (STE) and one float64 partial of sum(gy * dy/dnu) per block: float32 over runs of 16 units
 // of a thread, float64 across runs and threads.
-template <bool kWeight, bool kKnown, int kVec>
+template <bool kWeight, bool kKnown, int kVec, bool kStream>
 __global__ void __launch_bounds__(kThreads) fake_quant_backward_kernel(const float* __restrict__ x,
                                                                        const float* __restrict__ gy, int64_t n,
                                                                        const Quant k, float* __restrict__ gx,
                                                                        double* __restrict__ partial) {
+  using F = typename Unit<kVec>::F;
+  constexpr int kUnroll = Unit<kVec>::kUnroll;
+  static_assert(16 % kUnroll == 0, "a run is whole steps");
   __shared__ double red[kThreads / 32];
   float acc = 0.0f;
   double accd = 0.0;
   int run = 0;
   const int64_t units = n / kVec, step = (int64_t)gridDim.x * kThreads;
-  if constexpr (kVec == 4) {
-    for (int64_t u0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; u0 < units; u0 += step * kUnroll) {
-      float4 xv[kUnroll], gv[kUnroll];
+  for (int64_t u0 = (int64_t)blockIdx.x * kThreads + threadIdx.x; u0 < units; u0 += step * kUnroll) {
+    F xv[kUnroll], gv[kUnroll];
 #pragma unroll
-      for (int j = 0; j < kUnroll; ++j) {
-        if (u0 + j * step >= units) break;
-        xv[j] = __ldcs(reinterpret_cast<const float4*>(x) + u0 + j * step);
-        gv[j] = __ldcs(reinterpret_cast<const float4*>(gy) + u0 + j * step);
-      }
+    for (int j = 0; j < kUnroll; ++j) {
+      if (u0 + j * step >= units) break;
+      xv[j] = load<kStream>(reinterpret_cast<const F*>(x) + u0 + j * step);
+      gv[j] = load<kStream>(reinterpret_cast<const F*>(gy) + u0 + j * step);
+    }
 #pragma unroll
-      for (int j = 0; j < kUnroll; ++j) {
-        const int64_t u = u0 + j * step;
-        if (u >= units) break;
-        float d0, d1, d2, d3;
-        const float4 g = gv[j];
-        const float4 o = make_float4(dquant_one<kWeight, kKnown>(xv[j].x, g.x, k, d0), dquant_one<kWeight, kKnown>(xv[j].y, g.y, k, d1),
-                                     dquant_one<kWeight, kKnown>(xv[j].z, g.z, k, d2), dquant_one<kWeight, kKnown>(xv[j].w, g.w, k, d3));
-        if (gx) __stcs(reinterpret_cast<float4*>(gx) + u, o);
-        acc = __fadd_rn(acc, __fadd_rn(__fadd_rn(__fmul_rn(g.x, d0), __fmul_rn(g.y, d1)),
-                                       __fadd_rn(__fmul_rn(g.z, d2), __fmul_rn(g.w, d3))));
-      }
-      run += kUnroll;
-      if (run == 16) { accd += (double)acc; acc = 0.0f; run = 0; }
+    for (int j = 0; j < kUnroll; ++j) {
+      const int64_t u = u0 + j * step;
+      if (u >= units) break;
+      const F o = dquant_unit<kWeight, kKnown>(xv[j], gv[j], k, acc);
+      if (gx) store<kStream>(reinterpret_cast<F*>(gx) + u, o);
     }
-  } else {
-    for (int64_t u = (int64_t)blockIdx.x * kThreads + threadIdx.x; u < units; u += step) {
-      float d0;
-      const float g = __ldg(gy + u);
-      const float o = dquant_one<kWeight, kKnown>(__ldg(x + u), g, k, d0);
-      if (gx) gx[u] = o;
-      acc = __fadd_rn(acc, __fmul_rn(g, d0));
-      if (++run == 16) { accd += (double)acc; acc = 0.0f; run = 0; }
-    }
+    run += kUnroll;
+    if (run == 16) { accd += (double)acc; acc = 0.0f; run = 0; }
   }
   if (kVec > 1 && blockIdx.x == 0 && threadIdx.x < n - units * kVec) {
     const int64_t i = units * kVec + threadIdx.x;
@@ -390,9 +430,26 @@ inline Quant quant_of(float nu, int32_t bits) {
 // the intervals div_known takes (anything a trained network has); others use the division itself
 inline bool known_divisor(float nu) { return nu >= 0x1p-20f && nu <= 0x1p20f; }
 
-inline unsigned grid_for(int64_t units, int cap) {
-  const int64_t b = (units + kThreads - 1) / kThreads;
+// Blocks for a pass over n values: a step of kUnroll units per thread, but two blocks per SM before a thread
+// takes more than one (65,536 values forward in 16 blocks took 2.7 us, in 64 2.0); at most cap.
+template <int kVec>
+inline unsigned grid_for(int64_t n, int sms, int cap) {
+  const int64_t units = n / kVec, per = kThreads * Unit<kVec>::kUnroll;
+  const int64_t one = (units + kThreads - 1) / kThreads, full = (units + per - 1) / per;
+  int64_t b = one < 2 * sms ? one : 2 * sms;
+  if (full > b) b = full;
   return (unsigned)(b < 1 ? 1 : (b > cap ? cap : b));
+}
+// Tensors that leave L2 (129 MB) anyway
+inline bool stream_size(int64_t bytes) { return bytes > (int64_t)128 << 20; }
+
+// go(weight, known divisor, values per unit) with the choice as types
+template <class Go>
+void dispatch(bool weight, bool known, bool v4, Go&& go) {
+  using std::integral_constant;
+  auto vec = [&](auto w, auto kn) { v4 ? go(w, kn, integral_constant<int, 4>{}) : go(w, kn, integral_constant<int, 1>{}); };
+  auto kn = [&](auto w) { known ? vec(w, std::true_type{}) : vec(w, std::false_type{}); };
+  weight ? kn(std::true_type{}) : kn(std::false_type{});
 }
 
 }  // namespace trn
@@ -412,16 +469,14 @@ int launch_fake_quant(const float* x, int64_t n, float nu, int32_t bits, bool we
   const trn::Quant k = trn::quant_of(nu, bits);
   const bool known = trn::known_divisor(nu);
   const bool v4 = ((uintptr_t)x % 16 == 0) && ((uintptr_t)y % 16 == 0) && ((uintptr_t)codes % 4 == 0);
-  const int cap = (sms > 0 ? sms : 152) * 8;
-  const unsigned g = trn::grid_for(v4 ? (n / 4 + trn::kUnroll - 1) / trn::kUnroll : n, cap);
-  auto go = [&](auto kern) { kern<<<g, trn::kThreads, 0, stream>>>(x, n, k, y, codes); };
-  if (v4) {
-    if (weight) { known ? go(trn::fake_quant_kernel<true, true, 4>) : go(trn::fake_quant_kernel<true, false, 4>); }
-    else { known ? go(trn::fake_quant_kernel<false, true, 4>) : go(trn::fake_quant_kernel<false, false, 4>); }
-  } else {
-    if (weight) { known ? go(trn::fake_quant_kernel<true, true, 1>) : go(trn::fake_quant_kernel<true, false, 1>); }
-    else { known ? go(trn::fake_quant_kernel<false, true, 1>) : go(trn::fake_quant_kernel<false, false, 1>); }
-  }
+  if (sms <= 0) sms = 152;
+  const unsigned g = v4 ? trn::grid_for<4>(n, sms, sms * 8) : trn::grid_for<1>(n, sms, sms * 8);
+  const bool big = trn::stream_size(n * (4 + (y ? 4 : 0) + (codes ? 1 : 0)));
+  auto go = [&](auto w, auto kn, auto vec) {
+    if (big) trn::fake_quant_kernel<w.value, kn.value, vec.value, true><<<g, trn::kThreads, 0, stream>>>(x, n, k, y, codes);
+    else trn::fake_quant_kernel<w.value, kn.value, vec.value, false><<<g, trn::kThreads, 0, stream>>>(x, n, k, y, codes);
+  };
+  trn::dispatch(weight, known, v4, go);
   return check_launch_t("fake_quant launch", err);
 }
 
@@ -434,17 +489,16 @@ int launch_fake_quant_backward(const float* x, const float* gy, int64_t n, float
   const trn::Quant k = trn::quant_of(nu, bits);
   const bool known = trn::known_divisor(nu);
   const bool v4 = ((uintptr_t)x % 16 == 0) && ((uintptr_t)gy % 16 == 0) && ((uintptr_t)gx % 16 == 0);
-  int cap = (sms > 0 ? sms : 152) * 3;  // one wave
+  if (sms <= 0) sms = 152;
+  int cap = sms * 3;  // one wave
   if (cap > max_parts) cap = max_parts;
-  const unsigned g = trn::grid_for(v4 ? (n / 4 + trn::kUnroll - 1) / trn::kUnroll : n, cap);
-  auto go = [&](auto kern) { kern<<<g, trn::kThreads, 0, stream>>>(x, gy, n, k, gx, partial); };
-  if (v4) {
-    if (weight) { known ? go(trn::fake_quant_backward_kernel<true, true, 4>) : go(trn::fake_quant_backward_kernel<true, false, 4>); }
-    else { known ? go(trn::fake_quant_backward_kernel<false, true, 4>) : go(trn::fake_quant_backward_kernel<false, false, 4>); }
-  } else {
-    if (weight) { known ? go(trn::fake_quant_backward_kernel<true, true, 1>) : go(trn::fake_quant_backward_kernel<true, false, 1>); }
-    else { known ? go(trn::fake_quant_backward_kernel<false, true, 1>) : go(trn::fake_quant_backward_kernel<false, false, 1>); }
-  }
+  const unsigned g = v4 ? trn::grid_for<4>(n, sms, cap) : trn::grid_for<1>(n, sms, cap);
+  const bool big = trn::stream_size(n * (gx ? 12 : 8));
+  auto go = [&](auto w, auto kn, auto vec) {
+    if (big) trn::fake_quant_backward_kernel<w.value, kn.value, vec.value, true><<<g, trn::kThreads, 0, stream>>>(x, gy, n, k, gx, partial);
+    else trn::fake_quant_backward_kernel<w.value, kn.value, vec.value, false><<<g, trn::kThreads, 0, stream>>>(x, gy, n, k, gx, partial);
+  };
+  trn::dispatch(weight, known, v4, go);
   trn::sum_partials_kernel<<<1, trn::kThreads, 0, stream>>>(partial, (int)g, gnu);
   return check_launch_t("fake_quant_backward launch", err);
 }

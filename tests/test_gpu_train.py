@@ -71,6 +71,28 @@ def test_fake_quant_backward_matches_oracle(weight, bits, n):
         assert abs(got - want_gnu) <= 1e-5 * _gnu_scale(gy) + 1e-30
 
 
+# whole and partial steps of a thread's units, one and two blocks per SM, more than a grid pass; past the size from which
+# accesses are evict-first (38M values); at whole and at odd addresses
+@pytest.mark.parametrize("n", [255, 256 * 4 * 4 + 3, 256 * 8 * 2 + 1, 304 * 256 * 4 + 1, 152 * 8 * 256 * 8 + 5, 38_000_003])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("weight", [False, True])
+def test_fake_quant_steps_match_oracle(n, offset, weight):
+    rng = np.random.default_rng(n + offset)
+    nu = 0.9 if weight else 1.9
+    x, gy = (rng.standard_normal(n + 1, dtype=np.float32) for _ in range(2))
+    xd, gd = _cuda(x)[offset:offset + n], _cuda(gy)[offset:offset + n]
+    x, gy = x[offset:offset + n], gy[offset:offset + n]
+    want_y, want_c = (ot.fake_quant_weight if weight else ot.fake_quant_act)(x, nu, 4)
+    want_gx, want_gnu = (ot.fake_quant_weight_backward if weight else ot.fake_quant_act_backward)(x, gy, nu, 4)
+    y, c = aqd.fake_quant(xd, nu, 4, weight=weight)
+    gx, gnu = aqd.fake_quant_backward(xd, gd, nu, 4, weight=weight)
+    assert np.array_equal(c.cpu().numpy(), want_c)
+    assert np.array_equal(y.cpu().numpy().view(np.uint32), want_y.view(np.uint32))
+    assert np.array_equal(gx.cpu().numpy().view(np.uint32), want_gx.view(np.uint32))
+    # (float32 over runs of 16 units, 64 products: 64 * 2^-24 of their sum)
+    assert abs(float(gnu.cpu().item()) - want_gnu) <= 64 * 2.0 ** -24 * _gnu_scale(gy)
+
+
 def test_fake_quant_full_size_and_repeatable():
     """A 16x100x168x256 activation tensor (69M values): codes and values bit for bit, and the
     interval's gradient the same on a second run (fixed reduction order)."""
