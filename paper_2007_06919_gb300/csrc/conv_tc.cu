@@ -120,12 +120,12 @@ struct Params {
   uint64_t div_layer, div_nt;  // fast_div of layer_tiles and n_tiles
   int32_t acc_small;  // |acc| < 2^22 guaranteed by K * max|x| * max|w|
   int32_t cin_chunks; // cin / 128 (flat path)
-  int32_t dp_tiles;   // tiles [0, dp_tiles) are bn wide; later ones are the two bn/2 halves
+  int32_t dp_tiles;   // tiles [0, dp_tiles) are bn wide; later ones are the two bn/2 halves of the remaining
+                      // full tiles (the last, partial wave)
   int32_t tile_stride; // from one tile of a CTA (pair) to its next
-  int32_t share, extra; // contig: tiles per CTA, CTAs with one more
-  int32_t contig;     // each CTA takes one contiguous range of tiles (single CTAs, one layer,
-                      // no half tiles) instead of every gridDim-th tile
-                      // of the remaining full tiles (the last, partial wave)
+  int32_t contig;     // each CTA takes one contiguous range of tiles (single CTAs, one layer, no half tiles)
+                      // instead of every gridDim-th tile:
+  int32_t share, extra; // tiles per CTA, CTAs with one more
   // flat path: a ring of `stages` activation slabs and one of stages_b weight tiles (resident: all
   // weight tiles, loaded once)
   int32_t stages_b, resident;
@@ -1145,15 +1145,16 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
           const uint32_t un = lt * (uint32_t)nseg + (uint32_t)sg, b = un & buf_mask;
           if (!__all_sync(0xffffffffu, mbar_wait(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
           tc_fence_after();
+          // (8 columns a load: beside 64 sums, 16 spill)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if (c_lo + 16 * j >= c_hi) break;
-            uint32_t v[16];
-            tmem_ld16(lane_base() + b * (uint32_t)BN + (uint32_t)(c_lo + 16 * j), v);
+          for (int j = 0; j < 8; ++j) {
+            if (c_lo + 8 * j >= c_hi) break;
+            uint32_t v[8];
+            tmem_ld8(lane_base() + b * (uint32_t)BN + (uint32_t)(c_lo + 8 * j), v);
             tmem_wait_ld();
-            reg_fence16(v);
+            reg_fence8(v);
 #pragma unroll
-            for (int i = 0; i < 16; ++i) sum[16 * j + i] += __float2int_rn(__uint_as_float(v[i]));
+            for (int i = 0; i < 8; ++i) sum[8 * j + i] += __float2int_rn(__uint_as_float(v[i]));
           }
           tc_fence_before();
           __syncwarp();

@@ -19,8 +19,8 @@ def tables(rng, cout, std, out_bits):
     return synth.requant_params(rng, 1, cout, calib_std=std, out_bits=out_bits)
 
 
-# d at and beside the 32-bit form's limits: d + k >= 33 with k = 24 (2- to 4-bit codes), 23 (8-bit),
-# 3 (int32); from bits + 32 (codes) or 60 (int32) on the rescaled skip is 0
+# d at and beside the 32-bit rescale's limits: d + k >= 33 with k = 23 (8-bit codes) or 3 (int32); from 40 or 60 on the
+# rescaled skip is 0. (2- to 4-bit codes take a table whatever d is, within the limit of the next test.)
 @pytest.mark.parametrize("skip_bits,d_lo,d_hi", [(2, 8, 9), (2, 9, 33), (2, 34, 62), (3, 9, 36), (4, 8, 8), (4, 9, 12),
                                                  (4, 30, 40), (8, 9, 10), (8, 10, 12), (8, 30, 62), (32, 29, 33),
                                                  (32, 30, 34), (32, 55, 62)])
@@ -48,6 +48,27 @@ def test_skip_rescale_forms_bit_exact(skip_bits, d_lo, d_hi, ws, huge):
     got, want, _ = conv_pair(x, 4, wt, 4, out_bits=4, m0=m0, shift=sh, bias=b, skip=skip, skip_bits=skip_bits, skip_c=c,
                              skip_d=d, workspace=ws)
     assert_same(got, want, cout, 4, f"skip {skip_bits} bits, d {d_lo}..{d_hi}")
+
+
+# 2- to 4-bit skips: a table entry, bias + rescaled skip, at the table's limit of 2^30 and one beyond it, either sign
+@pytest.mark.parametrize("bits", [2, 3, 4])
+@pytest.mark.parametrize("over", [0, 1])
+@pytest.mark.parametrize("sign", [1, -1])
+@pytest.mark.parametrize("ws", [False, True])
+def test_skip_table_at_the_limit_bit_exact(bits, over, sign, ws):
+    rng = np.random.default_rng(bits + over)
+    n, h, w, cin, cout = 1, 9, 21, 64, 96
+    x = synth.act_codes(rng, (n, h, w, cin), 4)
+    wt = synth.weight_codes(rng, (cout, 1, 1, cin), 4)
+    skip = synth.act_codes(rng, (n, h, w, cout), bits)
+    top = (1 << bits) - 1
+    skip[0, 0, :3] = top
+    c = np.full((1, cout), sign << 20, np.int32)
+    b = np.full((1, cout), sign * ((1 << 30) + over - (top << 20)), np.int32)  # bias + top c = +-(2^30 + over)
+    got, want, _ = conv_pair(x, 4, wt, 4, pad=0, out_bits=4, m0=np.full((1, cout), I32.max, np.int32),
+                             shift=rng.integers(25, 29, size=(1, cout)).astype(np.int8), bias=b, skip=skip, skip_bits=bits,
+                             skip_c=c, skip_d=np.zeros((1, cout), np.int8), workspace=ws)
+    assert_same(got, want, cout, 4, f"{bits}-bit skip")
 
 
 # int32 skips at the 32-bit form's limit of 2^28 in magnitude: the one product of the largest multiplier that a shift of
