@@ -19,8 +19,8 @@
 // apart, 8-row groups 2560 B apart).
 //
 // Two kernels: stem_rows_kernel for stride 2 (a network's first conv), whose operand is the image
-// row itself, and stem_kernel for other strides and narrow outputs, which builds each pixel's
-// receptive field.
+// row itself, and stem_kernel for other strides, small maps and widths that leave strips of 128 columns
+// partly empty, which builds each pixel's receptive field.
 //
 // stem_kernel, per CTA (one per SM, persistent over tiles of 128 consecutive output pixels):
 //   warps 0..7   epilogue: tcgen05.ld (warp w reads TMEM lanes 32 (w % 4).., the two warps of a
@@ -787,12 +787,15 @@ int launch_stem(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   const uint32_t cst_bytes = (uint32_t)(256 * (sizeof(int4) + sizeof(EpiChan)));
   const uint32_t bar_rest = 16 + 1024;  // TMEM slot + 2 flags, alignment
   p.strips = (jb.wo + 127) / 128;
-  // Stride 2: image rows as the operand, unless the strips of 128 columns are mostly empty and there
-  // is more than one tile per SM. A tile of a strip costs 0.6 of a built one whatever its columns: 64
-  // images of 32 x 32 outputs 21.7 us against 17.1 built, of 32 x 48 21.9 / 20.9, of 64 x 64 35.2 /
-  // 37.3, 32 of 64 x 80 21.9 / 25.0, of 64 x 128 21.9 / 37.8, of 64 x 136 (two strips) 35.2 / 33.7; one
-  // image of 16 x 16 9.6 / 11.2.
-  const bool rows = a.stride == 2 && (jb.wo >= 72 * p.strips || (int64_t)jb.n * p.strips * jb.ho <= sms);
+  // Stride 2: image rows as the operand where there is more than one tile per SM and the strips of 128
+  // columns are full enough: a tile of a strip costs the same whatever its columns, 0.4 of a built tile of 128
+  // pixels with 16 channels, 0.55 with 32, 0.6, 0.75 and 0.95 with 64, 128 and 256 (the epilogue has the larger
+  // share). Rows / built in us, 4-bit or, with 16 channels, int32 outputs: 16 channels, 64 images of 32 x 48 outputs
+  // 11.3 / 13.4; 32 channels, 64 of 64 x 64 26.2 / 29.1; 64 channels, 32 of 64 x 72 20.1 / 19.2, of 64 x 80 20.3 /
+  // 20.9; 128 channels, 32 of 64 x 80 30.5 / 28.5, of 64 x 96 30.5 / 32.4; 256 channels, 32 of 64 x 96 58 / 54, of 64
+  // x 128 59 / 67. Within one tile per SM built tiles start sooner: 64 channels, one image of 100 x 128 8.4 / 7.6.
+  const int full = a.cout <= 16 ? 38 : (a.cout <= 32 ? 58 : (a.cout <= 64 ? 77 : (a.cout <= 128 ? 96 : 115)));
+  const bool rows = a.stride == 2 && jb.wo >= full * p.strips && (int64_t)jb.n * p.strips * jb.ho > sms;
   uint32_t total = 0;
   if (rows) {
     p.total_tiles = (int32_t)((int64_t)jb.n * p.strips * jb.ho);

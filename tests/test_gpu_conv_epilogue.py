@@ -286,8 +286,19 @@ def test_slabs_bit_exact(kh, kw, pad, cin, cout, bits, path):
     assert_same(got, want, cout, 4, f"{kh}x{kw} {cin}->{cout}")
 
 
-# the first conv at stride 2 (image rows as the operand): strips of 128 output columns and their edges, runs of
-# tiles that cross strips and images, more row pairs than the ring holds, images smaller than the kernel, wide padding
+# the first conv at stride 2: image rows as the operand (more than one tile per SM, strips of 128 output columns full
+# enough for the channels): strips and their edges, runs of tiles that cross strips and images, more row pairs than the ring
+# holds, images smaller than the kernel, wide padding
+@pytest.mark.parametrize("shape,pad,cout,out_bits", [((80, 5, 77), 3, 16, 32), ((200, 1, 80), 3, 16, 32), ((90, 3, 121), 6, 32, 3),
+                                                     ((24, 13, 257), 3, 32, 8), ((40, 9, 255), 3, 64, 2), ((21, 30, 307), 6, 64, 4),
+                                                     ((3, 211, 399), 0, 96, 8), ((2, 45, 1279), 3, 256, 4),
+                                                     ((1, 700, 313), 3, 48, 32), ((90, 7, 193), 2, 128, 4), ((30, 21, 151), 3, 64, 4),
+                                                     ((30, 21, 153), 3, 64, 4)])
+def test_first_conv_rows_of_many_tiles_bit_exact(shape, pad, cout, out_bits):
+    test_first_conv_rows_bit_exact(shape, pad, cout, out_bits)
+
+
+# the same at the sizes on either side of the line to built tiles, and small maps
 @pytest.mark.parametrize("shape,pad,cout,out_bits", [((1, 7, 7), 0, 16, 8), ((1, 1, 1), 3, 64, 4), ((2, 3, 5), 6, 32, 3),
                                                      ((1, 5, 259), 3, 64, 2), ((3, 61, 255), 3, 64, 4), ((1, 9, 257), 3, 96, 32),
                                                      ((2, 211, 262), 0, 48, 8), ((1, 30, 1031), 2, 256, 4),
