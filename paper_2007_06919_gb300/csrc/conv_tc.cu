@@ -1777,8 +1777,10 @@ static int launch_bits(const Params& prm, const Maps& maps, int grid, size_t sme
 bool conv_tc_uses_pair(const ConvArgs& a) {
   // every N tile width of the workspace path (BN is a multiple of 16, so each CTA's half of
   // the weight tile is whole 8-row swizzle atoms and M = 256 MMAs take N = BN), except narrow
-  // tiles on the FP4 pipe: the 256->84 output conv of the head measured 35.7 us on single
-  // CTAs against 39.4 us on pairs (same box, expansion included)
+  // tiles on the FP4 pipe. Single CTAs / pairs in us, five levels of a head, expansion included: 3x3 256 -> 84
+  // int32 at batch 1 11.3 / 11.9, 2 14.5 / 15.8, 4 21.5 / 23.3, 16 67 / 68; 3x3 256 -> 128 2-bit at batch 2 14.7 /
+  // 16.2; 1x1 256 -> 64 at batch 4 14.3 / 17.2. (Of 100 such layers pairs are ahead in three, by 5%: 3x3 to 16, 36 and
+  // 128 int32 outputs at batch 16.)
   if (a.fp4 && a.bn <= 128) return false;
   return a.ws != nullptr && a.bn >= 16 && a.bn % 16 == 0 && !a.no_pair;
 }
@@ -1950,7 +1952,10 @@ int launch_conv_tc(const ConvArgs& a, cudaStream_t stream, std::string* err) {
   int stages = 0, stages_b = 0;
   if (flat) {
     // Resident weights: every N tile's, where they leave at least 3 slabs and a third of the room. (A
-    // half-width tile takes other rows per CTA of a pair: a launch with such tiles streams.)
+    // half-width tile takes other rows per CTA of a pair: a launch with such tiles streams.) Resident / streamed
+    // in us, 4 bits, expansion included: 3x3 on eight 100 x 168 maps 64 -> 96 22.3 / 24.4, 256 -> 32 30.7 / 36.1, 512 -> 32
+    // 53 / 63; on one 25 x 42 map, where a CTA has a tile or none, 256 -> 96 9.2 / 8.8. With less room than a third
+    // for slabs, 3x3 64 -> 512 on two 50 x 84 maps, resident took 11.5 against 10.2 streamed.
     const size_t all_w = (size_t)prm.n_tiles * prm.num_kchunks * b_tile;
     prm.resident = nlayers <= 1 && prm.dp_tiles == tiles && all_w * 3 <= avail * 2 && all_w + 3 * slab <= avail;
     if (prm.resident) {

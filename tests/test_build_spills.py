@@ -1,26 +1,46 @@
-"""The tensor-core kernels that the benchmark step and the head run must compile without
-register spills (ptxas reports them by function in the build log): a spill in the tower's
-epilogue cost 46% of its time once."""
+"""Register spills, as ptxas reports them by function in the build log. The tensor-core kernels that the
+benchmark step and the head run must compile without any (a spill in the tower's epilogue cost 46%
+of its time once). The other instantiations that spill do so in the epilogue warps' per-tile code, at the
+register limit that their thread count sets; each may spill what it was measured with and no more."""
 import os
 import re
 
 import pytest
 
-LOG = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2007_06919_gb300", "_build",
-                   "conv_tc.log")
+BUILD = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2007_06919_gb300", "_build")
 
 # conv_tc_kernel<kXBits = 2, chunk in tap, workspace path, kPair, no skip, no split, 128-byte chunks, kFp4, kOStage>
 HOT = [f"conv_tc_kernelILi2ELb1ELb1ELb{pair}ELb0ELb0ELi128ELb{fp4}ELb{st}E"
        for pair in (0, 1) for fp4 in (0, 1) for st in (0, 1)]
 
+# (function, bytes of spill stores and loads it may have); anything else: none
+ALLOWED = [
+    (r"conv_tc_kernelILi[234]ELb[01]ELb0ELb0ELb1E", 20, 20),       # in-kernel unpack, with a skip
+    (r"conv_tc_kernelILi2ELb1ELb1ELb[01]ELb1E", 16, 20),           # workspace path, with a skip
+    (r"conv_tc_kernelILi8ELb1ELb1ELb[01]ELb0ELb0ELi128ELb0ELb0E", 68, 80),  # F16 pipe, codes: 64 sums a lane
+    (r"eltwise_lane_kernelILb1E", 4, 24),
+    (r"eltwise_staged_kernelILb1ELi\d+ELi[248]ELi[124]ELb1E", 28, 28),  # skips on another grid
+    (r"maxpool3s2_expand_kernelILi4E", 4, 4),
+    (r"fake_quant_backward_kernelILb[01]ELb0ELi1ELb[01]E", 8, 8),  # intervals and addresses of the rarest kind
+]
 
-def test_hot_conv_kernels_do_not_spill():
-    if not os.path.exists(LOG):
+
+def spills():
+    if not os.path.exists(os.path.join(BUILD, "conv_tc.log")):
         import __graft_entry__
         __graft_entry__.build()
-    if not os.path.exists(LOG):
+    if not os.path.exists(os.path.join(BUILD, "conv_tc.log")):
         pytest.skip("no build log")
-    text = open(LOG).read()
-    spilled = re.findall(r"spilled to local memory in function '([^']+)'", text)
-    bad = [h for h in HOT for f in spilled if h in f]
+    text = "".join(open(os.path.join(BUILD, f)).read() for f in sorted(os.listdir(BUILD)) if f.endswith(".log"))
+    return re.findall(r"spilled to local memory in function '([^']+)', (\d+) bytes spill stores, (\d+) bytes spill loads", text)
+
+
+def test_hot_conv_kernels_do_not_spill():
+    bad = [h for h in HOT for f, _, _ in spills() if h in f]
+    assert not bad, f"register spills in {bad}"
+
+
+def test_other_kernels_spill_no_more_than_measured():
+    bad = [(f, st, ld) for f, st, ld in spills()
+           if not any(re.search(p, f) and int(st) <= a and int(ld) <= b for p, a, b in ALLOWED)]
     assert not bad, f"register spills in {bad}"
