@@ -37,9 +37,9 @@ METRIC = "int-only conv TOPS & % of INT8 tensor peak; detector-head images/s at 
 # DRAM bytes (read + write) of one chained tower-layer conv_tc launch, from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum) of the build of conv_tc.cu whose SHA-256
 # prefix is recorded beside it; reported as null when the source differs from that build.
-TOWER_CONV_TRAFFIC = {"bytes": 15601920, "conv_tc_sha256": "5600194ecf4875f2",
+TOWER_CONV_TRAFFIC = {"bytes": 15579648, "conv_tc_sha256": "717a4d06e51f483c",
                       "profile": "profiles/conv_tc_retina_head_800x1333_b2_2bit_full.md (dram__bytes_read.sum "
-                                 "15.04 MB + dram__bytes_write.sum 0.57 MB, one fused tower launch)"}
+                                 "15.04 MB + dram__bytes_write.sum 0.54 MB, one fused tower launch)"}
 KTOWERS = 4  # chained 4-layer towers per timed kernel graph, each on its own workspaces
 WORKLOAD = "retina_head_800x1333_b2_2bit"
 

@@ -1143,7 +1143,8 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
 #pragma unroll 1
         for (int sg = 0; sg < nseg; ++sg) {
           const uint32_t un = lt * (uint32_t)nseg + (uint32_t)sg, b = un & buf_mask;
-          if (!__all_sync(0xffffffffu, mbar_wait(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
+          // (no call here, where 64 sums are live: 3x3 128 -> 128 on four 100 x 168 maps and below 40.4 -> 39.6 us)
+          if (!__all_sync(0xffffffffu, mbar_wait_inline(b_tfull + 8 * b, (un >> p.nbuf_log2) & 1, abort_flag))) { ok = false; break; }
           tc_fence_after();
           // (8 columns a load: beside 64 sums, 16 spill)
 #pragma unroll
@@ -1179,7 +1180,7 @@ conv_tc_kernel(const __grid_constant__ Maps maps, const __grid_constant__ Params
                                     : nullptr;
           const bool lean = kOStage ? (flags & kFlagBias) && (p.cout & 3) == 0
                                     : (flags & kFlagReq) && (out_bits != 8 || (p.cout & 31) == 0);
-          if (lean) {
+          if (__builtin_expect(lean, 1)) {
             // (|sum| < 2^28 and |bias| <= 2^30)
             uint32_t top = 0u;
 #pragma unroll

@@ -17,7 +17,8 @@ HOT = [f"conv_tc_kernelILi2ELb1ELb1ELb{pair}ELb0ELb0ELi128ELb{fp4}ELb{st}E"
 ALLOWED = [
     (r"conv_tc_kernelILi[234]ELb[01]ELb0ELb0ELb1E", 20, 20),       # in-kernel unpack, with a skip
     (r"conv_tc_kernelILi2ELb1ELb1ELb[01]ELb1E", 16, 20),           # workspace path, with a skip
-    (r"conv_tc_kernelILi8ELb1ELb1ELb[01]ELb0ELb0ELi128ELb0ELb0E", 68, 80),  # F16 pipe, codes: 64 sums a lane
+    (r"conv_tc_kernelILi8ELb1ELb1ELb1ELb0ELb0ELi128ELb0ELb0E", 40, 52),   # F16 pipe, codes: 64 sums a lane,
+    (r"conv_tc_kernelILi8ELb1ELb1ELb0ELb0ELb0ELi128ELb0ELb0E", 92, 172),  # on single CTAs (diagnostics only)
     (r"eltwise_lane_kernelILb1E", 4, 24),
     (r"eltwise_staged_kernelILb1ELi\d+ELi[248]ELi[124]ELb1E", 28, 28),  # skips on another grid
     (r"maxpool3s2_expand_kernelILi4E", 4, 4),
